@@ -184,6 +184,12 @@ wtconv_status wtconv_backward(const wtconv_desc *desc, const void *x, const void
  * Errors: NULL, the descriptor's own errors, ALIGNMENT (workspace), CUDA. */
 wtconv_status wtconv_read_status(const wtconv_desc *desc, void *workspace, int32_t *h_flag, void *stream);
 
+/* Calls that the calling host thread makes from now on report a bounded wait that runs out also by storing their tag (a
+ * non-zero number) in *h_alarm: pinned host memory that the device can write (cudaHostAlloc), owned by the caller and valid
+ * while such calls are in flight, or NULL (the default) for no report.  A host loop can then watch one word instead of
+ * enqueueing a status read per call.  Never fails. */
+wtconv_status wtconv_set_alarm(int32_t *h_alarm);
+
 /* Backward pass for callers that cannot hand over a workspace.  (The paper has no counterpart: it never
  * discusses where its kernels' scratch comes from.)
  *

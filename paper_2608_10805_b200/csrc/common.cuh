@@ -80,4 +80,15 @@ inline cudaError_t launch_overlapped(void (*kern)(P...), unsigned grid, unsigned
 // non-zero); a timeout of an earlier call leaves a different tag behind and reads as clean.
 constexpr int STATUS_TIMEOUT = 0, STATUS_LAUNCH = 1, STATUS_RESOLVED = 2;
 
+// Where the calls of this host thread report a timeout besides their status words: a word of pinned host memory the
+// caller watches (wtconv_set_alarm), or null.
+inline thread_local int *call_alarm = nullptr;
+__device__ __forceinline__ void raise_timeout(int *status, int *alarm, unsigned tag) {
+    atomicExch(status + STATUS_TIMEOUT, (int)tag);
+    if (alarm) {
+        *reinterpret_cast<volatile int *>(alarm) = (int)tag;
+        __threadfence_system();
+    }
+}
+
 }  // namespace wt

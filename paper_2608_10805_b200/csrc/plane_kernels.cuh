@@ -134,6 +134,7 @@ struct Geom {
     int nthreads, nblocks, blocks_per_sm;
     int vec;                               // 1: W % 4 == 0, rows are staged with 4-element vector loads
     int no_copy;                           // test mode: bulk copies are never issued and waits give up quickly (the timeout path)
+    int *alarm;                            // host word that hears of a timeout, or null
     unsigned tag;                          // non-zero tag of the call this launch belongs to (status words, see common.cuh)
     int taps;                              // taps per side in use: 5, or 3 for 3 x 3 kernels in the middle of 5 x 5 tables
     int bulk;                              // 1: planes are fetched ahead with cp.async.bulk into a ring of raw buffers at raw_off
@@ -594,7 +595,7 @@ __device__ __forceinline__ void start_prefetch(unsigned long long *bar, char *ra
 // copy lands in shared memory the block has already given back.
 __device__ __forceinline__ void give_up_after_timeout(unsigned long long *bar, const Geom &g, int ring, unsigned parity, int u,
                                                       int u_end, int *status) {
-    if (threadIdx.x == 0) atomicExch(status + STATUS_TIMEOUT, (int)g.tag);
+    if (threadIdx.x == 0) raise_timeout(status, g.alarm, g.tag);
     const unsigned limit = g.no_copy ? WAIT_LIMIT_TEST : WAIT_LIMIT;
     for (int s = 0; s < g.nstage && u + s < u_end; ++s) {
         mbar_wait(bar + ring, parity, limit);
@@ -1815,6 +1816,7 @@ cudaError_t forward(int B, int C, int H, int W, int L, const T *x, const float *
     if (!plan_forward(B, C, H, W, L, (int)sizeof(T), g, tune)) return cudaErrorInvalidValue;
     g.no_copy = no_copy;
     g.tag = tag;
+    g.alarm = call_alarm;
     g.taps = taps;
     return launch_fwd<T, false>(g, x, w0, s0, b0, wl, sl, out, reinterpret_cast<int *>(ws), st);
 }
@@ -1830,6 +1832,7 @@ cudaError_t backward(int B, int C, int H, int W, int L, const T *x, const T *go,
     if (plan_bwd_fused(B, C, H, W, L, (int)sizeof(T), gw, tune)) {
         gw.no_copy = no_copy;
         gw.tag = tag;
+        gw.alarm = call_alarm;
         gw.taps = taps;
         float *part0 = reinterpret_cast<float *>(ws + STATUS_BYTES);
         float *partl = part0 + (size_t)C * gw.np * (KK + 1);
@@ -1864,6 +1867,7 @@ cudaError_t backward(int B, int C, int H, int W, int L, const T *x, const T *go,
         return cudaErrorInvalidValue;
     gw.no_copy = gf.no_copy = no_copy;
     gw.tag = gf.tag = tag;
+    gw.alarm = gf.alarm = call_alarm;
     gw.taps = gf.taps = taps;
     int *status = reinterpret_cast<int *>(ws);
     float *part0 = reinterpret_cast<float *>(ws + STATUS_BYTES);

@@ -63,6 +63,7 @@ struct TGeom {
     int nteams, nthreads, nblocks, units, ngroups, np;
     int th;
     int no_copy;
+    int *alarm;                            // host word that hears of a timeout, or null
     unsigned tag;                           // non-zero tag of the call this launch belongs to (status words)
     double score;
 };
@@ -380,7 +381,7 @@ team_kernel(const __grid_constant__ TGeom g, const T *__restrict__ x, const T *_
             }
             if (team_sync_or(tw, bar_id, late)) {  // a copy never landed: record it and stop working (see the end of the kernel)
                 dead = true;
-                if (lt == 0) atomicExch(status + STATUS_TIMEOUT, (int)g.tag);
+                if (lt == 0) raise_timeout(status, g.alarm, g.tag);
                 break;
             }
             if (lt == 0 && u + NSTAGE * nteams < seg_end) {  // the ring entry is free again: fetch the unit two rounds ahead
@@ -723,6 +724,7 @@ cudaError_t forward(int B, int C, int H, int W, int L, const T *x, const float *
     if (!plan(B, C, H, W, L, (int)sizeof(T), false, g, forceG)) return cudaErrorInvalidValue;
     g.no_copy = no_copy;
     g.tag = tag;  // nothing is cleared: see the status words in common.cuh
+    g.alarm = call_alarm;
     return launch<T, false>(g, x, nullptr, w0, s0, b0, wl, sl, out, nullptr, nullptr, reinterpret_cast<int *>(ws), st);
 }
 
@@ -734,6 +736,7 @@ cudaError_t backward(int B, int C, int H, int W, int L, const T *x, const T *go,
     if (!plan(B, C, H, W, L, (int)sizeof(T), true, g, forceG)) return cudaErrorInvalidValue;
     g.no_copy = no_copy;
     g.tag = tag;
+    g.alarm = call_alarm;
     float *part0 = reinterpret_cast<float *>(ws + plane::STATUS_BYTES);
     float *partl = part0 + (size_t)C * g.np * (KK + 1);
     cudaError_t e;  // nothing is cleared: the epilogue is told which partial slots the blocks write

@@ -13,6 +13,7 @@
 
 #include <atomic>
 #include <chrono>
+#include <cstring>
 #include <mutex>
 
 namespace wt {
@@ -101,43 +102,33 @@ __global__ void resolve_status_kernel(int *status) {
 }
 
 // ------------------------------------------------------------------ dispatch
+// Which kernels serve a descriptor, and the scratch they need.  The answers come from the planners (searches of a few
+// thousand candidates behind process-wide caches of large plan structures), and one call asks many times over, so every
+// thread keeps the last few descriptors' answers in a small direct-mapped table (a lookup is some 20 ns; asking the
+// planners afresh cost a call of the smallest layer 3 us).
+struct Route {
+    wtconv_desc key;
+    bool set;
+    bool team, plane, window, k3;  // plane: any family that keeps whole planes on chip; k3: 3 x 3 kernels in 5 x 5 tables
+    size_t fwd_bytes, bwd_bytes;
+};
+const Route &route(const wtconv_desc *d);
+
 int team_force_g(const wtconv_desc *d) { return (int)((d->flags >> 16) & 63u); }  // "planes per work unit" override
 bool use_ref_chain(const wtconv_desc *d) { return (d->flags & WTCONV_FLAG_REFERENCE_CHAIN) != 0; }
-bool use_team_path(const wtconv_desc *d) {
-    if (d->flags & (WTCONV_FLAG_TILED_ONLY | WTCONV_FLAG_NO_TEAM | WTCONV_FLAG_REFERENCE_CHAIN)) return false;
-    if ((d->flags >> 8) & ~(63u << 8)) return false;  // other launch-plan overrides address the block-per-plane kernels
-    return wt::team::supported(d->B, d->C, d->H, d->W, d->k, d->L, d->dtype, team_force_g(d));
-}
-bool use_plane_path(const wtconv_desc *d) {  // any kernel family that keeps whole planes on chip (and a status word)
-    if (d->flags & (WTCONV_FLAG_TILED_ONLY | WTCONV_FLAG_REFERENCE_CHAIN)) return false;
-    return use_team_path(d) || wt::plane::supported(d->H, d->W, d->k, d->L, d->dtype);
-}
-
-// Large planes (k = 5): windows with levels 1-2 on chip, deeper levels on the whole-plane kernels over a carrier.
-bool use_window_path(const wtconv_desc *d) {
-    if (d->flags & (WTCONV_FLAG_TILED_ONLY | WTCONV_FLAG_NO_WINDOW | WTCONV_FLAG_REFERENCE_CHAIN)) return false;
-    if (d->flags >> 8) return false;
-    if (use_plane_path(d)) return false;
-    // Measured on B200: with 16-byte aligned rows the per-level tiled kernels are as fast or faster (they stream whole
-    // rows), with unaligned rows (225-wide 16-bit planes) they fall to element loads and the window kernels win.
-    if (((size_t)d->W * elem_bytes(d->dtype)) % 16 == 0 && !(d->flags & WTCONV_FLAG_PREFER_WINDOW)) return false;
-    return wt::window::supported(d->B, d->C, d->H, d->W, d->k, d->L, d->dtype);
-}
-
+bool use_team_path(const wtconv_desc *d) { return route(d).team; }
+bool use_plane_path(const wtconv_desc *d) { return route(d).plane; }
+bool use_window_path(const wtconv_desc *d) { return route(d).window; }
 // k = 3 through the k = 5 kernels.  A 3 x 3 depthwise kernel is a 5 x 5 kernel with a border of zeros, so wherever the
 // kernels that keep planes on chip (k = 5 only) serve the shape, the parameters are copied into 5 x 5 tables at the
 // head of the workspace, the k = 5 path runs on them, and the backward copies the inner 3 x 3 of the 5 x 5 weight
 // gradients out (the border's gradients are dropped; the scale and bias gradients are unaffected, since the border
 // weights are zero).  16 of 25 taps multiply zeros, and it is still 2-3 x faster than the per-level kernels.
+bool use_k3_embedding(const wtconv_desc *d) { return route(d).k3; }
 wtconv_desc as_k5(const wtconv_desc *d) {
     wtconv_desc d5 = *d;
     d5.k = 5;
     return d5;
-}
-bool use_k3_embedding(const wtconv_desc *d) {
-    if (d->k != 3 || (d->flags & (WTCONV_FLAG_TILED_ONLY | WTCONV_FLAG_REFERENCE_CHAIN))) return false;
-    const wtconv_desc d5 = as_k5(d);
-    return use_plane_path(&d5) || use_window_path(&d5);
 }
 // Workspace head of the embedding: w0 [C][25], wl [L][C][4][25], then the same two for the gradients; the k = 5
 // path's own workspace follows.
@@ -292,26 +283,71 @@ wtconv_status backward_tk(const wtconv_desc *d, const void *x, const void *g, co
         return WTCONV_ERR_DTYPE;                                                               \
     } while (0)
 
-size_t fwd_ws_bytes(const wtconv_desc *d) {
-    if (use_k3_embedding(d)) {
-        const wtconv_desc d5 = as_k5(d);
-        return embed_layout(d).inner + fwd_ws_bytes(&d5);
+size_t fwd_ws_bytes(const wtconv_desc *d) { return route(d).fwd_bytes; }
+size_t bwd_ws_bytes(const wtconv_desc *d) { return route(d).bwd_bytes; }
+
+Route find_route(const wtconv_desc *d) {
+    Route r = {};
+    r.key = *d;
+    r.set = true;
+    const int eb = (int)elem_bytes(d->dtype);
+    if (use_ref_chain(d)) {
+        const auto p = wt::refchain::make_plan(d);
+        r.fwd_bytes = p.fwd_bytes;
+        r.bwd_bytes = p.bwd_bytes;
+        return r;
     }
-    if (use_ref_chain(d)) return wt::refchain::make_plan(d).fwd_bytes;
-    if (use_plane_path(d)) return align_up(wt::plane::forward_workspace_bytes(d->B, d->C, d->H, d->W, d->L));
-    if (use_window_path(d)) return align_up(wt::window::ws_plan(d->B, d->C, d->H, d->W, d->L, (int)elem_bytes(d->dtype)).fwd_bytes);
-    return make_tiled_plan(d).fwd_bytes;
+    if (!(d->flags & WTCONV_FLAG_TILED_ONLY)) {
+        // launch-plan overrides other than the planes per unit address the block-per-plane kernels
+        if (!(d->flags & WTCONV_FLAG_NO_TEAM) && !((d->flags >> 8) & ~(63u << 8)))
+            r.team = wt::team::supported(d->B, d->C, d->H, d->W, d->k, d->L, d->dtype, team_force_g(d));
+        r.plane = r.team || wt::plane::supported(d->H, d->W, d->k, d->L, d->dtype);
+        // Large planes (k = 5): windows with levels 1-2 on chip, deeper levels on the whole-plane kernels over a carrier.
+        // Measured on B200: with 16-byte aligned rows the per-level tiled kernels are as fast or faster (they stream whole
+        // rows), with unaligned rows (225-wide 16-bit planes) they fall to element loads and the window kernels win.
+        if (!r.plane && !(d->flags & WTCONV_FLAG_NO_WINDOW) && !(d->flags >> 8) &&
+            (((size_t)d->W * eb) % 16 != 0 || (d->flags & WTCONV_FLAG_PREFER_WINDOW)))
+            r.window = wt::window::supported(d->B, d->C, d->H, d->W, d->k, d->L, d->dtype);
+    }
+    if (d->k == 3 && !(d->flags & WTCONV_FLAG_TILED_ONLY)) {
+        const wtconv_desc d5 = as_k5(d);
+        const Route r5 = route(&d5);
+        if (r5.plane || r5.window) {
+            r.k3 = true;
+            const size_t head = embed_layout(d).inner;
+            r.fwd_bytes = head + r5.fwd_bytes;
+            r.bwd_bytes = head + r5.bwd_bytes;
+            return r;
+        }
+    }
+    if (r.team) {
+        r.fwd_bytes = align_up(wt::plane::STATUS_BYTES);
+        r.bwd_bytes = align_up(wt::team::backward_workspace_bytes(d->B, d->C, d->H, d->W, d->L, eb, team_force_g(d)));
+    } else if (r.plane) {
+        r.fwd_bytes = align_up(wt::plane::forward_workspace_bytes(d->B, d->C, d->H, d->W, d->L));
+        r.bwd_bytes = align_up(wt::plane::backward_workspace_bytes(d->B, d->C, d->H, d->W, d->L, eb, d->flags >> 8));
+    } else if (r.window) {
+        const auto p = wt::window::ws_plan(d->B, d->C, d->H, d->W, d->L, eb);
+        r.fwd_bytes = align_up(p.fwd_bytes);
+        r.bwd_bytes = align_up(p.bwd_bytes);
+    } else {
+        const auto p = make_tiled_plan(d);
+        r.fwd_bytes = p.fwd_bytes;
+        r.bwd_bytes = p.bwd_bytes;
+    }
+    return r;
 }
-size_t bwd_ws_bytes(const wtconv_desc *d) {
-    if (use_k3_embedding(d)) {
-        const wtconv_desc d5 = as_k5(d);
-        return embed_layout(d).inner + bwd_ws_bytes(&d5);
+const Route &route(const wtconv_desc *d) {
+    thread_local Route table[64];
+    unsigned h = 2166136261u;
+    const unsigned v[8] = {(unsigned)d->B, (unsigned)d->C, (unsigned)d->H, (unsigned)d->W, (unsigned)d->k, (unsigned)d->L, (unsigned)d->dtype, d->flags};
+    for (unsigned x : v) h = (h ^ x) * 16777619u;
+    Route &r = table[(h ^ (h >> 15)) & 63u];
+    if (!r.set || memcmp(&r.key, d, sizeof *d) != 0) {
+        const Route found = find_route(d);  // (may look another descriptor up on the way)
+        r = found;
     }
-    if (use_ref_chain(d)) return wt::refchain::make_plan(d).bwd_bytes;
-    if (use_team_path(d)) return align_up(wt::team::backward_workspace_bytes(d->B, d->C, d->H, d->W, d->L, (int)elem_bytes(d->dtype), team_force_g(d)));
-    if (use_window_path(d)) return align_up(wt::window::ws_plan(d->B, d->C, d->H, d->W, d->L, (int)elem_bytes(d->dtype)).bwd_bytes);
-    if (use_plane_path(d)) return align_up(wt::plane::backward_workspace_bytes(d->B, d->C, d->H, d->W, d->L, (int)elem_bytes(d->dtype), d->flags >> 8));
-    return make_tiled_plan(d).bwd_bytes;
+    return r;
 }
 
 struct ParamSizes {
@@ -716,6 +752,11 @@ wtconv_status wtconv_step_host(const wtconv_desc *d, const void *h_x, const void
     d2h(h_gsl, gsl, ps.sl);
     ok = ok && cudaStreamWaitEvent(cs, out_home, 0) == cudaSuccess;  // join: the step ends when `out` is home too
     return ok ? WTCONV_OK : WTCONV_ERR_CUDA;
+}
+
+wtconv_status wtconv_set_alarm(int32_t *h_alarm) {
+    wt::call_alarm = h_alarm;
+    return WTCONV_OK;
 }
 
 wtconv_status wtconv_read_status(const wtconv_desc *d, void *workspace, int32_t *h_flag, void *stream) {

@@ -1,0 +1,236 @@
+// Native torch front end: the argument marshalling of the ctypes binding and the autograd layer in C++, so that a small
+// layer's call costs a few microseconds of host time instead of tens (a 7 x 7 layer's kernel takes about five).  Every
+// step of the operator still runs in libwtconv_b200.so through its C ABI; torch supplies memory, streams and autograd.
+#include <torch/csrc/autograd/custom_function.h>
+#include <torch/csrc/autograd/python_variable.h>
+#include <torch/csrc/Exceptions.h>
+#include <torch/torch.h>
+
+#include <c10/cuda/CUDAGuard.h>
+#include <c10/cuda/CUDAStream.h>
+#include <cuda_runtime_api.h>
+
+#include <atomic>
+
+#include "../../include/wtconv.h"
+
+namespace {
+
+PyObject *error_class = nullptr;  // WTConvError(code, message)
+
+PyObject *raise_status(int code, const char *msg) {
+    PyObject *exc = PyObject_CallFunction(error_class, "is", code, msg);
+    if (exc) {
+        PyErr_SetObject(error_class, exc);
+        Py_DECREF(exc);
+    }
+    return nullptr;
+}
+
+// One word of pinned memory per process that the layer's kernels write when a bounded wait runs out (wtconv_set_alarm).
+int32_t *alarm_word() {
+    static int32_t *word = [] {
+        void *p = nullptr;
+        TORCH_CHECK(cudaHostAlloc(&p, 64, cudaHostAllocPortable | cudaHostAllocMapped) == cudaSuccess, "cudaHostAlloc failed");
+        *static_cast<volatile int32_t *>(p) = 0;
+        return static_cast<int32_t *>(p);
+    }();
+    return word;
+}
+std::atomic<bool> layer_used{false};
+bool take_alarm() {
+    if (!layer_used.load(std::memory_order_relaxed)) return false;
+    volatile int32_t *w = alarm_word();
+    if (*w == 0) return false;
+    *w = 0;
+    return true;
+}
+struct AlarmScope {
+    AlarmScope() { wtconv_set_alarm(alarm_word()); }
+    ~AlarmScope() { wtconv_set_alarm(nullptr); }
+};
+
+// ------------------------------------------------------------------ C ABI calls on torch tensors
+struct Bad {};
+
+void *pointer(PyObject *o) {
+    if (o == Py_None) return nullptr;
+    if (!THPVariable_Check(o)) {
+        PyErr_SetString(PyExc_TypeError, "expected a tensor");
+        throw Bad{};
+    }
+    const at::Tensor &t = THPVariable_Unpack(o);
+    if (!t.is_cuda() || !t.is_contiguous()) {
+        PyErr_SetString(PyExc_ValueError, "expected contiguous CUDA tensors");
+        throw Bad{};
+    }
+    return t.data_ptr();
+}
+size_t bytes_of(PyObject *o) { return o == Py_None ? 0 : (size_t)THPVariable_Unpack(o).numel(); }
+void *stream_of(PyObject *o) {
+    if (o == Py_None) return c10::cuda::getCurrentCUDAStream().stream();
+    void *s = PyLong_AsVoidPtr(o);
+    if (PyErr_Occurred()) throw Bad{};
+    return s;
+}
+
+// forward(desc address, x, w0, s0, b0, wl, sl, out, workspace, stream) -> status
+PyObject *py_forward(PyObject *, PyObject *const *a, Py_ssize_t n) {
+    HANDLE_TH_ERRORS
+    if (n != 10) return PyErr_Format(PyExc_TypeError, "forward takes 10 arguments");
+    const wtconv_desc *d = static_cast<const wtconv_desc *>(PyLong_AsVoidPtr(a[0]));
+    void *p[8];
+    try {
+        for (int i = 0; i < 8; ++i) p[i] = pointer(a[i + 1]);
+        void *st = stream_of(a[9]);
+        return PyLong_FromLong(wtconv_forward(d, p[0], (const float *)p[1], (const float *)p[2], (const float *)p[3], (const float *)p[4],
+                                              (const float *)p[5], p[6], p[7], bytes_of(a[8]), st));
+    } catch (const Bad &) {
+        return nullptr;
+    }
+    END_HANDLE_TH_ERRORS
+}
+
+// backward(desc address, x, g, w0, s0, b0, wl, sl, gx, gw0, gs0, gb0, gwl, gsl, workspace, stream) -> status
+PyObject *py_backward(PyObject *, PyObject *const *a, Py_ssize_t n) {
+    HANDLE_TH_ERRORS
+    if (n != 16) return PyErr_Format(PyExc_TypeError, "backward takes 16 arguments");
+    const wtconv_desc *d = static_cast<const wtconv_desc *>(PyLong_AsVoidPtr(a[0]));
+    void *p[14];
+    try {
+        for (int i = 0; i < 14; ++i) p[i] = pointer(a[i + 1]);
+        void *st = stream_of(a[15]);
+        return PyLong_FromLong(wtconv_backward(d, p[0], p[1], (const float *)p[2], (const float *)p[3], (const float *)p[4], (const float *)p[5],
+                                               (const float *)p[6], p[7], (float *)p[8], (float *)p[9], (float *)p[10], (float *)p[11],
+                                               (float *)p[12], p[13], bytes_of(a[14]), st));
+    } catch (const Bad &) {
+        return nullptr;
+    }
+    END_HANDLE_TH_ERRORS
+}
+
+// ------------------------------------------------------------------ the autograd layer
+struct StatusError : std::runtime_error {
+    int code;
+    explicit StatusError(int c) : std::runtime_error(wtconv_status_string((wtconv_status)c)), code(c) {}
+};
+void check(wtconv_status s) {
+    if (s != WTCONV_OK) throw StatusError(s);
+}
+
+at::Tensor as_param(const at::Tensor &t) {
+    const at::Tensor d = t.detach();
+    return d.scalar_type() == at::kFloat && d.is_contiguous() ? d : d.to(at::kFloat).contiguous();
+}
+struct Layer {
+    wtconv_desc d;
+    at::Tensor x, w0, s0, b0, wl, sl;
+};
+Layer describe(const at::Tensor &x, const at::Tensor &w0, const at::Tensor &s0, const at::Tensor &b0, const at::Tensor &wl, const at::Tensor &sl) {
+    TORCH_CHECK(x.is_cuda(), "WTConvFunction runs on CUDA tensors only (there is no CPU path)");
+    TORCH_CHECK(x.dim() == 4, "WTConvFunction: expected an input [B, C, H, W]");
+    Layer l;
+    l.x = x.detach().contiguous();
+    const auto t = x.scalar_type();
+    TORCH_CHECK(t == at::kFloat || t == at::kHalf || t == at::kBFloat16, "WTConvFunction: float32, float16 or bfloat16 activations");
+    l.d = {(int32_t)x.size(0), (int32_t)x.size(1), (int32_t)x.size(2), (int32_t)x.size(3), (int32_t)w0.size(-1), (int32_t)wl.size(0),
+           t == at::kFloat ? WTCONV_F32 : t == at::kHalf ? WTCONV_F16 : WTCONV_BF16, 0u};
+    l.w0 = as_param(w0);
+    l.s0 = as_param(s0);
+    if (b0.defined()) l.b0 = as_param(b0);
+    l.wl = as_param(wl);
+    l.sl = as_param(sl);
+    return l;
+}
+const float *fp(const at::Tensor &t) { return t.defined() ? static_cast<const float *>(t.data_ptr()) : nullptr; }
+float *gp(const at::Tensor &t) { return t.defined() ? static_cast<float *>(t.data_ptr()) : nullptr; }
+
+at::Tensor run_forward(const Layer &l) {
+    const c10::cuda::CUDAGuard guard(l.x.device());
+    size_t fb = 0;
+    check(wtconv_workspace_bytes(&l.d, &fb, nullptr));
+    at::Tensor out = at::empty_like(l.x);
+    at::Tensor ws = at::empty({(int64_t)(fb < 256 ? 256 : fb)}, l.x.options().dtype(at::kByte));
+    AlarmScope scope;
+    layer_used.store(true, std::memory_order_relaxed);
+    check(wtconv_forward(&l.d, l.x.data_ptr(), fp(l.w0), fp(l.s0), fp(l.b0), fp(l.wl), fp(l.sl), out.data_ptr(), ws.data_ptr(),
+                         (size_t)ws.numel(), c10::cuda::getCurrentCUDAStream().stream()));
+    return out;
+}
+
+using torch::autograd::AutogradContext;
+using torch::autograd::variable_list;
+struct LayerFunction : public torch::autograd::Function<LayerFunction> {
+    static at::Tensor forward(AutogradContext *ctx, const at::Tensor &x, const at::Tensor &w0, const at::Tensor &s0,
+                              const std::optional<at::Tensor> &b0, const at::Tensor &wl, const at::Tensor &sl) {
+        const Layer l = describe(x, w0, s0, b0 ? *b0 : at::Tensor(), wl, sl);
+        at::Tensor out = run_forward(l);
+        ctx->save_for_backward({l.x, l.w0, l.s0, l.b0, l.wl, l.sl});
+        return out;
+    }
+    static variable_list backward(AutogradContext *ctx, variable_list grads) {
+        const variable_list v = ctx->get_saved_variables();
+        const Layer l = describe(v[0], v[1], v[2], v[3], v[4], v[5]);
+        const c10::cuda::CUDAGuard guard(l.x.device());
+        const at::Tensor g = grads[0].contiguous();
+        at::Tensor gx = at::empty_like(l.x), gw0 = at::empty_like(l.w0), gs0 = at::empty_like(l.s0), gwl = at::empty_like(l.wl),
+                   gsl = at::empty_like(l.sl), gb0;
+        if (l.b0.defined()) gb0 = at::empty_like(l.b0);
+        size_t bb = 0;
+        check(wtconv_workspace_bytes(&l.d, nullptr, &bb));
+        at::Tensor ws = at::empty({(int64_t)(bb < 256 ? 256 : bb)}, l.x.options().dtype(at::kByte));
+        AlarmScope scope;
+        check(wtconv_backward(&l.d, l.x.data_ptr(), g.data_ptr(), fp(l.w0), fp(l.s0), fp(l.b0), fp(l.wl), fp(l.sl), gx.data_ptr(), gp(gw0),
+                              gp(gs0), gp(gb0), gp(gwl), gp(gsl), ws.data_ptr(), (size_t)ws.numel(), c10::cuda::getCurrentCUDAStream().stream()));
+        return {gx, gw0, gs0, gb0, gwl, gsl};
+    }
+};
+
+// layer(x, w0, s0, b0, wl, sl) -> out
+PyObject *py_layer(PyObject *, PyObject *const *a, Py_ssize_t n) {
+    HANDLE_TH_ERRORS
+    if (n != 6) return PyErr_Format(PyExc_TypeError, "layer takes 6 arguments");
+    at::Tensor t[6];
+    bool grad = false;
+    for (int i = 0; i < 6; ++i) {
+        if (a[i] == Py_None && i == 3) continue;
+        if (!THPVariable_Check(a[i])) return PyErr_Format(PyExc_TypeError, "expected a tensor");
+        t[i] = THPVariable_Unpack(a[i]);
+        grad = grad || t[i].requires_grad();
+    }
+    if (take_alarm()) return raise_status(WTCONV_ERR_TIMEOUT, "a bounded device-side wait ran out in an earlier WTConv call; its outputs are not valid");
+    try {
+        if (grad && at::GradMode::is_enabled()) {
+            const std::optional<at::Tensor> b0 = t[3].defined() ? std::optional<at::Tensor>(t[3]) : std::nullopt;
+            return THPVariable_Wrap(LayerFunction::apply(t[0], t[1], t[2], b0, t[4], t[5]));
+        }
+        at::AutoDispatchBelowADInplaceOrView below;  // nothing here is recorded
+        return THPVariable_Wrap(run_forward(describe(t[0], t[1], t[2], t[3], t[4], t[5])));
+    } catch (const StatusError &e) {
+        return raise_status(e.code, e.what());
+    }
+    END_HANDLE_TH_ERRORS
+}
+
+PyObject *py_take_alarm(PyObject *, PyObject *) { return PyBool_FromLong(take_alarm()); }
+PyObject *py_used(PyObject *, PyObject *) { return PyBool_FromLong(layer_used.load()); }
+PyObject *py_set_error_class(PyObject *, PyObject *c) {
+    Py_INCREF(c);
+    Py_XDECREF(error_class);
+    error_class = c;
+    Py_RETURN_NONE;
+}
+
+PyMethodDef methods[] = {
+    {"forward", (PyCFunction)(void (*)(void))py_forward, METH_FASTCALL, "wtconv_forward on tensors"},
+    {"backward", (PyCFunction)(void (*)(void))py_backward, METH_FASTCALL, "wtconv_backward on tensors"},
+    {"layer", (PyCFunction)(void (*)(void))py_layer, METH_FASTCALL, "the layer as an autograd node"},
+    {"take_alarm", py_take_alarm, METH_NOARGS, "true if a bounded wait ran out since the last time (clears it)"},
+    {"used", py_used, METH_NOARGS, "true once a layer has run"},
+    {"set_error_class", py_set_error_class, METH_O, "the exception raised for a non-zero status"},
+    {nullptr, nullptr, 0, nullptr}};
+PyModuleDef module = {PyModuleDef_HEAD_INIT, "_wtconv_torch", nullptr, -1, methods, nullptr, nullptr, nullptr, nullptr};
+
+}  // namespace
+
+PyMODINIT_FUNC PyInit__wtconv_torch() { return PyModule_Create(&module); }

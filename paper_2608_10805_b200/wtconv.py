@@ -1,17 +1,21 @@
-"""Thin ctypes binding of libwtconv_b200.so (include/wtconv.h).
+"""Thin binding of libwtconv_b200.so (include/wtconv.h).
 
 Argument marshalling only: every step of the operator runs in the CUDA library.  Tensors
 are torch CUDA tensors (torch supplies device memory and streams); the functions below pass
-their raw pointers through the C ABI.  There is no CPU fallback: if the shared library is
-missing or fails to load, importing the symbols raises.
+their raw pointers through the C ABI.  The two calls of a training step go through the native
+marshalling of _wtconv_torch (converting fourteen arguments with ctypes costs more host time than a
+small layer's kernels take), the rest through ctypes.  There is no CPU fallback: if a shared library is
+missing or fails to load, the first use raises.
 """
 import ctypes
+import importlib.util
 import os
 
 import torch
 
 _HERE = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(_HERE, "libwtconv_b200.so")
+TORCH_EXT_PATH = os.path.join(_HERE, "_wtconv_torch.so")
 
 F32, F16, BF16 = 0, 1, 2
 FLAG_TILED_ONLY = 1
@@ -27,7 +31,7 @@ _DTYPES = {torch.float32: F32, torch.float16: F16, torch.bfloat16: BF16}
 DTYPE_NAMES = {"f32": torch.float32, "f16": torch.float16, "bf16": torch.bfloat16}
 
 EXPORTS = ["wtconv_status_string", "wtconv_level_shape", "wtconv_workspace_bytes", "wtconv_plan_name", "wtconv_plan_describe",
-           "wtconv_launch_count", "wtconv_forward", "wtconv_backward", "wtconv_read_status", "wtconv_backward_static",
+           "wtconv_launch_count", "wtconv_forward", "wtconv_backward", "wtconv_set_alarm", "wtconv_read_status", "wtconv_backward_static",
            "wtconv_step_host_workspace_bytes", "wtconv_step_host"]
 
 
@@ -65,11 +69,30 @@ def lib():
         L.wtconv_forward.argtypes = [dp] + [vp] * 7 + [vp, sz, vp]
         L.wtconv_backward.argtypes = [dp] + [vp] * 13 + [vp, sz, vp]
         L.wtconv_backward_static.argtypes = [dp] + [vp] * 13 + [vp]
+        L.wtconv_set_alarm.argtypes = [vp]
         L.wtconv_read_status.argtypes = [dp, vp, vp, vp]
         L.wtconv_step_host_workspace_bytes.argtypes = [dp, ctypes.POINTER(sz)]
         L.wtconv_step_host.argtypes = [dp] + [vp] * 14 + [vp, sz, vp]
         _lib = L
     return _lib
+
+
+_native = None
+
+
+def native():
+    """Load the native marshalling module (raises OSError if it has not been built)."""
+    global _native
+    if _native is None:
+        lib()
+        if not os.path.exists(TORCH_EXT_PATH):
+            raise OSError("%s not found: build it with `python -m paper_2608_10805_b200.build`" % TORCH_EXT_PATH)
+        spec = importlib.util.spec_from_file_location("_wtconv_torch", TORCH_EXT_PATH)
+        mod = importlib.util.module_from_spec(spec)
+        spec.loader.exec_module(mod)
+        mod.set_error_class(WTConvError)
+        _native = mod
+    return _native
 
 
 def _check(code):
@@ -129,19 +152,19 @@ def _need_cuda(*ts):
 
 def wtconv_forward(desc, x, w0, s0, b0, wl, sl, out, workspace, stream=None):
     """out <- WTConv(x) (Algorithm 1).  All tensors CUDA, contiguous; `workspace` a uint8 CUDA tensor."""
-    _need_cuda(x, w0, s0, b0, wl, sl, out, workspace)
-    _check(lib().wtconv_forward(ctypes.byref(desc), _ptr(x), _ptr(w0), _ptr(s0), _ptr(b0), _ptr(wl), _ptr(sl),
-                                _ptr(out), _ptr(workspace), workspace.numel() if workspace is not None else 0,
-                                _stream(stream)))
+    code = (_native or native()).forward(ctypes.addressof(desc), x, w0, s0, b0, wl, sl, out, workspace,
+                                         None if stream is None else stream.cuda_stream)
+    if code:
+        _check(code)
     return out
 
 
 def wtconv_backward(desc, x, grad_out, w0, s0, b0, wl, sl, grad_x, grad_w0, grad_s0, grad_b0, grad_wl, grad_sl,
                     workspace, stream=None):
-    _need_cuda(x, grad_out, w0, s0, b0, wl, sl, grad_x, grad_w0, grad_s0, grad_b0, grad_wl, grad_sl, workspace)
-    _check(lib().wtconv_backward(ctypes.byref(desc), _ptr(x), _ptr(grad_out), _ptr(w0), _ptr(s0), _ptr(b0), _ptr(wl),
-                                 _ptr(sl), _ptr(grad_x), _ptr(grad_w0), _ptr(grad_s0), _ptr(grad_b0), _ptr(grad_wl),
-                                 _ptr(grad_sl), _ptr(workspace), workspace.numel(), _stream(stream)))
+    code = (_native or native()).backward(ctypes.addressof(desc), x, grad_out, w0, s0, b0, wl, sl, grad_x, grad_w0, grad_s0,
+                                          grad_b0, grad_wl, grad_sl, workspace, None if stream is None else stream.cuda_stream)
+    if code:
+        _check(code)
 
 
 def wtconv_read_status(desc, workspace, h_flag, stream=None):

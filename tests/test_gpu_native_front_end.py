@@ -1,0 +1,52 @@
+"""The native marshalling and autograd node: argument errors, layouts that need a copy, and a timed-out call reported by the
+word of host memory that the layer watches."""
+import pytest
+import torch
+
+from paper_2608_10805_b200 import wtconv as wt
+from paper_2608_10805_b200.autograd import WTConv2d, WTConvFunction, status_watch
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("bias", [True, False])
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
+def test_strided_inputs_and_no_grad_agree_with_plain_calls(bias, dtype):
+    layer = WTConv2d(6, 5, 2, bias=bias)
+    x = torch.randn(3, 6, 12, 20, device="cuda").to(dtype)
+    ref = layer(x)
+    with torch.no_grad():
+        assert torch.equal(layer(x), ref) and not layer(x).requires_grad
+    assert torch.equal(layer(x.transpose(2, 3).contiguous().transpose(2, 3)), ref)
+    g = torch.randn_like(ref)
+    leaves = [p for p in layer.parameters()]
+    a = torch.autograd.grad(ref, leaves, g, retain_graph=True)
+    b = torch.autograd.grad(ref, leaves, g.transpose(2, 3).contiguous().transpose(2, 3))
+    assert all(torch.equal(u, v) for u, v in zip(a, b))
+
+
+def test_argument_errors():
+    layer = WTConv2d(4, 5, 1)
+    with pytest.raises(RuntimeError):
+        layer(torch.zeros(1, 4, 8, 8, dtype=torch.float64, device="cuda"))
+    with pytest.raises(TypeError):
+        WTConvFunction.apply(None, layer.w0, layer.s0, layer.b0, layer.wl, layer.sl)
+    d = wt.make_desc(1, 4, 8, 8, 5, 1, "f32")
+    x = torch.zeros(1, 4, 8, 16, device="cuda")[..., ::2]
+    with pytest.raises(ValueError):
+        wt.wtconv_forward(d, x, layer.w0, layer.s0, None, layer.wl, layer.sl, x, wt.alloc_workspace(d))
+
+
+def test_alarm_word_reports_a_timeout():
+    d = wt.make_desc(8, 12, 28, 28, 5, 2, "bf16", wt.FLAG_TEST_NO_COPY | wt.FLAG_NO_TEAM)
+    layer = WTConv2d(12, 5, 2, bias=False)
+    x = torch.randn(8, 12, 28, 28, device="cuda").to(torch.bfloat16)
+    word = torch.zeros(1, dtype=torch.int32).pin_memory()
+    wt.lib().wtconv_set_alarm(word.data_ptr())
+    with torch.no_grad():
+        wt.wtconv_forward(d, x, layer.w0.data, layer.s0.data, None, layer.wl.data, layer.sl.data, torch.empty_like(x), wt.alloc_workspace(d))
+    wt.lib().wtconv_set_alarm(None)
+    torch.cuda.synchronize()
+    assert int(word[0]) != 0
+    layer(x)  # the layer's own calls are clean
+    status_watch.drain()
