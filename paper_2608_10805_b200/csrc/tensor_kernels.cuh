@@ -1,0 +1,735 @@
+// Tensor-core kernels for 16-bit activations (k = 3, 5): the base convolution, one Haar level and its synthesis as ONE
+// convolution on tcgen05.
+//
+// Analysis, level convolution, synthesis and base convolution are all linear, so together they are a convolution whose
+// kernel depends on the output pixel's row and column parity (a, b):
+//     out[2i+a, 2j+b] = sum_{r,q < 10} M_ab[r][q] x[2i-4+r, 2j-4+q],
+//     M_ab[2u+a'][2v+b'] = 1/4 sum_sub s_sub(a,b) s_sub(a',b') W_sub[u][v]   (+ W_0[r-a-2][q-b-2] on the base taps)
+// with s_sub the Haar signs and W the folded weights (Eq. 8).  That is 100 multiply-adds a pixel instead of 50, but a
+// contraction: eight output columns x two rows of one position are 16 columns of a GEMM whose K runs over 16 window columns,
+// once per window row (ten MMAs of 128 x 48 x 16).  A 16-bit activation is an exact MMA operand; a weight is split into three
+// 16-bit parts (24 bits, the whole float), which are three groups of N columns added in fp32 afterwards.  Accumulation is
+// fp32 in tensor memory.  Scalar FMA tiles of the same work sat at 1.4 - 2.4 SM-cycles a pixel (their loads, stores,
+// butterflies and barriers included); the MMAs take 45 cycles each, 0.22 cycles a pixel at full tiles, and run beside the
+// staging and the stores of other blocks.
+//
+// Layout.  The A operand is the plane itself: shared memory holds [row][chunk of 8 columns][8 images][8 columns], so a core
+// matrix (8 rows of 16 bytes) is one chunk of eight images, the second half of K is the next chunk (128 bytes on) and the
+// sixteen groups of M are sixteen row pairs (two rows apart): neither im2col nor any copy of the window.  Planes of at most
+// 32 rows are whole items, taller ones are cut into items of 32 rows with four rows of halo; octets of items are stacked
+// above each other with four rows of zeros between them to fill the sixteen row pairs.
+//
+// Weight gradients are a contraction over positions: D[x row, x column][g row, g column] += sum over images and chunks; both
+// operands are read transposed from the same kind of array (16 x rows x 8 columns against 8 g rows x 8 columns, K = 8 images
+// x 2 groups of 8 rows).  Products of 16-bit values are exact, sums stay in tensor memory over all images a block has of a
+// channel; at the end the entries of equal offset are added in a fixed order, which gives dM, and dW follows from the formula
+// above read backwards.
+#pragma once
+#include <type_traits>
+#include "plane_kernels.cuh"
+
+namespace wt {
+namespace tensor {
+
+typedef unsigned long long u64;
+using plane::FastDiv;
+using plane::fdiv;
+using plane::make_fastdiv;
+
+constexpr int WORKERS = 256, THREADS = WORKERS + 32;  // eight staging / epilogue warps and the MMA issuer
+constexpr int TAPS = 10, NCOL = 48;                   // window rows; 3 weight parts x 2 rows x 8 columns
+constexpr int TAP_BYTES = NCOL * 16 * 2, TABLE_BYTES = TAPS * TAP_BYTES;
+constexpr int WG_COLS = 128;                          // weight-gradient accumulators: two window halves x 64
+constexpr int MAX_RING = 8;
+constexpr int SCR_PITCH = 65;                         // floats per lane of the gradient scratch
+constexpr unsigned WAIT_LIMIT = 1u << 20;
+
+struct KGeom {
+    int B, C, H, W, HW, L, K;
+    int th, nty;                 // rows per item, items per plane
+    int S, period, rows;         // octets per unit, array rows from one octet to the next, rows allocated
+    int T, n;                    // M tiles (16 row pairs) per unit, output chunks (8 columns)
+    int Pc, Px;                  // chunks per row of the convolved array and of x in the backward
+    int Ws;                      // weight gradients: groups of 16 g rows
+    int items, upc, units;       // items per channel, units per channel, units
+    int al;                      // bytes every item starts on a multiple of (2, 4, 8, 16)
+    int raw_stride, out_stride;  // bytes per item of the raw and of the output buffers
+    int conv_off, x_off, raw_off, out_off, table_off, misc_off, smem;  // byte offsets
+    int ring, cols;              // tensor-memory ring depth and columns allocated
+    int bps, nblocks, np;
+    int no_copy, bias, deep;
+    FastDiv d_period, d_nty;
+    int *alarm;
+    unsigned tag;
+    double cost;
+};
+
+// ------------------------------------------------------------------ tcgen05 helpers
+__device__ __forceinline__ u64 smem_desc(unsigned addr, unsigned lead, unsigned stride) {  // no swizzle
+    return (u64)((addr & 0x3ffffu) >> 4) | ((u64)(lead >> 4) << 16) | ((u64)(stride >> 4) << 32) | (1ull << 46);
+}
+template <typename T> __device__ __forceinline__ constexpr unsigned instr_desc(int n, bool transposed) {
+    return (1u << 4) | ((sizeof(T) == 2 && std::is_same<T, __nv_bfloat16>::value) ? (1u << 7) | (1u << 10) : 0u) |
+           (transposed ? (1u << 15) | (1u << 16) : 0u) | ((unsigned)(n >> 3) << 17) | ((128u >> 4) << 24);
+}
+__device__ __forceinline__ void mma(unsigned d, u64 a, u64 b, unsigned idesc, unsigned accumulate) {
+    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %4, 0;\n\ttcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d), "l"(a),
+                 "l"(b), "r"(idesc), "r"(accumulate)
+                 : "memory");
+}
+__device__ __forceinline__ void mma_commit(u64 *bar) {
+    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(plane::smem_addr(bar)) : "memory");
+}
+__device__ __forceinline__ void fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
+__device__ __forceinline__ void fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
+__device__ __forceinline__ void mbar_arrive(u64 *bar) {
+    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(plane::smem_addr(bar)) : "memory");
+}
+__device__ __forceinline__ void tmem_ld16(unsigned addr, float (&v)[16]) {
+    unsigned r[16];
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]), "=r"(r[9]),
+                   "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+                 : "r"(addr));
+#pragma unroll
+    for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
+}
+__device__ __forceinline__ void tmem_ld_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
+// Registers a load filled, as seen behind the wait: nothing that uses them may move above it.
+__device__ __forceinline__ void tmem_arrived(float (&v)[16]) {
+    asm volatile("" : "+f"(v[0]), "+f"(v[1]), "+f"(v[2]), "+f"(v[3]), "+f"(v[4]), "+f"(v[5]), "+f"(v[6]), "+f"(v[7]), "+f"(v[8]), "+f"(v[9]),
+                 "+f"(v[10]), "+f"(v[11]), "+f"(v[12]), "+f"(v[13]), "+f"(v[14]), "+f"(v[15]));
+}
+__device__ __forceinline__ void worker_sync() { asm volatile("bar.sync 1, 256;" ::: "memory"); }
+
+// ------------------------------------------------------------------ 16-bit packing
+__device__ __forceinline__ unsigned pack16(float a, float b, __nv_bfloat16) {
+    const __nv_bfloat162 h = __floats2bfloat162_rn(a, b);
+    return *reinterpret_cast<const unsigned *>(&h);
+}
+__device__ __forceinline__ unsigned pack16(float a, float b, __half) {
+    const __half2 h = __floats2half2_rn(a, b);
+    return *reinterpret_cast<const unsigned *>(&h);
+}
+__device__ __forceinline__ float2 unpack16(unsigned v, __nv_bfloat16) { return __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(&v)); }
+__device__ __forceinline__ float2 unpack16(unsigned v, __half) { return __half22float2(*reinterpret_cast<const __half2 *>(&v)); }
+// Part `sp` of a weight: bf16 keeps the float's exponent range, so the parts simply add up; half parts are scaled by 2^11 and
+// 2^22 (their columns are added with the inverse factors), the weight itself by the channel's power of two.
+template <typename T> __device__ __forceinline__ float weight_part(float w, int sp) {
+    constexpr bool half = std::is_same<T, __half>::value;
+    const float h0 = (float)(T)w;
+    if (sp == 0) return h0;
+    const float r1 = (w - h0) * (half ? 2048.f : 1.f), h1 = (float)(T)r1;
+    if (sp == 1) return h1;
+    return (r1 - h1) * (half ? 2048.f : 1.f);
+}
+
+// ------------------------------------------------------------------ loading
+template <int N> __device__ __forceinline__ void cp_async(void *dst, const void *src, int bytes) {
+    if (N == 16) asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(plane::smem_addr(dst)), "l"(src), "r"(bytes) : "memory");
+    else if (N == 8) asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"(plane::smem_addr(dst)), "l"(src), "r"(bytes) : "memory");
+    else asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(plane::smem_addr(dst)), "l"(src), "r"(bytes) : "memory");
+}
+struct Item {
+    int b, ty, ya, yb;   // image, item row, first row loaded, one past the last
+    size_t start;        // element index of the first loaded pixel
+    bool valid;
+};
+__device__ __forceinline__ Item find_item(const KGeom &g, int c, int k, int slot) {
+    Item it;
+    const int i = k * 8 * g.S + slot;
+    it.valid = i < g.items;
+    it.b = g.nty == 1 ? i : fdiv(i, g.d_nty);
+    it.ty = i - it.b * g.nty;
+    it.ya = it.ty * g.th - 4;
+    it.yb = it.ty * g.th + g.th + 4;
+    if (g.nty == 1 || it.ya < 0) it.ya = 0;
+    if (g.nty == 1 || it.yb > g.H) it.yb = g.H;
+    it.start = ((size_t)it.b * g.C + c) * g.HW + (size_t)it.ya * g.W;
+    return it;
+}
+// Enqueue the copies of one unit of one tensor: a warp per item, whole words of g.al bytes (rows that start on odd elements:
+// the aligned 4-byte words around the item).
+template <typename T>
+__device__ __forceinline__ void load_unit(char *raw, const KGeom &g, const T *__restrict__ src, int c, int k, int warp, int lane) {
+    const size_t total = (size_t)g.B * g.C * g.HW * 2;
+    for (int slot = warp; slot < 8 * g.S; slot += 8) {
+        const Item it = find_item(g, c, k, slot);
+        if (!it.valid) continue;
+        const size_t byte = it.start * 2, first = byte & ~(size_t)3;
+        const int bytes = (it.yb - it.ya) * g.W * 2 + (int)(byte - first);
+        const char *q = reinterpret_cast<const char *>(src) + first;
+        char *d = raw + slot * g.raw_stride;
+        if (g.al == 16)
+            for (int o = lane * 16; o < bytes; o += 512) cp_async<16>(d + o, q + o, 16);
+        else if (g.al == 8)
+            for (int o = lane * 8; o < bytes; o += 256) cp_async<8>(d + o, q + o, 8);
+        else
+            for (int o = lane * 4; o < bytes; o += 128) {
+                const size_t left = total - (first + o);
+                cp_async<4>(d + o, q + o, left < 4 ? (int)left : 4);
+            }
+    }
+}
+// Raw planes -> [row][chunk][image][8 columns].  Chunk j holds columns 8j - shift .. 8j - shift + 7 (zero outside the plane).
+// A warp takes one row of one octet: lanes = 8 images x 4 chunks, so a quarter warp stores 128 consecutive bytes.
+template <typename T, int VEC, bool SUM>
+__device__ __forceinline__ void repack(char *arr, const char *raw, const KGeom &g, int c, int k, int P, int shift, int warp, int lane, float &sum) {
+    const int img = lane & 7, cq = lane >> 3;
+    const int r0 = g.nty == 1 ? 0 : -4, nr = g.nty == 1 ? g.H : g.th + 8;
+    for (int o = 0; o < g.S; ++o) {
+        const Item it = find_item(g, c, k, o * 8 + img);
+        const T *src = reinterpret_cast<const T *>(raw + (o * 8 + img) * g.raw_stride) + (g.al < 4 ? (int)(it.start & 1) : 0);
+        for (int rr = warp; rr < nr; rr += 8) {
+            const int r = r0 + rr, y = it.ty * g.th + r;
+            const bool in = it.valid && y >= 0 && y < g.H;
+            const T *row = src + (y - it.ya) * g.W;
+            char *dst = arr + (((size_t)(o * g.period + 4 + r) * P) * 8 + img) * 16;
+            for (int j = cq; j < P; j += 4) {
+                const int x0 = 8 * j - shift;
+                unsigned v[4] = {0u, 0u, 0u, 0u};
+                if (in) {
+                    if (VEC == 4) {
+                        if (x0 >= 0 && x0 < g.W) { const uint2 t = *reinterpret_cast<const uint2 *>(row + x0); v[0] = t.x; v[1] = t.y; }
+                        if (x0 + 4 >= 0 && x0 + 4 < g.W) { const uint2 t = *reinterpret_cast<const uint2 *>(row + x0 + 4); v[2] = t.x; v[3] = t.y; }
+                    } else if (VEC == 2) {
+#pragma unroll
+                        for (int q = 0; q < 4; ++q)
+                            if (x0 + 2 * q >= 0 && x0 + 2 * q < g.W) v[q] = *reinterpret_cast<const unsigned *>(row + x0 + 2 * q);
+                    } else {
+                        const unsigned short *p = reinterpret_cast<const unsigned short *>(row);
+#pragma unroll
+                        for (int q = 0; q < 8; ++q)
+                            if (x0 + q >= 0 && x0 + q < g.W) v[q >> 1] |= (unsigned)p[x0 + q] << (16 * (q & 1));
+                    }
+                    if (SUM && r >= 0 && r < g.th) {
+#pragma unroll
+                        for (int q = 0; q < 4; ++q) {
+                            const float2 f = unpack16(v[q], T());
+                            sum += f.x + f.y;
+                        }
+                    }
+                }
+                *reinterpret_cast<uint4 *>(dst + (size_t)j * 128) = make_uint4(v[0], v[1], v[2], v[3]);
+            }
+        }
+    }
+}
+template <typename T, bool SUM>
+__device__ __forceinline__ void repack(char *arr, const char *raw, const KGeom &g, int c, int k, int P, int shift, int warp, int lane, float &sum) {
+    if ((g.W & 3) == 0) repack<T, 4, SUM>(arr, raw, g, c, k, P, shift, warp, lane, sum);
+    else if ((g.W & 1) == 0) repack<T, 2, SUM>(arr, raw, g, c, k, P, shift, warp, lane, sum);
+    else repack<T, 1, SUM>(arr, raw, g, c, k, P, shift, warp, lane, sum);
+}
+
+__device__ __forceinline__ float haar_sign(int sub, int a, int b) { return ((sub & 1) & a) ^ ((sub >> 1) & b) ? -1.f : 1.f; }
+
+// The B operand of channel c: folded weights -> M_ab -> parts.  `mis`: float scratch [128 folded | 400 M | scale at 544].
+template <typename T>
+__device__ __forceinline__ void build_table(char *table, float *mis, const KGeom &g, int c, bool flip, const float *__restrict__ w0,
+                                            const float *__restrict__ s0, const float *__restrict__ wl, const float *__restrict__ sl, int tid) {
+    const int KK = g.K * g.K, pad = (5 - g.K) / 2;
+    for (int e = tid; e < 125; e += WORKERS) {
+        const int cls = e / 25, t = e - cls * 25, tt = flip ? 24 - t : t, u = tt / 5 - pad, v = tt % 5 - pad;
+        float w = 0.f;
+        if (u >= 0 && u < g.K && v >= 0 && v < g.K) {
+            if (cls == 0) w = __ldg(w0 + (size_t)c * KK + u * g.K + v) * __ldg(s0 + c);
+            else if (g.L >= 1) w = __ldg(wl + ((size_t)c * 4 + cls - 1) * KK + u * g.K + v) * __ldg(sl + (size_t)c * 4 + cls - 1);
+        }
+        mis[e] = w;
+    }
+    worker_sync();
+    for (int e = tid; e < 400; e += WORKERS) {
+        const int ab = e / 100, rq = e - ab * 100, r = rq / 10, q = rq - r * 10, a = ab >> 1, b = ab & 1;
+        float m = 0.f;
+#pragma unroll
+        for (int sub = 0; sub < 4; ++sub)
+            m += haar_sign(sub, a, b) * haar_sign(sub, r & 1, q & 1) * mis[25 * (1 + sub) + (r >> 1) * 5 + (q >> 1)];
+        m *= 0.25f;
+        const int u = r - a - 2, v = q - b - 2;
+        if (u >= 0 && u < 5 && v >= 0 && v < 5) m += mis[u * 5 + v];
+        mis[128 + e] = m;
+    }
+    worker_sync();
+    float scale = 1.f;
+    if (std::is_same<T, __half>::value) {  // largest magnitude to [1/2, 1): no part overflows or loses bits to underflow
+        float big = 0.f;
+        for (int e = tid & 31; e < 400; e += 32) big = fmaxf(big, fabsf(mis[128 + e]));
+#pragma unroll
+        for (int o = 16; o; o >>= 1) big = fmaxf(big, __shfl_xor_sync(0xffffffffu, big, o));
+        int ex = (int)((__float_as_uint(big) >> 23) & 255u) - 126;
+        ex = ex < -100 ? -100 : ex > 120 ? 120 : ex;
+        scale = __uint_as_float((unsigned)(127 - ex) << 23);
+        if (tid == 0) mis[544] = __uint_as_float((unsigned)(127 + ex) << 23);
+    } else if (tid == 0) {
+        mis[544] = 1.f;
+    }
+    for (int e = tid; e < TAPS * 2 * NCOL; e += WORKERS) {  // 8 K entries of one column
+        const int nn = e % NCOL, rk = e / NCOL, kh = rk & 1, r = rk >> 1, sp = nn >> 4, a = (nn >> 3) & 1, oc = nn & 7;
+        const float *m = mis + 128 + (a * 2 + (oc & 1)) * 100 + r * 10;
+        unsigned v[4];
+#pragma unroll
+        for (int h = 0; h < 4; ++h) {
+            float p[2];
+#pragma unroll
+            for (int i = 0; i < 2; ++i) {
+                const int q = kh * 8 + 2 * h + i - 2 * (oc >> 1);
+                p[i] = q >= 0 && q < 10 ? weight_part<T>(m[q] * scale, sp) : 0.f;
+            }
+            v[h] = pack16(p[0], p[1], T());
+        }
+        *reinterpret_cast<uint4 *>(table + r * TAP_BYTES + (kh * (NCOL / 8) + (nn >> 3)) * 128 + (nn & 7) * 16) = make_uint4(v[0], v[1], v[2], v[3]);
+    }
+}
+
+// Eight pixels at p, `left` of them inside the row; VEC = pixels a store may cover.
+template <typename T>
+__device__ __forceinline__ void store8(T *p, const float *v, int left, int W) {
+    unsigned h[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) h[i] = pack16(v[2 * i], v[2 * i + 1], T());
+    if ((W & 7) == 0) {
+        *reinterpret_cast<uint4 *>(p) = make_uint4(h[0], h[1], h[2], h[3]);
+    } else if ((W & 3) == 0) {
+        *reinterpret_cast<uint2 *>(p) = make_uint2(h[0], h[1]);
+        if (left >= 8) *reinterpret_cast<uint2 *>(p + 4) = make_uint2(h[2], h[3]);
+    } else if ((W & 1) == 0) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+            if (2 * i < left) *reinterpret_cast<unsigned *>(p + 2 * i) = h[i];
+    } else {
+        unsigned short *q = reinterpret_cast<unsigned short *>(p);
+#pragma unroll
+        for (int i = 0; i < 8; ++i)
+            if (i < left) q[i] = (unsigned short)(h[i >> 1] >> (16 * (i & 1)));
+    }
+}
+
+// ------------------------------------------------------------------ the kernel
+// BWD = false: out = base + level 1 of x.  BWD = true: out = grad_x from go (rotated kernels) and the weight-gradient sums.
+template <typename T, bool BWD>
+__global__ void __launch_bounds__(THREADS, 2)
+tensor_kernel(const __grid_constant__ KGeom g, const T *__restrict__ x, const T *__restrict__ go, const float *__restrict__ w0,
+              const float *__restrict__ s0, const float *__restrict__ b0, const float *__restrict__ wl, const float *__restrict__ sl,
+              T *__restrict__ out, float *__restrict__ part0, float *__restrict__ partl, int *__restrict__ status) {
+    extern __shared__ __align__(128) char sb[];
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const bool worker = warp < 8;
+    char *conv = sb + g.conv_off, *xarr = sb + g.x_off, *raw = sb + g.raw_off, *table = sb + g.table_off;
+    float *mis = reinterpret_cast<float *>(sb + g.misc_off);
+    u64 *full = reinterpret_cast<u64 *>(mis + 560), *empty = full + MAX_RING, *done = empty + MAX_RING;
+    unsigned *tmem_slot = reinterpret_cast<unsigned *>(done + 1);
+    int *dead = reinterpret_cast<int *>(tmem_slot + 1);
+    const int u_begin = (int)((long long)blockIdx.x * g.units / gridDim.x), u_end = (int)((long long)(blockIdx.x + 1) * g.units / gridDim.x);
+    const unsigned limit = g.no_copy ? plane::WAIT_LIMIT_TEST : WAIT_LIMIT;
+    const int raw2 = 8 * g.S * g.raw_stride;  // bytes from x's raw planes to go's
+    {   // arrays start as zeros: halos, gaps and the rows beyond the last octet stay that way
+        uint4 *v = reinterpret_cast<uint4 *>(sb);
+        for (int i = tid; i < g.raw_off / 16; i += THREADS) v[i] = make_uint4(0u, 0u, 0u, 0u);
+    }
+    if (tid == 0) {
+        *dead = 0;
+        for (int i = 0; i < g.ring; ++i) {
+            plane::mbar_init(full + i, 1);
+            plane::mbar_init(empty + i, 4);
+        }
+        plane::mbar_init(done, 1);
+    }
+    if (warp == 8) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(plane::smem_addr(tmem_slot)), "r"(g.cols) : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+    }
+    fence_before();
+    __syncthreads();
+    fence_after();
+    const unsigned tmem = *tmem_slot;
+    const unsigned ring0 = tmem + (BWD ? WG_COLS : 0);
+    if (!BWD) dependents_may_start();
+    wait_for_predecessor();  // shared and tensor memory only up to here
+    if (blockIdx.x == 0 && tid == 0) status[STATUS_LAUNCH] = (int)g.tag;
+    int c = u_begin / g.upc, k = u_begin - c * g.upc, c_prev = -1;
+    const int jobs = g.T * g.n;
+    unsigned job0 = 0, unit = 0;  // jobs issued before this unit, units done
+    float gsum = 0.f;
+    auto fetch = [&](int cc, int kk) {
+        load_unit<T>(raw, g, x, cc, kk, warp, lane);
+        if (BWD) load_unit<T>(raw + raw2, g, go, cc, kk, warp, lane);
+    };
+    if (worker && u_begin < u_end) fetch(c, k);
+    for (int u = u_begin; u < u_end; ++u, ++unit, job0 += jobs) {
+        int cn = c, kn = k + 1;
+        if (kn == g.upc) { kn = 0; ++cn; }
+        if (worker) {
+            if (c != c_prev) {  // the MMAs that read the old table have completed (see the wait at the end of a unit)
+                build_table<T>(table, mis, g, c, BWD, w0, s0, wl, sl, tid);
+                if (tid == 0) mis[545] = !BWD && b0 ? __ldg(s0 + c) * __ldg(b0 + c) : 0.f;
+            }
+            asm volatile("cp.async.wait_all;" ::: "memory");
+        }
+        __syncthreads();  // the unit's raw planes have landed for everybody
+        if (worker) {
+            if (BWD) {
+                float none = 0.f;
+                if (g.bias) repack<T, true>(conv, raw + raw2, g, c, k, g.Pc, 4, warp, lane, gsum);
+                else repack<T, false>(conv, raw + raw2, g, c, k, g.Pc, 4, warp, lane, none);
+                repack<T, false>(xarr, raw, g, c, k, g.Px, 8, warp, lane, none);
+            } else {
+                float none = 0.f;
+                repack<T, false>(conv, raw, g, c, k, g.Pc, 4, warp, lane, none);
+            }
+            plane::fence_async_smem();
+        }
+        __syncthreads();
+        if (!worker) {
+            if (lane == 0 && !g.no_copy) {
+                fence_after();
+                const unsigned a0 = plane::smem_addr(conv);
+                const u64 b0d = smem_desc(plane::smem_addr(table), (NCOL / 8) * 128, 128);
+                const unsigned rowb = (unsigned)g.Pc * 128;
+                constexpr unsigned id = instr_desc<T>(NCOL, false);
+                int q = 0;
+                for (int t = 0; t < g.T; ++t)
+                    for (int j = 0; j < g.n; ++j, ++q) {
+                        const unsigned jc = job0 + q, s = jc % (unsigned)g.ring;
+                        if (!*reinterpret_cast<volatile int *>(dead) && !plane::mbar_wait(empty + s, ((jc / (unsigned)g.ring) & 1u) ^ 1u, limit))
+                            *reinterpret_cast<volatile int *>(dead) = 1;
+                        fence_after();
+                        const u64 ad = smem_desc(a0 + (unsigned)(32 * t) * rowb + (unsigned)j * 128, 128, 2 * rowb);
+#pragma unroll
+                        for (int r = 0; r < TAPS; ++r) mma(ring0 + s * NCOL, ad + (u64)(r * (rowb >> 4)), b0d + (u64)(r * (TAP_BYTES >> 4)), id, r > 0);
+                        mma_commit(full + s);
+                    }
+                if (BWD) {
+                    const unsigned xrow = (unsigned)g.Px * 128;
+                    const u64 xd = smem_desc(plane::smem_addr(xarr), 8 * xrow, xrow), gd = smem_desc(a0 + 4 * rowb, 8 * rowb, rowb);
+                    constexpr unsigned idw = instr_desc<T>(64, true);
+                    unsigned acc = c == c_prev;
+                    for (int w = 0; w < g.Ws; ++w) {
+                        // cut planes: only the item's own rows count, not its halo
+                        const unsigned row = g.nty == 1 ? 16 * w : (w >> 1) * g.period + (w & 1) * 16;
+                        for (int j = 0; j < g.Pc; ++j) {
+                            const u64 xa = xd + (u64)((row * xrow + (unsigned)j * 128) >> 4), gb = gd + (u64)((row * rowb + (unsigned)j * 128) >> 4);
+                            mma(tmem, xa, gb, idw, acc);
+                            mma(tmem + 64, xa + 8, gb, idw, acc);
+                            acc = 1;
+                        }
+                    }
+                }
+                mma_commit(done);
+            }
+        } else {
+            if (u + 1 < u_end) fetch(cn, kn);
+            // ---- epilogue: warps 0-3 take the even jobs, 4-7 the odd ones; a lane is one image of one row pair
+            const int m = (warp & 3) * 32 + lane, img = m & 7;
+            const float scale = mis[544], bias = mis[545];
+            for (int q = warp >> 2; q < jobs; q += 2) {
+                const int t = q / g.n, j = q - t * g.n;
+                const unsigned jc = job0 + q, s = jc % (unsigned)g.ring;
+                if (!*reinterpret_cast<volatile int *>(dead) && !plane::mbar_wait(full + s, (jc / (unsigned)g.ring) & 1u, limit)) {
+                    *reinterpret_cast<volatile int *>(dead) = 1;
+                    raise_timeout(status, g.alarm, g.tag);
+                }
+                __syncwarp();
+                fence_after();
+                float v[16], p1[16], p2[16];
+                const unsigned addr = ring0 + s * NCOL + ((unsigned)(warp & 3) << 21);
+                tmem_ld16(addr, v);
+                tmem_ld16(addr + 16, p1);
+                tmem_ld16(addr + 32, p2);
+                tmem_ld_wait();
+                tmem_arrived(v);
+                tmem_arrived(p1);
+                tmem_arrived(p2);
+                fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(empty + s);
+                const int row2 = 2 * (16 * t + (m >> 3)), o = fdiv(row2, g.d_period), r = row2 - o * g.period;
+                if (o >= g.S || r >= g.th) continue;
+                const Item it = find_item(g, c, k, o * 8 + img);
+                const int y = it.ty * g.th + r;
+                if (!it.valid || y >= g.H) continue;
+#pragma unroll
+                for (int i = 0; i < 16; ++i) {
+                    if (std::is_same<T, __half>::value) v[i] = fmaf(scale, fmaf(p2[i], 1.f / 4194304.f, fmaf(p1[i], 1.f / 2048.f, v[i])), bias);
+                    else v[i] = (v[i] + (p1[i] + p2[i])) + bias;
+                }
+                T *d = reinterpret_cast<T *>(sb + g.out_off + (o * 8 + img) * g.out_stride) + r * g.W + 8 * j;
+                store8<T>(d, v, g.W - 8 * j, g.W);
+                if (y + 1 < g.H) store8<T>(d + g.W, v + 8, g.W - 8 * j, g.W);
+            }
+            worker_sync();
+            // ---- the finished items to global memory, a warp per item
+            for (int slot = warp; slot < 8 * g.S; slot += 8) {
+                const Item it = find_item(g, c, k, slot);
+                if (!it.valid) continue;
+                const int y0 = it.ty * g.th, nrow = g.H - y0 < g.th ? g.H - y0 : g.th, bytes = nrow * g.W * 2;
+                const char *s = sb + g.out_off + slot * g.out_stride;
+                char *d = reinterpret_cast<char *>(out + ((size_t)it.b * g.C + c) * g.HW + (size_t)y0 * g.W);
+                if (g.al == 16)
+                    for (int e = lane * 16; e < bytes; e += 512) *reinterpret_cast<uint4 *>(d + e) = *reinterpret_cast<const uint4 *>(s + e);
+                else if (g.al == 8)
+                    for (int e = lane * 8; e < bytes; e += 256) *reinterpret_cast<uint2 *>(d + e) = *reinterpret_cast<const uint2 *>(s + e);
+                else if (g.al == 4)
+                    for (int e = lane * 4; e < bytes; e += 128) *reinterpret_cast<unsigned *>(d + e) = *reinterpret_cast<const unsigned *>(s + e);
+                else
+                    for (int e = lane * 2; e < bytes; e += 64) *reinterpret_cast<unsigned short *>(d + e) = *reinterpret_cast<const unsigned short *>(s + e);
+            }
+            // every MMA of the unit has completed: its arrays and (on a channel change) its table may be rewritten
+            if (!*reinterpret_cast<volatile int *>(dead) && !plane::mbar_wait(done, unit & 1u, limit)) {
+                *reinterpret_cast<volatile int *>(dead) = 1;
+                raise_timeout(status, g.alarm, g.tag);
+            }
+            if (BWD && (u + 1 == u_end || cn != c)) {
+                // ---- flush: accumulators to shared memory (the arrays are idle), entries of equal offset added in a fixed order
+                fence_after();
+                worker_sync();
+                float *scr = reinterpret_cast<float *>(sb);
+#pragma unroll 1
+                for (int half = 0; half < 2; ++half) {
+                    if (warp >> 2 == 0) {
+#pragma unroll 1
+                        for (int e = 0; e < 64; e += 16) {
+                            float v[16];
+                            tmem_ld16(tmem + half * 64 + e + ((unsigned)(warp & 3) << 21), v);
+                            tmem_ld_wait();
+                            tmem_arrived(v);
+#pragma unroll
+                            for (int i = 0; i < 16; ++i) scr[m * SCR_PITCH + e + i] = v[i];
+                        }
+                    }
+                    worker_sync();
+                    for (int e = tid; e < 400; e += WORKERS) {
+                        const int ab = e / 100, rq = e - ab * 100, r = rq / 10, qq = rq - r * 10;
+                        float sum = half ? mis[128 + e] : 0.f;
+#pragma unroll
+                        for (int gp = 0; gp < 4; ++gp)
+#pragma unroll
+                            for (int gq = 0; gq < 4; ++gq) {
+                                const int xc = qq + 2 * gq - 8 * half;
+                                if (xc >= 0 && xc < 8) sum += scr[((r + 2 * gp) * 8 + xc) * SCR_PITCH + (2 * gp + (ab >> 1)) * 8 + 2 * gq + (ab & 1)];
+                            }
+                        mis[128 + e] = sum;
+                    }
+                    worker_sync();
+                }
+                if (g.bias) {
+#pragma unroll
+                    for (int s = 16; s; s >>= 1) gsum += __shfl_xor_sync(0xffffffffu, gsum, s);
+                    if (lane == 0) mis[528 + warp] = gsum;
+                    gsum = 0.f;
+                }
+                worker_sync();
+                const int slotp = blockIdx.x - block_of_unit((long long)c * g.upc, gridDim.x, g.units);
+                const int KK = g.K * g.K, pad = (5 - g.K) / 2;
+                for (int e = tid; e < KK + 1 + (g.L >= 1 ? 4 * KK : 0); e += WORKERS) {
+                    const float *G = mis + 128;
+                    float sum = 0.f;
+                    if (e < KK) {
+                        const int uu = e / g.K + pad, vv = e % g.K + pad;
+#pragma unroll
+                        for (int ab = 0; ab < 4; ++ab) sum += G[ab * 100 + ((ab >> 1) + 2 + uu) * 10 + (ab & 1) + 2 + vv];
+                    } else if (e == KK) {
+                        if (g.bias)
+                            for (int w = 0; w < 8; ++w) sum += mis[528 + w];
+                    } else {
+                        const int sub = (e - KK - 1) / KK, t = (e - KK - 1) - sub * KK, uu = t / g.K + pad, vv = t % g.K + pad;
+                        for (int ab = 0; ab < 4; ++ab)
+                            for (int pq = 0; pq < 4; ++pq)
+                                sum += haar_sign(sub, ab >> 1, ab & 1) * haar_sign(sub, pq >> 1, pq & 1) * G[ab * 100 + (2 * uu + (pq >> 1)) * 10 + 2 * vv + (pq & 1)];
+                        sum *= 0.25f;
+                    }
+                    if (e <= KK) part0[((size_t)c * g.np + slotp) * (KK + 1) + e] = sum;
+                    else partl[((size_t)c * g.np + slotp) * 4 * KK + e - KK - 1] = sum;
+                }
+                fence_before();
+                uint4 *z = reinterpret_cast<uint4 *>(sb);  // the arrays' zeros are back before anybody stages
+                for (int i = tid; i < (128 * SCR_PITCH * 4 + 15) / 16; i += WORKERS) z[i] = make_uint4(0u, 0u, 0u, 0u);
+                worker_sync();
+            }
+        }
+        c_prev = c;
+        c = cn;
+        k = kn;
+    }
+    if (BWD) dependents_may_start();
+    fence_before();
+    __syncthreads();
+    if (warp == 8) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(g.cols));
+}
+
+// ------------------------------------------------------------------ host side
+struct Request {
+    int bwd, B, C, H, W, L, K;
+    bool operator==(const Request &o) const { return bwd == o.bwd && B == o.B && C == o.C && H == o.H && W == o.W && L == o.L && K == o.K; }
+};
+inline int up(int v, int m) { return (v + m - 1) / m * m; }
+
+inline bool search(const Request &q, KGeom &best) {
+    if ((q.K != 3 && q.K != 5) || q.L > 1 || q.W > 64 || q.H > 256 || q.H < 2 || q.W < 2) return false;
+    best = KGeom{};
+    best.cost = 1e30;
+    bool found = false;
+    KGeom g = {};
+    g.B = q.B; g.C = q.C; g.H = q.H; g.W = q.W; g.HW = q.H * q.W; g.L = q.L; g.K = q.K;
+    g.n = (q.W + 7) / 8;
+    g.Pc = g.n + 1;
+    g.Px = g.n + 2;
+    // taller planes: 32 rows an item (a multiple of 16, so that the rows the weight gradients sum over are the item's own)
+    g.nty = q.H <= 32 ? 1 : (q.H + 31) / 32;
+    g.th = g.nty == 1 ? up(q.H, 2) : 32;
+    g.period = g.th + (g.nty == 1 ? 4 : 8);
+    g.items = q.B * g.nty;
+    g.d_nty = make_fastdiv(g.nty);
+    g.d_period = make_fastdiv(g.period);
+    const long long st = g.nty == 1 ? (long long)g.HW * 2 : q.W * 8;  // every item starts on a multiple of this
+    const long long hw = (long long)g.HW * 2;
+    g.al = st % 16 == 0 && hw % 16 == 0 ? 16 : st % 8 == 0 && hw % 8 == 0 ? 8 : st % 4 == 0 && hw % 4 == 0 ? 4 : 2;
+    const int load_rows = g.nty == 1 ? q.H : g.th + 8, out_rows = g.nty == 1 ? q.H : g.th;
+    g.raw_stride = up(load_rows * q.W * 2 + 4, 128) + 16;  // items fall on different banks
+    g.out_stride = up(out_rows * q.W * 2, 128) + 16;
+    const int sides = q.bwd ? 2 : 1;
+    for (int S = 1; S <= 16; ++S) {
+        if (S > 1 && 8 * (S - 1) >= g.items) break;
+        KGeom h = g;
+        h.S = S;
+        const int used = (S - 1) * h.period + h.th;
+        h.T = (used + 31) / 32;
+        h.Ws = h.nty == 1 ? (used + 15) / 16 : 2 * S;
+        h.rows = 32 * h.T + 8;
+        if (h.rows < 16 * h.Ws + 16) h.rows = 16 * h.Ws + 16;
+        int off = 0;
+        h.conv_off = off; off += h.rows * h.Pc * 128;
+        h.x_off = off; if (q.bwd) off += h.rows * h.Px * 128;
+        if (q.bwd && off < 128 * SCR_PITCH * 4) off = up(128 * SCR_PITCH * 4, 128);
+        h.raw_off = off; off += sides * 8 * S * h.raw_stride;
+        h.out_off = off; off += 8 * S * h.out_stride;
+        off = up(off, 128);
+        h.table_off = off; off += TABLE_BYTES;
+        h.misc_off = off; off += 560 * 4 + (2 * MAX_RING + 1) * 8 + 16;
+        h.smem = up(off, 128);
+        if (h.smem > plane::SMEM_LIMIT) break;
+        h.upc = (h.items + 8 * S - 1) / (8 * S);
+        if ((long long)h.upc * q.C > 0x3fffffffLL) continue;
+        h.units = h.upc * q.C;
+        for (int bps = 1; bps <= 2; ++bps) {  // 112 registers a thread
+            if ((long long)bps * (h.smem + 1024) > plane::SMEM_PER_SM) break;
+            h.cols = 512 / bps;
+            h.ring = (h.cols - (q.bwd ? WG_COLS : 0)) / NCOL;
+            if (h.ring > MAX_RING) h.ring = MAX_RING;
+            h.bps = bps;
+            h.nblocks = plane::NUM_SMS * bps < h.units ? plane::NUM_SMS * bps : h.units;
+            // cycles: MMAs serialise over an SM's blocks; the workers' part and the hand-overs do not
+            const double tensor = (double)h.T * h.n * TAPS * 46 + (q.bwd ? (double)h.Ws * h.Pc * 2 * 50 : 0);
+            const double around = 3500.0 + 6.0 * S * (q.bwd ? 2.2 : 1.0) * load_rows * h.Pc + 0.25 * tensor;
+            const int active = (h.nblocks + plane::NUM_SMS - 1) / plane::NUM_SMS;
+            const int rounds = (h.units + h.nblocks - 1) / h.nblocks;
+            const double serial = tensor + around, per = active * tensor > serial ? active * tensor : serial;
+            const double switches = 1.0 + (double)q.C / h.nblocks;
+            const double cost = rounds * per + switches * (2500.0 + (q.bwd ? 5000.0 : 0.0));
+            if (cost < best.cost) {
+                best = h;
+                best.cost = cost;
+                found = true;
+            }
+        }
+    }
+    if (!found) return false;
+    best.np = 1;
+    for (int ch = 0; ch < best.C; ++ch) {
+        const int n = block_of_unit((long long)(ch + 1) * best.upc - 1, best.nblocks, best.units) - block_of_unit((long long)ch * best.upc, best.nblocks, best.units) + 1;
+        if (n > best.np) best.np = n;
+    }
+    return true;
+}
+
+struct Entry {
+    Request q;
+    bool ok;
+    KGeom g;
+};
+inline bool plan(const Request &q, KGeom &out) {  // searched once and kept (bounded)
+    static std::mutex mu;
+    static std::vector<Entry> cache;
+    {
+        std::lock_guard<std::mutex> lock(mu);
+        for (const Entry &e : cache)
+            if (e.q == q) {
+                if (e.ok) out = e.g;
+                return e.ok;
+            }
+    }
+    Entry e = {};
+    e.q = q;
+    e.ok = search(q, e.g);
+    {
+        std::lock_guard<std::mutex> lock(mu);
+        if (cache.size() >= 256) cache.clear();
+        cache.push_back(e);
+    }
+    if (e.ok) out = e.g;
+    return e.ok;
+}
+
+constexpr size_t STATUS_BYTES = 256;
+inline size_t backward_bytes(const Request &q) {
+    KGeom g;
+    if (!plan(q, g)) return 0;
+    const size_t KK = (size_t)q.K * q.K;
+    return STATUS_BYTES + sizeof(float) * (size_t)g.C * g.np * (KK + 1 + 4 * KK);
+}
+
+template <typename T>
+cudaError_t forward(const Request &q, const T *x, const float *w0, const float *s0, const float *b0, const float *wl, const float *sl, T *out,
+                    char *ws, cudaStream_t st, unsigned tag, bool no_copy) {
+    KGeom g;
+    if (!plan(q, g)) return cudaErrorInvalidValue;
+    g.tag = tag;
+    g.alarm = call_alarm;
+    g.no_copy = no_copy;
+    constexpr auto kern = tensor_kernel<T, false>;
+    const cudaError_t e = plane::opt_in_smem<kern>();
+    if (e != cudaSuccess) return e;
+    return launch_overlapped(kern, (unsigned)g.nblocks, (unsigned)THREADS, (size_t)g.smem, st, g, x, nullptr, w0, s0, b0, wl, sl, out, nullptr,
+                             nullptr, reinterpret_cast<int *>(ws));
+}
+
+template <typename T>
+cudaError_t backward(const Request &q, const T *x, const T *go, const float *w0, const float *s0, const float *wl, const float *sl, bool bias,
+                     T *gx, char *ws, EpiloguePtrs *ep, cudaStream_t st, unsigned tag, bool no_copy) {
+    KGeom g;
+    if (!plan(q, g)) return cudaErrorInvalidValue;
+    g.tag = tag;
+    g.alarm = call_alarm;
+    g.no_copy = no_copy;
+    g.bias = bias;
+    const size_t KK = (size_t)q.K * q.K;
+    float *part0 = reinterpret_cast<float *>(ws + STATUS_BYTES), *partl = part0 + (size_t)g.C * g.np * (KK + 1);
+    constexpr auto kern = tensor_kernel<T, true>;
+    cudaError_t e = plane::opt_in_smem<kern>();
+    if (e != cudaSuccess) return e;
+    e = launch_overlapped(kern, (unsigned)g.nblocks, (unsigned)THREADS, (size_t)g.smem, st, g, x, go, w0, s0, nullptr, wl, sl, gx, part0, partl,
+                          reinterpret_cast<int *>(ws));
+    if (e != cudaSuccess) return e;
+    ep->part0 = part0;
+    ep->np0 = g.np;
+    ep->partl[0] = partl;
+    ep->npl[0] = g.np;
+    ep->grp = 1; ep->B = g.upc; ep->units = g.units; ep->nblocks = g.nblocks;
+    return cudaSuccess;
+}
+
+inline int describe(const Request &q, char *buf, size_t n) {
+    KGeom g;
+    if (!plan(q, g)) return 0;
+    const int o = snprintf(buf, n, "%s[tensor S=%d T=%d n=%d bps=%d ring=%d np=%d smem=%d]", q.bwd ? "bwd" : "fwd", g.S, g.T, g.n, g.bps, g.ring, g.np, g.smem);
+    return o < 0 ? 0 : o;
+}
+
+#define WT_TENSOR_INSTANTIATE(T, EXTERN)                                                                                       \
+    EXTERN template cudaError_t forward<T>(const Request &, const T *, const float *, const float *, const float *, const float *, \
+                                           const float *, T *, char *, cudaStream_t, unsigned, bool);                           \
+    EXTERN template cudaError_t backward<T>(const Request &, const T *, const T *, const float *, const float *, const float *,    \
+                                            const float *, bool, T *, char *, EpiloguePtrs *, cudaStream_t, unsigned, bool);
+
+}  // namespace tensor
+}  // namespace wt

@@ -6,6 +6,7 @@
 #include "common.cuh"
 #include "tiled_kernels.cuh"
 #include "plane_kernels.cuh"
+#include "tensor_kernels.cuh"
 #include "team_kernels.cuh"
 #include "window_kernels.cuh"
 #include "tiled_host.cuh"
@@ -22,6 +23,10 @@ WT_PLANE_INSTANTIATE(float, extern)
 WT_PLANE_INSTANTIATE(__half, extern)
 WT_PLANE_INSTANTIATE(__nv_bfloat16, extern)
 }  // namespace plane
+namespace tensor {
+WT_TENSOR_INSTANTIATE(__half, extern)
+WT_TENSOR_INSTANTIATE(__nv_bfloat16, extern)
+}  // namespace tensor
 namespace team {
 WT_TEAM_INSTANTIATE(float, extern)
 WT_TEAM_INSTANTIATE(__half, extern)
@@ -109,7 +114,7 @@ __global__ void resolve_status_kernel(int *status) {
 struct Route {
     wtconv_desc key;
     bool set;
-    bool team, plane, window, k3;  // plane: any family that keeps whole planes on chip; k3: 3 x 3 kernels in 5 x 5 tables
+    bool team, plane, window, tensor, k3;  // plane: any family that keeps whole planes on chip; k3: 3 x 3 kernels in 5 x 5 tables
     size_t fwd_bytes, bwd_bytes;
 };
 const Route &route(const wtconv_desc *d);
@@ -119,6 +124,8 @@ bool use_ref_chain(const wtconv_desc *d) { return (d->flags & WTCONV_FLAG_REFERE
 bool use_team_path(const wtconv_desc *d) { return route(d).team; }
 bool use_plane_path(const wtconv_desc *d) { return route(d).plane; }
 bool use_window_path(const wtconv_desc *d) { return route(d).window; }
+bool use_tensor_path(const wtconv_desc *d) { return route(d).tensor; }
+wt::tensor::Request tensor_request(const wtconv_desc *d, int bwd) { return {bwd, d->B, d->C, d->H, d->W, d->L, d->k}; }
 // k = 3 through the k = 5 kernels.  A 3 x 3 depthwise kernel is a 5 x 5 kernel with a border of zeros, so wherever the
 // kernels that keep planes on chip (k = 5 only) serve the shape, the parameters are copied into 5 x 5 tables at the
 // head of the workspace, the k = 5 path runs on them, and the backward copies the inner 3 x 3 of the 5 x 5 weight
@@ -176,6 +183,14 @@ template <typename T, int K>
 wtconv_status forward_tk(const wtconv_desc *d, const void *x, const float *w0, const float *s0, const float *b0,
                          const float *wl, const float *sl, void *out, char *ws, cudaStream_t st, int taps = 5) {
     if (use_ref_chain(d)) return wt::refchain::forward<T, K>(d, (const T *)x, w0, s0, b0, wl, sl, (T *)out, ws, st);
+    if constexpr (K != 7 && sizeof(T) == 2) {
+        if (taps == 5 && use_tensor_path(d))
+            return wt::tensor::forward<T>(tensor_request(d, 0), (const T *)x, w0, s0, b0, wl, sl, (T *)out,
+                                          ws + (use_k3_embedding(d) ? embed_layout(d).inner : 0), st, next_status_tag(),
+                                          (d->flags & WTCONV_FLAG_TEST_NO_COPY) != 0) == cudaSuccess
+                       ? WTCONV_OK
+                       : WTCONV_ERR_CUDA;
+    }
     if constexpr (K == 3) {
         if (use_k3_embedding(d)) {
             const wtconv_desc d5 = as_k5(d);
@@ -220,6 +235,16 @@ wtconv_status backward_tk(const wtconv_desc *d, const void *x, const void *g, co
     if (use_ref_chain(d))
         return wt::refchain::backward<T, K>(d, (const T *)x, (const T *)g, w0, s0, b0, wl, sl, (T *)gx, gw0, gs0, gb0, gwl, gsl,
                                             ws, st);
+    if constexpr (K != 7 && sizeof(T) == 2) {
+        if (taps == 5 && use_tensor_path(d)) {
+            wt::EpiloguePtrs ep = {};
+            if (wt::tensor::backward<T>(tensor_request(d, 1), (const T *)x, (const T *)g, w0, s0, wl, sl, b0 != nullptr, (T *)gx,
+                                        ws + (use_k3_embedding(d) ? embed_layout(d).inner : 0), &ep, st, next_status_tag(),
+                                        (d->flags & WTCONV_FLAG_TEST_NO_COPY) != 0) != cudaSuccess)
+                return WTCONV_ERR_CUDA;
+            return launch_epilogue(d, ep, w0, s0, b0, wl, sl, gw0, gs0, gb0, gwl, gsl, st);
+        }
+    }
     if constexpr (K == 3) {
         if (use_k3_embedding(d)) {
             const wtconv_desc d5 = as_k5(d);
@@ -286,6 +311,12 @@ wtconv_status backward_tk(const wtconv_desc *d, const void *x, const void *g, co
 size_t fwd_ws_bytes(const wtconv_desc *d) { return route(d).fwd_bytes; }
 size_t bwd_ws_bytes(const wtconv_desc *d) { return route(d).bwd_bytes; }
 
+bool tensor_serves(const wtconv_desc *d, bool on_chip) {
+    if (d->dtype == WTCONV_F32 || !on_chip || (d->flags & ~WTCONV_FLAG_TEST_NO_COPY)) return false;
+    wt::tensor::KGeom g;
+    return wt::tensor::plan(tensor_request(d, 0), g) && wt::tensor::plan(tensor_request(d, 1), g);
+}
+
 Route find_route(const wtconv_desc *d) {
     Route r = {};
     r.key = *d;
@@ -315,12 +346,18 @@ Route find_route(const wtconv_desc *d) {
         if (r5.plane || r5.window) {
             r.k3 = true;
             const size_t head = embed_layout(d).inner;
+            r.tensor = tensor_serves(d, r5.plane);
+            const size_t own = r.tensor ? align_up(wt::tensor::backward_bytes(tensor_request(d, 1))) : 0;
             r.fwd_bytes = head + r5.fwd_bytes;
-            r.bwd_bytes = head + r5.bwd_bytes;
+            r.bwd_bytes = head + (own > r5.bwd_bytes ? own : r5.bwd_bytes);
             return r;
         }
     }
-    if (r.team) {
+    r.tensor = d->k == 5 && tensor_serves(d, r.plane);
+    if (r.tensor) {
+        r.fwd_bytes = align_up(wt::tensor::STATUS_BYTES);
+        r.bwd_bytes = align_up(wt::tensor::backward_bytes(tensor_request(d, 1)));
+    } else if (r.team) {
         r.fwd_bytes = align_up(wt::plane::STATUS_BYTES);
         r.bwd_bytes = align_up(wt::team::backward_workspace_bytes(d->B, d->C, d->H, d->W, d->L, eb, team_force_g(d)));
     } else if (r.plane) {
@@ -487,6 +524,16 @@ wtconv_status wtconv_plan_describe(const wtconv_desc *d, char *buf, size_t n) {
     if (st != WTCONV_OK) return st;
     if (!buf || n == 0) return WTCONV_ERR_NULL;
     buf[0] = 0;
+    if (use_tensor_path(d)) {  // the family's name as callers know it, then the plans that run
+        size_t o = (size_t)snprintf(buf, n, "%s%s ", use_k3_embedding(d) ? "3x3 kernels in 5x5 tables: " : "", wtconv_plan_name(d));
+        if (o < n) o += (size_t)wt::tensor::describe(tensor_request(d, 0), buf + o, n - o);
+        if (o + 1 < n) {
+            buf[o++] = ' ';
+            buf[o] = 0;
+            wt::tensor::describe(tensor_request(d, 1), buf + o, n - o);
+        }
+        return WTCONV_OK;
+    }
     if (use_k3_embedding(d)) {
         const wtconv_desc d5 = as_k5(d);
         const int o = snprintf(buf, n, "3x3 kernels in 5x5 tables: ");
@@ -539,7 +586,7 @@ wtconv_status wtconv_launch_count(const wtconv_desc *d, int32_t *fwd, int32_t *b
         if (bwd) {
             wt::plane::Geom gq;
             /* fused backward + epilogue, or weight-gradient + input-gradient + epilogue (and nothing else on the stream) */
-            *bwd = wt::plane::plan_bwd_fused(d->B, d->C, d->H, d->W, d->L, (int)elem_bytes(d->dtype), gq, d->flags >> 8) ? 2 : 3;
+            *bwd = use_tensor_path(d) || wt::plane::plan_bwd_fused(d->B, d->C, d->H, d->W, d->L, (int)elem_bytes(d->dtype), gq, d->flags >> 8) ? 2 : 3;
         }
     } else {
         if (fwd) *fwd = d->L + 1;
