@@ -52,13 +52,12 @@ struct KGeom {
     int Pc, Px;                  // chunks per row of the convolved array and of x in the backward
     int Ws;                      // weight gradients: groups of 16 g rows
     int items, upc, units;       // items per channel, units per channel, units
-    int al;                      // bytes every item starts on a multiple of (2, 4, 8, 16)
     int raw_stride, out_stride;  // bytes per item of the raw and of the output buffers
-    int conv_off, x_off, raw_off, out_off, table_off, misc_off, smem;  // byte offsets
+    int conv_off, x_off, parts_off, raw_off, out_off, table_off, misc_off, smem;  // byte offsets
     int ring, cols;              // tensor-memory ring depth and columns allocated
     int bps, nblocks, np;
     int no_copy, bias, deep;
-    FastDiv d_period, d_nty;
+    FastDiv d_period, d_nty, d_n, d_Pc, d_Px, d_ec, d_ex;  // d_ec / d_ex: chunks of one octet in the convolved / the x array
     int *alarm;
     unsigned tag;
     double cost;
@@ -100,6 +99,11 @@ __device__ __forceinline__ void tmem_arrived(float (&v)[16]) {
     asm volatile("" : "+f"(v[0]), "+f"(v[1]), "+f"(v[2]), "+f"(v[3]), "+f"(v[4]), "+f"(v[5]), "+f"(v[6]), "+f"(v[7]), "+f"(v[8]), "+f"(v[9]),
                  "+f"(v[10]), "+f"(v[11]), "+f"(v[12]), "+f"(v[13]), "+f"(v[14]), "+f"(v[15]));
 }
+__device__ __forceinline__ unsigned elect_one() {
+    unsigned p;
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(p));
+    return p;
+}
 __device__ __forceinline__ void worker_sync() { asm volatile("bar.sync 1, 256;" ::: "memory"); }
 
 // ------------------------------------------------------------------ 16-bit packing
@@ -125,119 +129,143 @@ template <typename T> __device__ __forceinline__ float weight_part(float w, int 
 }
 
 // ------------------------------------------------------------------ loading
-template <int N> __device__ __forceinline__ void cp_async(void *dst, const void *src, int bytes) {
-    if (N == 16) asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(plane::smem_addr(dst)), "l"(src), "r"(bytes) : "memory");
-    else if (N == 8) asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"(plane::smem_addr(dst)), "l"(src), "r"(bytes) : "memory");
-    else asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(plane::smem_addr(dst)), "l"(src), "r"(bytes) : "memory");
-}
-struct Item {
-    int b, ty, ya, yb;   // image, item row, first row loaded, one past the last
-    size_t start;        // element index of the first loaded pixel
-    bool valid;
+// An item of a unit, worked out once by the warp that fetches it.
+struct __align__(16) Item {
+    u64 start;  // element index of its first loaded pixel
+    int ty;     // item row, or -1: no such item
+    int ya;     // first row loaded
 };
-__device__ __forceinline__ Item find_item(const KGeom &g, int c, int k, int slot) {
-    Item it;
-    const int i = k * 8 * g.S + slot;
-    it.valid = i < g.items;
-    it.b = g.nty == 1 ? i : fdiv(i, g.d_nty);
-    it.ty = i - it.b * g.nty;
-    it.ya = it.ty * g.th - 4;
-    it.yb = it.ty * g.th + g.th + 4;
-    if (g.nty == 1 || it.ya < 0) it.ya = 0;
-    if (g.nty == 1 || it.yb > g.H) it.yb = g.H;
-    it.start = ((size_t)it.b * g.C + c) * g.HW + (size_t)it.ya * g.W;
-    return it;
-}
-// Enqueue the copies of one unit of one tensor: a warp per item, whole words of g.al bytes (rows that start on odd elements:
-// the aligned 4-byte words around the item).
-template <typename T>
-__device__ __forceinline__ void load_unit(char *raw, const KGeom &g, const T *__restrict__ src, int c, int k, int warp, int lane) {
-    const size_t total = (size_t)g.B * g.C * g.HW * 2;
-    for (int slot = warp; slot < 8 * g.S; slot += 8) {
-        const Item it = find_item(g, c, k, slot);
-        if (!it.valid) continue;
-        const size_t byte = it.start * 2, first = byte & ~(size_t)3;
-        const int bytes = (it.yb - it.ya) * g.W * 2 + (int)(byte - first);
-        const char *q = reinterpret_cast<const char *>(src) + first;
-        char *d = raw + slot * g.raw_stride;
-        if (g.al == 16)
-            for (int o = lane * 16; o < bytes; o += 512) cp_async<16>(d + o, q + o, 16);
-        else if (g.al == 8)
-            for (int o = lane * 8; o < bytes; o += 256) cp_async<8>(d + o, q + o, 8);
-        else
-            for (int o = lane * 4; o < bytes; o += 128) {
-                const size_t left = total - (first + o);
-                cp_async<4>(d + o, q + o, left < 4 ? (int)left : 4);
+// Bulk copies of one unit (one warp, a lane per item): the aligned 16-byte words around each item, so planes may start at any
+// element; repack() skips the bytes before the first pixel.
+template <typename T, bool BWD>
+__device__ __forceinline__ void fetch_unit(Item *items, char *raw, int raw2, u64 *bar, const KGeom &g, const T *__restrict__ x, const T *__restrict__ go,
+                                           int c, int k, int lane) {
+    const u64 total = (u64)g.B * g.C * g.HW * 2;
+    unsigned bytes_all = 0;
+    plane::fence_async_smem();
+#pragma unroll 1
+    for (int pass = 0; pass < 2; ++pass) {
+        for (int s0 = 0; s0 < 8 * g.S; s0 += 32) {
+            const int slot = s0 + lane, i = k * 8 * g.S + slot;
+            if (slot >= 8 * g.S) continue;
+            Item it;
+            it.ty = -1;
+            it.ya = 0;
+            it.start = 0;
+            if (i < g.items) {
+                const int b = g.nty == 1 ? i : fdiv(i, g.d_nty);
+                it.ty = i - b * g.nty;
+                int yb = g.H;
+                if (g.nty > 1) {
+                    it.ya = it.ty * g.th - 4 < 0 ? 0 : it.ty * g.th - 4;
+                    yb = it.ty * g.th + g.th + 4 > g.H ? g.H : it.ty * g.th + g.th + 4;
+                }
+                it.start = ((u64)b * g.C + c) * g.HW + (u64)(it.ya * g.W);
+                const u64 first = it.start * 2 & ~15ull, last = it.start * 2 + (unsigned)((yb - it.ya) * g.W * 2);
+                u64 end = (last + 15) & ~15ull;
+                const bool tail = end > total;
+                if (tail) end -= 16;
+                const unsigned n = (unsigned)(end - first);
+                if (pass == 0) {
+                    bytes_all += n;
+                } else {
+                    char *d = raw + slot * g.raw_stride;
+                    if (n) {
+                        plane::bulk_g2s(d, reinterpret_cast<const char *>(x) + first, n, bar);
+                        if (BWD) plane::bulk_g2s(d + raw2, reinterpret_cast<const char *>(go) + first, n, bar);
+                    }
+                    if (tail)  // the tensor ends inside a 16-byte word
+                        for (u64 o = end; o < last; o += 2) {
+                            *reinterpret_cast<T *>(d + (o - first)) = x[o / 2];
+                            if (BWD) *reinterpret_cast<T *>(d + raw2 + (o - first)) = go[o / 2];
+                        }
+                }
             }
+            if (pass == 0) items[slot] = it;
+        }
+        if (pass == 0) {
+#pragma unroll
+            for (int o = 16; o; o >>= 1) bytes_all += __shfl_xor_sync(0xffffffffu, bytes_all, o);
+            if (g.no_copy) return;  // test mode: the barrier is never armed, nothing is in flight
+            if (lane == 0) plane::mbar_expect_tx(bar, BWD ? 2 * bytes_all : bytes_all);
+            __syncwarp();
+        }
     }
 }
 // Raw planes -> [row][chunk][image][8 columns].  Chunk j holds columns 8j - shift .. 8j - shift + 7 (zero outside the plane).
-// A warp takes one row of one octet: lanes = 8 images x 4 chunks, so a quarter warp stores 128 consecutive bytes.
+// Eight lanes are the eight images of one chunk (a quarter warp stores 128 consecutive bytes); U chunks a thread in flight.
 template <typename T, int VEC, bool SUM>
-__device__ __forceinline__ void repack(char *arr, const char *raw, const KGeom &g, int c, int k, int P, int shift, int warp, int lane, float &sum) {
-    const int img = lane & 7, cq = lane >> 3;
-    const int r0 = g.nty == 1 ? 0 : -4, nr = g.nty == 1 ? g.H : g.th + 8;
-    for (int o = 0; o < g.S; ++o) {
-        const Item it = find_item(g, c, k, o * 8 + img);
-        const T *src = reinterpret_cast<const T *>(raw + (o * 8 + img) * g.raw_stride) + (g.al < 4 ? (int)(it.start & 1) : 0);
-        for (int rr = warp; rr < nr; rr += 8) {
-            const int r = r0 + rr, y = it.ty * g.th + r;
-            const bool in = it.valid && y >= 0 && y < g.H;
-            const T *row = src + (y - it.ya) * g.W;
-            char *dst = arr + (((size_t)(o * g.period + 4 + r) * P) * 8 + img) * 16;
-            for (int j = cq; j < P; j += 4) {
-                const int x0 = 8 * j - shift;
-                unsigned v[4] = {0u, 0u, 0u, 0u};
-                if (in) {
+__device__ __forceinline__ void repack(char *arr, const char *raw, const Item *items, const KGeom &g, int P, const FastDiv &dP, const FastDiv &dE,
+                                       int shift, int warp, int lane, float &sum) {
+    constexpr int U = VEC == 1 ? 2 : 4;
+    const int img = lane & 7, per = (int)dE.d, n = g.S * per, r0 = g.nty == 1 ? 0 : -4;
+    for (int e0 = warp * 4 + (lane >> 3); e0 < n; e0 += U * 32) {
+        unsigned v[U][4];
+        int dst[U];
+#pragma unroll
+        for (int i = 0; i < U; ++i) {
+            const int e = e0 + i * 32;
+            v[i][0] = v[i][1] = v[i][2] = v[i][3] = 0u;
+            dst[i] = -1;
+            if (e < n) {
+                const int o = fdiv(e, dE), ee = e - o * per, rr = fdiv(ee, dP), j = ee - rr * P, r = r0 + rr, x0 = 8 * j - shift;
+                const Item it = items[o * 8 + img];
+                dst[i] = (((o * g.period + 4 + r0) * P + ee) * 8 + img) * 16;
+                const int y = it.ty * g.th + r;
+                if (it.ty >= 0 && y >= 0 && y < g.H) {
+                    const T *row = reinterpret_cast<const T *>(raw + (o * 8 + img) * g.raw_stride + ((int)it.start & 7) * 2) + (y - it.ya) * g.W + x0;
                     if (VEC == 4) {
-                        if (x0 >= 0 && x0 < g.W) { const uint2 t = *reinterpret_cast<const uint2 *>(row + x0); v[0] = t.x; v[1] = t.y; }
-                        if (x0 + 4 >= 0 && x0 + 4 < g.W) { const uint2 t = *reinterpret_cast<const uint2 *>(row + x0 + 4); v[2] = t.x; v[3] = t.y; }
+                        if (x0 >= 0 && x0 < g.W) { const uint2 t = *reinterpret_cast<const uint2 *>(row); v[i][0] = t.x; v[i][1] = t.y; }
+                        if (x0 + 4 >= 0 && x0 + 4 < g.W) { const uint2 t = *reinterpret_cast<const uint2 *>(row + 4); v[i][2] = t.x; v[i][3] = t.y; }
                     } else if (VEC == 2) {
 #pragma unroll
                         for (int q = 0; q < 4; ++q)
-                            if (x0 + 2 * q >= 0 && x0 + 2 * q < g.W) v[q] = *reinterpret_cast<const unsigned *>(row + x0 + 2 * q);
+                            if (x0 + 2 * q >= 0 && x0 + 2 * q < g.W) v[i][q] = *reinterpret_cast<const unsigned *>(row + 2 * q);
                     } else {
                         const unsigned short *p = reinterpret_cast<const unsigned short *>(row);
 #pragma unroll
                         for (int q = 0; q < 8; ++q)
-                            if (x0 + q >= 0 && x0 + q < g.W) v[q >> 1] |= (unsigned)p[x0 + q] << (16 * (q & 1));
+                            if (x0 + q >= 0 && x0 + q < g.W) v[i][q >> 1] |= (unsigned)p[q] << (16 * (q & 1));
                     }
                     if (SUM && r >= 0 && r < g.th) {
 #pragma unroll
                         for (int q = 0; q < 4; ++q) {
-                            const float2 f = unpack16(v[q], T());
+                            const float2 f = unpack16(v[i][q], T());
                             sum += f.x + f.y;
                         }
                     }
                 }
-                *reinterpret_cast<uint4 *>(dst + (size_t)j * 128) = make_uint4(v[0], v[1], v[2], v[3]);
             }
         }
+#pragma unroll
+        for (int i = 0; i < U; ++i)
+            if (dst[i] >= 0) *reinterpret_cast<uint4 *>(arr + dst[i]) = make_uint4(v[i][0], v[i][1], v[i][2], v[i][3]);
     }
 }
 template <typename T, bool SUM>
-__device__ __forceinline__ void repack(char *arr, const char *raw, const KGeom &g, int c, int k, int P, int shift, int warp, int lane, float &sum) {
-    if ((g.W & 3) == 0) repack<T, 4, SUM>(arr, raw, g, c, k, P, shift, warp, lane, sum);
-    else if ((g.W & 1) == 0) repack<T, 2, SUM>(arr, raw, g, c, k, P, shift, warp, lane, sum);
-    else repack<T, 1, SUM>(arr, raw, g, c, k, P, shift, warp, lane, sum);
+__device__ __forceinline__ void repack(char *arr, const char *raw, const Item *items, const KGeom &g, int P, const FastDiv &dP, const FastDiv &dE,
+                                       int shift, int warp, int lane, float &sum) {
+    if ((g.W & 3) == 0) repack<T, 4, SUM>(arr, raw, items, g, P, dP, dE, shift, warp, lane, sum);
+    else if ((g.W & 1) == 0) repack<T, 2, SUM>(arr, raw, items, g, P, dP, dE, shift, warp, lane, sum);
+    else repack<T, 1, SUM>(arr, raw, items, g, P, dP, dE, shift, warp, lane, sum);
 }
 
 __device__ __forceinline__ float haar_sign(int sub, int a, int b) { return ((sub & 1) & a) ^ ((sub >> 1) & b) ? -1.f : 1.f; }
 
-// The B operand of channel c: folded weights -> M_ab -> parts.  `mis`: float scratch [128 folded | 400 M | scale at 544].
-template <typename T>
-__device__ __forceinline__ void build_table(char *table, float *mis, const KGeom &g, int c, bool flip, const float *__restrict__ w0,
-                                            const float *__restrict__ s0, const float *__restrict__ wl, const float *__restrict__ sl, int tid) {
+// One folded weight (Eq. 8) of channel c: classes base, LL, LH, HL, HH x 25 taps (3 x 3 kernels sit in the middle of 5 x 5).
+__device__ __forceinline__ float folded_weight(const KGeom &g, int c, int e, bool flip, const float *__restrict__ w0, const float *__restrict__ s0,
+                                               const float *__restrict__ wl, const float *__restrict__ sl) {
     const int KK = g.K * g.K, pad = (5 - g.K) / 2;
-    for (int e = tid; e < 125; e += WORKERS) {
-        const int cls = e / 25, t = e - cls * 25, tt = flip ? 24 - t : t, u = tt / 5 - pad, v = tt % 5 - pad;
-        float w = 0.f;
-        if (u >= 0 && u < g.K && v >= 0 && v < g.K) {
-            if (cls == 0) w = __ldg(w0 + (size_t)c * KK + u * g.K + v) * __ldg(s0 + c);
-            else if (g.L >= 1) w = __ldg(wl + ((size_t)c * 4 + cls - 1) * KK + u * g.K + v) * __ldg(sl + (size_t)c * 4 + cls - 1);
-        }
-        mis[e] = w;
-    }
+    const int cls = e / 25, t = e - cls * 25, tt = flip ? 24 - t : t, u = tt / 5 - pad, v = tt % 5 - pad;
+    if (u < 0 || u >= g.K || v < 0 || v >= g.K) return 0.f;
+    if (cls == 0) return __ldg(w0 + (size_t)c * KK + u * g.K + v) * __ldg(s0 + c);
+    return g.L >= 1 ? __ldg(wl + ((size_t)c * 4 + cls - 1) * KK + u * g.K + v) * __ldg(sl + (size_t)c * 4 + cls - 1) : 0.f;
+}
+// The B operand: folded weights (already in mis[0..124]) -> M_ab -> parts -> Toeplitz columns.  `parts`: [part][ab][r] rows of
+// 24 16-bit values, q = -6 .. 17, zero outside 0 .. 9, so that eight K entries of a column are four words of a row.
+// mis: [128 folded | 400 M | ... | 544 scale].
+template <typename T>
+__device__ __forceinline__ void build_table(char *table, char *parts, float *mis, int tid) {
     worker_sync();
     for (int e = tid; e < 400; e += WORKERS) {
         const int ab = e / 100, rq = e - ab * 100, r = rq / 10, q = rq - r * 10, a = ab >> 1, b = ab & 1;
@@ -250,9 +278,9 @@ __device__ __forceinline__ void build_table(char *table, float *mis, const KGeom
         if (u >= 0 && u < 5 && v >= 0 && v < 5) m += mis[u * 5 + v];
         mis[128 + e] = m;
     }
-    worker_sync();
     float scale = 1.f;
     if (std::is_same<T, __half>::value) {  // largest magnitude to [1/2, 1): no part overflows or loses bits to underflow
+        worker_sync();
         float big = 0.f;
         for (int e = tid & 31; e < 400; e += 32) big = fmaxf(big, fabsf(mis[128 + e]));
 #pragma unroll
@@ -264,21 +292,17 @@ __device__ __forceinline__ void build_table(char *table, float *mis, const KGeom
     } else if (tid == 0) {
         mis[544] = 1.f;
     }
+    for (int e = tid; e < 400; e += WORKERS) {
+        const int row = e / 10, q = e - row * 10;
+        const float m = mis[128 + e] * scale;
+#pragma unroll
+        for (int sp = 0; sp < 3; ++sp) reinterpret_cast<T *>(parts)[(sp * 40 + row) * 24 + 6 + q] = (T)weight_part<T>(m, sp);
+    }
+    worker_sync();
     for (int e = tid; e < TAPS * 2 * NCOL; e += WORKERS) {  // 8 K entries of one column
         const int nn = e % NCOL, rk = e / NCOL, kh = rk & 1, r = rk >> 1, sp = nn >> 4, a = (nn >> 3) & 1, oc = nn & 7;
-        const float *m = mis + 128 + (a * 2 + (oc & 1)) * 100 + r * 10;
-        unsigned v[4];
-#pragma unroll
-        for (int h = 0; h < 4; ++h) {
-            float p[2];
-#pragma unroll
-            for (int i = 0; i < 2; ++i) {
-                const int q = kh * 8 + 2 * h + i - 2 * (oc >> 1);
-                p[i] = q >= 0 && q < 10 ? weight_part<T>(m[q] * scale, sp) : 0.f;
-            }
-            v[h] = pack16(p[0], p[1], T());
-        }
-        *reinterpret_cast<uint4 *>(table + r * TAP_BYTES + (kh * (NCOL / 8) + (nn >> 3)) * 128 + (nn & 7) * 16) = make_uint4(v[0], v[1], v[2], v[3]);
+        const unsigned *p = reinterpret_cast<const unsigned *>(parts + ((sp * 40 + (a * 2 + (oc & 1)) * 10 + r) * 24 + 6 + kh * 8 - 2 * (oc >> 1)) * 2);
+        *reinterpret_cast<uint4 *>(table + r * TAP_BYTES + (kh * (NCOL / 8) + (nn >> 3)) * 128 + (nn & 7) * 16) = make_uint4(p[0], p[1], p[2], p[3]);
     }
 }
 
@@ -313,16 +337,18 @@ tensor_kernel(const __grid_constant__ KGeom g, const T *__restrict__ x, const T 
               const float *__restrict__ s0, const float *__restrict__ b0, const float *__restrict__ wl, const float *__restrict__ sl,
               T *__restrict__ out, float *__restrict__ part0, float *__restrict__ partl, int *__restrict__ status) {
     extern __shared__ __align__(128) char sb[];
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
     const bool worker = warp < 8;
     char *conv = sb + g.conv_off, *xarr = sb + g.x_off, *raw = sb + g.raw_off, *table = sb + g.table_off;
     float *mis = reinterpret_cast<float *>(sb + g.misc_off);
-    u64 *full = reinterpret_cast<u64 *>(mis + 560), *empty = full + MAX_RING, *done = empty + MAX_RING;
-    unsigned *tmem_slot = reinterpret_cast<unsigned *>(done + 1);
-    int *dead = reinterpret_cast<int *>(tmem_slot + 1);
+    u64 *full = reinterpret_cast<u64 *>(mis + 560), *empty = full + MAX_RING, *done = empty + MAX_RING, *landed = done + 1;
+    volatile int *dead = reinterpret_cast<volatile int *>(landed + 1);
+    unsigned *tmem_slot = reinterpret_cast<unsigned *>(landed + 1) + 1;
+    Item *items = reinterpret_cast<Item *>(mis + 600);  // two sets: a unit is fetched while the one before it is worked on
+    const int nslot = 8 * g.S;
     const int u_begin = (int)((long long)blockIdx.x * g.units / gridDim.x), u_end = (int)((long long)(blockIdx.x + 1) * g.units / gridDim.x);
     const unsigned limit = g.no_copy ? plane::WAIT_LIMIT_TEST : WAIT_LIMIT;
-    const int raw2 = 8 * g.S * g.raw_stride;  // bytes from x's raw planes to go's
+    const int raw2 = nslot * g.raw_stride;  // bytes from x's raw planes to go's
     {   // arrays start as zeros: halos, gaps and the rows beyond the last octet stay that way
         uint4 *v = reinterpret_cast<uint4 *>(sb);
         for (int i = tid; i < g.raw_off / 16; i += THREADS) v[i] = make_uint4(0u, 0u, 0u, 0u);
@@ -334,6 +360,7 @@ tensor_kernel(const __grid_constant__ KGeom g, const T *__restrict__ x, const T 
             plane::mbar_init(empty + i, 4);
         }
         plane::mbar_init(done, 1);
+        plane::mbar_init(landed, 1);
     }
     if (warp == 8) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(plane::smem_addr(tmem_slot)), "r"(g.cols) : "memory");
@@ -342,62 +369,78 @@ tensor_kernel(const __grid_constant__ KGeom g, const T *__restrict__ x, const T 
     fence_before();
     __syncthreads();
     fence_after();
-    const unsigned tmem = *tmem_slot;
+    const unsigned tmem = __shfl_sync(0xffffffffu, *tmem_slot, 0);
     const unsigned ring0 = tmem + (BWD ? WG_COLS : 0);
+    auto wait_for = [&](u64 *bar, unsigned parity) {  // bounded; a wait that runs out is recorded and ends all waiting
+        if (!*dead && !plane::mbar_wait(bar, parity, limit)) {
+            *dead = 1;
+            raise_timeout(status, g.alarm, g.tag);
+        }
+    };
     if (!BWD) dependents_may_start();
     wait_for_predecessor();  // shared and tensor memory only up to here
     if (blockIdx.x == 0 && tid == 0) status[STATUS_LAUNCH] = (int)g.tag;
     int c = u_begin / g.upc, k = u_begin - c * g.upc, c_prev = -1;
     const int jobs = g.T * g.n;
     unsigned job0 = 0, unit = 0;  // jobs issued before this unit, units done
-    float gsum = 0.f;
-    auto fetch = [&](int cc, int kk) {
-        load_unit<T>(raw, g, x, cc, kk, warp, lane);
-        if (BWD) load_unit<T>(raw + raw2, g, go, cc, kk, warp, lane);
+    float gsum = 0.f, wreg = 0.f, breg = 0.f;
+    auto fetch_weights = [&](int cc) {  // ahead of the channel that needs them
+        if (tid < 125) wreg = folded_weight(g, cc, tid, BWD, w0, s0, wl, sl);
+        if (tid == 0) breg = !BWD && b0 ? __ldg(s0 + cc) * __ldg(b0 + cc) : 0.f;
     };
-    if (worker && u_begin < u_end) fetch(c, k);
+    if (worker && u_begin < u_end) {
+        if (warp == 7) fetch_unit<T, BWD>(items, raw, raw2, landed, g, x, go, c, k, lane);
+        fetch_weights(c);
+    }
     for (int u = u_begin; u < u_end; ++u, ++unit, job0 += jobs) {
         int cn = c, kn = k + 1;
         if (kn == g.upc) { kn = 0; ++cn; }
+        const Item *it_u = items + (unit & 1u) * nslot;
         if (worker) {
             if (c != c_prev) {  // the MMAs that read the old table have completed (see the wait at the end of a unit)
-                build_table<T>(table, mis, g, c, BWD, w0, s0, wl, sl, tid);
-                if (tid == 0) mis[545] = !BWD && b0 ? __ldg(s0 + c) * __ldg(b0 + c) : 0.f;
+                if (tid < 125) mis[tid] = wreg;
+                if (tid == 0) mis[545] = breg;
+                build_table<T>(table, sb + g.parts_off, mis, tid);
             }
-            asm volatile("cp.async.wait_all;" ::: "memory");
+            wait_for(landed, unit & 1u);
+            plane::bulk_store_wait_read();  // the output image may be written again behind the next barriers
         }
-        __syncthreads();  // the unit's raw planes have landed for everybody
+        __syncthreads();  // the item list (and what its fetcher copied by hand) is visible
         if (worker) {
+            float none = 0.f;
             if (BWD) {
-                float none = 0.f;
-                if (g.bias) repack<T, true>(conv, raw + raw2, g, c, k, g.Pc, 4, warp, lane, gsum);
-                else repack<T, false>(conv, raw + raw2, g, c, k, g.Pc, 4, warp, lane, none);
-                repack<T, false>(xarr, raw, g, c, k, g.Px, 8, warp, lane, none);
+                if (g.bias) repack<T, true>(conv, raw + raw2, it_u, g, g.Pc, g.d_Pc, g.d_ec, 4, warp, lane, gsum);
+                else repack<T, false>(conv, raw + raw2, it_u, g, g.Pc, g.d_Pc, g.d_ec, 4, warp, lane, none);
+                repack<T, false>(xarr, raw, it_u, g, g.Px, g.d_Px, g.d_ex, 8, warp, lane, none);
             } else {
-                float none = 0.f;
-                repack<T, false>(conv, raw, g, c, k, g.Pc, 4, warp, lane, none);
+                repack<T, false>(conv, raw, it_u, g, g.Pc, g.d_Pc, g.d_ec, 4, warp, lane, none);
             }
             plane::fence_async_smem();
         }
         __syncthreads();
         if (!worker) {
-            if (lane == 0 && !g.no_copy) {
+            if (!g.no_copy) {
+                // The whole warp runs the loop (uniform control flow keeps the descriptors in uniform registers: 100 -> 45 cycles
+                // an MMA); one elected lane issues.
                 fence_after();
-                const unsigned a0 = plane::smem_addr(conv);
-                const u64 b0d = smem_desc(plane::smem_addr(table), (NCOL / 8) * 128, 128);
-                const unsigned rowb = (unsigned)g.Pc * 128;
+                const unsigned elected = elect_one();
+                const unsigned rowb = (unsigned)g.Pc * 128, a0 = plane::smem_addr(conv);
+                const u64 adesc = smem_desc(a0, 128, 2 * rowb), bdesc = smem_desc(plane::smem_addr(table), (NCOL / 8) * 128, 128);
                 constexpr unsigned id = instr_desc<T>(NCOL, false);
-                int q = 0;
+                unsigned s = job0 % (unsigned)g.ring, ph = (job0 / (unsigned)g.ring) & 1u;
                 for (int t = 0; t < g.T; ++t)
-                    for (int j = 0; j < g.n; ++j, ++q) {
-                        const unsigned jc = job0 + q, s = jc % (unsigned)g.ring;
-                        if (!*reinterpret_cast<volatile int *>(dead) && !plane::mbar_wait(empty + s, ((jc / (unsigned)g.ring) & 1u) ^ 1u, limit))
-                            *reinterpret_cast<volatile int *>(dead) = 1;
+                    for (int j = 0; j < g.n; ++j) {
+                        wait_for(empty + s, ph ^ 1u);
                         fence_after();
-                        const u64 ad = smem_desc(a0 + (unsigned)(32 * t) * rowb + (unsigned)j * 128, 128, 2 * rowb);
+                        const u64 ad = adesc + (u64)((unsigned)(32 * t) * rowb + (unsigned)j * 128 >> 4);
+                        const unsigned d = ring0 + s * NCOL;
+                        if (elected) {
 #pragma unroll
-                        for (int r = 0; r < TAPS; ++r) mma(ring0 + s * NCOL, ad + (u64)(r * (rowb >> 4)), b0d + (u64)(r * (TAP_BYTES >> 4)), id, r > 0);
-                        mma_commit(full + s);
+                            for (int r = 0; r < TAPS; ++r) mma(d, ad + (u64)((unsigned)r * (rowb >> 4)), bdesc + (u64)(r * (TAP_BYTES >> 4)), id, r > 0);
+                            mma_commit(full + s);
+                        }
+                        __syncwarp();
+                        if (++s == (unsigned)g.ring) { s = 0; ph ^= 1u; }
                     }
                 if (BWD) {
                     const unsigned xrow = (unsigned)g.Px * 128;
@@ -409,26 +452,29 @@ tensor_kernel(const __grid_constant__ KGeom g, const T *__restrict__ x, const T 
                         const unsigned row = g.nty == 1 ? 16 * w : (w >> 1) * g.period + (w & 1) * 16;
                         for (int j = 0; j < g.Pc; ++j) {
                             const u64 xa = xd + (u64)((row * xrow + (unsigned)j * 128) >> 4), gb = gd + (u64)((row * rowb + (unsigned)j * 128) >> 4);
-                            mma(tmem, xa, gb, idw, acc);
-                            mma(tmem + 64, xa + 8, gb, idw, acc);
+                            if (elected) {
+                                mma(tmem, xa, gb, idw, acc);
+                                mma(tmem + 64, xa + 8, gb, idw, acc);
+                            }
                             acc = 1;
                         }
                     }
                 }
-                mma_commit(done);
+                if (elected) mma_commit(done);
+                __syncwarp();
             }
         } else {
-            if (u + 1 < u_end) fetch(cn, kn);
+            if (u + 1 < u_end) {
+                if (warp == 7) fetch_unit<T, BWD>(items + ((unit + 1) & 1u) * nslot, raw, raw2, landed, g, x, go, cn, kn, lane);
+                if (cn != c) fetch_weights(cn);
+            }
             // ---- epilogue: warps 0-3 take the even jobs, 4-7 the odd ones; a lane is one image of one row pair
             const int m = (warp & 3) * 32 + lane, img = m & 7;
             const float scale = mis[544], bias = mis[545];
             for (int q = warp >> 2; q < jobs; q += 2) {
-                const int t = q / g.n, j = q - t * g.n;
+                const int t = fdiv(q, g.d_n), j = q - t * g.n;
                 const unsigned jc = job0 + q, s = jc % (unsigned)g.ring;
-                if (!*reinterpret_cast<volatile int *>(dead) && !plane::mbar_wait(full + s, (jc / (unsigned)g.ring) & 1u, limit)) {
-                    *reinterpret_cast<volatile int *>(dead) = 1;
-                    raise_timeout(status, g.alarm, g.tag);
-                }
+                wait_for(full + s, (jc / (unsigned)g.ring) & 1u);
                 __syncwarp();
                 fence_after();
                 float v[16], p1[16], p2[16];
@@ -436,6 +482,10 @@ tensor_kernel(const __grid_constant__ KGeom g, const T *__restrict__ x, const T 
                 tmem_ld16(addr, v);
                 tmem_ld16(addr + 16, p1);
                 tmem_ld16(addr + 32, p2);
+                const int row2 = 2 * (16 * t + (m >> 3)), o = fdiv(row2, g.d_period), r = row2 - o * g.period;
+                Item it;
+                it.ty = -1;
+                if (o < g.S && r < g.th) it = it_u[o * 8 + img];
                 tmem_ld_wait();
                 tmem_arrived(v);
                 tmem_arrived(p1);
@@ -443,42 +493,38 @@ tensor_kernel(const __grid_constant__ KGeom g, const T *__restrict__ x, const T 
                 fence_before();
                 __syncwarp();
                 if (lane == 0) mbar_arrive(empty + s);
-                const int row2 = 2 * (16 * t + (m >> 3)), o = fdiv(row2, g.d_period), r = row2 - o * g.period;
-                if (o >= g.S || r >= g.th) continue;
-                const Item it = find_item(g, c, k, o * 8 + img);
                 const int y = it.ty * g.th + r;
-                if (!it.valid || y >= g.H) continue;
+                if (it.ty < 0 || y >= g.H) continue;
 #pragma unroll
                 for (int i = 0; i < 16; ++i) {
                     if (std::is_same<T, __half>::value) v[i] = fmaf(scale, fmaf(p2[i], 1.f / 4194304.f, fmaf(p1[i], 1.f / 2048.f, v[i])), bias);
                     else v[i] = (v[i] + (p1[i] + p2[i])) + bias;
                 }
-                T *d = reinterpret_cast<T *>(sb + g.out_off + (o * 8 + img) * g.out_stride) + r * g.W + 8 * j;
+                // the output image keeps the item's place inside its 16-byte word of global memory
+                const int off = ((int)it.start + (it.ty * g.th - it.ya) * g.W) & 7;
+                T *d = reinterpret_cast<T *>(sb + g.out_off + (o * 8 + img) * g.out_stride) + off + r * g.W + 8 * j;
                 store8<T>(d, v, g.W - 8 * j, g.W);
                 if (y + 1 < g.H) store8<T>(d + g.W, v + 8, g.W - 8 * j, g.W);
             }
+            plane::fence_async_smem();
             worker_sync();
-            // ---- the finished items to global memory, a warp per item
-            for (int slot = warp; slot < 8 * g.S; slot += 8) {
-                const Item it = find_item(g, c, k, slot);
-                if (!it.valid) continue;
-                const int y0 = it.ty * g.th, nrow = g.H - y0 < g.th ? g.H - y0 : g.th, bytes = nrow * g.W * 2;
-                const char *s = sb + g.out_off + slot * g.out_stride;
-                char *d = reinterpret_cast<char *>(out + ((size_t)it.b * g.C + c) * g.HW + (size_t)y0 * g.W);
-                if (g.al == 16)
-                    for (int e = lane * 16; e < bytes; e += 512) *reinterpret_cast<uint4 *>(d + e) = *reinterpret_cast<const uint4 *>(s + e);
-                else if (g.al == 8)
-                    for (int e = lane * 8; e < bytes; e += 256) *reinterpret_cast<uint2 *>(d + e) = *reinterpret_cast<const uint2 *>(s + e);
-                else if (g.al == 4)
-                    for (int e = lane * 4; e < bytes; e += 128) *reinterpret_cast<unsigned *>(d + e) = *reinterpret_cast<const unsigned *>(s + e);
-                else
-                    for (int e = lane * 2; e < bytes; e += 64) *reinterpret_cast<unsigned short *>(d + e) = *reinterpret_cast<const unsigned short *>(s + e);
+            // ---- the finished items to global memory: whole 16-byte words by one bulk copy an item, the pixels before and behind
+            //      them one by one
+            for (int s0 = warp * 2; s0 < nslot; s0 += 16) {
+                const int slot = s0 + (lane >> 4), i = lane & 15;
+                const Item it = it_u[slot];
+                if (it.ty < 0) continue;
+                const int y0 = it.ty * g.th, nrow = g.H - y0 < g.th ? g.H - y0 : g.th;
+                const u64 first = it.start + (u64)((y0 - it.ya) * g.W), last = first + (unsigned)(nrow * g.W);
+                u64 lo = (first + 7) & ~7ull, hi = last & ~7ull;
+                if (hi < lo) hi = lo = lo < last ? lo : last;
+                const T *s = reinterpret_cast<const T *>(sb + g.out_off + slot * g.out_stride) + (int)(first & 7);  // the item's first pixel
+                if (i == 0 && hi > lo) plane::bulk_s2g(out + lo, s + (int)(lo - first), (unsigned)(hi - lo) * 2);
+                const u64 e = i < 8 ? first + i : hi + (i - 8);
+                if (i < 8 ? e < lo : e < last) out[e] = s[(int)(e - first)];
             }
             // every MMA of the unit has completed: its arrays and (on a channel change) its table may be rewritten
-            if (!*reinterpret_cast<volatile int *>(dead) && !plane::mbar_wait(done, unit & 1u, limit)) {
-                *reinterpret_cast<volatile int *>(dead) = 1;
-                raise_timeout(status, g.alarm, g.tag);
-            }
+            wait_for(done, unit & 1u);
             if (BWD && (u + 1 == u_end || cn != c)) {
                 // ---- flush: accumulators to shared memory (the arrays are idle), entries of equal offset added in a fixed order
                 fence_after();
@@ -551,6 +597,7 @@ tensor_kernel(const __grid_constant__ KGeom g, const T *__restrict__ x, const T 
         c = cn;
         k = kn;
     }
+    if (worker) plane::bulk_store_wait_read();  // shared memory must outlive the stores' reads
     if (BWD) dependents_may_start();
     fence_before();
     __syncthreads();
@@ -581,12 +628,14 @@ inline bool search(const Request &q, KGeom &best) {
     g.items = q.B * g.nty;
     g.d_nty = make_fastdiv(g.nty);
     g.d_period = make_fastdiv(g.period);
-    const long long st = g.nty == 1 ? (long long)g.HW * 2 : q.W * 8;  // every item starts on a multiple of this
-    const long long hw = (long long)g.HW * 2;
-    g.al = st % 16 == 0 && hw % 16 == 0 ? 16 : st % 8 == 0 && hw % 8 == 0 ? 8 : st % 4 == 0 && hw % 4 == 0 ? 4 : 2;
     const int load_rows = g.nty == 1 ? q.H : g.th + 8, out_rows = g.nty == 1 ? q.H : g.th;
-    g.raw_stride = up(load_rows * q.W * 2 + 4, 128) + 16;  // items fall on different banks
-    g.out_stride = up(out_rows * q.W * 2, 128) + 16;
+    g.raw_stride = up(load_rows * q.W * 2 + 30, 128) + 16;  // with the words' other pixels; items fall on different banks
+    g.out_stride = up(out_rows * q.W * 2 + 14, 128) + 16;
+    g.d_n = make_fastdiv(g.n);
+    g.d_Pc = make_fastdiv(g.Pc);
+    g.d_Px = make_fastdiv(g.Px);
+    g.d_ec = make_fastdiv(load_rows * g.Pc);
+    g.d_ex = make_fastdiv(load_rows * g.Px);
     const int sides = q.bwd ? 2 : 1;
     for (int S = 1; S <= 16; ++S) {
         if (S > 1 && 8 * (S - 1) >= g.items) break;
@@ -601,11 +650,13 @@ inline bool search(const Request &q, KGeom &best) {
         h.conv_off = off; off += h.rows * h.Pc * 128;
         h.x_off = off; if (q.bwd) off += h.rows * h.Px * 128;
         if (q.bwd && off < 128 * SCR_PITCH * 4) off = up(128 * SCR_PITCH * 4, 128);
+        h.parts_off = off; off += 5760;
+        off = up(off, 128);
         h.raw_off = off; off += sides * 8 * S * h.raw_stride;
         h.out_off = off; off += 8 * S * h.out_stride;
         off = up(off, 128);
         h.table_off = off; off += TABLE_BYTES;
-        h.misc_off = off; off += 560 * 4 + (2 * MAX_RING + 1) * 8 + 16;
+        h.misc_off = off; off += 600 * 4 + 2 * 8 * S * 16;
         h.smem = up(off, 128);
         if (h.smem > plane::SMEM_LIMIT) break;
         h.upc = (h.items + 8 * S - 1) / (8 * S);
