@@ -36,7 +36,9 @@ using plane::FastDiv;
 using plane::fdiv;
 using plane::make_fastdiv;
 
-constexpr int WORKERS = 256, THREADS = WORKERS + 32;  // eight staging / epilogue warps and the MMA issuer
+// Eight staging / epilogue warps and four that issue MMAs (an issue takes its warp about 100 cycles, the tensor cores 45).
+constexpr int WORKERS = 256, ISSUERS = 4, THREADS = WORKERS + 32 * ISSUERS;
+constexpr int BULK_WORDS = 48;
 constexpr int TAPS = 10, NCOL = 48;                   // window rows; 3 weight parts x 2 rows x 8 columns
 constexpr int TAP_BYTES = NCOL * 16 * 2, TABLE_BYTES = TAPS * TAP_BYTES;
 constexpr int WG_COLS = 128;                          // weight-gradient accumulators: two window halves x 64
@@ -53,11 +55,13 @@ struct KGeom {
     int Ws;                      // weight gradients: groups of 16 g rows
     int items, upc, units;       // items per channel, units per channel, units
     int raw_stride, out_stride;  // bytes per item of the raw and of the output buffers
+    int out_words;               // 16-byte words that can hold parts of an item's stored rows
+    int alias;                   // 1: the output image lies over the raw planes (the next unit is fetched behind the stores)
     int conv_off, x_off, parts_off, raw_off, out_off, table_off, misc_off, smem;  // byte offsets
     int ring, cols;              // tensor-memory ring depth and columns allocated
     int bps, nblocks, np;
     int no_copy, bias, deep;
-    FastDiv d_period, d_nty, d_n, d_Pc, d_Px, d_ec, d_ex;  // d_ec / d_ex: chunks of one octet in the convolved / the x array
+    FastDiv d_period, d_nty, d_n, d_Pc, d_Px, d_ec, d_ex, d_out_words;  // d_ec / d_ex: chunks of one octet in the convolved / the x array
     int *alarm;
     unsigned tag;
     double cost;
@@ -129,64 +133,63 @@ template <typename T> __device__ __forceinline__ float weight_part(float w, int 
 }
 
 // ------------------------------------------------------------------ loading
-// An item of a unit, worked out once by the warp that fetches it.
+// An item of a unit, worked out once for the whole block.
 struct __align__(16) Item {
     u64 start;  // element index of its first loaded pixel
     int ty;     // item row, or -1: no such item
     int ya;     // first row loaded
 };
+__device__ __forceinline__ Item find_item(const KGeom &g, int c, int k, int slot) {
+    Item it;
+    it.ty = -1;
+    it.ya = 0;
+    it.start = 0;
+    const int i = k * 8 * g.S + slot;
+    if (i < g.items) {
+        const int b = g.nty == 1 ? i : fdiv(i, g.d_nty);
+        it.ty = i - b * g.nty;
+        if (g.nty > 1 && it.ty > 0) it.ya = it.ty * g.th - 4;
+        it.start = ((u64)b * g.C + c) * g.HW + (u64)(it.ya * g.W);
+    }
+    return it;
+}
 // Bulk copies of one unit (one warp, a lane per item): the aligned 16-byte words around each item, so planes may start at any
-// element; repack() skips the bytes before the first pixel.
+// element (repack() skips the pixels before the first).
 template <typename T, bool BWD>
-__device__ __forceinline__ void fetch_unit(Item *items, char *raw, int raw2, u64 *bar, const KGeom &g, const T *__restrict__ x, const T *__restrict__ go,
-                                           int c, int k, int lane) {
+__device__ __forceinline__ void fetch_unit(const Item *items, char *raw, int raw2, u64 *bar, const KGeom &g, const T *__restrict__ x,
+                                           const T *__restrict__ go, int lane) {
+    if (g.no_copy) return;  // test mode: the barrier is never armed, nothing is in flight
     const u64 total = (u64)g.B * g.C * g.HW * 2;
     unsigned bytes_all = 0;
     plane::fence_async_smem();
 #pragma unroll 1
     for (int pass = 0; pass < 2; ++pass) {
-        for (int s0 = 0; s0 < 8 * g.S; s0 += 32) {
-            const int slot = s0 + lane, i = k * 8 * g.S + slot;
-            if (slot >= 8 * g.S) continue;
-            Item it;
-            it.ty = -1;
-            it.ya = 0;
-            it.start = 0;
-            if (i < g.items) {
-                const int b = g.nty == 1 ? i : fdiv(i, g.d_nty);
-                it.ty = i - b * g.nty;
-                int yb = g.H;
-                if (g.nty > 1) {
-                    it.ya = it.ty * g.th - 4 < 0 ? 0 : it.ty * g.th - 4;
-                    yb = it.ty * g.th + g.th + 4 > g.H ? g.H : it.ty * g.th + g.th + 4;
-                }
-                it.start = ((u64)b * g.C + c) * g.HW + (u64)(it.ya * g.W);
-                const u64 first = it.start * 2 & ~15ull, last = it.start * 2 + (unsigned)((yb - it.ya) * g.W * 2);
-                u64 end = (last + 15) & ~15ull;
-                const bool tail = end > total;
-                if (tail) end -= 16;
-                const unsigned n = (unsigned)(end - first);
-                if (pass == 0) {
-                    bytes_all += n;
-                } else {
-                    char *d = raw + slot * g.raw_stride;
-                    if (n) {
-                        plane::bulk_g2s(d, reinterpret_cast<const char *>(x) + first, n, bar);
-                        if (BWD) plane::bulk_g2s(d + raw2, reinterpret_cast<const char *>(go) + first, n, bar);
-                    }
-                    if (tail)  // the tensor ends inside a 16-byte word
-                        for (u64 o = end; o < last; o += 2) {
-                            *reinterpret_cast<T *>(d + (o - first)) = x[o / 2];
-                            if (BWD) *reinterpret_cast<T *>(d + raw2 + (o - first)) = go[o / 2];
-                        }
-                }
+        for (int slot = lane; slot < 8 * g.S; slot += 32) {
+            const Item it = items[slot];
+            if (it.ty < 0) continue;
+            int rows = g.H - it.ya;
+            if (g.nty > 1 && it.ty * g.th + g.th + 4 < g.H) rows = it.ty * g.th + g.th + 4 - it.ya;
+            const u64 first = it.start * 2 & ~15ull, last = it.start * 2 + (unsigned)(rows * g.W * 2);
+            u64 end = (last + 15) & ~15ull;
+            const bool tail = end > total;
+            if (tail) end -= 16;
+            const unsigned n = (unsigned)(end - first);
+            bytes_all += n;
+            if (pass == 0) continue;
+            char *d = raw + slot * g.raw_stride;
+            if (n) {
+                plane::bulk_g2s(d, reinterpret_cast<const char *>(x) + first, n, bar);
+                if (BWD) plane::bulk_g2s(d + raw2, reinterpret_cast<const char *>(go) + first, n, bar);
             }
-            if (pass == 0) items[slot] = it;
+            if (tail)  // the tensor ends inside a 16-byte word
+                for (u64 o = end; o < last; o += 2) {
+                    *reinterpret_cast<T *>(d + (o - first)) = x[o / 2];
+                    if (BWD) *reinterpret_cast<T *>(d + raw2 + (o - first)) = go[o / 2];
+                }
         }
         if (pass == 0) {
 #pragma unroll
             for (int o = 16; o; o >>= 1) bytes_all += __shfl_xor_sync(0xffffffffu, bytes_all, o);
-            if (g.no_copy) return;  // test mode: the barrier is never armed, nothing is in flight
             if (lane == 0) plane::mbar_expect_tx(bar, BWD ? 2 * bytes_all : bytes_all);
             __syncwarp();
         }
@@ -198,36 +201,37 @@ template <typename T, int VEC, bool SUM>
 __device__ __forceinline__ void repack(char *arr, const char *raw, const Item *items, const KGeom &g, int P, const FastDiv &dP, const FastDiv &dE,
                                        int shift, int warp, int lane, float &sum) {
     constexpr int U = VEC == 1 ? 2 : 4;
-    const int img = lane & 7, per = (int)dE.d, n = g.S * per, r0 = g.nty == 1 ? 0 : -4;
-    for (int e0 = warp * 4 + (lane >> 3); e0 < n; e0 += U * 32) {
-        unsigned v[U][4];
-        int dst[U];
+    const int img = lane & 7, per = (int)dE.d, r0 = g.nty == 1 ? 0 : -4;
+    const int wpo = g.S >= 8 ? 1 : g.S >= 4 ? 2 : g.S >= 2 ? 4 : 8, step = wpo * 4;  // warps to an octet
+    const int e_first = (warp & (wpo - 1)) * 4 + (lane >> 3);
+    for (int o = warp / wpo; o < g.S; o += 8 / wpo) {
+        const Item it = items[o * 8 + img];
+        const int ybase = it.ty * g.th + r0;
+        const char *src = raw + (o * 8 + img) * g.raw_stride + (((int)it.start & 7) + (ybase - it.ya) * g.W - shift) * 2;
+        char *dst = arr + (((o * g.period + 4 + r0) * P) * 8 + img) * 16;
+        for (int e0 = e_first; e0 < per; e0 += U * step) {
+            unsigned v[U][4];
 #pragma unroll
-        for (int i = 0; i < U; ++i) {
-            const int e = e0 + i * 32;
-            v[i][0] = v[i][1] = v[i][2] = v[i][3] = 0u;
-            dst[i] = -1;
-            if (e < n) {
-                const int o = fdiv(e, dE), ee = e - o * per, rr = fdiv(ee, dP), j = ee - rr * P, r = r0 + rr, x0 = 8 * j - shift;
-                const Item it = items[o * 8 + img];
-                dst[i] = (((o * g.period + 4 + r0) * P + ee) * 8 + img) * 16;
-                const int y = it.ty * g.th + r;
-                if (it.ty >= 0 && y >= 0 && y < g.H) {
-                    const T *row = reinterpret_cast<const T *>(raw + (o * 8 + img) * g.raw_stride + ((int)it.start & 7) * 2) + (y - it.ya) * g.W + x0;
+            for (int i = 0; i < U; ++i) {
+                const int e = e0 + i * step;
+                v[i][0] = v[i][1] = v[i][2] = v[i][3] = 0u;
+                const int rr = fdiv(e, dP), j = e - rr * P, x0 = 8 * j - shift, y = ybase + rr;
+                if (e < per && it.ty >= 0 && (unsigned)y < (unsigned)g.H) {
+                    const T *row = reinterpret_cast<const T *>(src) + rr * g.W + 8 * j;
                     if (VEC == 4) {
-                        if (x0 >= 0 && x0 < g.W) { const uint2 t = *reinterpret_cast<const uint2 *>(row); v[i][0] = t.x; v[i][1] = t.y; }
-                        if (x0 + 4 >= 0 && x0 + 4 < g.W) { const uint2 t = *reinterpret_cast<const uint2 *>(row + 4); v[i][2] = t.x; v[i][3] = t.y; }
+                        if ((unsigned)x0 < (unsigned)g.W) { const uint2 t = *reinterpret_cast<const uint2 *>(row); v[i][0] = t.x; v[i][1] = t.y; }
+                        if ((unsigned)(x0 + 4) < (unsigned)g.W) { const uint2 t = *reinterpret_cast<const uint2 *>(row + 4); v[i][2] = t.x; v[i][3] = t.y; }
                     } else if (VEC == 2) {
 #pragma unroll
                         for (int q = 0; q < 4; ++q)
-                            if (x0 + 2 * q >= 0 && x0 + 2 * q < g.W) v[i][q] = *reinterpret_cast<const unsigned *>(row + 2 * q);
+                            if ((unsigned)(x0 + 2 * q) < (unsigned)g.W) v[i][q] = *reinterpret_cast<const unsigned *>(row + 2 * q);
                     } else {
                         const unsigned short *p = reinterpret_cast<const unsigned short *>(row);
 #pragma unroll
                         for (int q = 0; q < 8; ++q)
-                            if (x0 + q >= 0 && x0 + q < g.W) v[i][q >> 1] |= (unsigned)p[q] << (16 * (q & 1));
+                            if ((unsigned)(x0 + q) < (unsigned)g.W) v[i][q >> 1] |= (unsigned)p[q] << (16 * (q & 1));
                     }
-                    if (SUM && r >= 0 && r < g.th) {
+                    if (SUM && r0 + rr >= 0 && r0 + rr < g.th) {
 #pragma unroll
                         for (int q = 0; q < 4; ++q) {
                             const float2 f = unpack16(v[i][q], T());
@@ -236,10 +240,12 @@ __device__ __forceinline__ void repack(char *arr, const char *raw, const Item *i
                     }
                 }
             }
-        }
 #pragma unroll
-        for (int i = 0; i < U; ++i)
-            if (dst[i] >= 0) *reinterpret_cast<uint4 *>(arr + dst[i]) = make_uint4(v[i][0], v[i][1], v[i][2], v[i][3]);
+            for (int i = 0; i < U; ++i) {
+                const int e = e0 + i * step;
+                if (e < per) *reinterpret_cast<uint4 *>(dst + e * 128) = make_uint4(v[i][0], v[i][1], v[i][2], v[i][3]);
+            }
+        }
     }
 }
 template <typename T, bool SUM>
@@ -359,7 +365,7 @@ tensor_kernel(const __grid_constant__ KGeom g, const T *__restrict__ x, const T 
             plane::mbar_init(full + i, 1);
             plane::mbar_init(empty + i, 4);
         }
-        plane::mbar_init(done, 1);
+        plane::mbar_init(done, ISSUERS);
         plane::mbar_init(landed, 1);
     }
     if (warp == 8) {
@@ -388,9 +394,17 @@ tensor_kernel(const __grid_constant__ KGeom g, const T *__restrict__ x, const T 
         if (tid < 125) wreg = folded_weight(g, cc, tid, BWD, w0, s0, wl, sl);
         if (tid == 0) breg = !BWD && b0 ? __ldg(s0 + cc) * __ldg(b0 + cc) : 0.f;
     };
+    auto list_items = [&](int set, int cc, int kk) {
+        if (tid < nslot) items[set * nslot + tid] = find_item(g, cc, kk, tid);
+    };
+    auto fetch = [&](int set) {
+        if (warp == 7) fetch_unit<T, BWD>(items + set * nslot, raw, raw2, landed, g, x, go, lane);
+    };
     if (worker && u_begin < u_end) {
-        if (warp == 7) fetch_unit<T, BWD>(items, raw, raw2, landed, g, x, go, c, k, lane);
         fetch_weights(c);
+        list_items(0, c, k);
+        worker_sync();
+        fetch(0);
     }
     for (int u = u_begin; u < u_end; ++u, ++unit, job0 += jobs) {
         int cn = c, kn = k + 1;
@@ -402,10 +416,11 @@ tensor_kernel(const __grid_constant__ KGeom g, const T *__restrict__ x, const T 
                 if (tid == 0) mis[545] = breg;
                 build_table<T>(table, sb + g.parts_off, mis, tid);
             }
+            if (u + 1 < u_end) list_items((unit + 1) & 1u, cn, kn);
             wait_for(landed, unit & 1u);
             plane::bulk_store_wait_read();  // the output image may be written again behind the next barriers
         }
-        __syncthreads();  // the item list (and what its fetcher copied by hand) is visible
+        __syncthreads();  // the next unit's item list (and what the fetcher copied by hand) is there for everybody
         if (worker) {
             float none = 0.f;
             if (BWD) {
@@ -420,42 +435,38 @@ tensor_kernel(const __grid_constant__ KGeom g, const T *__restrict__ x, const T 
         __syncthreads();
         if (!worker) {
             if (!g.no_copy) {
-                // The whole warp runs the loop (uniform control flow keeps the descriptors in uniform registers: 100 -> 45 cycles
-                // an MMA); one elected lane issues.
                 fence_after();
                 const unsigned elected = elect_one();
+                const int iw = warp - WORKERS / 32;
                 const unsigned rowb = (unsigned)g.Pc * 128, a0 = plane::smem_addr(conv);
                 const u64 adesc = smem_desc(a0, 128, 2 * rowb), bdesc = smem_desc(plane::smem_addr(table), (NCOL / 8) * 128, 128);
                 constexpr unsigned id = instr_desc<T>(NCOL, false);
-                unsigned s = job0 % (unsigned)g.ring, ph = (job0 / (unsigned)g.ring) & 1u;
-                for (int t = 0; t < g.T; ++t)
-                    for (int j = 0; j < g.n; ++j) {
-                        wait_for(empty + s, ph ^ 1u);
-                        fence_after();
-                        const u64 ad = adesc + (u64)((unsigned)(32 * t) * rowb + (unsigned)j * 128 >> 4);
-                        const unsigned d = ring0 + s * NCOL;
-                        if (elected) {
+                for (int q = iw; q < jobs; q += ISSUERS) {
+                    const int t = fdiv(q, g.d_n), j = q - t * g.n;
+                    const unsigned jc = job0 + q, s = jc % (unsigned)g.ring;
+                    wait_for(empty + s, ((jc / (unsigned)g.ring) & 1u) ^ 1u);
+                    fence_after();
+                    const u64 ad = adesc + (u64)((unsigned)(32 * t) * rowb + (unsigned)j * 128 >> 4);
+                    const unsigned d = ring0 + s * NCOL;
+                    if (elected) {
 #pragma unroll
-                            for (int r = 0; r < TAPS; ++r) mma(d, ad + (u64)((unsigned)r * (rowb >> 4)), bdesc + (u64)(r * (TAP_BYTES >> 4)), id, r > 0);
-                            mma_commit(full + s);
-                        }
-                        __syncwarp();
-                        if (++s == (unsigned)g.ring) { s = 0; ph ^= 1u; }
+                        for (int r = 0; r < TAPS; ++r) mma(d, ad + (u64)((unsigned)r * (rowb >> 4)), bdesc + (u64)(r * (TAP_BYTES >> 4)), id, r > 0);
+                        mma_commit(full + s);
                     }
-                if (BWD) {
+                    __syncwarp();
+                }
+                if (BWD && iw >= ISSUERS - 2) {  // weight gradients: one issuer for each half of the window (MMAs into one accumulator stay in order)
+                    const int half = iw - (ISSUERS - 2);
                     const unsigned xrow = (unsigned)g.Px * 128;
-                    const u64 xd = smem_desc(plane::smem_addr(xarr), 8 * xrow, xrow), gd = smem_desc(a0 + 4 * rowb, 8 * rowb, rowb);
+                    const u64 xd = smem_desc(plane::smem_addr(xarr) + half * 128, 8 * xrow, xrow), gd = smem_desc(a0 + 4 * rowb, 8 * rowb, rowb);
                     constexpr unsigned idw = instr_desc<T>(64, true);
                     unsigned acc = c == c_prev;
                     for (int w = 0; w < g.Ws; ++w) {
                         // cut planes: only the item's own rows count, not its halo
                         const unsigned row = g.nty == 1 ? 16 * w : (w >> 1) * g.period + (w & 1) * 16;
                         for (int j = 0; j < g.Pc; ++j) {
-                            const u64 xa = xd + (u64)((row * xrow + (unsigned)j * 128) >> 4), gb = gd + (u64)((row * rowb + (unsigned)j * 128) >> 4);
-                            if (elected) {
-                                mma(tmem, xa, gb, idw, acc);
-                                mma(tmem + 64, xa + 8, gb, idw, acc);
-                            }
+                            if (elected)
+                                mma(tmem + half * 64, xd + (u64)((row * xrow + (unsigned)j * 128) >> 4), gd + (u64)((row * rowb + (unsigned)j * 128) >> 4), idw, acc);
                             acc = 1;
                         }
                     }
@@ -465,7 +476,7 @@ tensor_kernel(const __grid_constant__ KGeom g, const T *__restrict__ x, const T 
             }
         } else {
             if (u + 1 < u_end) {
-                if (warp == 7) fetch_unit<T, BWD>(items + ((unit + 1) & 1u) * nslot, raw, raw2, landed, g, x, go, cn, kn, lane);
+                if (!g.alias) fetch((unit + 1) & 1u);
                 if (cn != c) fetch_weights(cn);
             }
             // ---- epilogue: warps 0-3 take the even jobs, 4-7 the odd ones; a lane is one image of one row pair
@@ -508,20 +519,45 @@ tensor_kernel(const __grid_constant__ KGeom g, const T *__restrict__ x, const T 
             }
             plane::fence_async_smem();
             worker_sync();
-            // ---- the finished items to global memory: whole 16-byte words by one bulk copy an item, the pixels before and behind
-            //      them one by one
-            for (int s0 = warp * 2; s0 < nslot; s0 += 16) {
-                const int slot = s0 + (lane >> 4), i = lane & 15;
-                const Item it = it_u[slot];
-                if (it.ty < 0) continue;
-                const int y0 = it.ty * g.th, nrow = g.H - y0 < g.th ? g.H - y0 : g.th;
-                const u64 first = it.start + (u64)((y0 - it.ya) * g.W), last = first + (unsigned)(nrow * g.W);
-                u64 lo = (first + 7) & ~7ull, hi = last & ~7ull;
-                if (hi < lo) hi = lo = lo < last ? lo : last;
-                const T *s = reinterpret_cast<const T *>(sb + g.out_off + slot * g.out_stride) + (int)(first & 7);  // the item's first pixel
-                if (i == 0 && hi > lo) plane::bulk_s2g(out + lo, s + (int)(lo - first), (unsigned)(hi - lo) * 2);
-                const u64 e = i < 8 ? first + i : hi + (i - 8);
-                if (i < 8 ? e < lo : e < last) out[e] = s[(int)(e - first)];
+            // ---- the finished items to global memory: whole 16-byte words (one bulk copy an item where that is much; a bulk copy
+            //      costs about 40 cycles whatever its size), the pixels before and behind them one by one
+            if (g.out_words >= BULK_WORDS) {
+                for (int s0 = warp * 2; s0 < nslot; s0 += 16) {
+                    const int slot = s0 + (lane >> 4), i = lane & 15;
+                    const Item it = it_u[slot];
+                    if (it.ty < 0) continue;
+                    const int y0 = it.ty * g.th, len = (g.H - y0 < g.th ? g.H - y0 : g.th) * g.W;
+                    const u64 first = it.start + (u64)((y0 - it.ya) * g.W);
+                    const int at = (int)(first & 7), lo = (8 - at) & 7, hi = ((at + len) & ~7) - at;  // whole words: [lo, hi) of [0, len)
+                    const T *s = reinterpret_cast<const T *>(sb + g.out_off + slot * g.out_stride) + at;
+                    if (i == 0) plane::bulk_s2g(out + first + lo, s + lo, (unsigned)(hi - lo) * 2);
+                    const int e = i < 8 ? i : hi + (i - 8);
+                    if (i < 8 ? e < lo : e < len) out[first + e] = s[e];
+                }
+            } else {
+                for (int e = tid; e < nslot * g.out_words; e += WORKERS) {
+                    const int slot = fdiv(e, g.d_out_words), w = e - slot * g.out_words;
+                    const Item it = it_u[slot];
+                    if (it.ty < 0) continue;
+                    const int y0 = it.ty * g.th, len = (g.H - y0 < g.th ? g.H - y0 : g.th) * g.W;
+                    const u64 first = it.start + (u64)((y0 - it.ya) * g.W);
+                    const int rel = 8 * w - (int)(first & 7);  // the word's first pixel, counted from the item's first
+                    const uint4 *s = reinterpret_cast<const uint4 *>(sb + g.out_off + slot * g.out_stride) + w;
+                    T *d = out + (first + rel);
+                    if (rel >= 0 && rel + 8 <= len) {
+                        *reinterpret_cast<uint4 *>(d) = *s;
+                    } else {
+                        const T *p = reinterpret_cast<const T *>(s);
+#pragma unroll
+                        for (int i = 0; i < 8; ++i)
+                            if (rel + i >= 0 && rel + i < len) d[i] = p[i];
+                    }
+                }
+            }
+            if (g.alias && u + 1 < u_end) {
+                plane::bulk_store_wait_read();
+                worker_sync();
+                fetch((unit + 1) & 1u);
             }
             // every MMA of the unit has completed: its arrays and (on a channel change) its table may be rewritten
             wait_for(done, unit & 1u);
@@ -629,6 +665,8 @@ inline bool search(const Request &q, KGeom &best) {
     g.d_nty = make_fastdiv(g.nty);
     g.d_period = make_fastdiv(g.period);
     const int load_rows = g.nty == 1 ? q.H : g.th + 8, out_rows = g.nty == 1 ? q.H : g.th;
+    g.out_words = (out_rows * q.W * 2 + 14 + 15) / 16;
+    g.d_out_words = make_fastdiv(g.out_words);
     g.raw_stride = up(load_rows * q.W * 2 + 30, 128) + 16;  // with the words' other pixels; items fall on different banks
     g.out_stride = up(out_rows * q.W * 2 + 14, 128) + 16;
     g.d_n = make_fastdiv(g.n);
@@ -637,6 +675,7 @@ inline bool search(const Request &q, KGeom &best) {
     g.d_ec = make_fastdiv(load_rows * g.Pc);
     g.d_ex = make_fastdiv(load_rows * g.Px);
     const int sides = q.bwd ? 2 : 1;
+    for (int alias = 0; alias < 2; ++alias)
     for (int S = 1; S <= 16; ++S) {
         if (S > 1 && 8 * (S - 1) >= g.items) break;
         KGeom h = g;
@@ -653,7 +692,8 @@ inline bool search(const Request &q, KGeom &best) {
         h.parts_off = off; off += 5760;
         off = up(off, 128);
         h.raw_off = off; off += sides * 8 * S * h.raw_stride;
-        h.out_off = off; off += 8 * S * h.out_stride;
+        h.alias = alias;
+        h.out_off = alias ? h.raw_off : off; if (!alias) off += 8 * S * h.out_stride;
         off = up(off, 128);
         h.table_off = off; off += TABLE_BYTES;
         h.misc_off = off; off += 600 * 4 + 2 * 8 * S * 16;
@@ -671,7 +711,7 @@ inline bool search(const Request &q, KGeom &best) {
             h.nblocks = plane::NUM_SMS * bps < h.units ? plane::NUM_SMS * bps : h.units;
             // cycles: MMAs serialise over an SM's blocks; the workers' part and the hand-overs do not
             const double tensor = (double)h.T * h.n * TAPS * 46 + (q.bwd ? (double)h.Ws * h.Pc * 2 * 50 : 0);
-            const double around = 3500.0 + 6.0 * S * (q.bwd ? 2.2 : 1.0) * load_rows * h.Pc + 0.25 * tensor;
+            const double around = 3500.0 + (alias ? 2500.0 : 0.0) + 6.0 * S * (q.bwd ? 2.2 : 1.0) * load_rows * h.Pc + 0.25 * tensor;
             const int active = (h.nblocks + plane::NUM_SMS - 1) / plane::NUM_SMS;
             const int rounds = (h.units + h.nblocks - 1) / h.nblocks;
             const double serial = tensor + around, per = active * tensor > serial ? active * tensor : serial;
