@@ -29,6 +29,10 @@
 #include "plane_kernels.cuh"
 
 namespace wt {
+namespace plane {
+WT_PLANE_DEEP_INSTANTIATE(__half, extern)  // levels >= 2, compiled in their own unit
+WT_PLANE_DEEP_INSTANTIATE(__nv_bfloat16, extern)
+}  // namespace plane
 namespace tensor {
 
 typedef unsigned long long u64;
@@ -511,6 +515,21 @@ tensor_kernel(const __grid_constant__ KGeom g, const T *__restrict__ x, const T 
                     if (std::is_same<T, __half>::value) v[i] = fmaf(scale, fmaf(p2[i], 1.f / 4194304.f, fmaf(p1[i], 1.f / 2048.f, v[i])), bias);
                     else v[i] = (v[i] + (p1[i] + p2[i])) + bias;
                 }
+                if (g.deep) {  // levels >= 2: one value (un-normalised LL of level 1, Proposition 2) per 2 x 2 pixels
+                    const u64 plane = (it.start - (u64)(it.ya * g.W)) / (unsigned)g.HW;
+                    const float *d = deep_plane(out, plane, g.HW) + (y >> 1) * ((g.W + 1) >> 1) + 4 * j;
+                    const int left = ((g.W + 1) >> 1) - 4 * j;
+                    float add[4];
+                    if (left >= 4 && ((g.W + 1) >> 1 & 3) == 0 && (g.HW & 7) == 0) {
+                        const float4 t4 = *reinterpret_cast<const float4 *>(d);
+                        add[0] = t4.x; add[1] = t4.y; add[2] = t4.z; add[3] = t4.w;
+                    } else {
+#pragma unroll
+                        for (int i = 0; i < 4; ++i) add[i] = i < left ? d[i] : 0.f;
+                    }
+#pragma unroll
+                    for (int i = 0; i < 16; ++i) v[i] = fmaf(0.5f, add[(i & 7) >> 1], v[i]);
+                }
                 // the output image keeps the item's place inside its 16-byte word of global memory
                 const int off = ((int)it.start + (it.ty * g.th - it.ya) * g.W) & 7;
                 T *d = reinterpret_cast<T *>(sb + g.out_off + (o * 8 + img) * g.out_stride) + off + r * g.W + 8 * j;
@@ -648,11 +667,17 @@ struct Request {
 inline int up(int v, int m) { return (v + m - 1) / m * m; }
 
 inline bool search(const Request &q, KGeom &best) {
-    if ((q.K != 3 && q.K != 5) || q.L > 1 || q.W > 64 || q.H > 256 || q.H < 2 || q.W < 2) return false;
+    if ((q.K != 3 && q.K != 5) || q.L > 8 || q.W > 64 || q.H > 256 || q.H < 2 || q.W < 2) return false;
     best = KGeom{};
     best.cost = 1e30;
     bool found = false;
     KGeom g = {};
+    g.deep = q.L > 1;
+    if (g.deep) {  // the addend lies in the planes' own place: a plane's items have to belong to one unit
+        plane::Geom d;
+        const int items = q.H <= 32 ? 1 : (q.H + 31) / 32;
+        if (q.K != 5 || items == 3 || (items > 4 && items != 8) || !plane::plan_deep(q.bwd, q.B, q.C, q.H, q.W, q.L, d)) return false;
+    }
     g.B = q.B; g.C = q.C; g.H = q.H; g.W = q.W; g.HW = q.H * q.W; g.L = q.L; g.K = q.K;
     g.n = (q.W + 7) / 8;
     g.Pc = g.n + 1;
@@ -766,7 +791,10 @@ inline size_t backward_bytes(const Request &q) {
     KGeom g;
     if (!plan(q, g)) return 0;
     const size_t KK = (size_t)q.K * q.K;
-    return STATUS_BYTES + sizeof(float) * (size_t)g.C * g.np * (KK + 1 + 4 * KK);
+    size_t floats = (size_t)g.C * g.np * (KK + 1 + 4 * KK);
+    plane::Geom d;
+    if (q.L > 1 && plane::plan_deep(true, q.B, q.C, q.H, q.W, q.L, d)) floats += (size_t)(q.L - 1) * q.C * d.np * 4 * KK;
+    return STATUS_BYTES + sizeof(float) * floats;
 }
 
 template <typename T>
@@ -778,8 +806,11 @@ cudaError_t forward(const Request &q, const T *x, const float *w0, const float *
     g.alarm = call_alarm;
     g.no_copy = no_copy;
     constexpr auto kern = tensor_kernel<T, false>;
-    const cudaError_t e = plane::opt_in_smem<kern>();
+    cudaError_t e = plane::opt_in_smem<kern>();
     if (e != cudaSuccess) return e;
+    if (q.L > 1 && (e = plane::deep_forward<T>(q.B, q.C, q.H, q.W, q.L, x, wl + (size_t)q.C * 4 * q.K * q.K, sl + (size_t)q.C * 4, out,
+                                               reinterpret_cast<int *>(ws), st, tag, no_copy)) != cudaSuccess)
+        return e;
     return launch_overlapped(kern, (unsigned)g.nblocks, (unsigned)THREADS, (size_t)g.smem, st, g, x, nullptr, w0, s0, b0, wl, sl, out, nullptr,
                              nullptr, reinterpret_cast<int *>(ws));
 }
@@ -798,6 +829,9 @@ cudaError_t backward(const Request &q, const T *x, const T *go, const float *w0,
     constexpr auto kern = tensor_kernel<T, true>;
     cudaError_t e = plane::opt_in_smem<kern>();
     if (e != cudaSuccess) return e;
+    if (q.L > 1 && (e = plane::deep_backward<T>(q.B, q.C, q.H, q.W, q.L, x, go, wl + (size_t)q.C * 4 * KK, sl + (size_t)q.C * 4, gx,
+                                                partl + (size_t)g.C * g.np * 4 * KK, ep, reinterpret_cast<int *>(ws), st, tag, no_copy)) != cudaSuccess)
+        return e;
     e = launch_overlapped(kern, (unsigned)g.nblocks, (unsigned)THREADS, (size_t)g.smem, st, g, x, go, w0, s0, nullptr, wl, sl, gx, part0, partl,
                           reinterpret_cast<int *>(ws));
     if (e != cudaSuccess) return e;
