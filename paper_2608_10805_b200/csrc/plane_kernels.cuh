@@ -269,6 +269,21 @@ __device__ __forceinline__ float at1(const T *plane, const Geom &g, int y, int x
     const float c = y1 ? ld1<T, RAW>(p + g.W0) : 0.f, d = x1 && y1 ? ld1<T, RAW>(p + g.W0 + 1) : 0.f;
     return 0.5f * ((a + b) + (c + d));
 }
+// Elements (y, x) and (y, x + 1), x even; the second is zero beyond the plane.  Where the pixel rows allow it, four pixels at a time.
+template <typename T, bool RAW, bool DEEP>
+__device__ __forceinline__ void at2(const T *plane, const Geom &g, int y, int x, float &v0, float &v1) {
+    if (DEEP && (g.W0 & 3) == 0 && (g.HW0 & 3) == 0) {
+        const T *p = plane + 2 * y * g.W0 + 2 * x;
+        float a[4], c[4] = {0.f, 0.f, 0.f, 0.f};
+        ld4<T, RAW>(p, a);
+        if (2 * y + 1 < g.H0) ld4<T, RAW>(p + g.W0, c);
+        v0 = 0.5f * ((a[0] + a[1]) + (c[0] + c[1]));
+        v1 = 0.5f * ((a[2] + a[3]) + (c[2] + c[3]));
+    } else {
+        v0 = at1<T, RAW, DEEP>(plane, g, y, x);
+        v1 = x + 1 < g.W ? at1<T, RAW, DEEP>(plane, g, y, x + 1) : 0.f;
+    }
+}
 // Elements (y, x .. x + 3), x a multiple of 4 (g.vec).
 template <typename T, bool RAW, bool DEEP>
 __device__ __forceinline__ void at4(const T *plane, const Geom &g, int y, int x, float (&v)[4]) {
@@ -562,10 +577,8 @@ __device__ __forceinline__ int stage_input(float *sm, const Geom &g, const int *
         float a = 0.f, bq = 0.f, cq = 0.f, d = 0.f;
         if (slot < nvalid) {
             const T *pa = gsrc + (size_t)slot * img_stride;
-            a = at1<T, RAW, DEEP>(pa, g, y, xx);
-            if (x1) bq = at1<T, RAW, DEEP>(pa, g, y, xx + 1);
-            if (y1) cq = at1<T, RAW, DEEP>(pa, g, y + 1, xx);
-            if (x1 && y1) d = at1<T, RAW, DEEP>(pa, g, y + 1, xx + 1);
+            at2<T, RAW, DEEP>(pa, g, y, xx, a, bq);
+            if (y1) at2<T, RAW, DEEP>(pa, g, y + 1, xx, cq, d);
         }
         const int S = slot * g.slot_stride;
         const int xi = S + off[0] + (y + 2) * p0 + xx + 2;

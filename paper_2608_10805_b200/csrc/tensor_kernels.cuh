@@ -52,7 +52,9 @@ constexpr unsigned WAIT_LIMIT = 1u << 20;
 
 struct KGeom {
     int B, C, H, W, HW, L, K;
-    int th, nty;                 // rows per item, items per plane
+    int th, nty;                 // rows per item, items per plane (of one panel)
+    int panels, tw;              // wide planes: column panels of tw columns
+    int halo;                    // rows of the neighbouring items above and below an item (0: the item is the whole plane)
     int S, period, rows;         // octets per unit, array rows from one octet to the next, rows allocated
     int T, n;                    // M tiles (16 row pairs) per unit, output chunks (8 columns)
     int Pc, Px;                  // chunks per row of the convolved array and of x in the backward
@@ -64,7 +66,7 @@ struct KGeom {
     int conv_off, x_off, parts_off, raw_off, out_off, table_off, misc_off, smem;  // byte offsets
     int ring, cols;              // tensor-memory ring depth and columns allocated
     int bps, nblocks, np;
-    int no_copy, bias, deep;
+    int no_copy, bias, deep;     // deep: 1 the addend lies in the planes' own place, 2 in a tensor of its own
     FastDiv d_period, d_nty, d_n, d_Pc, d_Px, d_ec, d_ex, d_out_words;  // d_ec / d_ex: chunks of one octet in the convolved / the x array
     int *alarm;
     unsigned tag;
@@ -152,7 +154,7 @@ __device__ __forceinline__ Item find_item(const KGeom &g, int c, int k, int slot
     if (i < g.items) {
         const int b = g.nty == 1 ? i : fdiv(i, g.d_nty);
         it.ty = i - b * g.nty;
-        if (g.nty > 1 && it.ty > 0) it.ya = it.ty * g.th - 4;
+        if (it.ty > 0) it.ya = it.ty * g.th - 4;
         it.start = ((u64)b * g.C + c) * g.HW + (u64)(it.ya * g.W);
     }
     return it;
@@ -172,7 +174,7 @@ __device__ __forceinline__ void fetch_unit(const Item *items, char *raw, int raw
             const Item it = items[slot];
             if (it.ty < 0) continue;
             int rows = g.H - it.ya;
-            if (g.nty > 1 && it.ty * g.th + g.th + 4 < g.H) rows = it.ty * g.th + g.th + 4 - it.ya;
+            if (g.halo && it.ty * g.th + g.th + 4 < g.H) rows = it.ty * g.th + g.th + 4 - it.ya;
             const u64 first = it.start * 2 & ~15ull, last = it.start * 2 + (unsigned)(rows * g.W * 2);
             u64 end = (last + 15) & ~15ull;
             const bool tail = end > total;
@@ -205,7 +207,7 @@ template <typename T, int VEC, bool SUM>
 __device__ __forceinline__ void repack(char *arr, const char *raw, const Item *items, const KGeom &g, int P, const FastDiv &dP, const FastDiv &dE,
                                        int shift, int warp, int lane, float &sum) {
     constexpr int U = VEC == 1 ? 2 : 4;
-    const int img = lane & 7, per = (int)dE.d, r0 = g.nty == 1 ? 0 : -4;
+    const int img = lane & 7, per = (int)dE.d, r0 = -g.halo;
     const int wpo = g.S >= 8 ? 1 : g.S >= 4 ? 2 : g.S >= 2 ? 4 : 8, step = wpo * 4;  // warps to an octet
     const int e_first = (warp & (wpo - 1)) * 4 + (lane >> 3);
     for (int o = warp / wpo; o < g.S; o += 8 / wpo) {
@@ -248,6 +250,96 @@ __device__ __forceinline__ void repack(char *arr, const char *raw, const Item *i
             for (int i = 0; i < U; ++i) {
                 const int e = e0 + i * step;
                 if (e < per) *reinterpret_cast<uint4 *>(dst + e * 128) = make_uint4(v[i][0], v[i][1], v[i][2], v[i][3]);
+            }
+        }
+    }
+}
+// The same for one column panel, straight from global memory (a panel's rows are short: staging them first costs a pass over
+// shared memory, whose bandwidth the MMAs need).  x0 = the panel's first column.
+template <typename T, bool SUM>
+__device__ __forceinline__ void repack_panel(char *arr, const T *__restrict__ src, const Item *items, const KGeom &g, int P, const FastDiv &dP,
+                                             const FastDiv &dE, int shift, int x0, int warp, int lane, float &sum) {
+    constexpr int U = 4;
+    const int img = lane & 7, per = (int)dE.d;
+    const int wpo = g.S >= 8 ? 1 : g.S >= 4 ? 2 : g.S >= 2 ? 4 : 8, step = wpo * 4;  // warps to an octet
+    const int e_first = (warp & (wpo - 1)) * 4 + (lane >> 3);
+    const bool quads = (g.W & 3) == 0;  // four pixels are one aligned word, wholly inside a row or wholly outside
+    const long long total = (long long)g.B * g.C * g.HW;
+    for (int o = warp / wpo; o < g.S; o += 8 / wpo) {
+        const Item it = items[o * 8 + img];
+        const int ybase = it.ty * g.th - 4;
+        const long long e_base = (long long)it.start + (long long)(ybase - it.ya) * g.W + x0 - shift;
+        char *dst = arr + ((o * g.period * P) * 8 + img) * 16;
+        for (int e0 = e_first; e0 < per; e0 += U * step) {
+            unsigned v[U][4], h[U][4];
+            int col[U];
+            int sh[U];
+#pragma unroll
+            for (int i = 0; i < U; ++i) {
+                const int e = e0 + i * step;
+                v[i][0] = v[i][1] = v[i][2] = v[i][3] = 0u;
+                h[i][0] = h[i][1] = h[i][2] = h[i][3] = 0u;
+                const int rr = fdiv(e, dP), j = e - rr * P, y = ybase + rr;
+                col[i] = x0 + 8 * j - shift;
+                sh[i] = 0;
+                if (e < per && it.ty >= 0 && (unsigned)y < (unsigned)g.H && col[i] > -8 && col[i] < g.W) {
+                    const long long at = e_base + (long long)rr * g.W + 8 * j;
+                    if (quads) {
+                        if ((unsigned)col[i] < (unsigned)g.W) { const uint2 t = __ldg(reinterpret_cast<const uint2 *>(src + at)); v[i][0] = t.x; v[i][1] = t.y; }
+                        if ((unsigned)(col[i] + 4) < (unsigned)g.W) { const uint2 t = __ldg(reinterpret_cast<const uint2 *>(src + at + 4)); v[i][2] = t.x; v[i][3] = t.y; }
+                    } else {  // two aligned words around the eight pixels; words that leave the tensor are read pixel by pixel
+                        const long long w = at >> 3;
+                        sh[i] = (int)(at & 7);
+                        if (w >= 0 && 8 * w + 16 <= total) {
+                            const uint4 t = __ldg(reinterpret_cast<const uint4 *>(src + 8 * w));
+                            v[i][0] = t.x; v[i][1] = t.y; v[i][2] = t.z; v[i][3] = t.w;
+                            if (sh[i]) {
+                                const uint4 t2 = __ldg(reinterpret_cast<const uint4 *>(src + 8 * w) + 1);
+                                h[i][0] = t2.x; h[i][1] = t2.y; h[i][2] = t2.z; h[i][3] = t2.w;
+                            }
+                        } else {
+                            sh[i] = 0;
+                            const unsigned short *p = reinterpret_cast<const unsigned short *>(src);
+#pragma unroll
+                            for (int q = 0; q < 8; ++q)
+                                if (at + q >= 0 && at + q < total) v[i][q >> 1] |= (unsigned)__ldg(p + at + q) << (16 * (q & 1));
+                        }
+                    }
+                } else {
+                    col[i] = -8;
+                }
+            }
+#pragma unroll
+            for (int i = 0; i < U; ++i) {
+                const int e = e0 + i * step;
+                if (e >= per) continue;
+                if (!quads && col[i] > -8) {
+                    unsigned *a = v[i], *b = h[i];
+                    if (sh[i] & 4) { a[0] = a[2]; a[1] = a[3]; a[2] = b[0]; a[3] = b[1]; b[0] = b[2]; b[1] = b[3]; }
+                    if (sh[i] & 2) { a[0] = a[1]; a[1] = a[2]; a[2] = a[3]; a[3] = b[0]; b[0] = b[1]; }
+                    if (sh[i] & 1) {
+                        a[0] = __funnelshift_r(a[0], a[1], 16);
+                        a[1] = __funnelshift_r(a[1], a[2], 16);
+                        a[2] = __funnelshift_r(a[2], a[3], 16);
+                        a[3] = __funnelshift_r(a[3], b[0], 16);
+                    }
+                    if (col[i] < 0 || col[i] + 8 > g.W) {  // pixels of the neighbouring rows
+#pragma unroll
+                        for (int q = 0; q < 8; ++q)
+                            if ((unsigned)(col[i] + q) >= (unsigned)g.W) a[q >> 1] &= q & 1 ? 0x0000ffffu : 0xffff0000u;
+                    }
+                }
+                if (SUM) {
+                    const int rr = fdiv(e, dP), j = e - rr * P;
+                    if (rr >= 4 && rr < 4 + g.th && (x0 == 0 || j > 0)) {
+#pragma unroll
+                        for (int q = 0; q < 4; ++q) {
+                            const float2 f = unpack16(v[i][q], T());
+                            sum += f.x + f.y;
+                        }
+                    }
+                }
+                *reinterpret_cast<uint4 *>(dst + e * 128) = make_uint4(v[i][0], v[i][1], v[i][2], v[i][3]);
             }
         }
     }
@@ -341,11 +433,11 @@ __device__ __forceinline__ void store8(T *p, const float *v, int left, int W) {
 
 // ------------------------------------------------------------------ the kernel
 // BWD = false: out = base + level 1 of x.  BWD = true: out = grad_x from go (rotated kernels) and the weight-gradient sums.
-template <typename T, bool BWD>
+template <typename T, bool BWD, bool PANEL>
 __global__ void __launch_bounds__(THREADS, 2)
 tensor_kernel(const __grid_constant__ KGeom g, const T *__restrict__ x, const T *__restrict__ go, const float *__restrict__ w0,
               const float *__restrict__ s0, const float *__restrict__ b0, const float *__restrict__ wl, const float *__restrict__ sl,
-              T *__restrict__ out, float *__restrict__ part0, float *__restrict__ partl, int *__restrict__ status) {
+              const float *__restrict__ add, T *__restrict__ out, float *__restrict__ part0, float *__restrict__ partl, int *__restrict__ status) {
     extern __shared__ __align__(128) char sb[];
     const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
     const bool worker = warp < 8;
@@ -390,7 +482,8 @@ tensor_kernel(const __grid_constant__ KGeom g, const T *__restrict__ x, const T 
     if (!BWD) dependents_may_start();
     wait_for_predecessor();  // shared and tensor memory only up to here
     if (blockIdx.x == 0 && tid == 0) status[STATUS_LAUNCH] = (int)g.tag;
-    int c = u_begin / g.upc, k = u_begin - c * g.upc, c_prev = -1;
+    const int per_channel = g.upc * g.panels;
+    int c = u_begin / per_channel, k = u_begin - c * per_channel, c_prev = -1;
     const int jobs = g.T * g.n;
     unsigned job0 = 0, unit = 0;  // jobs issued before this unit, units done
     float gsum = 0.f, wreg = 0.f, breg = 0.f;
@@ -399,10 +492,10 @@ tensor_kernel(const __grid_constant__ KGeom g, const T *__restrict__ x, const T 
         if (tid == 0) breg = !BWD && b0 ? __ldg(s0 + cc) * __ldg(b0 + cc) : 0.f;
     };
     auto list_items = [&](int set, int cc, int kk) {
-        if (tid < nslot) items[set * nslot + tid] = find_item(g, cc, kk, tid);
+        if (tid < nslot) items[set * nslot + tid] = find_item(g, cc, PANEL ? kk % g.upc : kk, tid);
     };
     auto fetch = [&](int set) {
-        if (warp == 7) fetch_unit<T, BWD>(items + set * nslot, raw, raw2, landed, g, x, go, lane);
+        if (!PANEL && warp == 7) fetch_unit<T, BWD>(items + set * nslot, raw, raw2, landed, g, x, go, lane);
     };
     if (worker && u_begin < u_end) {
         fetch_weights(c);
@@ -412,7 +505,8 @@ tensor_kernel(const __grid_constant__ KGeom g, const T *__restrict__ x, const T 
     }
     for (int u = u_begin; u < u_end; ++u, ++unit, job0 += jobs) {
         int cn = c, kn = k + 1;
-        if (kn == g.upc) { kn = 0; ++cn; }
+        if (kn == per_channel) { kn = 0; ++cn; }
+        const int panel = PANEL ? k / g.upc : 0, x0 = panel * g.tw;  // units of a channel: panel by panel
         const Item *it_u = items + (unit & 1u) * nslot;
         if (worker) {
             if (c != c_prev) {  // the MMAs that read the old table have completed (see the wait at the end of a unit)
@@ -421,13 +515,18 @@ tensor_kernel(const __grid_constant__ KGeom g, const T *__restrict__ x, const T 
                 build_table<T>(table, sb + g.parts_off, mis, tid);
             }
             if (u + 1 < u_end) list_items((unit + 1) & 1u, cn, kn);
-            wait_for(landed, unit & 1u);
+            if (!PANEL) wait_for(landed, unit & 1u);
             plane::bulk_store_wait_read();  // the output image may be written again behind the next barriers
         }
         __syncthreads();  // the next unit's item list (and what the fetcher copied by hand) is there for everybody
         if (worker) {
             float none = 0.f;
-            if (BWD) {
+            if (PANEL) {
+                const T *src = BWD ? go : x;
+                if (BWD && g.bias) repack_panel<T, true>(conv, src, it_u, g, g.Pc, g.d_Pc, g.d_ec, 4, x0, warp, lane, gsum);
+                else repack_panel<T, false>(conv, src, it_u, g, g.Pc, g.d_Pc, g.d_ec, 4, x0, warp, lane, none);
+                if (BWD) repack_panel<T, false>(xarr, x, it_u, g, g.Px, g.d_Px, g.d_ex, 8, x0, warp, lane, none);
+            } else if (BWD) {
                 if (g.bias) repack<T, true>(conv, raw + raw2, it_u, g, g.Pc, g.d_Pc, g.d_ec, 4, warp, lane, gsum);
                 else repack<T, false>(conv, raw + raw2, it_u, g, g.Pc, g.d_Pc, g.d_ec, 4, warp, lane, none);
                 repack<T, false>(xarr, raw, it_u, g, g.Px, g.d_Px, g.d_ex, 8, warp, lane, none);
@@ -467,8 +566,9 @@ tensor_kernel(const __grid_constant__ KGeom g, const T *__restrict__ x, const T 
                     unsigned acc = c == c_prev;
                     for (int w = 0; w < g.Ws; ++w) {
                         // cut planes: only the item's own rows count, not its halo
-                        const unsigned row = g.nty == 1 ? 16 * w : (w >> 1) * g.period + (w & 1) * 16;
-                        for (int j = 0; j < g.Pc; ++j) {
+                        const unsigned row = g.halo ? (w >> 1) * g.period + (w & 1) * 16 : 16 * w;
+                        // a panel's first chunk starts in the panel to its left, which has counted those columns
+                        for (int j = PANEL && panel > 0 ? 1 : 0; j < g.Pc; ++j) {
                             if (elected)
                                 mma(tmem + half * 64, xd + (u64)((row * xrow + (unsigned)j * 128) >> 4), gd + (u64)((row * rowb + (unsigned)j * 128) >> 4), idw, acc);
                             acc = 1;
@@ -517,10 +617,11 @@ tensor_kernel(const __grid_constant__ KGeom g, const T *__restrict__ x, const T 
                 }
                 if (g.deep) {  // levels >= 2: one value (un-normalised LL of level 1, Proposition 2) per 2 x 2 pixels
                     const u64 plane = (it.start - (u64)(it.ya * g.W)) / (unsigned)g.HW;
-                    const float *d = deep_plane(out, plane, g.HW) + (y >> 1) * ((g.W + 1) >> 1) + 4 * j;
-                    const int left = ((g.W + 1) >> 1) - 4 * j;
+                    const int W2 = (g.W + 1) >> 1, left = W2 - (x0 >> 1) - 4 * j;
+                    const float *d = (g.deep == 2 ? add + plane * (u64)(((g.H + 1) >> 1) * W2) : deep_plane(out, plane, g.HW)) + (y >> 1) * W2 +
+                                     (x0 >> 1) + 4 * j;
                     float add[4];
-                    if (left >= 4 && ((g.W + 1) >> 1 & 3) == 0 && (g.HW & 7) == 0) {
+                    if (left >= 4 && (W2 & 3) == 0 && (g.HW & 7) == 0) {
                         const float4 t4 = *reinterpret_cast<const float4 *>(d);
                         add[0] = t4.x; add[1] = t4.y; add[2] = t4.z; add[3] = t4.w;
                     } else {
@@ -531,16 +632,45 @@ tensor_kernel(const __grid_constant__ KGeom g, const T *__restrict__ x, const T 
                     for (int i = 0; i < 16; ++i) v[i] = fmaf(0.5f, add[(i & 7) >> 1], v[i]);
                 }
                 // the output image keeps the item's place inside its 16-byte word of global memory
+                // (panels: every row does; rows are tw + 8 pixels apart)
                 const int off = ((int)it.start + (it.ty * g.th - it.ya) * g.W) & 7;
-                T *d = reinterpret_cast<T *>(sb + g.out_off + (o * 8 + img) * g.out_stride) + off + r * g.W + 8 * j;
-                store8<T>(d, v, g.W - 8 * j, g.W);
-                if (y + 1 < g.H) store8<T>(d + g.W, v + 8, g.W - 8 * j, g.W);
+                T *d = reinterpret_cast<T *>(sb + g.out_off + (o * 8 + img) * g.out_stride);
+                if (PANEL) {
+                    const int first = (int)it.start + (y - it.ya) * g.W + x0;
+                    d += r * (g.tw + 8) + 8 * j;
+                    store8<T>(d + (first & 7), v, g.W - x0 - 8 * j, g.W);
+                    if (y + 1 < g.H) store8<T>(d + g.tw + 8 + ((first + g.W) & 7), v + 8, g.W - x0 - 8 * j, g.W);
+                } else {
+                    d += off + r * g.W + 8 * j;
+                    store8<T>(d, v, g.W - 8 * j, g.W);
+                    if (y + 1 < g.H) store8<T>(d + g.W, v + 8, g.W - 8 * j, g.W);
+                }
             }
             plane::fence_async_smem();
             worker_sync();
             // ---- the finished items to global memory: whole 16-byte words (one bulk copy an item where that is much; a bulk copy
             //      costs about 40 cycles whatever its size), the pixels before and behind them one by one
-            if (g.out_words >= BULK_WORDS) {
+            if (PANEL) {
+                const int words = g.n + 1, len = g.W - x0 < g.tw ? g.W - x0 : g.tw;
+                for (int e = tid; e < nslot * g.th * words; e += WORKERS) {
+                    const int rw = fdiv(e, g.d_out_words), w = e - rw * words, slot = rw / g.th, r = rw - slot * g.th;
+                    const Item it = it_u[slot];
+                    const int y = it.ty * g.th + r;
+                    if (it.ty < 0 || y >= g.H) continue;
+                    const u64 first = it.start + (u64)((y - it.ya) * g.W) + x0;
+                    const int rel = 8 * w - (int)(first & 7);
+                    const uint4 *s = reinterpret_cast<const uint4 *>(sb + g.out_off + slot * g.out_stride + r * (g.tw + 8) * 2) + w;
+                    T *d = out + (first + rel);
+                    if (rel >= 0 && rel + 8 <= len) {
+                        *reinterpret_cast<uint4 *>(d) = *s;
+                    } else {
+                        const T *p = reinterpret_cast<const T *>(s);
+#pragma unroll
+                        for (int i = 0; i < 8; ++i)
+                            if (rel + i >= 0 && rel + i < len) d[i] = p[i];
+                    }
+                }
+            } else if (g.out_words >= BULK_WORDS) {
                 for (int s0 = warp * 2; s0 < nslot; s0 += 16) {
                     const int slot = s0 + (lane >> 4), i = lane & 15;
                     const Item it = it_u[slot];
@@ -620,7 +750,7 @@ tensor_kernel(const __grid_constant__ KGeom g, const T *__restrict__ x, const T 
                     gsum = 0.f;
                 }
                 worker_sync();
-                const int slotp = blockIdx.x - block_of_unit((long long)c * g.upc, gridDim.x, g.units);
+                const int slotp = blockIdx.x - block_of_unit((long long)c * per_channel, gridDim.x, g.units);
                 const int KK = g.K * g.K, pad = (5 - g.K) / 2;
                 for (int e = tid; e < KK + 1 + (g.L >= 1 ? 4 * KK : 0); e += WORKERS) {
                     const float *G = mis + 128;
@@ -659,55 +789,103 @@ tensor_kernel(const __grid_constant__ KGeom g, const T *__restrict__ x, const T 
     if (warp == 8) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(g.cols));
 }
 
+// The level-1 low-pass band of every plane as floats: the carrier that levels >= 2 of wide planes are computed on.  One thread
+// makes four values of a row from 2 x 8 pixels.
+template <typename T>
+__global__ void __launch_bounds__(256) band_kernel(const T *__restrict__ x, int H, int W, int H2, int W2, u64 rows, float *__restrict__ X1) {
+    dependents_may_start();
+    wait_for_predecessor();
+    const int quads = (W2 + 3) >> 2;
+    for (u64 e = (u64)blockIdx.x * blockDim.x + threadIdx.x; e < rows * quads; e += (u64)gridDim.x * blockDim.x) {
+        const u64 row = e / quads;
+        const int j = (int)(e - row * quads), i = (int)(row % H2);
+        const T *p = x + (row / H2) * (u64)H * W + (u64)(2 * i) * W + 8 * j;
+        const bool y1 = 2 * i + 1 < H;
+        float a[8], c[8];
+        if ((W & 7) == 0) {
+            const uint4 t = __ldg(reinterpret_cast<const uint4 *>(p)), s = y1 ? __ldg(reinterpret_cast<const uint4 *>(p + W)) : make_uint4(0, 0, 0, 0);
+            const unsigned tv[4] = {t.x, t.y, t.z, t.w}, sv[4] = {s.x, s.y, s.z, s.w};
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const float2 f = unpack16(tv[q], T()), h = unpack16(sv[q], T());
+                a[2 * q] = f.x; a[2 * q + 1] = f.y; c[2 * q] = h.x; c[2 * q + 1] = h.y;
+            }
+        } else {
+#pragma unroll
+            for (int q = 0; q < 8; ++q) {
+                const bool in = 8 * j + q < W;
+                a[q] = in ? ldf(p + q) : 0.f;
+                c[q] = in && y1 ? ldf(p + W + q) : 0.f;
+            }
+        }
+        float *o = X1 + row * W2 + 4 * j;
+        float v[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) v[q] = 0.5f * ((a[2 * q] + a[2 * q + 1]) + (c[2 * q] + c[2 * q + 1]));
+        if ((W2 & 3) == 0) {
+            *reinterpret_cast<float4 *>(o) = make_float4(v[0], v[1], v[2], v[3]);
+        } else {
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+                if (4 * j + q < W2) o[q] = v[q];
+        }
+    }
+}
+template <typename T>
+cudaError_t band(int B, int C, int H, int W, const T *x, float *X1, cudaStream_t st) {
+    const int H2 = (H + 1) / 2, W2 = (W + 1) / 2;
+    const u64 rows = (u64)B * C * H2, n = rows * ((W2 + 3) / 4);
+    const u64 blocks = (n + 255) / 256;
+    return launch_overlapped(band_kernel<T>, (unsigned)(blocks < 148 * 8 * 8 ? blocks : 148 * 8 * 8), 256u, 0, st, x, H, W, H2, W2, rows, X1);
+}
+
 // ------------------------------------------------------------------ host side
 struct Request {
-    int bwd, B, C, H, W, L, K;
+    int bwd, B, C, H, W, L, K;  // L > 1 and planes beyond the on-chip kernels: levels >= 2 come as a tensor of addends
     bool operator==(const Request &o) const { return bwd == o.bwd && B == o.B && C == o.C && H == o.H && W == o.W && L == o.L && K == o.K; }
 };
 inline int up(int v, int m) { return (v + m - 1) / m * m; }
 
-inline bool search(const Request &q, KGeom &best) {
-    if ((q.K != 3 && q.K != 5) || q.L > 8 || q.W > 64 || q.H > 256 || q.H < 2 || q.W < 2) return false;
-    best = KGeom{};
-    best.cost = 1e30;
+inline bool wide(const Request &q) { return q.W > 64 || q.H > 128; }  // served in column panels
+
+inline bool search_n(const Request &q, KGeom &best, int n) {
     bool found = false;
     KGeom g = {};
-    g.deep = q.L > 1;
-    if (g.deep) {  // the addend lies in the planes' own place: a plane's items have to belong to one unit
-        plane::Geom d;
-        const int items = q.H <= 32 ? 1 : (q.H + 31) / 32;
-        if (q.K != 5 || items == 3 || (items > 4 && items != 8) || !plane::plan_deep(q.bwd, q.B, q.C, q.H, q.W, q.L, d)) return false;
-    }
+    g.deep = q.L > 1 ? (wide(q) ? 2 : 1) : 0;
     g.B = q.B; g.C = q.C; g.H = q.H; g.W = q.W; g.HW = q.H * q.W; g.L = q.L; g.K = q.K;
-    g.n = (q.W + 7) / 8;
+    g.n = n;
+    g.tw = 8 * n;
+    g.panels = (q.W + g.tw - 1) / g.tw;
     g.Pc = g.n + 1;
     g.Px = g.n + 2;
     // taller planes: 32 rows an item (a multiple of 16, so that the rows the weight gradients sum over are the item's own)
-    g.nty = q.H <= 32 ? 1 : (q.H + 31) / 32;
-    g.th = g.nty == 1 ? up(q.H, 2) : 32;
-    g.period = g.th + (g.nty == 1 ? 4 : 8);
+    const bool cut = q.H > 32 || wide(q);
+    g.nty = cut ? (q.H + 31) / 32 : 1;
+    g.th = cut ? 32 : up(q.H, 2);
+    g.period = g.th + (cut ? 8 : 4);
+    g.halo = cut ? 4 : 0;
     g.items = q.B * g.nty;
     g.d_nty = make_fastdiv(g.nty);
     g.d_period = make_fastdiv(g.period);
-    const int load_rows = g.nty == 1 ? q.H : g.th + 8, out_rows = g.nty == 1 ? q.H : g.th;
+    const int load_rows = cut ? g.th + 8 : q.H, out_rows = cut ? g.th : q.H;
     g.out_words = (out_rows * q.W * 2 + 14 + 15) / 16;
-    g.d_out_words = make_fastdiv(g.out_words);
-    g.raw_stride = up(load_rows * q.W * 2 + 30, 128) + 16;  // with the words' other pixels; items fall on different banks
-    g.out_stride = up(out_rows * q.W * 2 + 14, 128) + 16;
+    g.d_out_words = make_fastdiv(wide(q) ? n + 1 : g.out_words);
+    g.raw_stride = wide(q) ? 0 : up(load_rows * q.W * 2 + 30, 128) + 16;  // with the words' other pixels; items fall on different banks
+    g.out_stride = wide(q) ? up(g.th * (g.tw + 8) * 2, 128) + 16 : up(out_rows * q.W * 2 + 14, 128) + 16;
     g.d_n = make_fastdiv(g.n);
     g.d_Pc = make_fastdiv(g.Pc);
     g.d_Px = make_fastdiv(g.Px);
     g.d_ec = make_fastdiv(load_rows * g.Pc);
     g.d_ex = make_fastdiv(load_rows * g.Px);
     const int sides = q.bwd ? 2 : 1;
-    for (int alias = 0; alias < 2; ++alias)
+    for (int alias = 0; alias < (wide(q) ? 1 : 2); ++alias)
     for (int S = 1; S <= 16; ++S) {
         if (S > 1 && 8 * (S - 1) >= g.items) break;
         KGeom h = g;
         h.S = S;
         const int used = (S - 1) * h.period + h.th;
         h.T = (used + 31) / 32;
-        h.Ws = h.nty == 1 ? (used + 15) / 16 : 2 * S;
+        h.Ws = h.halo ? 2 * S : (used + 15) / 16;
         h.rows = 32 * h.T + 8;
         if (h.rows < 16 * h.Ws + 16) h.rows = 16 * h.Ws + 16;
         int off = 0;
@@ -725,8 +903,8 @@ inline bool search(const Request &q, KGeom &best) {
         h.smem = up(off, 128);
         if (h.smem > plane::SMEM_LIMIT) break;
         h.upc = (h.items + 8 * S - 1) / (8 * S);
-        if ((long long)h.upc * q.C > 0x3fffffffLL) continue;
-        h.units = h.upc * q.C;
+        if ((long long)h.upc * h.panels * q.C > 0x3fffffffLL) continue;
+        h.units = h.upc * h.panels * q.C;
         for (int bps = 1; bps <= 2; ++bps) {  // 112 registers a thread
             if ((long long)bps * (h.smem + 1024) > plane::SMEM_PER_SM) break;
             h.cols = 512 / bps;
@@ -749,10 +927,27 @@ inline bool search(const Request &q, KGeom &best) {
             }
         }
     }
+    return found;
+}
+inline bool search(const Request &q, KGeom &best) {
+    if ((q.K != 3 && q.K != 5) || q.L > 8 || q.H < 2 || q.W < 2 || (long long)q.H * q.W > 0x3fffffff) return false;
+    if (wide(q) ? q.W < 8 : false) return false;
+    if (q.L > 1 && !wide(q)) {  // the addend lies in the planes' own place: a plane's items have to belong to one unit
+        plane::Geom d;
+        if (q.K != 5 || (q.H > 64 && q.H <= 96) || !plane::plan_deep(q.bwd, q.B, q.C, q.H, q.W, q.L, d)) return false;
+    }
+    best = KGeom{};
+    best.cost = 1e30;
+    bool found = false;
+    if (wide(q))
+        for (int n = 3; n <= 8; ++n) found |= search_n(q, best, n);
+    else
+        found = search_n(q, best, (q.W + 7) / 8);
     if (!found) return false;
     best.np = 1;
+    const long long per = (long long)best.upc * best.panels;
     for (int ch = 0; ch < best.C; ++ch) {
-        const int n = block_of_unit((long long)(ch + 1) * best.upc - 1, best.nblocks, best.units) - block_of_unit((long long)ch * best.upc, best.nblocks, best.units) + 1;
+        const int n = block_of_unit((ch + 1) * per - 1, best.nblocks, best.units) - block_of_unit(ch * per, best.nblocks, best.units) + 1;
         if (n > best.np) best.np = n;
     }
     return true;
@@ -793,31 +988,37 @@ inline size_t backward_bytes(const Request &q) {
     const size_t KK = (size_t)q.K * q.K;
     size_t floats = (size_t)g.C * g.np * (KK + 1 + 4 * KK);
     plane::Geom d;
-    if (q.L > 1 && plane::plan_deep(true, q.B, q.C, q.H, q.W, q.L, d)) floats += (size_t)(q.L - 1) * q.C * d.np * 4 * KK;
+    if (q.L > 1 && !wide(q) && plane::plan_deep(true, q.B, q.C, q.H, q.W, q.L, d)) floats += (size_t)(q.L - 1) * q.C * d.np * 4 * KK;
     return STATUS_BYTES + sizeof(float) * floats;
 }
 
 template <typename T>
 cudaError_t forward(const Request &q, const T *x, const float *w0, const float *s0, const float *b0, const float *wl, const float *sl, T *out,
-                    char *ws, cudaStream_t st, unsigned tag, bool no_copy) {
+                    char *ws, cudaStream_t st, unsigned tag, bool no_copy, const float *add) {
     KGeom g;
     if (!plan(q, g)) return cudaErrorInvalidValue;
     g.tag = tag;
     g.alarm = call_alarm;
     g.no_copy = no_copy;
-    constexpr auto kern = tensor_kernel<T, false>;
-    cudaError_t e = plane::opt_in_smem<kern>();
-    if (e != cudaSuccess) return e;
+    cudaError_t e;
+    if (wide(q)) {
+        constexpr auto kern = tensor_kernel<T, false, true>;
+        if ((e = plane::opt_in_smem<kern>()) != cudaSuccess) return e;
+        return launch_overlapped(kern, (unsigned)g.nblocks, (unsigned)THREADS, (size_t)g.smem, st, g, x, nullptr, w0, s0, b0, wl, sl, add, out,
+                                 nullptr, nullptr, reinterpret_cast<int *>(ws));
+    }
+    constexpr auto kern = tensor_kernel<T, false, false>;
+    if ((e = plane::opt_in_smem<kern>()) != cudaSuccess) return e;
     if (q.L > 1 && (e = plane::deep_forward<T>(q.B, q.C, q.H, q.W, q.L, x, wl + (size_t)q.C * 4 * q.K * q.K, sl + (size_t)q.C * 4, out,
                                                reinterpret_cast<int *>(ws), st, tag, no_copy)) != cudaSuccess)
         return e;
-    return launch_overlapped(kern, (unsigned)g.nblocks, (unsigned)THREADS, (size_t)g.smem, st, g, x, nullptr, w0, s0, b0, wl, sl, out, nullptr,
+    return launch_overlapped(kern, (unsigned)g.nblocks, (unsigned)THREADS, (size_t)g.smem, st, g, x, nullptr, w0, s0, b0, wl, sl, add, out, nullptr,
                              nullptr, reinterpret_cast<int *>(ws));
 }
 
 template <typename T>
 cudaError_t backward(const Request &q, const T *x, const T *go, const float *w0, const float *s0, const float *wl, const float *sl, bool bias,
-                     T *gx, char *ws, EpiloguePtrs *ep, cudaStream_t st, unsigned tag, bool no_copy) {
+                     T *gx, char *ws, EpiloguePtrs *ep, cudaStream_t st, unsigned tag, bool no_copy, const float *add) {
     KGeom g;
     if (!plan(q, g)) return cudaErrorInvalidValue;
     g.tag = tag;
@@ -826,35 +1027,43 @@ cudaError_t backward(const Request &q, const T *x, const T *go, const float *w0,
     g.bias = bias;
     const size_t KK = (size_t)q.K * q.K;
     float *part0 = reinterpret_cast<float *>(ws + STATUS_BYTES), *partl = part0 + (size_t)g.C * g.np * (KK + 1);
-    constexpr auto kern = tensor_kernel<T, true>;
-    cudaError_t e = plane::opt_in_smem<kern>();
-    if (e != cudaSuccess) return e;
-    if (q.L > 1 && (e = plane::deep_backward<T>(q.B, q.C, q.H, q.W, q.L, x, go, wl + (size_t)q.C * 4 * KK, sl + (size_t)q.C * 4, gx,
-                                                partl + (size_t)g.C * g.np * 4 * KK, ep, reinterpret_cast<int *>(ws), st, tag, no_copy)) != cudaSuccess)
-        return e;
-    e = launch_overlapped(kern, (unsigned)g.nblocks, (unsigned)THREADS, (size_t)g.smem, st, g, x, go, w0, s0, nullptr, wl, sl, gx, part0, partl,
-                          reinterpret_cast<int *>(ws));
+    cudaError_t e;
+    if (wide(q)) {
+        constexpr auto kern = tensor_kernel<T, true, true>;
+        if ((e = plane::opt_in_smem<kern>()) != cudaSuccess) return e;
+        e = launch_overlapped(kern, (unsigned)g.nblocks, (unsigned)THREADS, (size_t)g.smem, st, g, x, go, w0, s0, nullptr, wl, sl, add, gx, part0,
+                              partl, reinterpret_cast<int *>(ws));
+    } else {
+        constexpr auto kern = tensor_kernel<T, true, false>;
+        if ((e = plane::opt_in_smem<kern>()) != cudaSuccess) return e;
+        if (q.L > 1 && (e = plane::deep_backward<T>(q.B, q.C, q.H, q.W, q.L, x, go, wl + (size_t)q.C * 4 * KK, sl + (size_t)q.C * 4, gx,
+                                                    partl + (size_t)g.C * g.np * 4 * KK, ep, reinterpret_cast<int *>(ws), st, tag, no_copy)) != cudaSuccess)
+            return e;
+        e = launch_overlapped(kern, (unsigned)g.nblocks, (unsigned)THREADS, (size_t)g.smem, st, g, x, go, w0, s0, nullptr, wl, sl, add, gx, part0,
+                              partl, reinterpret_cast<int *>(ws));
+    }
     if (e != cudaSuccess) return e;
     ep->part0 = part0;
     ep->np0 = g.np;
     ep->partl[0] = partl;
     ep->npl[0] = g.np;
-    ep->grp = 1; ep->B = g.upc; ep->units = g.units; ep->nblocks = g.nblocks;
+    ep->grp = 1; ep->B = g.upc * g.panels; ep->units = g.units; ep->nblocks = g.nblocks;
     return cudaSuccess;
 }
 
 inline int describe(const Request &q, char *buf, size_t n) {
     KGeom g;
     if (!plan(q, g)) return 0;
-    const int o = snprintf(buf, n, "%s[tensor S=%d T=%d n=%d bps=%d ring=%d np=%d smem=%d]", q.bwd ? "bwd" : "fwd", g.S, g.T, g.n, g.bps, g.ring, g.np, g.smem);
+    const int o = snprintf(buf, n, "%s[tensor S=%d T=%d n=%d panels=%d bps=%d ring=%d np=%d smem=%d]", q.bwd ? "bwd" : "fwd", g.S, g.T, g.n, g.panels, g.bps, g.ring, g.np, g.smem);
     return o < 0 ? 0 : o;
 }
 
-#define WT_TENSOR_INSTANTIATE(T, EXTERN)                                                                                       \
+#define WT_TENSOR_INSTANTIATE(T, EXTERN)                                                                                        \
+    EXTERN template cudaError_t band<T>(int, int, int, int, const T *, float *, cudaStream_t);                                                                                        \
     EXTERN template cudaError_t forward<T>(const Request &, const T *, const float *, const float *, const float *, const float *, \
-                                           const float *, T *, char *, cudaStream_t, unsigned, bool);                           \
+                                           const float *, T *, char *, cudaStream_t, unsigned, bool, const float *);            \
     EXTERN template cudaError_t backward<T>(const Request &, const T *, const T *, const float *, const float *, const float *,    \
-                                            const float *, bool, T *, char *, EpiloguePtrs *, cudaStream_t, unsigned, bool);
+                                            const float *, bool, T *, char *, EpiloguePtrs *, cudaStream_t, unsigned, bool, const float *);
 
 }  // namespace tensor
 }  // namespace wt

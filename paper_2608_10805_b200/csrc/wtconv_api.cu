@@ -114,7 +114,7 @@ __global__ void resolve_status_kernel(int *status) {
 struct Route {
     wtconv_desc key;
     bool set;
-    bool team, plane, window, tensor, k3;  // plane: any family that keeps whole planes on chip; k3: 3 x 3 kernels in 5 x 5 tables
+    bool team, plane, window, tensor[2], k3;  // plane: any family that keeps whole planes on chip; k3: 3 x 3 kernels in 5 x 5 tables
     size_t fwd_bytes, bwd_bytes;
 };
 const Route &route(const wtconv_desc *d);
@@ -124,7 +124,7 @@ bool use_ref_chain(const wtconv_desc *d) { return (d->flags & WTCONV_FLAG_REFERE
 bool use_team_path(const wtconv_desc *d) { return route(d).team; }
 bool use_plane_path(const wtconv_desc *d) { return route(d).plane; }
 bool use_window_path(const wtconv_desc *d) { return route(d).window; }
-bool use_tensor_path(const wtconv_desc *d) { return route(d).tensor; }
+bool use_tensor_path(const wtconv_desc *d, int bwd) { return route(d).tensor[bwd]; }
 wt::tensor::Request tensor_request(const wtconv_desc *d, int bwd) { return {bwd, d->B, d->C, d->H, d->W, d->L, d->k}; }
 // k = 3 through the k = 5 kernels.  A 3 x 3 depthwise kernel is a 5 x 5 kernel with a border of zeros, so wherever the
 // kernels that keep planes on chip (k = 5 only) serve the shape, the parameters are copied into 5 x 5 tables at the
@@ -184,10 +184,10 @@ wtconv_status forward_tk(const wtconv_desc *d, const void *x, const float *w0, c
                          const float *wl, const float *sl, void *out, char *ws, cudaStream_t st, int taps = 5) {
     if (use_ref_chain(d)) return wt::refchain::forward<T, K>(d, (const T *)x, w0, s0, b0, wl, sl, (T *)out, ws, st);
     if constexpr (K != 7 && sizeof(T) == 2) {
-        if (taps == 5 && use_tensor_path(d))
+        if (taps == 5 && use_tensor_path(d, 0))
             return wt::tensor::forward<T>(tensor_request(d, 0), (const T *)x, w0, s0, b0, wl, sl, (T *)out,
                                           ws + (use_k3_embedding(d) ? embed_layout(d).inner : 0), st, next_status_tag(),
-                                          (d->flags & WTCONV_FLAG_TEST_NO_COPY) != 0) == cudaSuccess
+                                          (d->flags & WTCONV_FLAG_TEST_NO_COPY) != 0, nullptr) == cudaSuccess
                        ? WTCONV_OK
                        : WTCONV_ERR_CUDA;
     }
@@ -236,11 +236,11 @@ wtconv_status backward_tk(const wtconv_desc *d, const void *x, const void *g, co
         return wt::refchain::backward<T, K>(d, (const T *)x, (const T *)g, w0, s0, b0, wl, sl, (T *)gx, gw0, gs0, gb0, gwl, gsl,
                                             ws, st);
     if constexpr (K != 7 && sizeof(T) == 2) {
-        if (taps == 5 && use_tensor_path(d)) {
+        if (taps == 5 && use_tensor_path(d, 1)) {
             wt::EpiloguePtrs ep = {};
             if (wt::tensor::backward<T>(tensor_request(d, 1), (const T *)x, (const T *)g, w0, s0, wl, sl, b0 != nullptr, (T *)gx,
                                         ws + (use_k3_embedding(d) ? embed_layout(d).inner : 0), &ep, st, next_status_tag(),
-                                        (d->flags & WTCONV_FLAG_TEST_NO_COPY) != 0) != cudaSuccess)
+                                        (d->flags & WTCONV_FLAG_TEST_NO_COPY) != 0, nullptr) != cudaSuccess)
                 return WTCONV_ERR_CUDA;
             return launch_epilogue(d, ep, w0, s0, b0, wl, sl, gw0, gs0, gb0, gwl, gsl, st);
         }
@@ -311,10 +311,10 @@ wtconv_status backward_tk(const wtconv_desc *d, const void *x, const void *g, co
 size_t fwd_ws_bytes(const wtconv_desc *d) { return route(d).fwd_bytes; }
 size_t bwd_ws_bytes(const wtconv_desc *d) { return route(d).bwd_bytes; }
 
-bool tensor_serves(const wtconv_desc *d, bool on_chip) {
+bool tensor_serves(const wtconv_desc *d, bool on_chip, int bwd) {
     if (d->dtype == WTCONV_F32 || !on_chip || (d->flags & ~WTCONV_FLAG_TEST_NO_COPY)) return false;
     wt::tensor::KGeom g;
-    return wt::tensor::plan(tensor_request(d, 0), g) && wt::tensor::plan(tensor_request(d, 1), g);
+    return wt::tensor::plan(tensor_request(d, bwd), g);
 }
 
 Route find_route(const wtconv_desc *d) {
@@ -346,18 +346,14 @@ Route find_route(const wtconv_desc *d) {
         if (r5.plane || r5.window) {
             r.k3 = true;
             const size_t head = embed_layout(d).inner;
-            r.tensor = tensor_serves(d, r5.plane);
-            const size_t own = r.tensor ? align_up(wt::tensor::backward_bytes(tensor_request(d, 1))) : 0;
+            for (int bwd = 0; bwd < 2; ++bwd) r.tensor[bwd] = tensor_serves(d, r5.plane, bwd);
+            const size_t own = r.tensor[1] ? align_up(wt::tensor::backward_bytes(tensor_request(d, 1))) : 0;
             r.fwd_bytes = head + r5.fwd_bytes;
             r.bwd_bytes = head + (own > r5.bwd_bytes ? own : r5.bwd_bytes);
             return r;
         }
     }
-    r.tensor = d->k == 5 && tensor_serves(d, r.plane);
-    if (r.tensor) {
-        r.fwd_bytes = align_up(wt::tensor::STATUS_BYTES);
-        r.bwd_bytes = align_up(wt::tensor::backward_bytes(tensor_request(d, 1)));
-    } else if (r.team) {
+    if (r.team) {
         r.fwd_bytes = align_up(wt::plane::STATUS_BYTES);
         r.bwd_bytes = align_up(wt::team::backward_workspace_bytes(d->B, d->C, d->H, d->W, d->L, eb, team_force_g(d)));
     } else if (r.plane) {
@@ -372,6 +368,9 @@ Route find_route(const wtconv_desc *d) {
         r.fwd_bytes = p.fwd_bytes;
         r.bwd_bytes = p.bwd_bytes;
     }
+    for (int bwd = 0; bwd < 2; ++bwd) r.tensor[bwd] = d->k == 5 && tensor_serves(d, r.plane, bwd);
+    if (r.tensor[0]) r.fwd_bytes = align_up(wt::tensor::STATUS_BYTES);
+    if (r.tensor[1]) r.bwd_bytes = align_up(wt::tensor::backward_bytes(tensor_request(d, 1)));
     return r;
 }
 const Route &route(const wtconv_desc *d) {
@@ -524,15 +523,19 @@ wtconv_status wtconv_plan_describe(const wtconv_desc *d, char *buf, size_t n) {
     if (st != WTCONV_OK) return st;
     if (!buf || n == 0) return WTCONV_ERR_NULL;
     buf[0] = 0;
-    if (use_tensor_path(d)) {  // the family's name as callers know it, then the plans that run
-        size_t o = (size_t)snprintf(buf, n, "%s%s ", use_k3_embedding(d) ? "3x3 kernels in 5x5 tables: " : "", wtconv_plan_name(d));
-        if (o < n) o += (size_t)wt::tensor::describe(tensor_request(d, 0), buf + o, n - o);
-        if (o + 1 < n) {
-            buf[o++] = ' ';
-            buf[o] = 0;
-            wt::tensor::describe(tensor_request(d, 1), buf + o, n - o);
-        }
-        return WTCONV_OK;
+    if (use_tensor_path(d, 0) || use_tensor_path(d, 1)) {  // the family's name as callers know it, then the plans that run
+        size_t o = (size_t)snprintf(buf, n, "%s%s", use_k3_embedding(d) ? "3x3 kernels in 5x5 tables: " : "", wtconv_plan_name(d));
+        for (int bwd = 0; bwd < 2; ++bwd)
+            if (use_tensor_path(d, bwd) && o + 1 < n) {
+                buf[o++] = ' ';
+                buf[o] = 0;
+                o += (size_t)wt::tensor::describe(tensor_request(d, bwd), buf + o, n - o);
+            }
+        if (use_tensor_path(d, 0) && use_tensor_path(d, 1)) return WTCONV_OK;
+        if (o < n) o += (size_t)snprintf(buf + o, n - o, "; the other direction: ");
+        if (o >= n) return WTCONV_OK;
+        buf += o;
+        n -= o;
     }
     if (use_k3_embedding(d)) {
         const wtconv_desc d5 = as_k5(d);
@@ -586,7 +589,7 @@ wtconv_status wtconv_launch_count(const wtconv_desc *d, int32_t *fwd, int32_t *b
         if (bwd) {
             wt::plane::Geom gq;
             /* fused backward + epilogue, or weight-gradient + input-gradient + epilogue (and nothing else on the stream) */
-            *bwd = use_tensor_path(d) || wt::plane::plan_bwd_fused(d->B, d->C, d->H, d->W, d->L, (int)elem_bytes(d->dtype), gq, d->flags >> 8) ? 2 : 3;
+            *bwd = use_tensor_path(d, 1) || wt::plane::plan_bwd_fused(d->B, d->C, d->H, d->W, d->L, (int)elem_bytes(d->dtype), gq, d->flags >> 8) ? 2 : 3;
         }
     } else {
         if (fwd) *fwd = d->L + 1;
