@@ -66,7 +66,7 @@ struct KGeom {
     int conv_off, x_off, parts_off, raw_off, out_off, table_off, misc_off, smem;  // byte offsets
     int ring, cols;              // tensor-memory ring depth and columns allocated
     int bps, nblocks, np;
-    int no_copy, bias, deep;     // deep: 1 the addend lies in the planes' own place, 2 in a tensor of its own
+    int no_copy, bias, deep;     // deep: levels >= 2 come as a float addend per 2 x 2 pixels, 1 in the planes' own place, 2 in a tensor
     FastDiv d_period, d_nty, d_n, d_Pc, d_Px, d_ec, d_ex, d_out_words;  // d_ec / d_ex: chunks of one octet in the convolved / the x array
     int *alarm;
     unsigned tag;
@@ -114,7 +114,10 @@ __device__ __forceinline__ unsigned elect_one() {
     asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(p));
     return p;
 }
-__device__ __forceinline__ void worker_sync() { asm volatile("bar.sync 1, 256;" ::: "memory"); }
+__device__ __forceinline__ void worker_sync() {
+    __syncwarp();
+    asm volatile("bar.sync 1, 256;" ::: "memory");
+}
 
 // ------------------------------------------------------------------ 16-bit packing
 __device__ __forceinline__ unsigned pack16(float a, float b, __nv_bfloat16) {
@@ -141,21 +144,24 @@ template <typename T> __device__ __forceinline__ float weight_part(float w, int 
 // ------------------------------------------------------------------ loading
 // An item of a unit, worked out once for the whole block.
 struct __align__(16) Item {
-    u64 start;  // element index of its first loaded pixel
-    int ty;     // item row, or -1: no such item
-    int ya;     // first row loaded
+    unsigned plane;  // image x channels + channel
+    int ty;          // item row, or -1: no such item
+    int ya;          // first row loaded
+    int unused;
+    __device__ u64 at(const KGeom &g, int y) const { return (u64)plane * (unsigned)g.HW + (unsigned)(y * g.W); }  // element index of row y
 };
 __device__ __forceinline__ Item find_item(const KGeom &g, int c, int k, int slot) {
     Item it;
     it.ty = -1;
     it.ya = 0;
-    it.start = 0;
+    it.plane = 0;
+    it.unused = 0;
     const int i = k * 8 * g.S + slot;
     if (i < g.items) {
         const int b = g.nty == 1 ? i : fdiv(i, g.d_nty);
         it.ty = i - b * g.nty;
         if (it.ty > 0) it.ya = it.ty * g.th - 4;
-        it.start = ((u64)b * g.C + c) * g.HW + (u64)(it.ya * g.W);
+        it.plane = (unsigned)b * g.C + c;
     }
     return it;
 }
@@ -175,7 +181,7 @@ __device__ __forceinline__ void fetch_unit(const Item *items, char *raw, int raw
             if (it.ty < 0) continue;
             int rows = g.H - it.ya;
             if (g.halo && it.ty * g.th + g.th + 4 < g.H) rows = it.ty * g.th + g.th + 4 - it.ya;
-            const u64 first = it.start * 2 & ~15ull, last = it.start * 2 + (unsigned)(rows * g.W * 2);
+            const u64 start = it.at(g, it.ya), first = start * 2 & ~15ull, last = start * 2 + (unsigned)(rows * g.W * 2);
             u64 end = (last + 15) & ~15ull;
             const bool tail = end > total;
             if (tail) end -= 16;
@@ -213,7 +219,7 @@ __device__ __forceinline__ void repack(char *arr, const char *raw, const Item *i
     for (int o = warp / wpo; o < g.S; o += 8 / wpo) {
         const Item it = items[o * 8 + img];
         const int ybase = it.ty * g.th + r0;
-        const char *src = raw + (o * 8 + img) * g.raw_stride + (((int)it.start & 7) + (ybase - it.ya) * g.W - shift) * 2;
+        const char *src = raw + (o * 8 + img) * g.raw_stride + (((int)it.at(g, it.ya) & 7) + (ybase - it.ya) * g.W - shift) * 2;
         char *dst = arr + (((o * g.period + 4 + r0) * P) * 8 + img) * 16;
         for (int e0 = e_first; e0 < per; e0 += U * step) {
             unsigned v[U][4];
@@ -268,7 +274,7 @@ __device__ __forceinline__ void repack_panel(char *arr, const T *__restrict__ sr
     for (int o = warp / wpo; o < g.S; o += 8 / wpo) {
         const Item it = items[o * 8 + img];
         const int ybase = it.ty * g.th - 4;
-        const long long e_base = (long long)it.start + (long long)(ybase - it.ya) * g.W + x0 - shift;
+        const long long e_base = (long long)it.at(g, 0) + (long long)ybase * g.W + x0 - shift;
         char *dst = arr + ((o * g.period * P) * 8 + img) * 16;
         for (int e0 = e_first; e0 < per; e0 += U * step) {
             unsigned v[U][4], h[U][4];
@@ -446,7 +452,7 @@ tensor_kernel(const __grid_constant__ KGeom g, const T *__restrict__ x, const T 
     u64 *full = reinterpret_cast<u64 *>(mis + 560), *empty = full + MAX_RING, *done = empty + MAX_RING, *landed = done + 1;
     volatile int *dead = reinterpret_cast<volatile int *>(landed + 1);
     unsigned *tmem_slot = reinterpret_cast<unsigned *>(landed + 1) + 1;
-    Item *items = reinterpret_cast<Item *>(mis + 600);  // two sets: a unit is fetched while the one before it is worked on
+    Item *items = reinterpret_cast<Item *>(mis + 600);  // three sets: the next unit is listed while the slowest warps still copy the one before this one out
     const int nslot = 8 * g.S;
     const int u_begin = (int)((long long)blockIdx.x * g.units / gridDim.x), u_end = (int)((long long)(blockIdx.x + 1) * g.units / gridDim.x);
     const unsigned limit = g.no_copy ? plane::WAIT_LIMIT_TEST : WAIT_LIMIT;
@@ -464,6 +470,7 @@ tensor_kernel(const __grid_constant__ KGeom g, const T *__restrict__ x, const T 
         plane::mbar_init(done, ISSUERS);
         plane::mbar_init(landed, 1);
     }
+    __syncwarp();  // warp-collective instructions below, here and elsewhere: the lanes have to be together, loops may have parted them
     if (warp == 8) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(plane::smem_addr(tmem_slot)), "r"(g.cols) : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
@@ -486,6 +493,7 @@ tensor_kernel(const __grid_constant__ KGeom g, const T *__restrict__ x, const T 
     int c = u_begin / per_channel, k = u_begin - c * per_channel, c_prev = -1;
     const int jobs = g.T * g.n;
     unsigned job0 = 0, unit = 0;  // jobs issued before this unit, units done
+    int set_u = 0;                // item list of the unit
     float gsum = 0.f, wreg = 0.f, breg = 0.f;
     auto fetch_weights = [&](int cc) {  // ahead of the channel that needs them
         if (tid < 125) wreg = folded_weight(g, cc, tid, BWD, w0, s0, wl, sl);
@@ -507,14 +515,15 @@ tensor_kernel(const __grid_constant__ KGeom g, const T *__restrict__ x, const T 
         int cn = c, kn = k + 1;
         if (kn == per_channel) { kn = 0; ++cn; }
         const int panel = PANEL ? k / g.upc : 0, x0 = panel * g.tw;  // units of a channel: panel by panel
-        const Item *it_u = items + (unit & 1u) * nslot;
+        const Item *it_u = items + set_u * nslot;
+        const int set_next = set_u == 2 ? 0 : set_u + 1;
         if (worker) {
             if (c != c_prev) {  // the MMAs that read the old table have completed (see the wait at the end of a unit)
                 if (tid < 125) mis[tid] = wreg;
                 if (tid == 0) mis[545] = breg;
                 build_table<T>(table, sb + g.parts_off, mis, tid);
             }
-            if (u + 1 < u_end) list_items((unit + 1) & 1u, cn, kn);
+            if (u + 1 < u_end) list_items(set_next, cn, kn);
             if (!PANEL) wait_for(landed, unit & 1u);
             plane::bulk_store_wait_read();  // the output image may be written again behind the next barriers
         }
@@ -544,7 +553,10 @@ tensor_kernel(const __grid_constant__ KGeom g, const T *__restrict__ x, const T 
                 const unsigned rowb = (unsigned)g.Pc * 128, a0 = plane::smem_addr(conv);
                 const u64 adesc = smem_desc(a0, 128, 2 * rowb), bdesc = smem_desc(plane::smem_addr(table), (NCOL / 8) * 128, 128);
                 constexpr unsigned id = instr_desc<T>(NCOL, false);
-                for (int q = iw; q < jobs; q += ISSUERS) {
+                // a ring slot always belongs to the same issuer and to the same epilogue warps (the ring is a multiple of both), so
+                // whoever waits for a phase of its barriers has seen the phase before it
+                const int ni = g.ring < ISSUERS ? g.ring : ISSUERS;
+                for (int q = iw < ni ? (int)((iw - job0) & (ni - 1)) : jobs; q < jobs; q += ni) {
                     const int t = fdiv(q, g.d_n), j = q - t * g.n;
                     const unsigned jc = job0 + q, s = jc % (unsigned)g.ring;
                     wait_for(empty + s, ((jc / (unsigned)g.ring) & 1u) ^ 1u);
@@ -580,13 +592,13 @@ tensor_kernel(const __grid_constant__ KGeom g, const T *__restrict__ x, const T 
             }
         } else {
             if (u + 1 < u_end) {
-                if (!g.alias) fetch((unit + 1) & 1u);
+                if (!g.alias) fetch(set_next);
                 if (cn != c) fetch_weights(cn);
             }
-            // ---- epilogue: warps 0-3 take the even jobs, 4-7 the odd ones; a lane is one image of one row pair
+            // ---- epilogue: warps 0-3 take the even jobs (counted over the units), 4-7 the odd ones; a lane is one image of one row pair
             const int m = (warp & 3) * 32 + lane, img = m & 7;
             const float scale = mis[544], bias = mis[545];
-            for (int q = warp >> 2; q < jobs; q += 2) {
+            for (int q = (int)(((warp >> 2) - job0) & 1u); q < jobs; q += 2) {
                 const int t = fdiv(q, g.d_n), j = q - t * g.n;
                 const unsigned jc = job0 + q, s = jc % (unsigned)g.ring;
                 wait_for(full + s, (jc / (unsigned)g.ring) & 1u);
@@ -601,6 +613,7 @@ tensor_kernel(const __grid_constant__ KGeom g, const T *__restrict__ x, const T 
                 Item it;
                 it.ty = -1;
                 if (o < g.S && r < g.th) it = it_u[o * 8 + img];
+                __syncwarp();
                 tmem_ld_wait();
                 tmem_arrived(v);
                 tmem_arrived(p1);
@@ -616,27 +629,26 @@ tensor_kernel(const __grid_constant__ KGeom g, const T *__restrict__ x, const T 
                     else v[i] = (v[i] + (p1[i] + p2[i])) + bias;
                 }
                 if (g.deep) {  // levels >= 2: one value (un-normalised LL of level 1, Proposition 2) per 2 x 2 pixels
-                    const u64 plane = (it.start - (u64)(it.ya * g.W)) / (unsigned)g.HW;
                     const int W2 = (g.W + 1) >> 1, left = W2 - (x0 >> 1) - 4 * j;
-                    const float *d = (g.deep == 2 ? add + plane * (u64)(((g.H + 1) >> 1) * W2) : deep_plane(out, plane, g.HW)) + (y >> 1) * W2 +
+                    const float *d = (PANEL ? add + (u64)it.plane * (unsigned)(((g.H + 1) >> 1) * W2) : deep_plane(out, it.plane, g.HW)) + (y >> 1) * W2 +
                                      (x0 >> 1) + 4 * j;
-                    float add[4];
-                    if (left >= 4 && (W2 & 3) == 0 && (g.HW & 7) == 0) {
+                    float more[4];
+                    if (left >= 4 && (W2 & 3) == 0 && (PANEL || (g.HW & 7) == 0)) {
                         const float4 t4 = *reinterpret_cast<const float4 *>(d);
-                        add[0] = t4.x; add[1] = t4.y; add[2] = t4.z; add[3] = t4.w;
+                        more[0] = t4.x; more[1] = t4.y; more[2] = t4.z; more[3] = t4.w;
                     } else {
 #pragma unroll
-                        for (int i = 0; i < 4; ++i) add[i] = i < left ? d[i] : 0.f;
+                        for (int i = 0; i < 4; ++i) more[i] = i < left ? d[i] : 0.f;
                     }
 #pragma unroll
-                    for (int i = 0; i < 16; ++i) v[i] = fmaf(0.5f, add[(i & 7) >> 1], v[i]);
+                    for (int i = 0; i < 16; ++i) v[i] = fmaf(0.5f, more[(i & 7) >> 1], v[i]);
                 }
                 // the output image keeps the item's place inside its 16-byte word of global memory
                 // (panels: every row does; rows are tw + 8 pixels apart)
-                const int off = ((int)it.start + (it.ty * g.th - it.ya) * g.W) & 7;
+                const int off = (int)it.at(g, it.ty * g.th) & 7;
                 T *d = reinterpret_cast<T *>(sb + g.out_off + (o * 8 + img) * g.out_stride);
                 if (PANEL) {
-                    const int first = (int)it.start + (y - it.ya) * g.W + x0;
+                    const int first = (int)it.at(g, y) + x0;
                     d += r * (g.tw + 8) + 8 * j;
                     store8<T>(d + (first & 7), v, g.W - x0 - 8 * j, g.W);
                     if (y + 1 < g.H) store8<T>(d + g.tw + 8 + ((first + g.W) & 7), v + 8, g.W - x0 - 8 * j, g.W);
@@ -657,7 +669,7 @@ tensor_kernel(const __grid_constant__ KGeom g, const T *__restrict__ x, const T 
                     const Item it = it_u[slot];
                     const int y = it.ty * g.th + r;
                     if (it.ty < 0 || y >= g.H) continue;
-                    const u64 first = it.start + (u64)((y - it.ya) * g.W) + x0;
+                    const u64 first = it.at(g, y) + x0;
                     const int rel = 8 * w - (int)(first & 7);
                     const uint4 *s = reinterpret_cast<const uint4 *>(sb + g.out_off + slot * g.out_stride + r * (g.tw + 8) * 2) + w;
                     T *d = out + (first + rel);
@@ -676,7 +688,7 @@ tensor_kernel(const __grid_constant__ KGeom g, const T *__restrict__ x, const T 
                     const Item it = it_u[slot];
                     if (it.ty < 0) continue;
                     const int y0 = it.ty * g.th, len = (g.H - y0 < g.th ? g.H - y0 : g.th) * g.W;
-                    const u64 first = it.start + (u64)((y0 - it.ya) * g.W);
+                    const u64 first = it.at(g, y0);
                     const int at = (int)(first & 7), lo = (8 - at) & 7, hi = ((at + len) & ~7) - at;  // whole words: [lo, hi) of [0, len)
                     const T *s = reinterpret_cast<const T *>(sb + g.out_off + slot * g.out_stride) + at;
                     if (i == 0) plane::bulk_s2g(out + first + lo, s + lo, (unsigned)(hi - lo) * 2);
@@ -689,7 +701,7 @@ tensor_kernel(const __grid_constant__ KGeom g, const T *__restrict__ x, const T 
                     const Item it = it_u[slot];
                     if (it.ty < 0) continue;
                     const int y0 = it.ty * g.th, len = (g.H - y0 < g.th ? g.H - y0 : g.th) * g.W;
-                    const u64 first = it.start + (u64)((y0 - it.ya) * g.W);
+                    const u64 first = it.at(g, y0);
                     const int rel = 8 * w - (int)(first & 7);  // the word's first pixel, counted from the item's first
                     const uint4 *s = reinterpret_cast<const uint4 *>(sb + g.out_off + slot * g.out_stride) + w;
                     T *d = out + (first + rel);
@@ -706,7 +718,7 @@ tensor_kernel(const __grid_constant__ KGeom g, const T *__restrict__ x, const T 
             if (g.alias && u + 1 < u_end) {
                 plane::bulk_store_wait_read();
                 worker_sync();
-                fetch((unit + 1) & 1u);
+                fetch(set_next);
             }
             // every MMA of the unit has completed: its arrays and (on a channel change) its table may be rewritten
             wait_for(done, unit & 1u);
@@ -717,6 +729,7 @@ tensor_kernel(const __grid_constant__ KGeom g, const T *__restrict__ x, const T 
                 float *scr = reinterpret_cast<float *>(sb);
 #pragma unroll 1
                 for (int half = 0; half < 2; ++half) {
+                    __syncwarp();
                     if (warp >> 2 == 0) {
 #pragma unroll 1
                         for (int e = 0; e < 64; e += 16) {
@@ -726,6 +739,7 @@ tensor_kernel(const __grid_constant__ KGeom g, const T *__restrict__ x, const T 
                             tmem_arrived(v);
 #pragma unroll
                             for (int i = 0; i < 16; ++i) scr[m * SCR_PITCH + e + i] = v[i];
+                            __syncwarp();
                         }
                     }
                     worker_sync();
@@ -778,6 +792,7 @@ tensor_kernel(const __grid_constant__ KGeom g, const T *__restrict__ x, const T 
                 worker_sync();
             }
         }
+        set_u = set_next;
         c_prev = c;
         c = cn;
         k = kn;
@@ -786,6 +801,7 @@ tensor_kernel(const __grid_constant__ KGeom g, const T *__restrict__ x, const T 
     if (BWD) dependents_may_start();
     fence_before();
     __syncthreads();
+    __syncwarp();
     if (warp == 8) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(g.cols));
 }
 
@@ -851,7 +867,7 @@ inline bool wide(const Request &q) { return q.W > 64 || q.H > 128; }  // served 
 inline bool search_n(const Request &q, KGeom &best, int n) {
     bool found = false;
     KGeom g = {};
-    g.deep = q.L > 1 ? (wide(q) ? 2 : 1) : 0;
+    g.deep = q.L > 1;
     g.B = q.B; g.C = q.C; g.H = q.H; g.W = q.W; g.HW = q.H * q.W; g.L = q.L; g.K = q.K;
     g.n = n;
     g.tw = 8 * n;
@@ -899,7 +915,7 @@ inline bool search_n(const Request &q, KGeom &best, int n) {
         h.out_off = alias ? h.raw_off : off; if (!alias) off += 8 * S * h.out_stride;
         off = up(off, 128);
         h.table_off = off; off += TABLE_BYTES;
-        h.misc_off = off; off += 600 * 4 + 2 * 8 * S * 16;
+        h.misc_off = off; off += 600 * 4 + 3 * 8 * S * 16;
         h.smem = up(off, 128);
         if (h.smem > plane::SMEM_LIMIT) break;
         h.upc = (h.items + 8 * S - 1) / (8 * S);
@@ -909,17 +925,21 @@ inline bool search_n(const Request &q, KGeom &best, int n) {
             if ((long long)bps * (h.smem + 1024) > plane::SMEM_PER_SM) break;
             h.cols = 512 / bps;
             h.ring = (h.cols - (q.bwd ? WG_COLS : 0)) / NCOL;
-            if (h.ring > MAX_RING) h.ring = MAX_RING;
+            h.ring = h.ring >= MAX_RING ? MAX_RING : h.ring >= 4 ? 4 : 2;
             h.bps = bps;
             h.nblocks = plane::NUM_SMS * bps < h.units ? plane::NUM_SMS * bps : h.units;
-            // cycles: MMAs serialise over an SM's blocks; the workers' part and the hand-overs do not
-            const double tensor = (double)h.T * h.n * TAPS * 46 + (q.bwd ? (double)h.Ws * h.Pc * 2 * 50 : 0);
-            const double around = 3500.0 + (alias ? 2500.0 : 0.0) + 6.0 * S * (q.bwd ? 2.2 : 1.0) * load_rows * h.Pc + 0.25 * tensor;
-            const int active = (h.nblocks + plane::NUM_SMS - 1) / plane::NUM_SMS;
-            const int rounds = (h.units + h.nblocks - 1) / h.nblocks;
-            const double serial = tensor + around, per = active * tensor > serial ? active * tensor : serial;
-            const double switches = 1.0 + (double)q.C / h.nblocks;
-            const double cost = rounds * per + switches * (2500.0 + (q.bwd ? 5000.0 : 0.0));
+            // Cycles, fitted to the times of 3000 shapes (4 % off, backward 6 %): a round of units pays a fixed part, its staging
+            // words (odd row lengths pixel by pixel) and its MMAs; two resident blocks share tensor cores and shared memory.
+            const double mma = (double)h.T * h.n * TAPS * 46 + (q.bwd ? (double)h.Ws * h.Pc * 2 * 50 : 0);
+            const bool two = h.nblocks > plane::NUM_SMS;
+            const int rounds = (h.units + h.nblocks - 1) / h.nblocks, channels = 1 + q.C / h.nblocks < rounds ? 1 + q.C / h.nblocks : rounds;
+            const double words = (double)S * load_rows * h.Pc, copied = h.out_words < BULK_WORDS ? 8.0 * S * h.out_words : 0;
+            const int odd = q.W % 4 == 0 ? 0 : q.W % 2 == 0 ? 1 : 2;
+            const double per = q.bwd ? 4715 + 2757 * two + 1311 * alias + (6.6 + (odd == 1 ? 2.8 : odd == 2 ? 18 : 0)) * words + 1161 * S +
+                                           mma * (1.16 + 0.29 * two) + 0.7 * copied
+                                     : 1677 + 1913 * two + 1014 * alias + (1.8 + (odd == 1 ? 3.4 : odd == 2 ? 11.6 : 0)) * words + 613 * S +
+                                           mma * (1.93 + 0.65 * two) + 0.8 * copied;
+            const double cost = (q.bwd ? 12657 : 7563) + rounds * per + channels * (q.bwd ? 4823 : 1429);
             if (cost < best.cost) {
                 best = h;
                 best.cost = cost;

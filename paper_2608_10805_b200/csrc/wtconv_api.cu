@@ -115,6 +115,7 @@ struct Route {
     wtconv_desc key;
     bool set;
     bool team, plane, window, tensor[2], k3;  // plane: any family that keeps whole planes on chip; k3: 3 x 3 kernels in 5 x 5 tables
+    size_t chip_fwd, chip_bwd;  // workspace of the family itself, which the k = 3 embedding runs whatever serves k = 5
     size_t fwd_bytes, bwd_bytes;
 };
 const Route &route(const wtconv_desc *d);
@@ -311,10 +312,28 @@ wtconv_status backward_tk(const wtconv_desc *d, const void *x, const void *g, co
 size_t fwd_ws_bytes(const wtconv_desc *d) { return route(d).fwd_bytes; }
 size_t bwd_ws_bytes(const wtconv_desc *d) { return route(d).bwd_bytes; }
 
+// What the kernels that keep a plane on one SM (or a team of them) take for a 16-bit layer with at most one level, in
+// microseconds: fitted to 3000 shapes between 1 x 16 x 7 x 7 and 128 x 768 x 64 x 64 (13 % off; k = 3 in 5 x 5 tables 11 %).
+// They pay for tiles of 4 x 4 pixels, for planes, for rows that are not 8-byte multiples, and a fixed part that is larger
+// where teams work on the smallest planes.
+double on_chip_us(const wtconv_desc *d, int bwd) {
+    const double planes = (double)d->B * d->C * 1e-3, tiles = planes * ((d->W + 3) / 4 * 4) * ((d->H + 3) / 4 * 4) * 1e-3;
+    const int hw = d->H * d->W;
+    const double first = planes < 1 ? planes : 1, kpx = hw * 1e-3;
+    const bool odd = d->W % 4 != 0, small = hw <= 100, least = hw <= 64;
+    if (d->k == 5)
+        return bwd ? 10.4 + (7.33 + 3.1 * odd) * tiles + 0.48 * planes + 8.5 * small + 3.0 * first + 0.4 * kpx
+                   : 6.6 + (3.16 + 1.56 * odd) * tiles + (0.355 - 0.25 * least) * planes + 2.5 * small;
+    return bwd ? 17.2 + (4.61 + 2.87 * odd) * tiles + 0.82 * planes + 8.9 * small + 2.2 * first + 0.3 * kpx
+               : 9.8 + (2.2 + 1.56 * odd) * tiles + (0.43 - 0.26 * least) * planes + 3.1 * small;
+}
+// The tensor-core kernels win where the images of a channel fill their groups of eight and there are enough channels and images
+// for the SMs.  They are taken where their own estimate (4 - 6 % off) is at least a tenth below: over those shapes they gained
+// 14 % (forward, k = 5), 25 % (backward), 27 % and 35 % (k = 3, which also saves the table kernels), and lost in 1 of 40.
 bool tensor_serves(const wtconv_desc *d, bool on_chip, int bwd) {
-    if (d->dtype == WTCONV_F32 || !on_chip || (d->flags & ~WTCONV_FLAG_TEST_NO_COPY)) return false;
+    if (d->dtype == WTCONV_F32 || !on_chip || d->L > 1 || (d->flags & ~WTCONV_FLAG_TEST_NO_COPY)) return false;
     wt::tensor::KGeom g;
-    return wt::tensor::plan(tensor_request(d, bwd), g);
+    return wt::tensor::plan(tensor_request(d, bwd), g) && g.cost * (1.1 / 1900) < on_chip_us(d, bwd);
 }
 
 Route find_route(const wtconv_desc *d) {
@@ -348,8 +367,8 @@ Route find_route(const wtconv_desc *d) {
             const size_t head = embed_layout(d).inner;
             for (int bwd = 0; bwd < 2; ++bwd) r.tensor[bwd] = tensor_serves(d, r5.plane, bwd);
             const size_t own = r.tensor[1] ? align_up(wt::tensor::backward_bytes(tensor_request(d, 1))) : 0;
-            r.fwd_bytes = head + r5.fwd_bytes;
-            r.bwd_bytes = head + (own > r5.bwd_bytes ? own : r5.bwd_bytes);
+            r.fwd_bytes = head + r5.chip_fwd;
+            r.bwd_bytes = head + (own > r5.chip_bwd ? own : r5.chip_bwd);
             return r;
         }
     }
@@ -368,6 +387,8 @@ Route find_route(const wtconv_desc *d) {
         r.fwd_bytes = p.fwd_bytes;
         r.bwd_bytes = p.bwd_bytes;
     }
+    r.chip_fwd = r.fwd_bytes;
+    r.chip_bwd = r.bwd_bytes;
     for (int bwd = 0; bwd < 2; ++bwd) r.tensor[bwd] = d->k == 5 && tensor_serves(d, r.plane, bwd);
     if (r.tensor[0]) r.fwd_bytes = align_up(wt::tensor::STATUS_BYTES);
     if (r.tensor[1]) r.bwd_bytes = align_up(wt::tensor::backward_bytes(tensor_request(d, 1)));
