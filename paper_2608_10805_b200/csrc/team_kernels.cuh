@@ -333,6 +333,7 @@ team_kernel(const __grid_constant__ TGeom g, const T *__restrict__ x, const T *_
         if (lt == 0 && !dead)
             for (int s = 0; s < NSTAGE; ++s)
                 if (seg + team_id + s * nteams < seg_end) issue(seg + team_id + s * nteams, cg, it + s);
+        if (!BWD && seg > u_begin) __syncthreads();  // a slower team may still be reading the last channel group's bias
         build_table(wtab, g, c0, BWD, w0, s0, BWD ? nullptr : b0, wl, sl);
         __syncthreads();
         if (has_tile) plane::load_weights(wtab + (q * ncls + cls) * WT_STRIDE, w);
