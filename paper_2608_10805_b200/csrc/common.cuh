@@ -74,12 +74,6 @@ inline cudaError_t launch_overlapped(void (*kern)(P...), unsigned grid, unsigned
     return cudaLaunchKernelEx(&cfg, kern, static_cast<P>(args)...);
 }
 
-// The float plane that a deeper-levels kernel leaves in the place of plane `plane` (HW elements of T) of an output tensor: at
-// its first byte, rounded up to a float.
-template <typename T> __device__ __forceinline__ float *deep_plane(T *out, size_t plane, int HW) {
-    return reinterpret_cast<float *>((reinterpret_cast<uintptr_t>(out + plane * HW) + 3) & ~(uintptr_t)3);
-}
-
 // ---- Status words at the start of a workspace whose kernels wait for bulk copies.  No launch clears them: every
 // call carries a fresh non-zero tag; block 0 of each kernel of the call stores it in STATUS_LAUNCH, a block whose
 // bounded wait ran out stores it in STATUS_TIMEOUT.  The last call timed out iff the two words are equal (and

@@ -1,0 +1,176 @@
+// Wide planes on the tensor-core kernels (k = 3 or 5, 16-bit activations): base convolution and level 1 in column panels,
+// levels >= 2 on fp32 carriers.
+//
+//   band_kernel            X1 = low-pass band of level 1 (fp32, a quarter of the plane)
+//   level kernels          levels 2 .. L on the carriers, as in the tiled path (one launch a level)
+//   synthesis_kernel       R = what levels >= 2 add to X1's reconstruction (Proposition 2, un-normalised LL of level 1)
+//   tensor kernel, panels  out = base + level 1 + R / 2 per 2 x 2 pixels
+//
+// The tiled path runs base convolution and level 1 as fp32 FMAs and passes all of level 1's coefficients through HBM; here a
+// level-1 coefficient never leaves the SM and its products run on the tensor cores.
+#pragma once
+#include "tensor_kernels.cuh"
+#include "tiled_host.cuh"
+
+namespace wt {
+namespace tensor {
+
+struct WidePlan {
+    size_t X[9], G[9], Z[9], part[9], R, fwd_bytes, bwd_bytes;  // by level; X[1], G[1]: the level-1 carriers
+    int Hs[9], Ws[9], bsplit[9], npl[9];
+};
+inline WidePlan wide_plan(const Request &q) {
+    using host::align_up;
+    WidePlan p = {};
+    p.Hs[0] = q.H;
+    p.Ws[0] = q.W;
+    for (int l = 1; l <= 8; ++l) { p.Hs[l] = (p.Hs[l - 1] + 1) / 2; p.Ws[l] = (p.Ws[l - 1] + 1) / 2; }
+    const size_t P = (size_t)q.B * q.C, KK = (size_t)q.K * q.K;
+    Request b = q;
+    b.bwd = 1;
+    // the tensor kernel's part (status words, partial sums) opens the workspace in both directions
+    const size_t head = align_up(backward_bytes(b));
+    size_t off = head;
+    auto floats = [&](size_t n) { const size_t at = off; off = align_up(off + sizeof(float) * n); return at; };
+    if (q.L > 1) {
+        for (int l = 1; l <= q.L; ++l) {
+            const size_t S = (size_t)p.Hs[l] * p.Ws[l];
+            if (l < q.L) p.X[l] = floats(S * P);
+            if (l > 1) p.Z[l] = floats(4 * S * P);
+        }
+        p.R = floats((size_t)p.Hs[1] * p.Ws[1] * P);
+    }
+    p.fwd_bytes = off;
+    for (int l = 1; l < q.L; ++l) p.G[l] = floats((size_t)p.Hs[l] * p.Ws[l] * P);
+    for (int l = 2; l <= q.L; ++l) {
+        const int tiles = host::cdiv(p.Ws[l], tiled::TW) * host::cdiv(p.Hs[l], tiled::TH);
+        p.bsplit[l] = host::pick_bsplit(q.B, (long long)tiles * q.C);
+        p.npl[l] = tiles * p.bsplit[l];
+        p.part[l] = floats((size_t)q.C * p.npl[l] * 4 * KK);
+    }
+    p.bwd_bytes = off;
+    return p;
+}
+
+// R from Z^2 .. Z^L.  Bound by memory (Z^2 read, R written); a thread makes 2 x 4 values from two level-2 coefficients, so its
+// stores are 16 bytes wide and every deeper coefficient is read once by neighbouring threads of a warp.
+struct SynthPtrs {
+    const float *z[9];
+    int H[9], W[9], L;
+};
+static __global__ void __launch_bounds__(256) synthesis_kernel(const __grid_constant__ SynthPtrs s, u64 rows, float *__restrict__ R) {
+    const int H1 = s.H[1], W1 = s.W[1], H2 = s.H[2], W2 = s.W[2], pairs = (W2 + 1) >> 1;
+    for (u64 e = (u64)blockIdx.x * blockDim.x + threadIdx.x; e < rows * pairs; e += (u64)gridDim.x * blockDim.x) {
+        const u64 row = e / pairs, p = row / H2;
+        const int j = (int)(e - row * pairs), i = (int)(row - p * H2);
+        float v[2][4];
+        const size_t S2 = (size_t)H2 * W2;
+        const float *z = s.z[2] + p * 4 * S2 + (size_t)i * W2 + 2 * j;
+        const bool second = 2 * j + 1 < W2;
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            float ll = 0.f, lh = 0.f, hl = 0.f, hh = 0.f;
+            if (h == 0 || second) { ll = __ldg(z + h); lh = __ldg(z + S2 + h); hl = __ldg(z + 2 * S2 + h); hh = __ldg(z + 3 * S2 + h); }
+            const float pp = ll + lh, pm = ll - lh, qp = hl + hh, qm = hl - hh;
+            v[0][2 * h] = 0.5f * (pp + qp); v[0][2 * h + 1] = 0.5f * (pp - qp);
+            v[1][2 * h] = 0.5f * (pm + qm); v[1][2 * h + 1] = 0.5f * (pm - qm);
+        }
+        float deep[2] = {0.f, 0.f}, scale = 0.5f;  // constant over a level-2 coefficient's 2 x 2 values
+        for (int l = 3; l <= s.L; ++l) {
+            scale *= 0.5f;
+            const size_t S = (size_t)s.H[l] * s.W[l];
+            const float *q = s.z[l] + p * 4 * S + (size_t)(i >> (l - 2)) * s.W[l] + (2 * j >> (l - 2));
+            const float ll = __ldg(q), lh = __ldg(q + S), hl = __ldg(q + 2 * S), hh = __ldg(q + 3 * S);
+#pragma unroll
+            for (int h = 0; h < 2; ++h) deep[h] += synth_term(ll, lh, hl, hh, (i >> (l - 3)) & 1, ((2 * j + h) >> (l - 3)) & 1, scale);
+        }
+#pragma unroll
+        for (int r = 0; r < 2; ++r)
+#pragma unroll
+            for (int c = 0; c < 4; ++c) v[r][c] += deep[c >> 1];
+        float *o = R + (p * H1 + 2 * i) * (u64)W1 + 4 * j;
+#pragma unroll
+        for (int r = 0; r < 2; ++r, o += W1) {
+            if (2 * i + r >= H1) break;
+            if ((W1 & 3) == 0) {
+                *reinterpret_cast<float4 *>(o) = make_float4(v[r][0], v[r][1], v[r][2], v[r][3]);
+            } else {
+#pragma unroll
+                for (int c = 0; c < 4; ++c)
+                    if (4 * j + c < W1) o[c] = v[r][c];
+            }
+        }
+    }
+}
+inline cudaError_t synthesize(const Request &q, const WidePlan &p, char *ws, cudaStream_t st) {
+    SynthPtrs s = {};
+    s.L = q.L;
+    for (int l = 1; l <= q.L; ++l) { s.z[l] = reinterpret_cast<const float *>(ws + p.Z[l]); s.H[l] = p.Hs[l]; s.W[l] = p.Ws[l]; }
+    const u64 rows = (u64)q.B * q.C * p.Hs[2], n = rows * ((p.Ws[2] + 1) / 2), blocks = (n + 255) / 256;
+    synthesis_kernel<<<(unsigned)(blocks < 148 * 64 ? blocks : 148 * 64), 256, 0, st>>>(s, rows, reinterpret_cast<float *>(ws + p.R));
+    return cudaGetLastError();
+}
+
+template <typename T, int K>
+cudaError_t wide_forward_k(const Request &q, const T *x, const float *w0, const float *s0, const float *b0, const float *wl, const float *sl,
+                           T *out, char *ws, cudaStream_t st, unsigned tag) {
+    const WidePlan p = wide_plan(q);
+    cudaError_t e;
+    if (q.L > 1) {
+        if ((e = band<T>(q.B, q.C, q.H, q.W, x, reinterpret_cast<float *>(ws + p.X[1]), st)) != cudaSuccess) return e;
+        for (int l = 2; l <= q.L; ++l) {
+            dim3 grid((unsigned)((size_t)q.B * q.C * host::cdiv(p.Ws[l], tiled::TW) * host::cdiv(p.Hs[l], tiled::TH)));
+            tiled::level_fwd_kernel<float, K><<<grid, tiled::NTHREADS, 0, st>>>(
+                reinterpret_cast<const float *>(ws + p.X[l - 1]), p.Hs[l - 1], p.Ws[l - 1], p.Hs[l], p.Ws[l], q.C, wl + (size_t)(l - 1) * q.C * 4 * K * K,
+                sl + (size_t)(l - 1) * q.C * 4, reinterpret_cast<float *>(ws + p.Z[l]), l < q.L ? reinterpret_cast<float *>(ws + p.X[l]) : nullptr);
+        }
+        if ((e = synthesize(q, p, ws, st)) != cudaSuccess) return e;
+    }
+    return forward<T>(q, x, w0, s0, b0, wl, sl, out, ws, st, tag, false, reinterpret_cast<const float *>(ws + p.R));
+}
+template <typename T, int K>
+cudaError_t wide_backward_k(const Request &q, const T *x, const T *go, const float *w0, const float *s0, const float *wl, const float *sl, bool bias,
+                            T *gx, char *ws, EpiloguePtrs *ep, cudaStream_t st, unsigned tag) {
+    const WidePlan p = wide_plan(q);
+    cudaError_t e;
+    if (q.L > 1) {
+        if ((e = band<T>(q.B, q.C, q.H, q.W, x, reinterpret_cast<float *>(ws + p.X[1]), st)) != cudaSuccess) return e;
+        if ((e = band<T>(q.B, q.C, q.H, q.W, go, reinterpret_cast<float *>(ws + p.G[1]), st)) != cudaSuccess) return e;
+        constexpr auto kern = tiled::level_bwd_kernel<float, K>;
+        constexpr size_t smem = tiled::level_bwd_smem_bytes<K>();
+        if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess) return e;
+        for (int l = 2; l <= q.L; ++l) {
+            dim3 grid((unsigned)((size_t)q.C * p.npl[l]));
+            kern<<<grid, tiled::NTHREADS, smem, st>>>(
+                reinterpret_cast<const float *>(ws + p.X[l - 1]), reinterpret_cast<const float *>(ws + p.G[l - 1]), p.Hs[l - 1], p.Ws[l - 1], p.Hs[l],
+                p.Ws[l], q.B, q.C, p.bsplit[l], wl + (size_t)(l - 1) * q.C * 4 * K * K, sl + (size_t)(l - 1) * q.C * 4,
+                reinterpret_cast<float *>(ws + p.Z[l]), l < q.L ? reinterpret_cast<float *>(ws + p.X[l]) : nullptr,
+                l < q.L ? reinterpret_cast<float *>(ws + p.G[l]) : nullptr, reinterpret_cast<float *>(ws + p.part[l]));
+            ep->partl[l - 1] = reinterpret_cast<const float *>(ws + p.part[l]);
+            ep->npl[l - 1] = p.npl[l];
+        }
+        if ((e = synthesize(q, p, ws, st)) != cudaSuccess) return e;
+        ep->deep_all = true;
+    }
+    return backward<T>(q, x, go, w0, s0, wl, sl, bias, gx, ws, ep, st, tag, false, reinterpret_cast<const float *>(ws + p.R));
+}
+template <typename T>
+cudaError_t wide_forward(const Request &q, const T *x, const float *w0, const float *s0, const float *b0, const float *wl, const float *sl, T *out,
+                         char *ws, cudaStream_t st, unsigned tag) {
+    return q.K == 3 ? wide_forward_k<T, 3>(q, x, w0, s0, b0, wl, sl, out, ws, st, tag) : wide_forward_k<T, 5>(q, x, w0, s0, b0, wl, sl, out, ws, st, tag);
+}
+template <typename T>
+cudaError_t wide_backward(const Request &q, const T *x, const T *go, const float *w0, const float *s0, const float *wl, const float *sl, bool bias,
+                          T *gx, char *ws, EpiloguePtrs *ep, cudaStream_t st, unsigned tag) {
+    return q.K == 3 ? wide_backward_k<T, 3>(q, x, go, w0, s0, wl, sl, bias, gx, ws, ep, st, tag)
+                    : wide_backward_k<T, 5>(q, x, go, w0, s0, wl, sl, bias, gx, ws, ep, st, tag);
+}
+
+#define WT_WIDE_INSTANTIATE(T, EXTERN)                                                                                               \
+    EXTERN template cudaError_t wide_forward<T>(const Request &, const T *, const float *, const float *, const float *, const float *, \
+                                                const float *, T *, char *, cudaStream_t, unsigned);                                 \
+    EXTERN template cudaError_t wide_backward<T>(const Request &, const T *, const T *, const float *, const float *, const float *,  \
+                                                 const float *, bool, T *, char *, EpiloguePtrs *, cudaStream_t, unsigned);
+
+}  // namespace tensor
+}  // namespace wt

@@ -115,7 +115,6 @@ __device__ __forceinline__ int fdiv(int e, const FastDiv &f) { return f.d == 1 ?
 
 struct Geom {
     int B, C, H, W, L;
-    int H0, W0, HW0, deep;                 // the tensor's planes: H x W, or (deep) the planes whose level-1 low-pass band is H x W
     int Hl[MAXL + 1], Wl[MAXL + 1];        // level grids, index 0 = input
     int rows[MAXL + 1], pitch[MAXL + 1];   // haloed arrays: ty*TH+4 rows, pitch pad4(Wl)+4 floats; element (y,x) at (y+2, x+2)
     int offA[MAXL + 1];                    // slot-relative offset of x (l=0) / Y^l subband 0 (subband stride rows*pitch)
@@ -183,10 +182,8 @@ __device__ __forceinline__ void build_weight_table(float *wtab, const Geom &g, i
                 dst[k] = sc * WT_STRIDE + t;
                 if (c < g.C) {
                     if (cls == 0) {
-                        if (w0) {
-                            wv[k] = __ldg(w0 + c * KK + src);
-                            sv[k] = __ldg(s0 + c);
-                        }
+                        wv[k] = __ldg(w0 + c * KK + src);
+                        sv[k] = __ldg(s0 + c);
                     } else {
                         const int l = (cls - 1) >> 2, sub = (cls - 1) & 3;
                         const size_t i = ((size_t)l * g.C + c) * 4 + sub;
@@ -258,62 +255,13 @@ template <typename T, bool RAW>
 __device__ __forceinline__ void ld4(const T *p, float (&v)[4]) {
     if (RAW) load4s(p, v); else load4(p, v);
 }
-// Element (y, x) of the plane the kernel works on.  DEEP: that plane is the level-1 low-pass band of the tensor's plane, its
-// elements are worked out from the pixels as they are read (Eq. 5's LL, in the butterfly's own order).
-template <typename T, bool RAW, bool DEEP>
-__device__ __forceinline__ float at1(const T *plane, const Geom &g, int y, int x) {
-    if (!DEEP) return ld1<T, RAW>(plane + y * g.W + x);
-    const T *p = plane + 2 * y * g.W0 + 2 * x;
-    const bool x1 = 2 * x + 1 < g.W0, y1 = 2 * y + 1 < g.H0;
-    const float a = ld1<T, RAW>(p), b = x1 ? ld1<T, RAW>(p + 1) : 0.f;
-    const float c = y1 ? ld1<T, RAW>(p + g.W0) : 0.f, d = x1 && y1 ? ld1<T, RAW>(p + g.W0 + 1) : 0.f;
-    return 0.5f * ((a + b) + (c + d));
-}
-// Elements (y, x) and (y, x + 1), x even; the second is zero beyond the plane.  Where the pixel rows allow it, four pixels at a time.
-template <typename T, bool RAW, bool DEEP>
-__device__ __forceinline__ void at2(const T *plane, const Geom &g, int y, int x, float &v0, float &v1) {
-    if (DEEP && (g.W0 & 3) == 0 && (g.HW0 & 3) == 0) {
-        const T *p = plane + 2 * y * g.W0 + 2 * x;
-        float a[4], c[4] = {0.f, 0.f, 0.f, 0.f};
-        ld4<T, RAW>(p, a);
-        if (2 * y + 1 < g.H0) ld4<T, RAW>(p + g.W0, c);
-        v0 = 0.5f * ((a[0] + a[1]) + (c[0] + c[1]));
-        v1 = 0.5f * ((a[2] + a[3]) + (c[2] + c[3]));
-    } else {
-        v0 = at1<T, RAW, DEEP>(plane, g, y, x);
-        v1 = x + 1 < g.W ? at1<T, RAW, DEEP>(plane, g, y, x + 1) : 0.f;
-    }
-}
-// Elements (y, x .. x + 3), x a multiple of 4 (g.vec).
-template <typename T, bool RAW, bool DEEP>
-__device__ __forceinline__ void at4(const T *plane, const Geom &g, int y, int x, float (&v)[4]) {
-    if (!DEEP) {
-        ld4<T, RAW>(plane + y * g.W + x, v);
-    } else if ((g.W0 & 3) == 0) {
-        const T *p = plane + 2 * y * g.W0 + 2 * x;
-        float a[4], b[4], c[4] = {0.f, 0.f, 0.f, 0.f}, d[4] = {0.f, 0.f, 0.f, 0.f};
-        ld4<T, RAW>(p, a);
-        ld4<T, RAW>(p + 4, b);
-        if (2 * y + 1 < g.H0) {
-            ld4<T, RAW>(p + g.W0, c);
-            ld4<T, RAW>(p + g.W0 + 4, d);
-        }
-        v[0] = 0.5f * ((a[0] + a[1]) + (c[0] + c[1]));
-        v[1] = 0.5f * ((a[2] + a[3]) + (c[2] + c[3]));
-        v[2] = 0.5f * ((b[0] + b[1]) + (d[0] + d[1]));
-        v[3] = 0.5f * ((b[2] + b[3]) + (d[2] + d[3]));
-    } else {
-#pragma unroll
-        for (int i = 0; i < 4; ++i) v[i] = at1<T, RAW, true>(plane, g, y, x + i);
-    }
-}
 
 __device__ __forceinline__ void decode_level_item(const Geom &g, int r, int &l, int &sub, int &tyy, int &txx);
 
 // ---- per-thread work descriptors.  A thread's tiles and staging patches are the same for every unit, so
 // ---- they are decoded once, before the unit loop, and live in registers.
 struct PatchD {   // 4x4 pixel staging patch (vector path, L >= 2)
-    int so;       // element offset of the patch inside its plane: y*W + 4q (deep: y << 16 | 4q)
+    int so;       // element offset of the patch inside its plane: y*W + 4q
     int xi, yi, y2;  // float indices of its first x / level-1 / level-2 element in shared memory
     int meta;     // bit 31 valid, bits 0-7 plane slot, bits 8-10 rows inside the image (1..4)
 };
@@ -327,7 +275,7 @@ __device__ __forceinline__ PatchD decode_patch(const Geom &g, const int *off, in
         const int y = 4 * i2, S = slot * g.slot_stride;
         int nrows = g.H - y;
         if (nrows > 4) nrows = 4;
-        p.so = g.deep ? y << 16 | 4 * q : y * g.W + 4 * q;
+        p.so = y * g.W + 4 * q;
         p.xi = S + off[0] + (y + 2) * g.pitch[0] + 4 * q + 2;
         p.yi = S + off[1] + (2 * i2 + 2) * g.pitch[1] + 2 * q + 2;
         p.y2 = S + off[2] + (i2 + 2) * g.pitch[2] + q + 2;
@@ -336,7 +284,7 @@ __device__ __forceinline__ PatchD decode_patch(const Geom &g, const int *off, in
     return p;
 }
 // The 4 x 4 pixels of a patch (zero where the patch leaves the image or the plane slot is not in use).
-template <typename T, bool RAW, bool DEEP>
+template <typename T, bool RAW>
 __device__ __forceinline__ void load_patch(const Geom &g, const PatchD &p, const T *__restrict__ gsrc, int nvalid,
                                            float (&a)[4][4]) {
     const int slot = p.meta & 0xff, nrows = (p.meta >> 8) & 7;
@@ -345,13 +293,10 @@ __device__ __forceinline__ void load_patch(const Geom &g, const PatchD &p, const
 #pragma unroll
         for (int cc = 0; cc < 4; ++cc) a[rr][cc] = 0.f;
     if (slot < nvalid) {
-        const T *pa = gsrc + slot * g.HW0;  // the unit's planes are contiguous
+        const T *pa = gsrc + slot * (g.H * g.W) + p.so;  // the unit's planes are contiguous
 #pragma unroll
         for (int rr = 0; rr < 4; ++rr)
-            if (rr < nrows) {
-                if (DEEP) at4<T, RAW, true>(pa, g, (p.so >> 16) + rr, p.so & 0xffff, a[rr]);
-                else ld4<T, RAW>(pa + p.so + rr * g.W, a[rr]);
-            }
+            if (rr < nrows) ld4<T, RAW>(pa + rr * g.W, a[rr]);
     }
 }
 // x, level 1 and level 2 of one patch into the haloed arrays; d0/d1/d2 shift the targets to another set of
@@ -390,23 +335,23 @@ __device__ __forceinline__ void store_patch(float *sm, const Geom &g, const Patc
     sm[p.y2 + 2 * sub2] = h2.hl;
     sm[p.y2 + 3 * sub2] = h2.hh;
 }
-template <typename T, bool RAW, bool DEEP = false>
+template <typename T, bool RAW>
 __device__ __forceinline__ void run_patch(float *sm, const Geom &g, const PatchD &p, const T *__restrict__ gsrc,
                                           int nvalid, int d0 = 0, int d1 = 0, int d2 = 0) {
     if (p.meta >= 0) return;
     float a[4][4];
-    load_patch<T, RAW, DEEP>(g, p, gsrc, nvalid, a);
+    load_patch<T, RAW>(g, p, gsrc, nvalid, a);
     store_patch(sm, g, p, a, d0, d1, d2);
 }
 // The same patch of two tensors (x and grad_out): both sets of loads are issued before either is used, so
 // their global-memory latencies overlap.
-template <typename T, bool RAW, bool DEEP = false>
+template <typename T, bool RAW>
 __device__ __forceinline__ void run_patch_pair(float *sm, const Geom &g, const PatchD &p, const T *__restrict__ xsrc,
                                                const T *__restrict__ gsrc, int nvalid, int d0, int d1, int d2) {
     if (p.meta >= 0) return;
     float a[4][4], b[4][4];
-    load_patch<T, RAW, DEEP>(g, p, xsrc, nvalid, a);
-    load_patch<T, RAW, DEEP>(g, p, gsrc, nvalid, b);
+    load_patch<T, RAW>(g, p, xsrc, nvalid, a);
+    load_patch<T, RAW>(g, p, gsrc, nvalid, b);
     store_patch(sm, g, p, a, 0, 0, 0);
     store_patch(sm, g, p, b, d0, d1, d2);
 }
@@ -468,13 +413,13 @@ __device__ __forceinline__ ItemD decode_item(const Geom &g, int it, int nlevel_i
 // plane slot s from the raw shared buffer at src + s * slot_elems (a bulk copy put it there); RAW = false
 // reads global memory.  Pixels beyond H x W are never written and stay zero (odd-size padding and conv
 // halo); images beyond the batch are written as zeros.
-template <typename T, bool RAW, bool DEEP = false>
+template <typename T, bool RAW>
 __device__ __forceinline__ int stage_input(float *sm, const Geom &g, const int *off, const T *__restrict__ src, int c,
                                            int b, int srank, int nstagers) {
     const int H = g.H, W = g.W, HW = H * W;
     const int p0 = g.pitch[0];
-    const T *gsrc = RAW ? src : src + ((size_t)b * g.C + c) * g.HW0;  // channel c (first of the unit) of image b
-    const int img_stride = g.HW0;                                     // the unit's planes are contiguous
+    const T *gsrc = RAW ? src : src + ((size_t)b * g.C + c) * HW;  // channel c (first of the unit) of image b
+    const int img_stride = HW;                                     // the unit's planes are contiguous
     const int nvalid = g.C - c < g.NPL ? g.C - c : g.NPL;
     if (g.L == 0) {
         for (int e = srank; e < g.NPL * HW; e += nstagers) {
@@ -499,10 +444,10 @@ __device__ __forceinline__ int stage_input(float *sm, const Geom &g, const int *
 #pragma unroll
                 for (int cc = 0; cc < 4; ++cc) a[rr][cc] = 0.f;
             if (slot < nvalid) {
-                const T *pa = gsrc + (size_t)slot * img_stride;
+                const T *pa = gsrc + (size_t)slot * img_stride + y * W + 4 * q;
 #pragma unroll
                 for (int rr = 0; rr < 4; ++rr)
-                    if (y + rr < H) at4<T, RAW, DEEP>(pa, g, y + rr, 4 * q, a[rr]);
+                    if (y + rr < H) ld4<T, RAW>(pa + rr * W, a[rr]);
             }
             const int S = slot * g.slot_stride;
             const int xi = S + off[0] + (y + 2) * p0 + 4 * q + 2;  // 8-byte aligned
@@ -546,9 +491,9 @@ __device__ __forceinline__ int stage_input(float *sm, const Geom &g, const int *
             const bool y1 = y + 1 < H;
             float a0[4] = {0.f, 0.f, 0.f, 0.f}, a1[4] = {0.f, 0.f, 0.f, 0.f};
             if (slot < nvalid) {
-                const T *pa = gsrc + (size_t)slot * img_stride;
-                at4<T, RAW, DEEP>(pa, g, y, 4 * q, a0);
-                if (y1) at4<T, RAW, DEEP>(pa, g, y + 1, 4 * q, a1);
+                const T *pa = gsrc + (size_t)slot * img_stride + y * W + 4 * q;
+                ld4<T, RAW>(pa, a0);
+                if (y1) ld4<T, RAW>(pa + W, a1);
             }
             const int S = slot * g.slot_stride;
             const int xi = S + off[0] + (y + 2) * p0 + 4 * q + 2;  // 8-byte aligned
@@ -576,9 +521,11 @@ __device__ __forceinline__ int stage_input(float *sm, const Geom &g, const int *
         const bool x1 = xx + 1 < W, y1 = y + 1 < H;
         float a = 0.f, bq = 0.f, cq = 0.f, d = 0.f;
         if (slot < nvalid) {
-            const T *pa = gsrc + (size_t)slot * img_stride;
-            at2<T, RAW, DEEP>(pa, g, y, xx, a, bq);
-            if (y1) at2<T, RAW, DEEP>(pa, g, y + 1, xx, cq, d);
+            const T *pa = gsrc + (size_t)slot * img_stride + y * W + xx;
+            a = ld1<T, RAW>(pa);
+            if (x1) bq = ld1<T, RAW>(pa + 1);
+            if (y1) cq = ld1<T, RAW>(pa + W);
+            if (x1 && y1) d = ld1<T, RAW>(pa + W + 1);
         }
         const int S = slot * g.slot_stride;
         const int xi = S + off[0] + (y + 2) * p0 + xx + 2;
@@ -608,7 +555,7 @@ __device__ __forceinline__ void zero_fill(float *sm, const Geom &g) {
 // the unit's 128-byte lines (prefetch only; no registers or shared memory are tied up).
 template <typename T>
 __device__ __forceinline__ void prefetch_unit_l2(const Geom &g, const T *__restrict__ src, int c0, int b) {
-    const char *base = reinterpret_cast<const char *>(src + ((size_t)b * g.C + c0) * g.HW0);
+    const char *base = reinterpret_cast<const char *>(src + ((size_t)b * g.C + c0) * g.H * g.W);
     const int bytes = g.NPL * g.plane_bytes;
     for (int o = threadIdx.x * 128; o < bytes; o += blockDim.x * 128)
         asm volatile("prefetch.global.L2 [%0];" ::"l"(base + o));
@@ -623,7 +570,7 @@ __device__ __forceinline__ void issue_unit_copies(unsigned long long *bar, char 
     const unsigned bytes = (unsigned)g.NPL * g.plane_bytes;
     if (g.no_copy) return;  // test mode: the barrier is never armed, nothing is in flight
     mbar_expect_tx(bar, bytes * (src2 ? 2u : 1u));
-    const size_t po = ((size_t)b * g.C + c0) * g.HW0;
+    const size_t po = ((size_t)b * g.C + c0) * g.H * g.W;
     bulk_g2s(raw, src + po, bytes, bar);
     if (src2) bulk_g2s(raw + bytes, src2 + po, bytes, bar);
 }
@@ -816,17 +763,6 @@ __device__ __forceinline__ void store_tile(const Geom &g, float *sm, T *__restri
     }
 }
 
-// DEEP: the result is a float plane in the place of the tensor's plane (an addend that the kernel behind this one reads before
-// it stores the plane).
-template <typename T, int TH>
-__device__ __forceinline__ void store_deep(const Geom &g, T *out, size_t plane, int tyy, int txx, float (&acc)[TH][4]) {
-    float *o = deep_plane(out, plane, g.HW0) + (TH * tyy) * g.W + 4 * txx;
-    const bool vec = g.vec && (g.HW0 & 7) == 0 && 4 * txx + 3 < g.W;
-#pragma unroll
-    for (int r = 0; r < TH; ++r)
-        if (TH * tyy + r < g.H) store_row4(o + r * g.W, 4 * txx, g.W, vec, acc[r]);
-}
-
 // ------------------------------------------------------------------ forward / input-gradient kernel
 // Adds the Proposition 2 terms of all levels to one 4x4 pixel block (block row t4, block column tx of
 // the plane) held in a[0..3][0..3]; `bias` is the folded bias.
@@ -889,7 +825,7 @@ __device__ __forceinline__ void synth_block(const float *S, const Geom &g, int t
 
 // FLIP = false: out = WTConv(x).  FLIP = true: the same dataflow on grad_out with every kernel rotated
 // by 180 degrees and no bias gives grad_x.  MINB = resident blocks per SM the register budget is sized for.
-template <typename T, bool FLIP, int MAXT, int MINB, int TH, int KT, bool DEEP = false>
+template <typename T, bool FLIP, int MAXT, int MINB, int TH, int KT>
 __global__ void __launch_bounds__(MAXT, MINB)
 plane_fwd_kernel(const __grid_constant__ Geom g, const T *__restrict__ x, const float *__restrict__ w0,
                  const float *__restrict__ s0, const float *__restrict__ b0, const float *__restrict__ wl,
@@ -907,7 +843,7 @@ plane_fwd_kernel(const __grid_constant__ Geom g, const T *__restrict__ x, const 
     const unsigned wait_limit = g.no_copy ? WAIT_LIMIT_TEST : WAIT_LIMIT;
     const int L = g.L, nlv = g.lvl_start[L + 1];
     const int nlevel_items = g.NPL * nlv, nitems = nlevel_items + g.NPL * g.nbase;
-    const size_t HW = (size_t)g.HW0;
+    const size_t HW = (size_t)g.H * g.W;
     int c_prev = -1;
     // Staging order: the threads that hold a base tile (the last `nbase_thr` items of the list) are busy with
     // the synthesis of the previous unit when the next one is staged, so the others stage, two patches each
@@ -958,19 +894,19 @@ plane_fwd_kernel(const __grid_constant__ Geom g, const T *__restrict__ x, const 
             late = !mbar_wait(bar + ring, parity, wait_limit);
             const T *rx = reinterpret_cast<const T *>(raw + ring * g.stage_bytes);
             if (hoist_patch) {
-                run_patch<T, true, DEEP>(sm, g, patch0, rx, nvalid);
-                run_patch<T, true, DEEP>(sm, g, patch1, rx, nvalid);
+                run_patch<T, true>(sm, g, patch0, rx, nvalid);
+                run_patch<T, true>(sm, g, patch1, rx, nvalid);
                 lnext = 3;
             } else {
-                lnext = stage_input<T, true, DEEP>(sm, g, g.offA, rx, c, b, srank, nstagers);
+                lnext = stage_input<T, true>(sm, g, g.offA, rx, c, b, srank, nstagers);
             }
         } else if (hoist_patch) {
             const T *gsrc = x + ((size_t)b * g.C + c) * HW;
-            run_patch<T, false, DEEP>(sm, g, patch0, gsrc, nvalid);
-            run_patch<T, false, DEEP>(sm, g, patch1, gsrc, nvalid);
+            run_patch<T, false>(sm, g, patch0, gsrc, nvalid);
+            run_patch<T, false>(sm, g, patch1, gsrc, nvalid);
             lnext = 3;
         } else {
-            lnext = stage_input<T, false, DEEP>(sm, g, g.offA, x, c, b, srank, nstagers);
+            lnext = stage_input<T, false>(sm, g, g.offA, x, c, b, srank, nstagers);
         }
         if (g.bulk) {
             if (__syncthreads_or(late)) {
@@ -1015,12 +951,7 @@ plane_fwd_kernel(const __grid_constant__ Geom g, const T *__restrict__ x, const 
                     d = decode_item(g, tid + k * nthr, nlevel_items, nitems, bslot, tyy, txx, isb);
                     has_base = isb;
                 }
-                if (DEEP && d.z == -1) {  // no base convolution: the tile is the synthesis alone
-#pragma unroll
-                    for (int r = 0; r < TH; ++r)
-#pragma unroll
-                        for (int q = 0; q < 4; ++q) acc[r][q] = 0.f;
-                } else if (d.meta < 0) {
+                if (d.meta < 0) {
                     float w[KK];
                     load_weights(sm + d.wt, w);
                     conv_tile<TH, false, KT>(sm + d.src, d.meta & 0x3ff, w, acc);
@@ -1041,10 +972,7 @@ plane_fwd_kernel(const __grid_constant__ Geom g, const T *__restrict__ x, const 
             const float *S = sm + bslot * g.slot_stride;
 #pragma unroll
             for (int hb = 0; hb < TH / 4; ++hb) synth_block(S, g, (TH / 4) * tyy + hb, txx, bias, &acc[4 * hb]);
-            if (bslot < nvalid) {
-                if (DEEP) store_deep<T, TH>(g, out, (size_t)b * g.C + c + bslot, tyy, txx, acc);
-                else store_tile<T, TH>(g, sm, out + ((size_t)b * g.C + c + bslot) * HW, bslot, tyy, txx, acc);
-            }
+            if (bslot < nvalid) store_tile<T, TH>(g, sm, out + ((size_t)b * g.C + c + bslot) * HW, bslot, tyy, txx, acc);
         }
         if (g.bulk_out) {  // the unit is contiguous in global memory: one bulk store once every tile is in place
             fence_async_smem();  // every writer orders its shared-memory writes before the async proxy's reads
@@ -1197,7 +1125,7 @@ plane_wgrad_kernel(const __grid_constant__ Geom g, const T *__restrict__ x, cons
 //                    closed-form synthesis of Proposition 2 and the store of grad_x.
 // Used when a unit's item list fits one round of the block (<= 256 tiles); otherwise the separate weight-
 // gradient and input-gradient kernels run.
-template <typename T, int TH, int BULK, int KT, bool DEEP = false>  // BULK: tensors prefetched by bulk copy (0 none, 2 x and grad_out)
+template <typename T, int TH, int BULK, int KT>  // BULK: tensors prefetched by bulk copy (0 none, 2 x and grad_out)
 __global__ void __launch_bounds__(256, 2)
 plane_bwd_kernel(const __grid_constant__ Geom g, const T *__restrict__ x, const T *__restrict__ go,
                  const float *__restrict__ w0, const float *__restrict__ s0, const float *__restrict__ wl,
@@ -1214,7 +1142,7 @@ plane_bwd_kernel(const __grid_constant__ Geom g, const T *__restrict__ x, const 
     unsigned parity = 0;
     const int L = g.L, nlv = g.lvl_start[L + 1], ncls = 1 + 4 * L;
     const int nlevel_items = g.NPL * nlv, nitems = nlevel_items + g.NPL * g.nbase;
-    const size_t HW = (size_t)g.HW0;
+    const size_t HW = (size_t)g.H * g.W;
     int bslot = 0, tyy = 0, txx = 0;
     bool has_base = false;
     const ItemD item = decode_item(g, tid, nlevel_items, nitems, bslot, tyy, txx, has_base);
@@ -1256,23 +1184,23 @@ plane_bwd_kernel(const __grid_constant__ Geom g, const T *__restrict__ x, const 
             const T *rx = reinterpret_cast<const T *>(raw + ring * g.stage_bytes);
             const T *rg = reinterpret_cast<const T *>(raw + ring * g.stage_bytes + (size_t)g.NPL * g.plane_bytes);
             if (hoist_patch) {
-                run_patch<T, true, DEEP>(sm, g, patch0, rx, nvalid);
-                run_patch<T, true, DEEP>(sm, g, patch0, rg, nvalid, dA0, dA1, dA2);
-                run_patch<T, true, DEEP>(sm, g, patch1, rx, nvalid);
-                run_patch<T, true, DEEP>(sm, g, patch1, rg, nvalid, dA0, dA1, dA2);
+                run_patch<T, true>(sm, g, patch0, rx, nvalid);
+                run_patch<T, true>(sm, g, patch0, rg, nvalid, dA0, dA1, dA2);
+                run_patch<T, true>(sm, g, patch1, rx, nvalid);
+                run_patch<T, true>(sm, g, patch1, rg, nvalid, dA0, dA1, dA2);
                 lnext = 3;
             } else {
-                lnext = stage_input<T, true, DEEP>(sm, g, g.offA, rx, c, b, tid, nthr);
-                stage_input<T, true, DEEP>(sm, g, g.offG, rg, c, b, tid, nthr);
+                lnext = stage_input<T, true>(sm, g, g.offA, rx, c, b, tid, nthr);
+                stage_input<T, true>(sm, g, g.offG, rg, c, b, tid, nthr);
             }
         } else if (hoist_patch) {
             const size_t po = ((size_t)b * g.C + c) * HW;
-            run_patch_pair<T, false, DEEP>(sm, g, patch0, x + po, go + po, nvalid, dA0, dA1, dA2);
-            run_patch_pair<T, false, DEEP>(sm, g, patch1, x + po, go + po, nvalid, dA0, dA1, dA2);
+            run_patch_pair<T, false>(sm, g, patch0, x + po, go + po, nvalid, dA0, dA1, dA2);
+            run_patch_pair<T, false>(sm, g, patch1, x + po, go + po, nvalid, dA0, dA1, dA2);
             lnext = 3;
         } else {
-            lnext = stage_input<T, false, DEEP>(sm, g, g.offA, x, c, b, tid, nthr);
-            stage_input<T, false, DEEP>(sm, g, g.offG, go, c, b, tid, nthr);
+            lnext = stage_input<T, false>(sm, g, g.offA, x, c, b, tid, nthr);
+            stage_input<T, false>(sm, g, g.offG, go, c, b, tid, nthr);
         }
         if (BULK) {
             if (__syncthreads_or(late)) {
@@ -1304,12 +1232,7 @@ plane_bwd_kernel(const __grid_constant__ Geom g, const T *__restrict__ x, const 
             __syncthreads();
         }
         float acc[TH][4];
-        if (DEEP && has_base) {  // no base convolution: the tile is the synthesis alone
-#pragma unroll
-            for (int r = 0; r < TH; ++r)
-#pragma unroll
-                for (int q = 0; q < 4; ++q) acc[r][q] = 0.f;
-        } else if (item.meta < 0) {
+        if (item.meta < 0) {
             const int pitch = item.meta & 0x3ff;
             const float *ysrc = sm + item.src;            // Y window (x side)
             const float *gsrc = sm + item.src + item.dg;  // D window (grad_out side)
@@ -1358,10 +1281,7 @@ plane_bwd_kernel(const __grid_constant__ Geom g, const T *__restrict__ x, const 
             const float *S = sm + bslot * g.slot_stride;
 #pragma unroll
             for (int hb = 0; hb < TH / 4; ++hb) synth_block(S, g, (TH / 4) * tyy + hb, txx, 0.f, &acc[4 * hb]);
-            if (bslot < nvalid) {
-                if (DEEP) store_deep<T, TH>(g, gx, (size_t)b * g.C + c + bslot, tyy, txx, acc);
-                else store_tile<T, TH>(g, sm, gx + ((size_t)b * g.C + c + bslot) * HW, bslot, tyy, txx, acc);
-            }
+            if (bslot < nvalid) store_tile<T, TH>(g, sm, gx + ((size_t)b * g.C + c + bslot) * HW, bslot, tyy, txx, acc);
         }
         if (BULK && g.bulk_out) {
             fence_async_smem();  // every writer orders its shared-memory writes before the async proxy's reads
@@ -1390,7 +1310,7 @@ plane_bwd_kernel(const __grid_constant__ Geom g, const T *__restrict__ x, const 
             const int slotp = blockIdx.x - block_of_unit((long long)cg * g.B, gridDim.x, g.units);
             for (int e = tid; e < nvalid * ncls * (KK + 1); e += nthr) {
                 const int sc = e / (KK + 1), t = e - sc * (KK + 1), slot = sc / ncls, c2 = sc - slot * ncls;
-                if ((c2 > 0 && t == KK) || (DEEP && c2 == 0)) continue;
+                if (c2 > 0 && t == KK) continue;
                 const int ch = c + slot;
                 float sacc = 0.f;
                 const int th1 = run_end[sc];  // known trip count: the loads of the sum do not wait for one another
@@ -1424,12 +1344,7 @@ plane_bwd_kernel(const __grid_constant__ Geom g, const T *__restrict__ x, const 
 }
 
 // ------------------------------------------------------------------ host-side planning
-// `deep` > 0: the tensor's planes are (deep >> 16) x (deep & 0xffff), the kernel works on their level-1 low-pass band H x W.
-inline void fill_common(Geom &g, int B, int C, int H, int W, int L, int elem_bytes, int TH, int deep = 0) {
-    g.deep = deep > 0;
-    g.H0 = deep > 0 ? deep >> 16 : H;
-    g.W0 = deep > 0 ? deep & 0xffff : W;
-    g.HW0 = g.H0 * g.W0;
+inline void fill_common(Geom &g, int B, int C, int H, int W, int L, int elem_bytes, int TH) {
     g.B = B; g.C = C; g.H = H; g.W = W; g.L = L; g.th = TH;
     g.Hl[0] = H; g.Wl[0] = W;
     for (int l = 1; l <= MAXL; ++l) { g.Hl[l] = (g.Hl[l - 1] + 1) / 2; g.Wl[l] = (g.Wl[l - 1] + 1) / 2; }
@@ -1463,7 +1378,7 @@ inline void fill_common(Geom &g, int B, int C, int H, int W, int L, int elem_byt
     g.d_nbase = make_fastdiv(g.nbase);
     g.npatch4 = ((H + 3) / 4) * (W / 4 > 0 ? W / 4 : 1);
     g.d_npatch4 = make_fastdiv(g.npatch4);
-    g.plane_bytes = g.HW0 * elem_bytes;
+    g.plane_bytes = H * W * elem_bytes;
     g.bulk = 0;  // decided per plan: a unit of NPL planes must be a 16-byte multiple and C a multiple of NPL
     g.raw_slot_bytes = g.plane_bytes;
 }
@@ -1481,7 +1396,7 @@ inline long long finish_layout(Geom &g, long long arrays_floats, int wtab_floats
     if (use_bulk) off += ((long long)g.nstage * g.stage_bytes + 3) / 4;
     off = pad4((int)off);
     g.out_off = (int)off;
-    g.bulk_out = (use_bulk && !g.vec && !g.deep) ? 1 : 0;  // rows that are not 16-byte multiples: assemble the unit on chip
+    g.bulk_out = (use_bulk && !g.vec) ? 1 : 0;  // rows that are not 16-byte multiples: assemble the unit on chip
     if (g.bulk_out) off += ((long long)g.NPL * g.plane_bytes + 3) / 4;
     off = pad4((int)off);
     g.bar_off = (int)off;
@@ -1541,11 +1456,11 @@ inline double tile_score(const Geom &g, double short_tiles = 0.93) {
 }
 
 // Forward plan.  `tune` (0 = automatic): bits 0-4 threads/32, bits 5-7 blocks per SM, bits 8-13 planes per unit.
-inline bool plan_forward_th(int B, int C, int H, int W, int L, int elem_bytes, Geom &best, unsigned tune, int th, int deep) {
+inline bool plan_forward_th(int B, int C, int H, int W, int L, int elem_bytes, Geom &best, unsigned tune, int th) {
     const int fT = (tune & 31) * 32, fBps = (tune >> 5) & 7, fNpl = (tune >> 8) & 63;
     const bool no_bulk = (tune >> 20) & 1;
     Geom g = {};
-    fill_common(g, B, C, H, W, L, elem_bytes, th, deep);
+    fill_common(g, B, C, H, W, L, elem_bytes, th);
     const int slot = layout_slot(g, false, true);
     const int M = g.lvl_start[L + 1] + g.nbase;
     const double teff = tile_score(g);
@@ -1601,11 +1516,11 @@ inline bool plan_forward_th(int B, int C, int H, int W, int L, int elem_bytes, G
 
 // Weight-gradient plan: per class c with n_c tiles (x NPL) allocate ceil(n_c NPL / rounds) threads, smallest
 // `rounds` that fits the thread limit.  tune bits 14-19: planes per unit.
-inline bool plan_wgrad_th(int B, int C, int H, int W, int L, int elem_bytes, Geom &best, unsigned tune, int th, int deep) {
+inline bool plan_wgrad_th(int B, int C, int H, int W, int L, int elem_bytes, Geom &best, unsigned tune, int th) {
     const int fNpl = (tune >> 14) & 63, fBps = 0;
     const bool no_bulk = (tune >> 20) & 1;
     Geom g = {};
-    fill_common(g, B, C, H, W, L, elem_bytes, th, deep);
+    fill_common(g, B, C, H, W, L, elem_bytes, th);
     const int slot = layout_slot(g, true, false);
     const int ncls = 1 + 4 * L;
     const double teff = tile_score(g);
@@ -1675,10 +1590,10 @@ inline bool plan_wgrad_th(int B, int C, int H, int W, int L, int elem_bytes, Geo
 
 // Fused-backward plan: one round (every tile its own thread), both input pyramids plus Z in shared memory, no
 // bulk prefetch unless it fits.  tune bits 14-19: planes per unit (shared with the weight-gradient plan).
-inline bool plan_bwd_fused_th(int B, int C, int H, int W, int L, int elem_bytes, Geom &best, unsigned tune, int th, int deep) {
+inline bool plan_bwd_fused_th(int B, int C, int H, int W, int L, int elem_bytes, Geom &best, unsigned tune, int th) {
     const int fNpl = (tune >> 14) & 63, fBps = 0;
     Geom g = {};
-    fill_common(g, B, C, H, W, L, elem_bytes, th, deep);
+    fill_common(g, B, C, H, W, L, elem_bytes, th);
     const int slot = layout_slot(g, true, true);
     const int M = g.lvl_start[L + 1] + g.nbase;
     const double teff = tile_score(g, 1.03);
@@ -1738,28 +1653,28 @@ inline bool plan_bwd_fused_th(int B, int C, int H, int W, int L, int elem_bytes,
 }
 
 // Each plan is searched for both tile heights; tune bit 22 forces 8 rows, bit 23 forces 4 rows.
-inline bool search_forward(int B, int C, int H, int W, int L, int elem_bytes, Geom &best, unsigned tune, int deep) {
+inline bool search_forward(int B, int C, int H, int W, int L, int elem_bytes, Geom &best, unsigned tune) {
     best.score = -1.0;
     bool ok = false;
-    if (!((tune >> 23) & 1)) ok |= plan_forward_th(B, C, H, W, L, elem_bytes, best, tune, 8, deep);
-    if (!((tune >> 22) & 1)) ok |= plan_forward_th(B, C, H, W, L, elem_bytes, best, tune, 4, deep);
+    if (!((tune >> 23) & 1)) ok |= plan_forward_th(B, C, H, W, L, elem_bytes, best, tune, 8);
+    if (!((tune >> 22) & 1)) ok |= plan_forward_th(B, C, H, W, L, elem_bytes, best, tune, 4);
     if (ok) deepen_prefetch(best);
     return ok;
 }
-inline bool search_wgrad(int B, int C, int H, int W, int L, int elem_bytes, Geom &best, unsigned tune, int deep) {
+inline bool search_wgrad(int B, int C, int H, int W, int L, int elem_bytes, Geom &best, unsigned tune) {
     best.score = -1.0;
     bool ok = false;
-    if (!((tune >> 23) & 1)) ok |= plan_wgrad_th(B, C, H, W, L, elem_bytes, best, tune, 8, deep);
-    if (!((tune >> 22) & 1)) ok |= plan_wgrad_th(B, C, H, W, L, elem_bytes, best, tune, 4, deep);
+    if (!((tune >> 23) & 1)) ok |= plan_wgrad_th(B, C, H, W, L, elem_bytes, best, tune, 8);
+    if (!((tune >> 22) & 1)) ok |= plan_wgrad_th(B, C, H, W, L, elem_bytes, best, tune, 4);
     if (ok) deepen_prefetch(best);
     return ok;
 }
-inline bool search_bwd_fused(int B, int C, int H, int W, int L, int elem_bytes, Geom &best, unsigned tune, int deep) {
+inline bool search_bwd_fused(int B, int C, int H, int W, int L, int elem_bytes, Geom &best, unsigned tune) {
     if ((tune >> 21) & 1) return false;  // bit 21: never fuse
     best.score = -1.0;
     bool ok = false;
-    if (!((tune >> 23) & 1)) ok |= plan_bwd_fused_th(B, C, H, W, L, elem_bytes, best, tune, 8, deep);
-    if (!((tune >> 22) & 1)) ok |= plan_bwd_fused_th(B, C, H, W, L, elem_bytes, best, tune, 4, deep);
+    if (!((tune >> 23) & 1)) ok |= plan_bwd_fused_th(B, C, H, W, L, elem_bytes, best, tune, 8);
+    if (!((tune >> 22) & 1)) ok |= plan_bwd_fused_th(B, C, H, W, L, elem_bytes, best, tune, 4);
     if (ok) deepen_prefetch(best);
     return ok;
 }
@@ -1767,11 +1682,11 @@ inline bool search_bwd_fused(int B, int C, int H, int W, int L, int elem_bytes, 
 // The searches above walk a few thousand candidates (tens of microseconds of host time), more than a small
 // layer's kernels take on the GPU, so every entry point looks its plan up in a small process-wide cache first.
 struct PlanKey {
-    int kind, B, C, H, W, L, elem_bytes, deep;
+    int kind, B, C, H, W, L, elem_bytes;
     unsigned tune;
     bool operator==(const PlanKey &o) const {
         return kind == o.kind && B == o.B && C == o.C && H == o.H && W == o.W && L == o.L && elem_bytes == o.elem_bytes &&
-               deep == o.deep && tune == o.tune;
+               tune == o.tune;
     }
 };
 struct PlanEntry {
@@ -1779,10 +1694,10 @@ struct PlanEntry {
     bool ok;
     Geom g;
 };
-inline bool cached_plan(int kind, int B, int C, int H, int W, int L, int elem_bytes, Geom &best, unsigned tune, int deep = 0) {
+inline bool cached_plan(int kind, int B, int C, int H, int W, int L, int elem_bytes, Geom &best, unsigned tune) {
     static std::mutex mu;
     static std::vector<PlanEntry> cache;
-    const PlanKey key = {kind, B, C, H, W, L, elem_bytes, deep, tune};
+    const PlanKey key = {kind, B, C, H, W, L, elem_bytes, tune};
     {
         std::lock_guard<std::mutex> lock(mu);
         for (const PlanEntry &e : cache)
@@ -1794,9 +1709,9 @@ inline bool cached_plan(int kind, int B, int C, int H, int W, int L, int elem_by
     PlanEntry e;
     e.key = key;
     e.g = Geom{};
-    e.ok = kind == 0   ? search_forward(B, C, H, W, L, elem_bytes, e.g, tune, deep)
-           : kind == 1 ? search_wgrad(B, C, H, W, L, elem_bytes, e.g, tune, deep)
-                       : search_bwd_fused(B, C, H, W, L, elem_bytes, e.g, tune, deep);
+    e.ok = kind == 0   ? search_forward(B, C, H, W, L, elem_bytes, e.g, tune)
+           : kind == 1 ? search_wgrad(B, C, H, W, L, elem_bytes, e.g, tune)
+                       : search_bwd_fused(B, C, H, W, L, elem_bytes, e.g, tune);
     {
         std::lock_guard<std::mutex> lock(mu);
         if (cache.size() >= 256) cache.clear();  // bounded: a process cycling through more shapes just searches again
@@ -1986,77 +1901,6 @@ cudaError_t backward(int B, int C, int H, int W, int L, const T *x, const T *go,
     return cudaSuccess;
 }
 
-// ------------------------------------------------------------------ levels >= 2 of a larger layer
-// For a kernel that does the base convolution and level 1 itself (tensor_kernels.cuh): levels 2 .. L of the planes' level-1
-// low-pass bands, which are worked out from the pixels on the way in.  The result is left as a float plane in the place of
-// each plane of `out`; the weight gradients of levels 2 .. L go to `partl` ([L - 1][C][np][4][25]).
-inline int deep_key(int H, int W) { return H << 16 | W; }
-inline bool plan_deep(bool bwd, int B, int C, int H, int W, int L, Geom &g) {
-    // a float plane of the band has to fit the 16-bit plane, whatever byte it starts on
-    if (((H + 1) / 2) * ((W + 1) / 2) * 4 + 2 > H * W * 2 && ((H & 1) || (W & 1))) return false;
-    return cached_plan(bwd ? 2 : 0, B, C, (H + 1) / 2, (W + 1) / 2, L - 1, 2, g, 0, deep_key(H, W));
-}
-template <typename T>
-cudaError_t deep_forward(int B, int C, int H, int W, int L, const T *x, const float *wl, const float *sl, T *out, int *status, cudaStream_t st,
-                         unsigned tag, bool no_copy) {
-    Geom g;
-    cudaError_t e;
-    if (!plan_deep(false, B, C, H, W, L, g)) return cudaErrorInvalidValue;
-    g.no_copy = no_copy;
-    g.tag = tag;
-    g.alarm = call_alarm;
-    const float *none = nullptr;
-#define WT_LAUNCH_DEEP(MAXT_, MINB_, TH_)                                                                                       \
-    {                                                                                                                           \
-        constexpr auto kern = plane_fwd_kernel<T, false, MAXT_, MINB_, TH_, 5, true>;                                           \
-        if ((e = opt_in_smem<kern>()) != cudaSuccess) return e;                                                                 \
-        return launch_overlapped(kern, (unsigned)g.nblocks, (unsigned)g.nthreads, (size_t)g.smem_floats * 4, st, g, x, none, none, none, wl, \
-                                 sl, out, status);                                                                              \
-    }
-    if (g.nthreads <= 128 && g.nthreads * g.blocks_per_sm <= 512) {
-        if (g.th == 8) WT_LAUNCH_DEEP(128, 4, 8) else WT_LAUNCH_DEEP(128, 4, 4)
-    } else if (g.nthreads * g.blocks_per_sm <= 512) {
-        if (g.th == 8) WT_LAUNCH_DEEP(256, 2, 8) else WT_LAUNCH_DEEP(256, 2, 4)
-    } else if (g.nthreads <= 128) {
-        if (g.th == 8) WT_LAUNCH_DEEP(128, 6, 8) else WT_LAUNCH_DEEP(128, 6, 4)
-    } else {
-        if (g.th == 8) WT_LAUNCH_DEEP(256, 3, 8) else WT_LAUNCH_DEEP(256, 3, 4)
-    }
-#undef WT_LAUNCH_DEEP
-}
-template <typename T>
-cudaError_t deep_backward(int B, int C, int H, int W, int L, const T *x, const T *go, const float *wl, const float *sl, T *gx, float *partl,
-                          EpiloguePtrs *ep, int *status, cudaStream_t st, unsigned tag, bool no_copy) {
-    Geom g;
-    cudaError_t e;
-    if (!plan_deep(true, B, C, H, W, L, g)) return cudaErrorInvalidValue;
-    g.no_copy = no_copy;
-    g.tag = tag;
-    g.alarm = call_alarm;
-    const float *none = nullptr;
-    float *nowhere = nullptr;
-#define WT_LAUNCH_DEEP(TH_, BULK_)                                                                                              \
-    {                                                                                                                           \
-        constexpr auto kern = plane_bwd_kernel<T, TH_, BULK_, 5, true>;                                                         \
-        if ((e = opt_in_smem<kern>()) != cudaSuccess) return e;                                                                 \
-        e = launch_overlapped(kern, (unsigned)g.nblocks, (unsigned)g.nthreads, (size_t)g.smem_floats * 4, st, g, x, go, none, none, wl, sl, \
-                              gx, nowhere, partl, status);                                                                      \
-    }
-    if (g.th == 8) {
-        if (g.bulk == 2) WT_LAUNCH_DEEP(8, 2) else WT_LAUNCH_DEEP(8, 0)
-    } else {
-        if (g.bulk == 2) WT_LAUNCH_DEEP(4, 2) else WT_LAUNCH_DEEP(4, 0)
-    }
-#undef WT_LAUNCH_DEEP
-    if (e != cudaSuccess) return e;
-    for (int l = 1; l < L; ++l) {
-        ep->partl[l] = partl + (size_t)(l - 1) * C * g.np * 4 * KK;
-        ep->npl[l] = g.np;
-    }
-    ep->deep = EpiloguePtrs::Split{g.NPL, B, g.units, g.nblocks};
-    return cudaSuccess;
-}
-
 // Explicit instantiation (EXTERN empty) or its declaration (EXTERN = extern) of the host entry points for one
 // activation type: the kernels are compiled once, in the instantiation unit of that type.
 #define WT_PLANE_INSTANTIATE(T, EXTERN)                                                                                    \
@@ -2066,12 +1910,6 @@ cudaError_t deep_backward(int B, int C, int H, int W, int L, const T *x, const T
     EXTERN template cudaError_t backward<T>(int, int, int, int, int, const T *, const T *, const float *, const float *,    \
                                             const float *, const float *, T *, char *, EpiloguePtrs *, cudaStream_t,       \
                                             unsigned, unsigned, bool, int);
-
-#define WT_PLANE_DEEP_INSTANTIATE(T, EXTERN)                                                                                  \
-    EXTERN template cudaError_t deep_forward<T>(int, int, int, int, int, const T *, const float *, const float *, T *, int *,   \
-                                                cudaStream_t, unsigned, bool);                                                  \
-    EXTERN template cudaError_t deep_backward<T>(int, int, int, int, int, const T *, const T *, const float *, const float *, T *, float *, \
-                                                 EpiloguePtrs *, int *, cudaStream_t, unsigned, bool);
 
 }  // namespace plane
 }  // namespace wt

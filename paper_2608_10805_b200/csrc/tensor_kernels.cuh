@@ -29,10 +29,6 @@
 #include "plane_kernels.cuh"
 
 namespace wt {
-namespace plane {
-WT_PLANE_DEEP_INSTANTIATE(__half, extern)  // levels >= 2, compiled in their own unit
-WT_PLANE_DEEP_INSTANTIATE(__nv_bfloat16, extern)
-}  // namespace plane
 namespace tensor {
 
 typedef unsigned long long u64;
@@ -66,7 +62,7 @@ struct KGeom {
     int conv_off, x_off, parts_off, raw_off, out_off, table_off, misc_off, smem;  // byte offsets
     int ring, cols;              // tensor-memory ring depth and columns allocated
     int bps, nblocks, np;
-    int no_copy, bias, deep;     // deep: levels >= 2 come as a float addend per 2 x 2 pixels, 1 in the planes' own place, 2 in a tensor
+    int no_copy, bias, deep;     // deep: levels >= 2 come as a float addend per 2 x 2 pixels (panels only)
     FastDiv d_period, d_nty, d_n, d_Pc, d_Px, d_ec, d_ex, d_out_words;  // d_ec / d_ex: chunks of one octet in the convolved / the x array
     int *alarm;
     unsigned tag;
@@ -262,14 +258,13 @@ __device__ __forceinline__ void repack(char *arr, const char *raw, const Item *i
 }
 // The same for one column panel, straight from global memory (a panel's rows are short: staging them first costs a pass over
 // shared memory, whose bandwidth the MMAs need).  x0 = the panel's first column.
-template <typename T, bool SUM>
-__device__ __forceinline__ void repack_panel(char *arr, const T *__restrict__ src, const Item *items, const KGeom &g, int P, const FastDiv &dP,
+template <typename T, bool SUM, bool QUADS>
+__device__ __forceinline__ void repack_panel_t(char *arr, const T *__restrict__ src, const Item *items, const KGeom &g, int P, const FastDiv &dP,
                                              const FastDiv &dE, int shift, int x0, int warp, int lane, float &sum) {
-    constexpr int U = 4;
+    constexpr int U = QUADS ? 6 : 4;  // words in flight: the loads' latency is what this phase costs
     const int img = lane & 7, per = (int)dE.d;
     const int wpo = g.S >= 8 ? 1 : g.S >= 4 ? 2 : g.S >= 2 ? 4 : 8, step = wpo * 4;  // warps to an octet
     const int e_first = (warp & (wpo - 1)) * 4 + (lane >> 3);
-    const bool quads = (g.W & 3) == 0;  // four pixels are one aligned word, wholly inside a row or wholly outside
     const long long total = (long long)g.B * g.C * g.HW;
     for (int o = warp / wpo; o < g.S; o += 8 / wpo) {
         const Item it = items[o * 8 + img];
@@ -277,20 +272,20 @@ __device__ __forceinline__ void repack_panel(char *arr, const T *__restrict__ sr
         const long long e_base = (long long)it.at(g, 0) + (long long)ybase * g.W + x0 - shift;
         char *dst = arr + ((o * g.period * P) * 8 + img) * 16;
         for (int e0 = e_first; e0 < per; e0 += U * step) {
-            unsigned v[U][4], h[U][4];
+            unsigned v[U][4], h[QUADS ? 1 : U][4];
             int col[U];
             int sh[U];
 #pragma unroll
             for (int i = 0; i < U; ++i) {
                 const int e = e0 + i * step;
                 v[i][0] = v[i][1] = v[i][2] = v[i][3] = 0u;
-                h[i][0] = h[i][1] = h[i][2] = h[i][3] = 0u;
+                if (!QUADS) h[i][0] = h[i][1] = h[i][2] = h[i][3] = 0u;
                 const int rr = fdiv(e, dP), j = e - rr * P, y = ybase + rr;
                 col[i] = x0 + 8 * j - shift;
                 sh[i] = 0;
                 if (e < per && it.ty >= 0 && (unsigned)y < (unsigned)g.H && col[i] > -8 && col[i] < g.W) {
                     const long long at = e_base + (long long)rr * g.W + 8 * j;
-                    if (quads) {
+                    if (QUADS) {  // four pixels are one aligned word, wholly inside a row or wholly outside
                         if ((unsigned)col[i] < (unsigned)g.W) { const uint2 t = __ldg(reinterpret_cast<const uint2 *>(src + at)); v[i][0] = t.x; v[i][1] = t.y; }
                         if ((unsigned)(col[i] + 4) < (unsigned)g.W) { const uint2 t = __ldg(reinterpret_cast<const uint2 *>(src + at + 4)); v[i][2] = t.x; v[i][3] = t.y; }
                     } else {  // two aligned words around the eight pixels; words that leave the tensor are read pixel by pixel
@@ -301,7 +296,8 @@ __device__ __forceinline__ void repack_panel(char *arr, const T *__restrict__ sr
                             v[i][0] = t.x; v[i][1] = t.y; v[i][2] = t.z; v[i][3] = t.w;
                             if (sh[i]) {
                                 const uint4 t2 = __ldg(reinterpret_cast<const uint4 *>(src + 8 * w) + 1);
-                                h[i][0] = t2.x; h[i][1] = t2.y; h[i][2] = t2.z; h[i][3] = t2.w;
+                                unsigned *b = h[QUADS ? 0 : i];
+                                b[0] = t2.x; b[1] = t2.y; b[2] = t2.z; b[3] = t2.w;
                             }
                         } else {
                             sh[i] = 0;
@@ -319,8 +315,8 @@ __device__ __forceinline__ void repack_panel(char *arr, const T *__restrict__ sr
             for (int i = 0; i < U; ++i) {
                 const int e = e0 + i * step;
                 if (e >= per) continue;
-                if (!quads && col[i] > -8) {
-                    unsigned *a = v[i], *b = h[i];
+                if (!QUADS && col[i] > -8) {
+                    unsigned *a = v[i], *b = h[QUADS ? 0 : i];
                     if (sh[i] & 4) { a[0] = a[2]; a[1] = a[3]; a[2] = b[0]; a[3] = b[1]; b[0] = b[2]; b[1] = b[3]; }
                     if (sh[i] & 2) { a[0] = a[1]; a[1] = a[2]; a[2] = a[3]; a[3] = b[0]; b[0] = b[1]; }
                     if (sh[i] & 1) {
@@ -348,6 +344,27 @@ __device__ __forceinline__ void repack_panel(char *arr, const T *__restrict__ sr
                 *reinterpret_cast<uint4 *>(dst + e * 128) = make_uint4(v[i][0], v[i][1], v[i][2], v[i][3]);
             }
         }
+    }
+}
+template <typename T, bool SUM>
+__device__ __forceinline__ void repack_panel(char *arr, const T *__restrict__ src, const Item *items, const KGeom &g, int P, const FastDiv &dP,
+                                             const FastDiv &dE, int shift, int x0, int warp, int lane, float &sum) {
+    if ((g.W & 3) == 0) repack_panel_t<T, SUM, true>(arr, src, items, g, P, dP, dE, shift, x0, warp, lane, sum);
+    else repack_panel_t<T, SUM, false>(arr, src, items, g, P, dP, dE, shift, x0, warp, lane, sum);
+}
+// The next unit's rows on their way to L2 (a request, nothing is tied up): what is left of the loads' latency is L2's.
+template <typename T>
+__device__ __forceinline__ void prefetch_panel(const T *__restrict__ src, const Item *items, const KGeom &g, int x0, int tid) {
+    const int rows = g.th + 8, cols = g.tw + 8;
+    for (int e = tid; e < 8 * g.S * rows; e += WORKERS) {
+        const int slot = e / rows, rr = e - slot * rows;
+        const Item it = items[slot];
+        const int y = it.ty * g.th - 4 + rr;
+        if (it.ty < 0 || (unsigned)y >= (unsigned)g.H) continue;
+        const int c0 = x0 >= 8 ? x0 - 8 : 0, c1 = x0 + cols < g.W ? x0 + cols : g.W;
+        const char *a = reinterpret_cast<const char *>(src + it.at(g, y) + c0), *b = reinterpret_cast<const char *>(src + it.at(g, y) + c1);
+        for (const char *p = reinterpret_cast<const char *>(reinterpret_cast<uintptr_t>(a) & ~(uintptr_t)127); p < b; p += 128)
+            asm volatile("prefetch.global.L2 [%0];" ::"l"(p));
     }
 }
 template <typename T, bool SUM>
@@ -592,7 +609,11 @@ tensor_kernel(const __grid_constant__ KGeom g, const T *__restrict__ x, const T 
             }
         } else {
             if (u + 1 < u_end) {
-                if (!g.alias) fetch(set_next);
+                if (PANEL) {
+                    const int next0 = kn / g.upc * g.tw;
+                    prefetch_panel<T>(x, items + set_next * nslot, g, next0, tid);
+                    if (BWD) prefetch_panel<T>(go, items + set_next * nslot, g, next0, tid);
+                } else if (!g.alias) fetch(set_next);
                 if (cn != c) fetch_weights(cn);
             }
             // ---- epilogue: warps 0-3 take the even jobs (counted over the units), 4-7 the odd ones; a lane is one image of one row pair
@@ -628,12 +649,11 @@ tensor_kernel(const __grid_constant__ KGeom g, const T *__restrict__ x, const T 
                     if (std::is_same<T, __half>::value) v[i] = fmaf(scale, fmaf(p2[i], 1.f / 4194304.f, fmaf(p1[i], 1.f / 2048.f, v[i])), bias);
                     else v[i] = (v[i] + (p1[i] + p2[i])) + bias;
                 }
-                if (g.deep) {  // levels >= 2: one value (un-normalised LL of level 1, Proposition 2) per 2 x 2 pixels
+                if (PANEL && g.deep) {  // levels >= 2: one value (un-normalised LL of level 1, Proposition 2) per 2 x 2 pixels
                     const int W2 = (g.W + 1) >> 1, left = W2 - (x0 >> 1) - 4 * j;
-                    const float *d = (PANEL ? add + (u64)it.plane * (unsigned)(((g.H + 1) >> 1) * W2) : deep_plane(out, it.plane, g.HW)) + (y >> 1) * W2 +
-                                     (x0 >> 1) + 4 * j;
+                    const float *d = add + (u64)it.plane * (unsigned)(((g.H + 1) >> 1) * W2) + (y >> 1) * W2 + (x0 >> 1) + 4 * j;
                     float more[4];
-                    if (left >= 4 && (W2 & 3) == 0 && (PANEL || (g.HW & 7) == 0)) {
+                    if (left >= 4 && (W2 & 3) == 0) {
                         const float4 t4 = *reinterpret_cast<const float4 *>(d);
                         more[0] = t4.x; more[1] = t4.y; more[2] = t4.z; more[3] = t4.w;
                     } else {
@@ -952,10 +972,7 @@ inline bool search_n(const Request &q, KGeom &best, int n) {
 inline bool search(const Request &q, KGeom &best) {
     if ((q.K != 3 && q.K != 5) || q.L > 8 || q.H < 2 || q.W < 2 || (long long)q.H * q.W > 0x3fffffff) return false;
     if (wide(q) ? q.W < 8 : false) return false;
-    if (q.L > 1 && !wide(q)) {  // the addend lies in the planes' own place: a plane's items have to belong to one unit
-        plane::Geom d;
-        if (q.K != 5 || (q.H > 64 && q.H <= 96) || !plane::plan_deep(q.bwd, q.B, q.C, q.H, q.W, q.L, d)) return false;
-    }
+    if (q.L > 1 && !wide(q)) return false;
     best = KGeom{};
     best.cost = 1e30;
     bool found = false;
@@ -1007,8 +1024,6 @@ inline size_t backward_bytes(const Request &q) {
     if (!plan(q, g)) return 0;
     const size_t KK = (size_t)q.K * q.K;
     size_t floats = (size_t)g.C * g.np * (KK + 1 + 4 * KK);
-    plane::Geom d;
-    if (q.L > 1 && !wide(q) && plane::plan_deep(true, q.B, q.C, q.H, q.W, q.L, d)) floats += (size_t)(q.L - 1) * q.C * d.np * 4 * KK;
     return STATUS_BYTES + sizeof(float) * floats;
 }
 
@@ -1029,9 +1044,6 @@ cudaError_t forward(const Request &q, const T *x, const float *w0, const float *
     }
     constexpr auto kern = tensor_kernel<T, false, false>;
     if ((e = plane::opt_in_smem<kern>()) != cudaSuccess) return e;
-    if (q.L > 1 && (e = plane::deep_forward<T>(q.B, q.C, q.H, q.W, q.L, x, wl + (size_t)q.C * 4 * q.K * q.K, sl + (size_t)q.C * 4, out,
-                                               reinterpret_cast<int *>(ws), st, tag, no_copy)) != cudaSuccess)
-        return e;
     return launch_overlapped(kern, (unsigned)g.nblocks, (unsigned)THREADS, (size_t)g.smem, st, g, x, nullptr, w0, s0, b0, wl, sl, add, out, nullptr,
                              nullptr, reinterpret_cast<int *>(ws));
 }
@@ -1056,9 +1068,6 @@ cudaError_t backward(const Request &q, const T *x, const T *go, const float *w0,
     } else {
         constexpr auto kern = tensor_kernel<T, true, false>;
         if ((e = plane::opt_in_smem<kern>()) != cudaSuccess) return e;
-        if (q.L > 1 && (e = plane::deep_backward<T>(q.B, q.C, q.H, q.W, q.L, x, go, wl + (size_t)q.C * 4 * KK, sl + (size_t)q.C * 4, gx,
-                                                    partl + (size_t)g.C * g.np * 4 * KK, ep, reinterpret_cast<int *>(ws), st, tag, no_copy)) != cudaSuccess)
-            return e;
         e = launch_overlapped(kern, (unsigned)g.nblocks, (unsigned)THREADS, (size_t)g.smem, st, g, x, go, w0, s0, nullptr, wl, sl, add, gx, part0,
                               partl, reinterpret_cast<int *>(ws));
     }

@@ -817,9 +817,7 @@ struct EpiloguePtrs {
     // of one image each, channel-group major) into contiguous ranges; slot i of a channel belongs to the i-th block
     // whose range meets the channel's group, later slots were never written and are not read.
     int grp, B, units, nblocks;
-    struct Split {
-        int grp, B, units, nblocks;
-    } deep;  // the same for levels >= 2 where another kernel produced them (grp == 0: the kernel above did)
+    bool deep_all;  // levels >= 2 come from kernels that write every slot, whatever the one above does
 };
 
 template <int UNUSED>  // a template only so that every translation unit may include this header
@@ -837,11 +835,6 @@ unfold_epilogue_kernel(int C, int K, int L, EpiloguePtrs ep, const float *__rest
     if (ep.grp > 0) {
         const long long first_unit = (long long)(c / ep.grp) * ep.B;
         written = block_of_unit(first_unit + ep.B - 1, ep.nblocks, ep.units) - block_of_unit(first_unit, ep.nblocks, ep.units) + 1;
-    }
-    int written_deep = written;
-    if (ep.deep.grp > 0) {
-        const long long first_unit = (long long)(c / ep.deep.grp) * ep.deep.B;
-        written_deep = block_of_unit(first_unit + ep.deep.B - 1, ep.deep.nblocks, ep.deep.units) - block_of_unit(first_unit, ep.deep.nblocks, ep.deep.units) + 1;
     }
     // One entry per thread and pass: its partial sums, the parameter it meets in the scale gradient and its scale are
     // all requested before the first is used, so the block pays one memory round trip.
@@ -862,8 +855,7 @@ unfold_epilogue_kernel(int C, int K, int L, EpiloguePtrs ep, const float *__rest
             const int l = (e - n0) / nl, t = (e - n0) - l * nl;
             q = ep.partl[l] + (size_t)c * ep.npl[l] * nl + t;
             stride = nl;
-            const int have = l >= 1 ? written_deep : written;
-            n = ep.npl[l] < have ? ep.npl[l] : have;
+            n = ep.npl[l] < written || (l >= 1 && ep.deep_all) ? ep.npl[l] : written;
             wv = wl[((size_t)l * C + c) * nl + t];
             sv = sl[((size_t)l * C + c) * 4 + t / KK];
             dst = dwl + ((size_t)l * C + c) * nl + t;

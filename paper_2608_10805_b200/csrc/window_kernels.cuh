@@ -386,7 +386,7 @@ window_kernel(const __grid_constant__ WGeom w, const T *__restrict__ x, const T 
 #pragma unroll
             for (int t = 0; t < KK; ++t) scr[tid * (KK + 2) + t] = accw[t];
             scr[tid * (KK + 2) + KK] = gsum;
-            scr[tid * (KK + 2) + KK + 1] = __int_as_float(item.meta < 0 ? cls : -1);
+            scr[tid * (KK + 2) + KK + 1] = (float)(item.meta < 0 ? cls : -1);  // (a finite number: it may stay in an array's padding)
             __syncthreads();
             const long long first_unit = (long long)c * g.B * nwin;
             const int slotp = blockIdx.x - (int)(((first_unit + 1) * gridDim.x - 1) / w.units);
@@ -395,7 +395,7 @@ window_kernel(const __grid_constant__ WGeom w, const T *__restrict__ x, const T 
                 if (c2 > 0 && t == KK) continue;
                 float sacc = 0.f;
                 for (int th = 0; th < nthr; ++th)
-                    if (__float_as_int(scr[th * (KK + 2) + KK + 1]) == c2) sacc += scr[th * (KK + 2) + t];
+                    if (scr[th * (KK + 2) + KK + 1] == (float)c2) sacc += scr[th * (KK + 2) + t];
                 if (c2 == 0) {
                     part0[((size_t)c * g.np + slotp) * (KK + 1) + t] = sacc;
                 } else {

@@ -6,7 +6,7 @@
 #include "common.cuh"
 #include "tiled_kernels.cuh"
 #include "plane_kernels.cuh"
-#include "tensor_kernels.cuh"
+#include "panel_host.cuh"
 #include "team_kernels.cuh"
 #include "window_kernels.cuh"
 #include "tiled_host.cuh"
@@ -26,6 +26,8 @@ WT_PLANE_INSTANTIATE(__nv_bfloat16, extern)
 namespace tensor {
 WT_TENSOR_INSTANTIATE(__half, extern)
 WT_TENSOR_INSTANTIATE(__nv_bfloat16, extern)
+WT_WIDE_INSTANTIATE(__half, extern)
+WT_WIDE_INSTANTIATE(__nv_bfloat16, extern)
 }  // namespace tensor
 namespace team {
 WT_TEAM_INSTANTIATE(float, extern)
@@ -114,7 +116,7 @@ __global__ void resolve_status_kernel(int *status) {
 struct Route {
     wtconv_desc key;
     bool set;
-    bool team, plane, window, tensor[2], k3;  // plane: any family that keeps whole planes on chip; k3: 3 x 3 kernels in 5 x 5 tables
+    bool team, plane, window, tensor[2], wide, k3;  // wide: tensor-core kernels in column panels, both directions; plane: any family that keeps whole planes on chip; k3: 3 x 3 kernels in 5 x 5 tables
     size_t chip_fwd, chip_bwd;  // workspace of the family itself, which the k = 3 embedding runs whatever serves k = 5
     size_t fwd_bytes, bwd_bytes;
 };
@@ -125,6 +127,7 @@ bool use_ref_chain(const wtconv_desc *d) { return (d->flags & WTCONV_FLAG_REFERE
 bool use_team_path(const wtconv_desc *d) { return route(d).team; }
 bool use_plane_path(const wtconv_desc *d) { return route(d).plane; }
 bool use_window_path(const wtconv_desc *d) { return route(d).window; }
+bool use_wide_path(const wtconv_desc *d) { return route(d).wide; }
 bool use_tensor_path(const wtconv_desc *d, int bwd) { return route(d).tensor[bwd]; }
 wt::tensor::Request tensor_request(const wtconv_desc *d, int bwd) { return {bwd, d->B, d->C, d->H, d->W, d->L, d->k}; }
 // k = 3 through the k = 5 kernels.  A 3 x 3 depthwise kernel is a 5 x 5 kernel with a border of zeros, so wherever the
@@ -185,6 +188,10 @@ wtconv_status forward_tk(const wtconv_desc *d, const void *x, const float *w0, c
                          const float *wl, const float *sl, void *out, char *ws, cudaStream_t st, int taps = 5) {
     if (use_ref_chain(d)) return wt::refchain::forward<T, K>(d, (const T *)x, w0, s0, b0, wl, sl, (T *)out, ws, st);
     if constexpr (K != 7 && sizeof(T) == 2) {
+        if (taps == 5 && use_wide_path(d))
+            return wt::tensor::wide_forward<T>(tensor_request(d, 0), (const T *)x, w0, s0, b0, wl, sl, (T *)out, ws, st, next_status_tag()) == cudaSuccess
+                       ? WTCONV_OK
+                       : WTCONV_ERR_CUDA;
         if (taps == 5 && use_tensor_path(d, 0))
             return wt::tensor::forward<T>(tensor_request(d, 0), (const T *)x, w0, s0, b0, wl, sl, (T *)out,
                                           ws + (use_k3_embedding(d) ? embed_layout(d).inner : 0), st, next_status_tag(),
@@ -237,6 +244,13 @@ wtconv_status backward_tk(const wtconv_desc *d, const void *x, const void *g, co
         return wt::refchain::backward<T, K>(d, (const T *)x, (const T *)g, w0, s0, b0, wl, sl, (T *)gx, gw0, gs0, gb0, gwl, gsl,
                                             ws, st);
     if constexpr (K != 7 && sizeof(T) == 2) {
+        if (taps == 5 && use_wide_path(d)) {
+            wt::EpiloguePtrs ep = {};
+            if (wt::tensor::wide_backward<T>(tensor_request(d, 1), (const T *)x, (const T *)g, w0, s0, wl, sl, b0 != nullptr, (T *)gx, ws, &ep, st,
+                                             next_status_tag()) != cudaSuccess)
+                return WTCONV_ERR_CUDA;
+            return launch_epilogue(d, ep, w0, s0, b0, wl, sl, gw0, gs0, gb0, gwl, gsl, st);
+        }
         if (taps == 5 && use_tensor_path(d, 1)) {
             wt::EpiloguePtrs ep = {};
             if (wt::tensor::backward<T>(tensor_request(d, 1), (const T *)x, (const T *)g, w0, s0, wl, sl, b0 != nullptr, (T *)gx,
@@ -336,6 +350,13 @@ bool tensor_serves(const wtconv_desc *d, bool on_chip, int bwd) {
     return wt::tensor::plan(tensor_request(d, bwd), g) && g.cost * (1.1 / 1900) < on_chip_us(d, bwd);
 }
 
+// Planes beyond the on-chip kernels.
+bool wide_serves(const wtconv_desc *d, bool on_chip) {
+    if (d->dtype == WTCONV_F32 || on_chip || d->k == 7 || d->flags) return false;
+    wt::tensor::KGeom g;
+    return wt::tensor::wide(tensor_request(d, 0)) && wt::tensor::plan(tensor_request(d, 0), g) && wt::tensor::plan(tensor_request(d, 1), g);
+}
+
 Route find_route(const wtconv_desc *d) {
     Route r = {};
     r.key = *d;
@@ -358,6 +379,17 @@ Route find_route(const wtconv_desc *d) {
         if (!r.plane && !(d->flags & WTCONV_FLAG_NO_WINDOW) && !(d->flags >> 8) &&
             (((size_t)d->W * eb) % 16 != 0 || (d->flags & WTCONV_FLAG_PREFER_WINDOW)))
             r.window = wt::window::supported(d->B, d->C, d->H, d->W, d->k, d->L, d->dtype);
+    }
+    if (wide_serves(d, [&] {
+            if (d->k != 3) return r.plane;
+            const wtconv_desc d5 = as_k5(d);
+            return route(&d5).plane;
+        }())) {
+        const auto p = wt::tensor::wide_plan(tensor_request(d, 1));
+        r.wide = true;
+        r.fwd_bytes = r.chip_fwd = p.fwd_bytes;
+        r.bwd_bytes = r.chip_bwd = p.bwd_bytes;
+        return r;
     }
     if (d->k == 3 && !(d->flags & WTCONV_FLAG_TILED_ONLY)) {
         const wtconv_desc d5 = as_k5(d);
@@ -544,6 +576,14 @@ wtconv_status wtconv_plan_describe(const wtconv_desc *d, char *buf, size_t n) {
     if (st != WTCONV_OK) return st;
     if (!buf || n == 0) return WTCONV_ERR_NULL;
     buf[0] = 0;
+    if (use_wide_path(d)) {
+        size_t o = (size_t)snprintf(buf, n, "%s ", wtconv_plan_name(d));
+        for (int bwd = 0; bwd < 2 && o + 1 < n; ++bwd) {
+            if (bwd) buf[o++] = ' ';
+            o += (size_t)wt::tensor::describe(tensor_request(d, bwd), buf + o, n - o);
+        }
+        return WTCONV_OK;
+    }
     if (use_tensor_path(d, 0) || use_tensor_path(d, 1)) {  // the family's name as callers know it, then the plans that run
         size_t o = (size_t)snprintf(buf, n, "%s%s", use_k3_embedding(d) ? "3x3 kernels in 5x5 tables: " : "", wtconv_plan_name(d));
         for (int bwd = 0; bwd < 2; ++bwd)
@@ -847,7 +887,9 @@ wtconv_status wtconv_read_status(const wtconv_desc *d, void *workspace, int32_t 
         d5 = as_k5(d);
         d = &d5;
     }
-    if (use_window_path(d) && d->L > 2)  // the carrier's whole-plane kernels keep the only status word of this path
+    if (use_wide_path(d)) {
+        // the status words open the workspace
+    } else if (use_window_path(d) && d->L > 2)  // the carrier's whole-plane kernels keep the only status word of this path
         workspace = (char *)workspace + wt::window::ws_plan(d->B, d->C, d->H, d->W, d->L, (int)elem_bytes(d->dtype)).deep;
     else if (!use_plane_path(d)) {  // the tiled, window (L <= 2) and reference kernels wait for nothing and keep no status word
         *h_flag = 0;
