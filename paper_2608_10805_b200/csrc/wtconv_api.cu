@@ -346,15 +346,37 @@ double on_chip_us(const wtconv_desc *d, int bwd) {
 // 14 % (forward, k = 5), 25 % (backward), 27 % and 35 % (k = 3, which also saves the table kernels), and lost in 1 of 40.
 bool tensor_serves(const wtconv_desc *d, bool on_chip, int bwd) {
     if (d->dtype == WTCONV_F32 || !on_chip || d->L > 1 || (d->flags & ~WTCONV_FLAG_TEST_NO_COPY)) return false;
+    if (d->W > 64 && d->W % 4 != 0) return false;  // panels whose rows are not 8-byte multiples: element shifts, often slower
     wt::tensor::KGeom g;
     return wt::tensor::plan(tensor_request(d, bwd), g) && g.cost * (1.1 / 1900) < on_chip_us(d, bwd);
 }
 
-// Planes beyond the on-chip kernels.
+// Planes beyond the on-chip kernels: tensor-core panels against the per-level (tiled) kernels, which need rows of whole 16-byte
+// words to be fast, and the window kernels, which take the others.  Measured over 3500 shapes between 60 x 60 and 256 x 256:
+// against the tiled kernels panels win nearly everywhere (forward 1.5 x, backward 1.7 x; the exceptions are small 3 x 3 layers
+// of several levels, all launches).  Against the windows the backward wins everywhere (1.4 x) and the forward where the
+// launches of the levels do not count and the panels are well filled: both directions follow the forward's estimate, because a
+// workspace keeps its status words in one place.  The estimates (microseconds, fitted, 10 % off) count pixels (n, millions),
+// 64 x 64 pixel tiles (t1) and the 32 x 32 coefficient tiles of levels 2, 3 and deeper (t2, t3, t4).
+bool panels_win(const wtconv_desc *d, double cost) {
+    const double n = (double)d->B * d->C * d->H * d->W * 1e-6, planes = (double)d->B * d->C * 1e-3;
+    if (d->W % 8 == 0) return d->k == 5 || d->L <= 1 || n >= 4;
+    auto tiles = [&](int px, int side) { return planes * ((d->W + px - 1) / px) * ((d->H + px - 1) / px) * side * side * 1e-3; };
+    const int L = d->L;
+    const double t1 = tiles(64, 64), t2 = L > 1 ? tiles(128, 32) : 0, t3 = L > 2 ? tiles(256, 32) : 0, t4 = (L > 3 ? tiles(512, 32) : 0) + (L > 4) * planes;
+    const bool odd = d->W % 4 != 0, deep = L > 1, deeper = L > 2;
+    const double c = cost / 1900;
+    if (d->k == 5)
+        return 1.03 * ((1.35 + 0.08 * odd) * c + 2.86 * n * deep + 6.56 * t2 + 5.97 * t3 + 10.0 * t4 + 10.3 * deep + 1.7 * L) <
+               8.9 + (5.13 + 0.6 * odd + 0.7 * deep + 0.69 * deeper) * n + (0.13 + 0.96 * deep) * t1 + 4.4 * t3 + 1.5 * t4 + 0.58 * L + 15.9 * deeper;
+    return 1.1 * ((1.34 + 0.09 * odd) * c + 2.94 * n * deep + 3.36 * t2 + 1.78 * t3 + 9.0 * t4 + 11.9 * deep + 1.3 * L) <
+           10.2 + (4.68 + 0.93 * odd + 0.58 * deep + 0.86 * deeper) * n + 1.16 * deep * t1 + 5.7 * t3 + 1.65 * L + 13.2 * deeper;
+}
 bool wide_serves(const wtconv_desc *d, bool on_chip) {
     if (d->dtype == WTCONV_F32 || on_chip || d->k == 7 || d->flags) return false;
     wt::tensor::KGeom g;
-    return wt::tensor::wide(tensor_request(d, 0)) && wt::tensor::plan(tensor_request(d, 0), g) && wt::tensor::plan(tensor_request(d, 1), g);
+    return wt::tensor::wide(tensor_request(d, 0)) && wt::tensor::plan(tensor_request(d, 1), g) && wt::tensor::plan(tensor_request(d, 0), g) &&
+           panels_win(d, g.cost);
 }
 
 Route find_route(const wtconv_desc *d) {

@@ -1,0 +1,75 @@
+"""The tensor-core kernels against the fp64 oracle at the edges of their tiles: batches that do not fill groups of eight images,
+planes of one 8-column chunk and of several, odd rows, planes cut into 32-row slices, column panels with a narrow last one,
+no level, one level, carriers for the others, 3 x 3 kernels."""
+import pytest
+
+from helpers import GRAD_NAMES, TOL, rel_err, run_gpu, run_oracle
+from paper_2608_10805_b200 import inputs, wtconv as wt
+
+pytestmark = pytest.mark.gpu
+
+ON_CHIP = [  # B, C, H, W, k, L, directions on the tensor cores
+    (11, 16, 7, 7, 5, 1, "both"),      # one chunk, a group of three images
+    (40, 33, 9, 9, 5, 1, "both"),      # odd rows, two chunks, several planes stacked
+    (21, 40, 14, 14, 5, 0, "both"),    # no level
+    (24, 40, 31, 30, 5, 1, "both"),    # rows of pairs
+    (19, 20, 25, 27, 3, 1, "both"),    # 3 x 3, odd rows
+    (10, 64, 64, 64, 5, 1, "bwd"),     # two slices, the widest plane that is not cut into panels
+    (16, 37, 33, 60, 5, 1, "bwd"),     # a slice of one row
+    (12, 64, 100, 64, 3, 1, "bwd"),   # four slices, the last of four rows
+    (33, 48, 50, 56, 3, 1, "both"),    # slices, both directions
+    (9, 48, 80, 72, 5, 1, "both"),     # panels of a plane the on-chip kernels also serve
+]
+WIDE = [
+    (3, 6, 130, 136, 5, 0),
+    (8, 16, 161, 137, 3, 1),            # odd rows, a narrow last panel
+    (9, 3, 128, 160, 5, 2),            # a second group of images
+    (3, 16, 136, 200, 5, 3),
+    (2, 24, 161, 138, 5, 1),           # rows of pairs
+    (2, 40, 233, 225, 5, 4),
+    (2, 8, 256, 256, 5, 8),            # every level there is
+    (4, 33, 200, 152, 3, 3),
+    (1, 5, 300, 48, 5, 1),             # tall and narrow: one panel
+]
+
+
+def check(B, C, H, W, k, L, dtype, seed):
+    w = inputs.Workload("tensor", B, C, H, W, k, L, dtype, seed)
+    data = inputs.make_inputs(w, bias=seed % 2 == 0)
+    out, grads = run_gpu(w, data)
+    ref, ref_grads = run_oracle(w, data)
+    assert rel_err(out, ref) < TOL[dtype]
+    for n in GRAD_NAMES:
+        if ref_grads.get(n) is not None and ref_grads[n].size:
+            # parameter gradients are sums in fp32 of exact products: far inside the storage type's tolerance
+            assert rel_err(grads[n], ref_grads[n]) < (TOL[dtype] if n == "dx" else 1e-5), n
+
+
+@pytest.mark.parametrize("dtype", ["f16", "bf16"])
+@pytest.mark.parametrize("shape", ON_CHIP, ids=lambda s: "x".join(map(str, s[:6])))
+def test_planes_and_slices(shape, dtype):
+    B, C, H, W, k, L, where = shape
+    plan = wt.wtconv_plan_describe(wt.make_desc(B, C, H, W, k, L, dtype))
+    assert ("fwd[tensor" in plan) == (where != "bwd") and ("bwd[tensor" in plan) == (where != "fwd")
+    check(B, C, H, W, k, L, dtype, 900 + ON_CHIP.index(shape))
+
+
+@pytest.mark.parametrize("dtype", ["f16", "bf16"])
+@pytest.mark.parametrize("shape", WIDE, ids=lambda s: "x".join(map(str, s)))
+def test_column_panels(shape, dtype):
+    plan = wt.wtconv_plan_describe(wt.make_desc(*shape, dtype))
+    assert "fwd[tensor" in plan and "bwd[tensor" in plan
+    check(*shape, dtype, 950 + WIDE.index(shape))
+
+
+def test_many_units_per_channel_repeat_to_the_bit():
+    """Units of one channel follow one another without a block-wide barrier in between: item lists, ring slots and output
+    images must not meet."""
+    w = inputs.Workload("tensor", 84, 160, 18, 18, 5, 1, "bf16", 990)
+    data = inputs.make_inputs(w)
+    first = run_gpu(w, data, guarded=False)
+    plain = run_gpu(w, data, flags=wt.FLAG_PREFER_WINDOW, guarded=False)
+    assert rel_err(first[0], plain[0]) < TOL["bf16"] and rel_err(first[1]["dx"], plain[1]["dx"]) < TOL["bf16"]
+    for _ in range(20):
+        again = run_gpu(w, data, guarded=False)
+        assert (again[0] == first[0]).all() and all((again[1][n] == first[1][n]).all() for n in ("dx", "dw0", "dwl"))
