@@ -86,7 +86,8 @@ typedef enum {
 #define WTCONV_FLAG_NO_WINDOW 64u /* never take the window kernels for large planes (used to test the tiled path on them) */
 /* Large planes are served by the window kernels (levels 1-2 on chip, about 2.2 N elements of HBM traffic) when their
  * rows are not 16-byte multiples, and by the tiled kernels (per-level launches, Q_fused - 2 N of traffic, but faster
- * on this GPU when rows are aligned) otherwise; this flag takes the window kernels wherever they apply. */
+ * on this GPU when rows are aligned) otherwise, unless column panels on the tensor cores are faster (16-bit activations,
+ * k = 3 or 5); this flag takes the window kernels wherever they apply. */
 #define WTCONV_FLAG_PREFER_WINDOW 128u
 /* Comparator: run the layer as the chain of separate operators of Sec. 3.1 (analysis, depthwise conv, scale pass,
  * slice, add, concatenate, synthesis per level; base conv, scale pass, add), every intermediate in HBM, as plain
@@ -145,7 +146,9 @@ const char *wtconv_plan_name(const wtconv_desc *desc);
  * tile rows, prefetch ring depth; "ring=0" = the kernel waits for no copy).  Host call.  Errors: NULL, desc. */
 wtconv_status wtconv_plan_describe(const wtconv_desc *desc, char *buf, size_t n);
 
-/* Number of kernel launches one wtconv_forward / wtconv_backward call enqueues. */
+/* Number of kernel launches one wtconv_forward / wtconv_backward call of the family wtconv_plan_name() names enqueues.
+ * Where wtconv_plan_describe() shows tensor-core plans in the family's place: 1 and 2, in column panels with more than one
+ * level L + 2 and L + 4. */
 wtconv_status wtconv_launch_count(const wtconv_desc *desc, int32_t *fwd_launches, int32_t *bwd_launches);
 
 /* Forward pass of Algorithm 1 (device pointers).  out must not overlap x. */

@@ -10,8 +10,11 @@
 // once per window row (ten MMAs of 128 x 48 x 16).  A 16-bit activation is an exact MMA operand; a weight is split into three
 // 16-bit parts (24 bits, the whole float), which are three groups of N columns added in fp32 afterwards.  Accumulation is
 // fp32 in tensor memory.  Scalar FMA tiles of the same work sat at 1.4 - 2.4 SM-cycles a pixel (their loads, stores,
-// butterflies and barriers included); the MMAs take 45 cycles each, 0.22 cycles a pixel at full tiles, and run beside the
-// staging and the stores of other blocks.
+// butterflies and barriers included); an MMA takes 46 - 48 cycles (it is bound by the A operand's shared-memory reads), 0.22
+// cycles a pixel at full tiles, and runs beside the staging and the stores of other blocks.  Measured (128 images, one level,
+// forward / backward, against the on-chip FMA kernels): 96 x 56 x 56 149 -> 91 / 345 -> 148 us, 192 x 28 x 28 89 -> 56 / 193 ->
+// 93, 384 x 14 x 14 63 -> 47 / 114 -> 78, 768 x 7 x 7 (backward only) 102 -> 93.  What bounds it now is latency: load, staging,
+// MMAs, epilogue and copy-out of a unit follow one another and two blocks per SM hide only part of that (issue slots 25 % used).
 //
 // Layout.  The A operand is the plane itself: shared memory holds [row][chunk of 8 columns][8 images][8 columns], so a core
 // matrix (8 rows of 16 bytes) is one chunk of eight images, the second half of K is the next chunk (128 bytes on) and the
@@ -36,7 +39,7 @@ using plane::FastDiv;
 using plane::fdiv;
 using plane::make_fastdiv;
 
-// Eight staging / epilogue warps and four that issue MMAs (an issue takes its warp about 100 cycles, the tensor cores 45).
+// Eight staging / epilogue warps and four that issue MMAs (an issue takes its warp about 100 cycles, the tensor cores 46).
 constexpr int WORKERS = 256, ISSUERS = 4, THREADS = WORKERS + 32 * ISSUERS;
 constexpr int BULK_WORDS = 48;
 constexpr int TAPS = 10, NCOL = 48;                   // window rows; 3 weight parts x 2 rows x 8 columns
@@ -257,7 +260,9 @@ __device__ __forceinline__ void repack(char *arr, const char *raw, const Item *i
     }
 }
 // The same for one column panel, straight from global memory (a panel's rows are short: staging them first costs a pass over
-// shared memory, whose bandwidth the MMAs need).  x0 = the panel's first column.
+// shared memory, whose bandwidth the MMAs need).  x0 = the panel's first column.  Bound by the latency of the loads; six words in
+// flight and the rows requested for L2 a unit ahead took 16 x 64 x 256 x 256 (one level, f16) from 222 / 456 to 206 / 378 us
+// (tiled kernels: 360 / 799).
 template <typename T, bool SUM, bool QUADS>
 __device__ __forceinline__ void repack_panel_t(char *arr, const T *__restrict__ src, const Item *items, const KGeom &g, int P, const FastDiv &dP,
                                              const FastDiv &dE, int shift, int x0, int warp, int lane, float &sum) {
