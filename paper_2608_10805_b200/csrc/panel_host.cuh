@@ -24,7 +24,7 @@ inline WidePlan wide_plan(const Request &q) {
     WidePlan p = {};
     p.Hs[0] = q.H;
     p.Ws[0] = q.W;
-    for (int l = 1; l <= 8; ++l) { p.Hs[l] = (p.Hs[l - 1] + 1) / 2; p.Ws[l] = (p.Ws[l - 1] + 1) / 2; }
+    for (int l = 1; l <= 8; ++l) { p.Hs[l] = (p.Hs[l - 1] + 1) / 2; p.Ws[l] = l == 1 ? band_pitch(q.W) : (p.Ws[l - 1] + 1) / 2; }
     const size_t P = (size_t)q.B * q.C, KK = (size_t)q.K * q.K;
     Request b = q;
     b.bwd = 1;
@@ -59,18 +59,18 @@ struct SynthPtrs {
     int H[9], W[9], L;
 };
 static __global__ void __launch_bounds__(256) synthesis_kernel(const __grid_constant__ SynthPtrs s, u64 rows, float *__restrict__ R) {
-    const int H1 = s.H[1], W1 = s.W[1], H2 = s.H[2], W2 = s.W[2], pairs = (W2 + 1) >> 1;
+    const int H1 = s.H[1], W1 = s.W[1], H2 = s.H[2], W2 = s.W[2], pairs = W2 >> 1;  // W1 is a multiple of eight
     for (u64 e = (u64)blockIdx.x * blockDim.x + threadIdx.x; e < rows * pairs; e += (u64)gridDim.x * blockDim.x) {
         const u64 row = e / pairs, p = row / H2;
         const int j = (int)(e - row * pairs), i = (int)(row - p * H2);
         float v[2][4];
         const size_t S2 = (size_t)H2 * W2;
         const float *z = s.z[2] + p * 4 * S2 + (size_t)i * W2 + 2 * j;
-        const bool second = 2 * j + 1 < W2;
+        const float2 ll2 = __ldg(reinterpret_cast<const float2 *>(z)), lh2 = __ldg(reinterpret_cast<const float2 *>(z + S2));
+        const float2 hl2 = __ldg(reinterpret_cast<const float2 *>(z + 2 * S2)), hh2 = __ldg(reinterpret_cast<const float2 *>(z + 3 * S2));
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
-            float ll = 0.f, lh = 0.f, hl = 0.f, hh = 0.f;
-            if (h == 0 || second) { ll = __ldg(z + h); lh = __ldg(z + S2 + h); hl = __ldg(z + 2 * S2 + h); hh = __ldg(z + 3 * S2 + h); }
+            const float ll = h ? ll2.y : ll2.x, lh = h ? lh2.y : lh2.x, hl = h ? hl2.y : hl2.x, hh = h ? hh2.y : hh2.x;
             const float pp = ll + lh, pm = ll - lh, qp = hl + hh, qm = hl - hh;
             v[0][2 * h] = 0.5f * (pp + qp); v[0][2 * h + 1] = 0.5f * (pp - qp);
             v[1][2 * h] = 0.5f * (pm + qm); v[1][2 * h + 1] = 0.5f * (pm - qm);
@@ -92,13 +92,7 @@ static __global__ void __launch_bounds__(256) synthesis_kernel(const __grid_cons
 #pragma unroll
         for (int r = 0; r < 2; ++r, o += W1) {
             if (2 * i + r >= H1) break;
-            if ((W1 & 3) == 0) {
-                *reinterpret_cast<float4 *>(o) = make_float4(v[r][0], v[r][1], v[r][2], v[r][3]);
-            } else {
-#pragma unroll
-                for (int c = 0; c < 4; ++c)
-                    if (4 * j + c < W1) o[c] = v[r][c];
-            }
+            *reinterpret_cast<float4 *>(o) = make_float4(v[r][0], v[r][1], v[r][2], v[r][3]);
         }
     }
 }
@@ -106,7 +100,7 @@ inline cudaError_t synthesize(const Request &q, const WidePlan &p, char *ws, cud
     SynthPtrs s = {};
     s.L = q.L;
     for (int l = 1; l <= q.L; ++l) { s.z[l] = reinterpret_cast<const float *>(ws + p.Z[l]); s.H[l] = p.Hs[l]; s.W[l] = p.Ws[l]; }
-    const u64 rows = (u64)q.B * q.C * p.Hs[2], n = rows * ((p.Ws[2] + 1) / 2), blocks = (n + 255) / 256;
+    const u64 rows = (u64)q.B * q.C * p.Hs[2], n = rows * (p.Ws[2] / 2), blocks = (n + 255) / 256;
     synthesis_kernel<<<(unsigned)(blocks < 148 * 64 ? blocks : 148 * 64), 256, 0, st>>>(s, rows, reinterpret_cast<float *>(ws + p.R));
     return cudaGetLastError();
 }

@@ -65,6 +65,7 @@ struct KGeom {
     int conv_off, x_off, parts_off, raw_off, out_off, table_off, misc_off, smem;  // byte offsets
     int ring, cols;              // tensor-memory ring depth and columns allocated
     int bps, nblocks, np;
+    int pitch;                   // floats in a row of the addend (band_pitch)
     int no_copy, bias, deep;     // deep: levels >= 2 come as a float addend per 2 x 2 pixels (panels only)
     FastDiv d_period, d_nty, d_n, d_Pc, d_Px, d_ec, d_ex, d_out_words;  // d_ec / d_ex: chunks of one octet in the convolved / the x array
     int *alarm;
@@ -655,18 +656,13 @@ tensor_kernel(const __grid_constant__ KGeom g, const T *__restrict__ x, const T 
                     else v[i] = (v[i] + (p1[i] + p2[i])) + bias;
                 }
                 if (PANEL && g.deep) {  // levels >= 2: one value (un-normalised LL of level 1, Proposition 2) per 2 x 2 pixels
-                    const int W2 = (g.W + 1) >> 1, left = W2 - (x0 >> 1) - 4 * j;
-                    const float *d = add + (u64)it.plane * (unsigned)(((g.H + 1) >> 1) * W2) + (y >> 1) * W2 + (x0 >> 1) + 4 * j;
-                    float more[4];
-                    if (left >= 4 && (W2 & 3) == 0) {
-                        const float4 t4 = *reinterpret_cast<const float4 *>(d);
-                        more[0] = t4.x; more[1] = t4.y; more[2] = t4.z; more[3] = t4.w;
-                    } else {
+                    const int left = g.pitch - (x0 >> 1) - 4 * j;
+                    const float *d = add + (u64)it.plane * (unsigned)(((g.H + 1) >> 1) * g.pitch) + (y >> 1) * g.pitch + (x0 >> 1) + 4 * j;
+                    float4 more = make_float4(0.f, 0.f, 0.f, 0.f);
+                    if (left > 0) more = *reinterpret_cast<const float4 *>(d);  // (left is a multiple of four)
+                    const float m4[4] = {more.x, more.y, more.z, more.w};
 #pragma unroll
-                        for (int i = 0; i < 4; ++i) more[i] = i < left ? d[i] : 0.f;
-                    }
-#pragma unroll
-                    for (int i = 0; i < 16; ++i) v[i] = fmaf(0.5f, more[(i & 7) >> 1], v[i]);
+                    for (int i = 0; i < 16; ++i) v[i] = fmaf(0.5f, m4[(i & 7) >> 1], v[i]);
                 }
                 // the output image keeps the item's place inside its 16-byte word of global memory
                 // (panels: every row does; rows are tw + 8 pixels apart)
@@ -830,20 +826,25 @@ tensor_kernel(const __grid_constant__ KGeom g, const T *__restrict__ x, const T 
     if (warp == 8) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(g.cols));
 }
 
+// Rows of the level-1 carriers are padded with zeros to eight floats: beyond the plane the transform sees zeros anyway (an odd
+// row's last pair, the convolution's border), so every level keeps its values, and the level kernels load and store whole words
+// however wide the plane is (16 x 256 x 225 x 225, five levels: 1738 -> 1672 us forward, 3210 -> 2921 backward).
+inline int band_pitch(int W) { return ((W + 1) / 2 + 7) / 8 * 8; }
+
 // The level-1 low-pass band of every plane as floats: the carrier that levels >= 2 of wide planes are computed on.  One thread
 // makes four values of a row from 2 x 8 pixels.
 template <typename T>
-__global__ void __launch_bounds__(256) band_kernel(const T *__restrict__ x, int H, int W, int H2, int W2, u64 rows, float *__restrict__ X1) {
+__global__ void __launch_bounds__(256) band_kernel(const T *__restrict__ x, int H, int W, int H2, int pitch, u64 rows, float *__restrict__ X1) {
     dependents_may_start();
     wait_for_predecessor();
-    const int quads = (W2 + 3) >> 2;
+    const int quads = pitch >> 2;
     for (u64 e = (u64)blockIdx.x * blockDim.x + threadIdx.x; e < rows * quads; e += (u64)gridDim.x * blockDim.x) {
         const u64 row = e / quads;
         const int j = (int)(e - row * quads), i = (int)(row % H2);
         const T *p = x + (row / H2) * (u64)H * W + (u64)(2 * i) * W + 8 * j;
         const bool y1 = 2 * i + 1 < H;
         float a[8], c[8];
-        if ((W & 7) == 0) {
+        if ((W & 7) == 0 && 8 * j < W) {
             const uint4 t = __ldg(reinterpret_cast<const uint4 *>(p)), s = y1 ? __ldg(reinterpret_cast<const uint4 *>(p + W)) : make_uint4(0, 0, 0, 0);
             const unsigned tv[4] = {t.x, t.y, t.z, t.w}, sv[4] = {s.x, s.y, s.z, s.w};
 #pragma unroll
@@ -859,25 +860,19 @@ __global__ void __launch_bounds__(256) band_kernel(const T *__restrict__ x, int 
                 c[q] = in && y1 ? ldf(p + W + q) : 0.f;
             }
         }
-        float *o = X1 + row * W2 + 4 * j;
+        float *o = X1 + row * pitch + 4 * j;
         float v[4];
 #pragma unroll
         for (int q = 0; q < 4; ++q) v[q] = 0.5f * ((a[2 * q] + a[2 * q + 1]) + (c[2 * q] + c[2 * q + 1]));
-        if ((W2 & 3) == 0) {
-            *reinterpret_cast<float4 *>(o) = make_float4(v[0], v[1], v[2], v[3]);
-        } else {
-#pragma unroll
-            for (int q = 0; q < 4; ++q)
-                if (4 * j + q < W2) o[q] = v[q];
-        }
+        *reinterpret_cast<float4 *>(o) = make_float4(v[0], v[1], v[2], v[3]);
     }
 }
 template <typename T>
 cudaError_t band(int B, int C, int H, int W, const T *x, float *X1, cudaStream_t st) {
-    const int H2 = (H + 1) / 2, W2 = (W + 1) / 2;
-    const u64 rows = (u64)B * C * H2, n = rows * ((W2 + 3) / 4);
+    const int H2 = (H + 1) / 2, pitch = band_pitch(W);
+    const u64 rows = (u64)B * C * H2, n = rows * (pitch / 4);
     const u64 blocks = (n + 255) / 256;
-    return launch_overlapped(band_kernel<T>, (unsigned)(blocks < 148 * 8 * 8 ? blocks : 148 * 8 * 8), 256u, 0, st, x, H, W, H2, W2, rows, X1);
+    return launch_overlapped(band_kernel<T>, (unsigned)(blocks < 148 * 8 * 8 ? blocks : 148 * 8 * 8), 256u, 0, st, x, H, W, H2, pitch, rows, X1);
 }
 
 // ------------------------------------------------------------------ host side
@@ -893,6 +888,7 @@ inline bool search_n(const Request &q, KGeom &best, int n) {
     bool found = false;
     KGeom g = {};
     g.deep = q.L > 1;
+    g.pitch = ((q.W + 1) / 2 + 7) / 8 * 8;
     g.B = q.B; g.C = q.C; g.H = q.H; g.W = q.W; g.HW = q.H * q.W; g.L = q.L; g.K = q.K;
     g.n = n;
     g.tw = 8 * n;
