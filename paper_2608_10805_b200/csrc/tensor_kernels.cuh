@@ -665,16 +665,14 @@ tensor_kernel(const __grid_constant__ KGeom g, const T *__restrict__ x, const T 
                     for (int i = 0; i < 16; ++i) v[i] = fmaf(0.5f, m4[(i & 7) >> 1], v[i]);
                 }
                 // the output image keeps the item's place inside its 16-byte word of global memory
-                // (panels: every row does; rows are tw + 8 pixels apart)
-                const int off = (int)it.at(g, it.ty * g.th) & 7;
+                // (panels: rows start at whole words, tw + 8 pixels apart, and are shifted into place on the way out)
                 T *d = reinterpret_cast<T *>(sb + g.out_off + (o * 8 + img) * g.out_stride);
                 if (PANEL) {
-                    const int first = (int)it.at(g, y) + x0;
                     d += r * (g.tw + 8) + 8 * j;
-                    store8<T>(d + (first & 7), v, g.W - x0 - 8 * j, g.W);
-                    if (y + 1 < g.H) store8<T>(d + g.tw + 8 + ((first + g.W) & 7), v + 8, g.W - x0 - 8 * j, g.W);
+                    store8<T>(d, v, 8, 8);
+                    if (y + 1 < g.H) store8<T>(d + g.tw + 8, v + 8, 8, 8);
                 } else {
-                    d += off + r * g.W + 8 * j;
+                    d += ((int)it.at(g, it.ty * g.th) & 7) + r * g.W + 8 * j;
                     store8<T>(d, v, g.W - 8 * j, g.W);
                     if (y + 1 < g.H) store8<T>(d + g.W, v + 8, g.W - 8 * j, g.W);
                 }
@@ -691,16 +689,30 @@ tensor_kernel(const __grid_constant__ KGeom g, const T *__restrict__ x, const T 
                     const int y = it.ty * g.th + r;
                     if (it.ty < 0 || y >= g.H) continue;
                     const u64 first = it.at(g, y) + x0;
-                    const int rel = 8 * w - (int)(first & 7);
+                    const int sh = (int)(first & 7), rel = 8 * w - sh;
                     const uint4 *s = reinterpret_cast<const uint4 *>(sb + g.out_off + slot * g.out_stride + r * (g.tw + 8) * 2) + w;
+                    uint4 q = *s;
+                    if (sh) {  // pixels 8 - sh .. 15 - sh of the word before and this one
+                        const uint4 p = w ? s[-1] : q;
+                        unsigned a[8] = {p.x, p.y, p.z, p.w, q.x, q.y, q.z, q.w};
+                        const int by = 8 - sh;
+                        if (by & 4) { a[0] = a[2]; a[1] = a[3]; a[2] = a[4]; a[3] = a[5]; a[4] = a[6]; a[5] = a[7]; }
+                        if (by & 2) { a[0] = a[1]; a[1] = a[2]; a[2] = a[3]; a[3] = a[4]; a[4] = a[5]; }
+                        if (by & 1) {
+#pragma unroll
+                            for (int i = 0; i < 4; ++i) a[i] = __funnelshift_r(a[i], a[i + 1], 16);
+                        }
+                        q = make_uint4(a[0], a[1], a[2], a[3]);
+                    }
                     T *d = out + (first + rel);
                     if (rel >= 0 && rel + 8 <= len) {
-                        *reinterpret_cast<uint4 *>(d) = *s;
+                        *reinterpret_cast<uint4 *>(d) = q;
                     } else {
-                        const T *p = reinterpret_cast<const T *>(s);
+                        const unsigned a[4] = {q.x, q.y, q.z, q.w};
+                        unsigned short *u = reinterpret_cast<unsigned short *>(d);
 #pragma unroll
                         for (int i = 0; i < 8; ++i)
-                            if (rel + i >= 0 && rel + i < len) d[i] = p[i];
+                            if (rel + i >= 0 && rel + i < len) u[i] = (unsigned short)(a[i >> 1] >> (16 * (i & 1)));
                     }
                 }
             } else if (g.out_words >= BULK_WORDS) {
