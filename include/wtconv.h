@@ -142,7 +142,8 @@ wtconv_status wtconv_workspace_bytes(const wtconv_desc *desc, size_t *fwd_bytes,
 
 /* Name of the kernels a descriptor dispatches to ("team" = small planes, several per thread team; "plane" =
  * one block per whole plane in shared memory; "window" = large planes cut into windows with levels 1-2 on chip;
- * "tiled" = per-level tiled kernels; "tensor" = base convolution, level 1 and synthesis as one contraction on the
+ * "tiled" = per-level tiled kernels, and the name of all 7 x 7 kernels, whose planes of up to about 70 x 70 stay on one SM too
+ * (wtconv_plan_describe tells which kernels run); "tensor" = base convolution, level 1 and synthesis as one contraction on the
  * tensor cores (16-bit activations), "panel" = the same in column panels of wide planes, levels >= 2 through HBM;
  * "reference-chain" = the comparator).  Where the two directions are served differently: both names, forward/backward
  * ("team/tensor").  Host call; returns NULL for an invalid desc. */

@@ -1,4 +1,4 @@
-// Whole-plane WTConv kernels for sm_100a (k = 5, and k = 3 as the inner taps of 5 x 5 tables: KT = 3 builds of the
+// Whole-plane WTConv kernels for sm_100a (k = 5 and 7, and k = 3 as the inner taps of 5 x 5 tables: KT = 3 builds of the
 // kernels leave the zero border out of the tap loops): every (b, c) plane's entire decomposition lives
 // in shared memory, so the only HBM traffic is the compulsory one (read x, write out; in the backward
 // read x and grad_out, write grad_x).
@@ -28,6 +28,10 @@
 //    rotated-kernel convolution, synthesis and store on the same window.  Shapes whose tiles do not fit
 //    one pass of 256 threads take the split pair instead: a weight-gradient kernel with class-major
 //    thread allocation plus the FLIP instantiation of the forward kernel.
+//  * 7 x 7 kernels take the forward and the split pair (49 weight-gradient sums, 49 weights and a tile are more than the 128
+//    registers of the fused kernel).  The per-level kernels they were on stage every level's coefficients through memory and
+//    give a grid of 7 x 7 coefficients a tile of 32 x 32: 16 x 96 x 56 x 56 f32, three levels, forward + backward 426 -> 180 us;
+//    over 60 random shapes of up to 72 x 72 forward 3.6 x and backward 4.1 x (geometric means), no shape slower.
 //  * Launches overlap: every kernel here is started with programmatic stream serialisation (common.cuh), does its
 //    set-up in shared memory and registers beside the tail of the kernel before it and only then waits for that
 //    kernel; no call puts a clearing operation between two kernels (status words are tagged per call, the epilogue
@@ -53,6 +57,17 @@ constexpr int NUM_SMS = 148;                 // planning constant (B200); plans 
 constexpr int SMEM_LIMIT = 227 * 1024;       // opt-in dynamic shared memory per block
 constexpr int SMEM_PER_SM = 228 * 1024;      // per SM, 1 KB reserved per resident block
 constexpr int WT_STRIDE = 28;                // floats per class in the weight table (25 taps, 16-byte padded)
+// What the tile code is built for.  KT: taps per side in use.  3 x 3 kernels sit in the middle of 5 x 5 tables and windows; 7 x 7
+// kernels have arrays with a halo of three rows and four columns, so that a window row is three aligned 16-byte loads whose
+// first column no tap uses.
+template <int KT> struct Taps {
+    static constexpr int K = KT == 7 ? 7 : 5, KK = K * K;
+    static constexpr int HY = K / 2, HX = KT == 7 ? 4 : 2;  // halo rows and columns: element (y, x) at (y + HY, x + HX)
+    static constexpr int C0 = HX - HY, NQ = KT == 7 ? 3 : 2;  // window column of the first tap, 16-byte loads in a window row
+    static constexpr int T0 = (K - KT) / 2, T1 = K - T0;      // taps T0 .. T1 - 1 per side
+    static constexpr int WS = KT == 7 ? 52 : WT_STRIDE;       // floats per class in the weight table
+};
+__host__ __device__ inline int table_stride(int k) { return k == 7 ? Taps<7>::WS : WT_STRIDE; }
 constexpr int MAX_STAGES = 4;               // deepest prefetch ring (units in flight per block)
 constexpr unsigned WAIT_LIMIT = 1u << 20;    // bounded number of (suspending) waits on the copy barrier: never an endless loop
 constexpr unsigned WAIT_LIMIT_TEST = 64;     // the same under WTCONV_FLAG_TEST_NO_COPY (no copy is ever issued: every wait runs out)
@@ -116,7 +131,7 @@ __device__ __forceinline__ int fdiv(int e, const FastDiv &f) { return f.d == 1 ?
 struct Geom {
     int B, C, H, W, L;
     int Hl[MAXL + 1], Wl[MAXL + 1];        // level grids, index 0 = input
-    int rows[MAXL + 1], pitch[MAXL + 1];   // haloed arrays: ty*TH+4 rows, pitch pad4(Wl)+4 floats; element (y,x) at (y+2, x+2)
+    int rows[MAXL + 1], pitch[MAXL + 1];   // haloed arrays: ty*TH+2*HY rows, pitch pad4(Wl)+2*HX floats; element (y,x) at (y+HY, x+HX)
     int offA[MAXL + 1];                    // slot-relative offset of x (l=0) / Y^l subband 0 (subband stride rows*pitch)
     int offG[MAXL + 1];                    // same for grad_out / D^l (weight-gradient kernel only)
     int zrows[MAXL + 1], zpitch[MAXL + 1]; // conv outputs Z^l (forward kernel only)
@@ -127,7 +142,7 @@ struct Geom {
     int tx[MAXL + 1], ty[MAXL + 1];        // 4 x TH tiles per level grid (index 0 = base)
     int lvl_start[MAXL + 2];               // per plane: first level-item of level l (1..L); [L+1] = count
     int nbase;                             // base tiles per plane
-    int wtab_off;                          // offset of the folded weight table [(1+4L)][WT_STRIDE] (bias at [0][25])
+    int wtab_off;                          // offset of the folded weight table [(1+4L)][WS] (bias at [0][KK])
     int smem_floats;
     int ngroups, units;                    // work units = ngroups channel groups x B images, group-major (a block keeps a group's
                                            // weights and gradient accumulators while it walks through the images)
@@ -136,7 +151,8 @@ struct Geom {
     int no_copy;                           // test mode: bulk copies are never issued and waits give up quickly (the timeout path)
     int *alarm;                            // host word that hears of a timeout, or null
     unsigned tag;                          // non-zero tag of the call this launch belongs to (status words, see common.cuh)
-    int taps;                              // taps per side in use: 5, or 3 for 3 x 3 kernels in the middle of 5 x 5 tables
+    int k;                                 // side of the tables: 5 or 7
+    int taps;                              // taps per side in use: k, or 3 for 3 x 3 kernels in the middle of 5 x 5 tables
     int bulk;                              // 1: planes are fetched ahead with cp.async.bulk into a ring of raw buffers at raw_off
     int nstage, stage_bytes;               // ring depth (units in flight) and bytes per ring entry
     int raw_off, raw_slot_bytes, plane_bytes;  // raw staging buffer (float offset), bytes per plane slot / per plane
@@ -159,11 +175,13 @@ __host__ __device__ inline int pad4(int n) { return (n + 3) & ~3; }
 using wt::block_of_unit;
 
 // ------------------------------------------------------------------ shared device pieces
+template <int KT = 5>
 __device__ __forceinline__ void build_weight_table(float *wtab, const Geom &g, int c0, bool flip,
                                                    const float *__restrict__ w0, const float *__restrict__ s0,
                                                    const float *__restrict__ b0, const float *__restrict__ wl,
                                                    const float *__restrict__ sl) {
-    // one table per plane slot (channel c0 + slot): [slot][class][WT_STRIDE], folded bias at [slot][0][25]
+    // one table per plane slot (channel c0 + slot): [slot][class][WS], folded bias at [slot][0][KK]
+    constexpr int KK = Taps<KT>::KK, WT_STRIDE = Taps<KT>::WS;
     const int ncls = 1 + 4 * g.L, n = g.NPL * ncls * KK;
     constexpr int WB = 4;
     // four entries per step, all eight loads issued before the first product: a 16-plane unit's table has 2000
@@ -201,14 +219,15 @@ __device__ __forceinline__ void build_weight_table(float *wtab, const Geom &g, i
         wtab[slot * ncls * WT_STRIDE + KK] = (b0 && c0 + slot < g.C) ? __ldg(s0 + c0 + slot) * __ldg(b0 + c0 + slot) : 0.f;
 }
 
-__device__ __forceinline__ void load_weights(const float *wt, float (&w)[KK]) {
+template <int N>
+__device__ __forceinline__ void load_weights(const float *wt, float (&w)[N]) {
     const float4 *q = reinterpret_cast<const float4 *>(wt);
 #pragma unroll
-    for (int t = 0; t < 6; ++t) {
+    for (int t = 0; t < N / 4; ++t) {
         const float4 v = q[t];
         w[4 * t] = v.x; w[4 * t + 1] = v.y; w[4 * t + 2] = v.z; w[4 * t + 3] = v.w;
     }
-    w[24] = wt[24];
+    w[N - 1] = wt[N - 1];  // 25 or 49
 }
 
 // four consecutive activations (16-byte aligned for float, 8-byte for the 16-bit types)
@@ -265,7 +284,9 @@ struct PatchD {   // 4x4 pixel staging patch (vector path, L >= 2)
     int xi, yi, y2;  // float indices of its first x / level-1 / level-2 element in shared memory
     int meta;     // bit 31 valid, bits 0-7 plane slot, bits 8-10 rows inside the image (1..4)
 };
+template <int KT>
 __device__ __forceinline__ PatchD decode_patch(const Geom &g, const int *off, int e) {
+    constexpr int HY = Taps<KT>::HY, HX = Taps<KT>::HX;
     PatchD p;
     p.meta = 0;
     p.so = p.xi = p.yi = p.y2 = 0;
@@ -276,9 +297,9 @@ __device__ __forceinline__ PatchD decode_patch(const Geom &g, const int *off, in
         int nrows = g.H - y;
         if (nrows > 4) nrows = 4;
         p.so = y * g.W + 4 * q;
-        p.xi = S + off[0] + (y + 2) * g.pitch[0] + 4 * q + 2;
-        p.yi = S + off[1] + (2 * i2 + 2) * g.pitch[1] + 2 * q + 2;
-        p.y2 = S + off[2] + (i2 + 2) * g.pitch[2] + q + 2;
+        p.xi = S + off[0] + (y + HY) * g.pitch[0] + 4 * q + HX;
+        p.yi = S + off[1] + (2 * i2 + HY) * g.pitch[1] + 2 * q + HX;
+        p.y2 = S + off[2] + (i2 + HY) * g.pitch[2] + q + HX;
         p.meta = (int)(0x80000000u | (unsigned)slot | ((unsigned)nrows << 8));
     }
     return p;
@@ -366,6 +387,7 @@ struct ItemD {    // one 4 x TH conv tile
     int slot;     // plane slot of the tile
     int dg;       // float offset from this tile's x-side array to the matching grad_out-side array (backward kernel)
 };
+template <int KT = 5>
 __device__ __forceinline__ ItemD decode_item(const Geom &g, int it, int nlevel_items, int nitems, int &bslot, int &tyy,
                                              int &txx, bool &is_base) {
     ItemD d;
@@ -380,7 +402,7 @@ __device__ __forceinline__ ItemD decode_item(const Geom &g, int it, int nlevel_i
         decode_level_item(g, it - slot * nlv, l, sub, ty2, tx2);
         const int pitch = g.pitch[l], zp = g.zpitch[l];
         d.src = slot * g.slot_stride + g.offA[l] + sub * g.rows[l] * pitch + g.th * ty2 * pitch + 4 * tx2;
-        d.wt = g.wtab_off + (slot * (1 + 4 * g.L) + 1 + (l - 1) * 4 + sub) * WT_STRIDE;
+        d.wt = g.wtab_off + (slot * (1 + 4 * g.L) + 1 + (l - 1) * 4 + sub) * Taps<KT>::WS;
         int zleft = g.zrows[l] - g.th * ty2;
         if (zleft > g.th) zleft = g.th;
         if (4 * tx2 < zp && zleft > 0) d.z = slot * g.slot_stride + g.offZ[l] + sub * g.zrows[l] * zp + g.th * ty2 * zp + 4 * tx2;
@@ -397,7 +419,7 @@ __device__ __forceinline__ ItemD decode_item(const Geom &g, int it, int nlevel_i
         txx = r - tyy * g.tx[0];
         const int pitch = g.pitch[0];
         d.src = bslot * g.slot_stride + g.offA[0] + g.th * tyy * pitch + 4 * txx;
-        d.wt = g.wtab_off + bslot * (1 + 4 * g.L) * WT_STRIDE;
+        d.wt = g.wtab_off + bslot * (1 + 4 * g.L) * Taps<KT>::WS;
         d.z = -1;
         d.meta = (int)(0x80000000u | (unsigned)pitch);
         d.dg = g.offG[0] - g.offA[0];
@@ -413,9 +435,10 @@ __device__ __forceinline__ ItemD decode_item(const Geom &g, int it, int nlevel_i
 // plane slot s from the raw shared buffer at src + s * slot_elems (a bulk copy put it there); RAW = false
 // reads global memory.  Pixels beyond H x W are never written and stay zero (odd-size padding and conv
 // halo); images beyond the batch are written as zeros.
-template <typename T, bool RAW>
+template <typename T, bool RAW, int KT>
 __device__ __forceinline__ int stage_input(float *sm, const Geom &g, const int *off, const T *__restrict__ src, int c,
                                            int b, int srank, int nstagers) {
+    constexpr int HY = Taps<KT>::HY, HX = Taps<KT>::HX;
     const int H = g.H, W = g.W, HW = H * W;
     const int p0 = g.pitch[0];
     const T *gsrc = RAW ? src : src + ((size_t)b * g.C + c) * HW;  // channel c (first of the unit) of image b
@@ -425,7 +448,7 @@ __device__ __forceinline__ int stage_input(float *sm, const Geom &g, const int *
         for (int e = srank; e < g.NPL * HW; e += nstagers) {
             const int slot = fdiv(e, g.d_npatch), r = e - slot * HW, y = fdiv(r, g.d_prow), xx = r - y * W;
             const bool valid = slot < nvalid;
-            sm[slot * g.slot_stride + off[0] + (y + 2) * p0 + xx + 2] =
+            sm[slot * g.slot_stride + off[0] + (y + HY) * p0 + xx + HX] =
                 valid ? ld1<T, RAW>(gsrc + (size_t)slot * img_stride + r) : 0.f;
         }
         return 1;
@@ -450,7 +473,7 @@ __device__ __forceinline__ int stage_input(float *sm, const Geom &g, const int *
                     if (y + rr < H) ld4<T, RAW>(pa + rr * W, a[rr]);
             }
             const int S = slot * g.slot_stride;
-            const int xi = S + off[0] + (y + 2) * p0 + 4 * q + 2;  // 8-byte aligned
+            const int xi = S + off[0] + (y + HY) * p0 + 4 * q + HX;  // 8-byte aligned
 #pragma unroll
             for (int rr = 0; rr < 4; ++rr) {
                 if (y + rr < H) {
@@ -465,7 +488,7 @@ __device__ __forceinline__ int stage_input(float *sm, const Geom &g, const int *
                 for (int bj = 0; bj < 2; ++bj)
                     h[bi][bj] = haar_butterfly(a[2 * bi][2 * bj], a[2 * bi][2 * bj + 1], a[2 * bi + 1][2 * bj],
                                                a[2 * bi + 1][2 * bj + 1]);
-            const int yi = S + off[1] + (2 * i2 + 2) * p1 + 2 * q + 2;
+            const int yi = S + off[1] + (2 * i2 + HY) * p1 + 2 * q + HX;
 #pragma unroll
             for (int bi = 0; bi < 2; ++bi) {
                 *reinterpret_cast<float2 *>(&sm[yi + bi * p1]) = make_float2(h[bi][0].ll, h[bi][1].ll);
@@ -474,7 +497,7 @@ __device__ __forceinline__ int stage_input(float *sm, const Geom &g, const int *
                 *reinterpret_cast<float2 *>(&sm[yi + bi * p1 + 3 * sub1]) = make_float2(h[bi][0].hh, h[bi][1].hh);
             }
             const Haar4 h2 = haar_butterfly(h[0][0].ll, h[0][1].ll, h[1][0].ll, h[1][1].ll);
-            const int y2 = S + off[2] + (i2 + 2) * p2 + q + 2;
+            const int y2 = S + off[2] + (i2 + HY) * p2 + q + HX;
             sm[y2] = h2.ll;
             sm[y2 + sub2] = h2.lh;
             sm[y2 + 2 * sub2] = h2.hl;
@@ -496,7 +519,7 @@ __device__ __forceinline__ int stage_input(float *sm, const Geom &g, const int *
                 if (y1) ld4<T, RAW>(pa + W, a1);
             }
             const int S = slot * g.slot_stride;
-            const int xi = S + off[0] + (y + 2) * p0 + 4 * q + 2;  // 8-byte aligned
+            const int xi = S + off[0] + (y + HY) * p0 + 4 * q + HX;  // 8-byte aligned
             *reinterpret_cast<float2 *>(&sm[xi]) = make_float2(a0[0], a0[1]);
             *reinterpret_cast<float2 *>(&sm[xi + 2]) = make_float2(a0[2], a0[3]);
             if (y1) {
@@ -504,7 +527,7 @@ __device__ __forceinline__ int stage_input(float *sm, const Geom &g, const int *
                 *reinterpret_cast<float2 *>(&sm[xi + p0 + 2]) = make_float2(a1[2], a1[3]);
             }
             const Haar4 ha = haar_butterfly(a0[0], a0[1], a1[0], a1[1]), hb = haar_butterfly(a0[2], a0[3], a1[2], a1[3]);
-            const int yi = S + off[1] + (i + 2) * p1 + 2 * q + 2;
+            const int yi = S + off[1] + (i + HY) * p1 + 2 * q + HX;
             *reinterpret_cast<float2 *>(&sm[yi]) = make_float2(ha.ll, hb.ll);
             *reinterpret_cast<float2 *>(&sm[yi + sub1]) = make_float2(ha.lh, hb.lh);
             *reinterpret_cast<float2 *>(&sm[yi + 2 * sub1]) = make_float2(ha.hl, hb.hl);
@@ -528,13 +551,13 @@ __device__ __forceinline__ int stage_input(float *sm, const Geom &g, const int *
             if (x1 && y1) d = ld1<T, RAW>(pa + W + 1);
         }
         const int S = slot * g.slot_stride;
-        const int xi = S + off[0] + (y + 2) * p0 + xx + 2;
+        const int xi = S + off[0] + (y + HY) * p0 + xx + HX;
         sm[xi] = a;
         if (x1) sm[xi + 1] = bq;
         if (y1) sm[xi + p0] = cq;
         if (x1 && y1) sm[xi + p0 + 1] = d;
         const Haar4 h = haar_butterfly(a, bq, cq, d);
-        const int yi = S + off[1] + (i + 2) * p1 + j + 2;
+        const int yi = S + off[1] + (i + HY) * p1 + j + HX;
         sm[yi] = h.ll;
         sm[yi + sub1] = h.lh;
         sm[yi + 2 * sub1] = h.hl;
@@ -605,17 +628,19 @@ __device__ __forceinline__ void give_up_after_timeout(unsigned long long *bar, c
 
 // Level l >= 2 from the raw LL band of level l-1 (already in shared memory).  Reads one element past
 // an odd grid land in the zero padding.
+template <int KT>
 __device__ __forceinline__ void stage_level(float *sm, const Geom &g, const int *off, int l) {
+    constexpr int HY = Taps<KT>::HY, HX = Taps<KT>::HX;
     const int Wl = g.Wl[l], n = (int)g.d_lvl[l].d;
     const int pp = g.pitch[l - 1], pl = g.pitch[l], subl = g.rows[l] * pl;
     for (int e = threadIdx.x; e < g.NPL * n; e += blockDim.x) {
         const int slot = fdiv(e, g.d_lvl[l]), r = e - slot * n, i = fdiv(r, g.d_lvlw[l]), j = r - i * Wl;
         const int S = slot * g.slot_stride;
-        const int si = S + off[l - 1] + (2 * i + 2) * pp + 2 * j + 2;  // even column: 8-byte aligned
+        const int si = S + off[l - 1] + (2 * i + HY) * pp + 2 * j + HX;  // even column: 8-byte aligned
         const float2 top = *reinterpret_cast<const float2 *>(&sm[si]);
         const float2 bot = *reinterpret_cast<const float2 *>(&sm[si + pp]);
         const Haar4 h = haar_butterfly(top.x, top.y, bot.x, bot.y);
-        const int yi = S + off[l] + (i + 2) * pl + j + 2;
+        const int yi = S + off[l] + (i + HY) * pl + j + HX;
         sm[yi] = h.ll;
         sm[yi + subl] = h.lh;
         sm[yi + 2 * subl] = h.hl;
@@ -623,34 +648,44 @@ __device__ __forceinline__ void stage_level(float *sm, const Geom &g, const int 
     }
 }
 
-// 4-column x TH-row output tile of a 5x5 correlation.  `src` = array + (TH*ty)*pitch + 4*tx is the
-// window's top-left element (the array's halo of 2 makes window row rr = output row + tap row), 16-byte
-// aligned; eight floats per window row.
-// KEEP: the window's interior (rows 2 .. TH+1, columns 2 .. 5: the tile's own elements) is copied to `keep` on the
-// way through the registers.  KT: taps per side that are in use, 5 or 3 - a 3 x 3 kernel sits in the middle of the
+// One window row of a tile: Taps<KT>::NQ aligned 16-byte loads.
+template <int KT>
+__device__ __forceinline__ void load_row(const float *__restrict__ p, float4 (&n)[Taps<KT>::NQ]) {
+#pragma unroll
+    for (int q = 0; q < Taps<KT>::NQ; ++q) n[q] = *reinterpret_cast<const float4 *>(p + 4 * q);
+}
+template <int KT>
+__device__ __forceinline__ void spread_row(const float4 (&n)[Taps<KT>::NQ], float (&in)[4 * Taps<KT>::NQ]) {
+#pragma unroll
+    for (int q = 0; q < Taps<KT>::NQ; ++q) { in[4 * q] = n[q].x; in[4 * q + 1] = n[q].y; in[4 * q + 2] = n[q].z; in[4 * q + 3] = n[q].w; }
+}
+// 4-column x TH-row output tile of a 5x5 (7x7) correlation.  `src` = array + (TH*ty)*pitch + 4*tx is the
+// window's top-left element (the array's halo makes window row rr = output row + tap row), 16-byte
+// aligned; eight (twelve) floats per window row.
+// KEEP: the window's interior (rows HY .. TH+HY-1, columns HX .. HX+3: the tile's own elements) is copied to `keep` on the
+// way through the registers.  KT: taps per side that are in use - a 3 x 3 kernel sits in the middle of the
 // 5 x 5 table and of the 5 x 5 window, its zero border is neither read nor multiplied.
 template <int TH, bool KEEP = false, int KT = 5>
-__device__ __forceinline__ void conv_tile(const float *__restrict__ src, int pitch, const float (&w)[KK],
+__device__ __forceinline__ void conv_tile(const float *__restrict__ src, int pitch, const float (&w)[Taps<KT>::KK],
                                           float (&acc)[TH][4], float (*keep)[4] = nullptr) {
-    constexpr int T0 = (5 - KT) / 2, T1 = 5 - T0;  // taps T0 .. T1-1 per side; window rows T0 .. TH+3-T0
+    using Q = Taps<KT>;
+    constexpr int T0 = Q::T0, T1 = Q::T1, LAST = TH + Q::K - 1 - T0;  // window rows T0 .. LAST - 1
 #pragma unroll
     for (int r = 0; r < TH; ++r)
 #pragma unroll
         for (int c = 0; c < 4; ++c) acc[r][c] = 0.f;
     // the next window row is fetched while the current one is being used (software pipelining by hand)
-    float4 n0 = *reinterpret_cast<const float4 *>(src + T0 * pitch);
-    float4 n1 = *reinterpret_cast<const float4 *>(src + T0 * pitch + 4);
+    float4 n[Q::NQ];
+    load_row<KT>(src + T0 * pitch, n);
 #pragma unroll
-    for (int rr = T0; rr < TH + 4 - T0; ++rr) {
-        const float in[8] = {n0.x, n0.y, n0.z, n0.w, n1.x, n1.y, n1.z, n1.w};
-        if (KEEP && rr >= 2 && rr < TH + 2) {
+    for (int rr = T0; rr < LAST; ++rr) {
+        float in[4 * Q::NQ];
+        spread_row<KT>(n, in);
+        if (KEEP && rr >= Q::HY && rr < TH + Q::HY) {
 #pragma unroll
-            for (int c = 0; c < 4; ++c) keep[rr - 2][c] = in[c + 2];
+            for (int c = 0; c < 4; ++c) keep[rr - Q::HY][c] = in[c + Q::HX];
         }
-        if (rr + 1 < TH + 4 - T0) {
-            n0 = *reinterpret_cast<const float4 *>(src + (rr + 1) * pitch);
-            n1 = *reinterpret_cast<const float4 *>(src + (rr + 1) * pitch + 4);
-        }
+        if (rr + 1 < LAST) load_row<KT>(src + (rr + 1) * pitch, n);
 #pragma unroll
         for (int u = T0; u < T1; ++u) {
             const int r = rr - u;
@@ -658,7 +693,7 @@ __device__ __forceinline__ void conv_tile(const float *__restrict__ src, int pit
 #pragma unroll
                 for (int v = T0; v < T1; ++v)
 #pragma unroll
-                    for (int c = 0; c < 4; ++c) acc[r][c] = fmaf(w[u * 5 + v], in[c + v], acc[r][c]);
+                    for (int c = 0; c < 4; ++c) acc[r][c] = fmaf(w[u * Q::K + v], in[c + v + Q::C0], acc[r][c]);
             }
         }
     }
@@ -667,18 +702,17 @@ __device__ __forceinline__ void conv_tile(const float *__restrict__ src, int pit
 // The weight-gradient taps of one tile: accw[u][v] += sum over the tile of D[r][c] * Y[r + u][c + v] (window
 // coordinates; `d` = the tile's D values, `ysrc` = the window's top-left element).
 template <int TH, int KT>
-__device__ __forceinline__ void wgrad_taps(const float *__restrict__ ysrc, int pitch, const float (&d)[TH][4], float (&accw)[KK]) {
-    constexpr int T0 = (5 - KT) / 2, T1 = 5 - T0;
+__device__ __forceinline__ void wgrad_taps(const float *__restrict__ ysrc, int pitch, const float (&d)[TH][4], float (&accw)[Taps<KT>::KK]) {
+    using Q = Taps<KT>;
+    constexpr int T0 = Q::T0, T1 = Q::T1, LAST = TH + Q::K - 1 - T0;
     // the next window row is fetched while the current one is used
-    float4 n0 = *reinterpret_cast<const float4 *>(ysrc + T0 * pitch);
-    float4 n1 = *reinterpret_cast<const float4 *>(ysrc + T0 * pitch + 4);
+    float4 n[Q::NQ];
+    load_row<KT>(ysrc + T0 * pitch, n);
 #pragma unroll
-    for (int rr = T0; rr < TH + 4 - T0; ++rr) {
-        const float in[8] = {n0.x, n0.y, n0.z, n0.w, n1.x, n1.y, n1.z, n1.w};
-        if (rr + 1 < TH + 4 - T0) {
-            n0 = *reinterpret_cast<const float4 *>(ysrc + (rr + 1) * pitch);
-            n1 = *reinterpret_cast<const float4 *>(ysrc + (rr + 1) * pitch + 4);
-        }
+    for (int rr = T0; rr < LAST; ++rr) {
+        float in[4 * Q::NQ];
+        spread_row<KT>(n, in);
+        if (rr + 1 < LAST) load_row<KT>(ysrc + (rr + 1) * pitch, n);
 #pragma unroll
         for (int uu = T0; uu < T1; ++uu) {
             const int dr = rr - uu;
@@ -686,7 +720,7 @@ __device__ __forceinline__ void wgrad_taps(const float *__restrict__ ysrc, int p
 #pragma unroll
                 for (int v = T0; v < T1; ++v)
 #pragma unroll
-                    for (int cc = 0; cc < 4; ++cc) accw[uu * 5 + v] = fmaf(d[dr][cc], in[cc + v], accw[uu * 5 + v]);
+                    for (int cc = 0; cc < 4; ++cc) accw[uu * Q::K + v] = fmaf(d[dr][cc], in[cc + v + Q::C0], accw[uu * Q::K + v]);
             }
         }
     }
@@ -866,9 +900,9 @@ plane_fwd_kernel(const __grid_constant__ Geom g, const T *__restrict__ x, const 
     bool has_base = false;
 #pragma unroll
     for (int k = 0; k < MAXI; ++k)
-        items[k] = decode_item(g, hoist_items ? tid + k * nthr : 0x3fffffff, nlevel_items, nitems, bslot, tyy, txx, has_base);
-    PatchD patch0 = decode_patch(g, g.offA, hoist_patch ? srank : 0x3fffffff);
-    PatchD patch1 = decode_patch(g, g.offA, hoist_patch && srank < nstagers ? srank + nstagers : 0x3fffffff);
+        items[k] = decode_item<KT>(g, hoist_items ? tid + k * nthr : 0x3fffffff, nlevel_items, nitems, bslot, tyy, txx, has_base);
+    PatchD patch0 = decode_patch<KT>(g, g.offA, hoist_patch ? srank : 0x3fffffff);
+    PatchD patch1 = decode_patch<KT>(g, g.offA, hoist_patch && srank < nstagers ? srank + nstagers : 0x3fffffff);
     // Everything above touched shared memory and registers only and may have run beside the tail of the kernel
     // before this one; global memory is used from here on.  The input-gradient instantiation is followed by the small
     // epilogue and releases it at the end (see plane_bwd_kernel).
@@ -883,7 +917,7 @@ plane_fwd_kernel(const __grid_constant__ Geom g, const T *__restrict__ x, const 
         const int c = cg * g.NPL;
         const int nvalid = g.C - c < g.NPL ? g.C - c : g.NPL;
         if (c != c_prev) {  // units are group-major: the tables survive all images of a channel group
-            build_weight_table(wtab, g, c, FLIP, w0, s0, FLIP ? nullptr : b0, wl, sl);
+            build_weight_table<KT>(wtab, g, c, FLIP, w0, s0, FLIP ? nullptr : b0, wl, sl);
             c_prev = c;
         }
         int lnext;
@@ -898,7 +932,7 @@ plane_fwd_kernel(const __grid_constant__ Geom g, const T *__restrict__ x, const 
                 run_patch<T, true>(sm, g, patch1, rx, nvalid);
                 lnext = 3;
             } else {
-                lnext = stage_input<T, true>(sm, g, g.offA, rx, c, b, srank, nstagers);
+                lnext = stage_input<T, true, KT>(sm, g, g.offA, rx, c, b, srank, nstagers);
             }
         } else if (hoist_patch) {
             const T *gsrc = x + ((size_t)b * g.C + c) * HW;
@@ -906,7 +940,7 @@ plane_fwd_kernel(const __grid_constant__ Geom g, const T *__restrict__ x, const 
             run_patch<T, false>(sm, g, patch1, gsrc, nvalid);
             lnext = 3;
         } else {
-            lnext = stage_input<T, false>(sm, g, g.offA, x, c, b, srank, nstagers);
+            lnext = stage_input<T, false, KT>(sm, g, g.offA, x, c, b, srank, nstagers);
         }
         if (g.bulk) {
             if (__syncthreads_or(late)) {
@@ -930,7 +964,7 @@ plane_fwd_kernel(const __grid_constant__ Geom g, const T *__restrict__ x, const 
             if (cgn * g.NPL + g.NPL <= g.C) prefetch_unit_l2<T>(g, x, cgn * g.NPL, (u + 1) - cgn * g.B);
         }
         for (int l = lnext; l <= L; ++l) {
-            stage_level(sm, g, g.offA, l);
+            stage_level<KT>(sm, g, g.offA, l);
             __syncthreads();
         }
         // ---- one item list: level tiles (Z^l = Wfold^l (*) Y^l) first, base tiles last; a thread's last
@@ -948,11 +982,11 @@ plane_fwd_kernel(const __grid_constant__ Geom g, const T *__restrict__ x, const 
                     d = k == 0 ? items[0] : items[1];
                 } else {
                     bool isb = false;
-                    d = decode_item(g, tid + k * nthr, nlevel_items, nitems, bslot, tyy, txx, isb);
+                    d = decode_item<KT>(g, tid + k * nthr, nlevel_items, nitems, bslot, tyy, txx, isb);
                     has_base = isb;
                 }
                 if (d.meta < 0) {
-                    float w[KK];
+                    float w[Taps<KT>::KK];
                     load_weights(sm + d.wt, w);
                     conv_tile<TH, false, KT>(sm + d.src, d.meta & 0x3ff, w, acc);
                     if (d.z >= 0) {
@@ -965,7 +999,7 @@ plane_fwd_kernel(const __grid_constant__ Geom g, const T *__restrict__ x, const 
                 }
             }
         }
-        const float bias = wtab[bslot * (1 + 4 * L) * WT_STRIDE + KK];
+        const float bias = wtab[bslot * (1 + 4 * L) * Taps<KT>::WS + Taps<KT>::KK];
         if (g.bulk_out && tid == 0) bulk_store_wait_read();  // the previous unit's store has drained the output image
         __syncthreads();
         if (has_base) {
@@ -993,8 +1027,9 @@ plane_fwd_kernel(const __grid_constant__ Geom g, const T *__restrict__ x, const 
 template <typename T, int MAXT, int MINB, int TH, int KT>
 __global__ void __launch_bounds__(MAXT, MINB)
 plane_wgrad_kernel(const __grid_constant__ Geom g, const T *__restrict__ x, const T *__restrict__ go,
-                   float *__restrict__ part0, float *__restrict__ partl /* level l at l*C*np*100 */,
+                   float *__restrict__ part0, float *__restrict__ partl /* level l at l*C*np*4*KK */,
                    int *__restrict__ status) {
+    constexpr int KK = Taps<KT>::KK;
     extern __shared__ __align__(16) float sm[];
     const int tid = threadIdx.x, nthr = blockDim.x;
     unsigned long long *bar = reinterpret_cast<unsigned long long *>(sm + g.bar_off);
@@ -1029,15 +1064,15 @@ plane_wgrad_kernel(const __grid_constant__ Geom g, const T *__restrict__ x, cons
             const bool late = !mbar_wait(bar + ring, parity, g.no_copy ? WAIT_LIMIT_TEST : WAIT_LIMIT);
             const T *rx = reinterpret_cast<const T *>(raw + ring * g.stage_bytes);
             const T *rg = reinterpret_cast<const T *>(raw + ring * g.stage_bytes + (size_t)g.NPL * g.plane_bytes);
-            lnext = stage_input<T, true>(sm, g, g.offA, rx, c, b, tid, nthr);
-            stage_input<T, true>(sm, g, g.offG, rg, c, b, tid, nthr);
+            lnext = stage_input<T, true, KT>(sm, g, g.offA, rx, c, b, tid, nthr);
+            stage_input<T, true, KT>(sm, g, g.offG, rg, c, b, tid, nthr);
             if (__syncthreads_or(late)) {
                 give_up_after_timeout(bar, g, ring, parity, u, u_end, status);
                 break;
             }
         } else {
-            lnext = stage_input<T, false>(sm, g, g.offA, x, c, b, tid, nthr);
-            stage_input<T, false>(sm, g, g.offG, go, c, b, tid, nthr);
+            lnext = stage_input<T, false, KT>(sm, g, g.offA, x, c, b, tid, nthr);
+            stage_input<T, false, KT>(sm, g, g.offG, go, c, b, tid, nthr);
             __syncthreads();
         }
         if (g.bulk) {
@@ -1054,8 +1089,8 @@ plane_wgrad_kernel(const __grid_constant__ Geom g, const T *__restrict__ x, cons
             prefetch_unit_l2<T>(g, go, cn, bn);
         }
         for (int l = lnext; l <= L; ++l) {
-            stage_level(sm, g, g.offA, l);
-            stage_level(sm, g, g.offG, l);
+            stage_level<KT>(sm, g, g.offA, l);
+            stage_level<KT>(sm, g, g.offG, l);
             __syncthreads();
         }
         if (active) {
@@ -1064,8 +1099,8 @@ plane_wgrad_kernel(const __grid_constant__ Geom g, const T *__restrict__ x, cons
                 const int tyy = fdiv(r, g.d_tx[lvl]), txx = r - tyy * g.tx[lvl];
                 const float *S = sm + slot * g.slot_stride;
                 const float *ysrc = S + g.offA[lvl] + suboff + TH * tyy * pl + 4 * txx;
-                // D tile = columns 4tx+2..4tx+5 of rows TH*ty+2.. (8-byte aligned)
-                const float *dsrc = S + g.offG[lvl] + suboff + (TH * tyy + 2) * pl + 4 * txx + 2;
+                // D tile = columns 4tx+HX..4tx+HX+3 of rows TH*ty+HY.. (8-byte aligned)
+                const float *dsrc = S + g.offG[lvl] + suboff + (TH * tyy + Taps<KT>::HY) * pl + 4 * txx + Taps<KT>::HX;
                 float d[TH][4];
 #pragma unroll
                 for (int rr = 0; rr < TH; ++rr) {
@@ -1130,7 +1165,7 @@ __global__ void __launch_bounds__(256, 2)
 plane_bwd_kernel(const __grid_constant__ Geom g, const T *__restrict__ x, const T *__restrict__ go,
                  const float *__restrict__ w0, const float *__restrict__ s0, const float *__restrict__ wl,
                  const float *__restrict__ sl, T *__restrict__ gx, float *__restrict__ part0,
-                 float *__restrict__ partl /* level l at l*C*np*100 */, int *__restrict__ status) {
+                 float *__restrict__ partl /* level l at l*C*np*4*KK */, int *__restrict__ status) {
     extern __shared__ __align__(16) float sm[];
     const int tid = threadIdx.x, nthr = blockDim.x;
     float *wtab = sm + g.wtab_off;
@@ -1145,7 +1180,7 @@ plane_bwd_kernel(const __grid_constant__ Geom g, const T *__restrict__ x, const 
     const size_t HW = (size_t)g.H * g.W;
     int bslot = 0, tyy = 0, txx = 0;
     bool has_base = false;
-    const ItemD item = decode_item(g, tid, nlevel_items, nitems, bslot, tyy, txx, has_base);
+    const ItemD item = decode_item<KT>(g, tid, nlevel_items, nitems, bslot, tyy, txx, has_base);
     const int cls = (item.meta >> 24) & 0x3f;
     // No barrier separates a unit's synthesis (which reads only Z and registers) from the next unit's staging.
     // With the planes already in shared memory (BULK == 2) the staging is left to the whole warps that hold
@@ -1157,8 +1192,8 @@ plane_bwd_kernel(const __grid_constant__ Geom g, const T *__restrict__ x, const 
     if (BULK != 2 || nstagers * 4 < nthr || g.NPL * g.npatch4 > nstagers) nstagers = nthr;
     const int srank = tid < nstagers ? tid : 0x3fffffff;
     const bool hoist_patch = g.vec && L >= 2 && g.NPL * g.npatch4 <= 2 * nstagers;
-    const PatchD patch0 = decode_patch(g, g.offA, hoist_patch ? srank : 0x3fffffff);
-    const PatchD patch1 = decode_patch(g, g.offA, hoist_patch && srank < nstagers ? srank + nstagers : 0x3fffffff);
+    const PatchD patch0 = decode_patch<KT>(g, g.offA, hoist_patch ? srank : 0x3fffffff);
+    const PatchD patch1 = decode_patch<KT>(g, g.offA, hoist_patch && srank < nstagers ? srank + nstagers : 0x3fffffff);
     const int dA0 = g.offG[0] - g.offA[0], dA1 = L >= 1 ? g.offG[1] - g.offA[1] : 0, dA2 = L >= 2 ? g.offG[2] - g.offA[2] : 0;
     float accw[KK], gsum = 0.f;
 #pragma unroll
@@ -1174,7 +1209,7 @@ plane_bwd_kernel(const __grid_constant__ Geom g, const T *__restrict__ x, const 
         const int c = cg * g.NPL;
         const int nvalid = g.C - c < g.NPL ? g.C - c : g.NPL;
         if (c != c_prev) {
-            build_weight_table(wtab, g, c, true, w0, s0, nullptr, wl, sl);
+            build_weight_table<KT>(wtab, g, c, true, w0, s0, nullptr, wl, sl);
             c_prev = c;
         }
         int lnext;
@@ -1190,8 +1225,8 @@ plane_bwd_kernel(const __grid_constant__ Geom g, const T *__restrict__ x, const 
                 run_patch<T, true>(sm, g, patch1, rg, nvalid, dA0, dA1, dA2);
                 lnext = 3;
             } else {
-                lnext = stage_input<T, true>(sm, g, g.offA, rx, c, b, tid, nthr);
-                stage_input<T, true>(sm, g, g.offG, rg, c, b, tid, nthr);
+                lnext = stage_input<T, true, KT>(sm, g, g.offA, rx, c, b, tid, nthr);
+                stage_input<T, true, KT>(sm, g, g.offG, rg, c, b, tid, nthr);
             }
         } else if (hoist_patch) {
             const size_t po = ((size_t)b * g.C + c) * HW;
@@ -1199,8 +1234,8 @@ plane_bwd_kernel(const __grid_constant__ Geom g, const T *__restrict__ x, const 
             run_patch_pair<T, false>(sm, g, patch1, x + po, go + po, nvalid, dA0, dA1, dA2);
             lnext = 3;
         } else {
-            lnext = stage_input<T, false>(sm, g, g.offA, x, c, b, tid, nthr);
-            stage_input<T, false>(sm, g, g.offG, go, c, b, tid, nthr);
+            lnext = stage_input<T, false, KT>(sm, g, g.offA, x, c, b, tid, nthr);
+            stage_input<T, false, KT>(sm, g, g.offG, go, c, b, tid, nthr);
         }
         if (BULK) {
             if (__syncthreads_or(late)) {
@@ -1227,8 +1262,8 @@ plane_bwd_kernel(const __grid_constant__ Geom g, const T *__restrict__ x, const 
             }
         }
         for (int l = lnext; l <= L; ++l) {
-            stage_level(sm, g, g.offA, l);
-            stage_level(sm, g, g.offG, l);
+            stage_level<KT>(sm, g, g.offA, l);
+            stage_level<KT>(sm, g, g.offG, l);
             __syncthreads();
         }
         float acc[TH][4];
@@ -1241,7 +1276,7 @@ plane_bwd_kernel(const __grid_constant__ Geom g, const T *__restrict__ x, const 
             // are loaded on their own.
             float d[TH][4];
             if (TH == 4) {
-                float w[KK];
+                float w[Taps<KT>::KK];
                 load_weights(sm + item.wt, w);
                 conv_tile<TH, true, KT>(gsrc, pitch, w, acc, d);
             } else {
@@ -1263,7 +1298,7 @@ plane_bwd_kernel(const __grid_constant__ Geom g, const T *__restrict__ x, const 
                 wgrad_taps<TH, KT>(ysrc, pitch, d, accw);
             }
             if (TH != 4) {  // input gradient: rotated-kernel conv of the D window
-                float w[KK];
+                float w[Taps<KT>::KK];
                 load_weights(sm + item.wt, w);
                 conv_tile<TH, false, KT>(gsrc, pitch, w, acc);
             }
@@ -1344,15 +1379,17 @@ plane_bwd_kernel(const __grid_constant__ Geom g, const T *__restrict__ x, const 
 }
 
 // ------------------------------------------------------------------ host-side planning
-inline void fill_common(Geom &g, int B, int C, int H, int W, int L, int elem_bytes, int TH) {
+inline void fill_common(Geom &g, int B, int C, int H, int W, int L, int elem_bytes, int TH, int k = 5) {
+    const int hy = k == 7 ? Taps<7>::HY : Taps<5>::HY, hx = k == 7 ? Taps<7>::HX : Taps<5>::HX;
+    g.k = g.taps = k;
     g.B = B; g.C = C; g.H = H; g.W = W; g.L = L; g.th = TH;
     g.Hl[0] = H; g.Wl[0] = W;
     for (int l = 1; l <= MAXL; ++l) { g.Hl[l] = (g.Hl[l - 1] + 1) / 2; g.Wl[l] = (g.Wl[l - 1] + 1) / 2; }
     for (int l = 0; l <= L; ++l) {
         g.ty[l] = (g.Hl[l] + TH - 1) / TH;
         g.tx[l] = pad4(g.Wl[l]) / 4;
-        g.rows[l] = g.ty[l] * TH + 4;
-        g.pitch[l] = pad4(g.Wl[l]) + 4;
+        g.rows[l] = g.ty[l] * TH + 2 * hy;
+        g.pitch[l] = pad4(g.Wl[l]) + 2 * hx;
     }
     g.nbase = g.tx[0] * g.ty[0];
     g.lvl_start[0] = 0; g.lvl_start[1] = 0;
@@ -1456,11 +1493,11 @@ inline double tile_score(const Geom &g, double short_tiles = 0.93) {
 }
 
 // Forward plan.  `tune` (0 = automatic): bits 0-4 threads/32, bits 5-7 blocks per SM, bits 8-13 planes per unit.
-inline bool plan_forward_th(int B, int C, int H, int W, int L, int elem_bytes, Geom &best, unsigned tune, int th) {
+inline bool plan_forward_th(int k, int B, int C, int H, int W, int L, int elem_bytes, Geom &best, unsigned tune, int th) {
     const int fT = (tune & 31) * 32, fBps = (tune >> 5) & 7, fNpl = (tune >> 8) & 63;
     const bool no_bulk = (tune >> 20) & 1;
     Geom g = {};
-    fill_common(g, B, C, H, W, L, elem_bytes, th);
+    fill_common(g, B, C, H, W, L, elem_bytes, th, k);
     const int slot = layout_slot(g, false, true);
     const int M = g.lvl_start[L + 1] + g.nbase;
     const double teff = tile_score(g);
@@ -1468,7 +1505,7 @@ inline bool plan_forward_th(int B, int C, int H, int W, int L, int elem_bytes, G
     for (int npl = 1; npl <= 64; ++npl) {
         if (npl > 1 && npl > C) break;
         if (fNpl && npl != fNpl) continue;
-        const int wtab = npl * (1 + 4 * L) * WT_STRIDE;
+        const int wtab = npl * (1 + 4 * L) * table_stride(k);
         const bool can_bulk = (C % npl == 0) && (((long long)npl * g.plane_bytes) % 16 == 0) && !no_bulk;
         for (int use_bulk = can_bulk ? 1 : 0; use_bulk >= 0; --use_bulk) {
         Geom cg = g;
@@ -1480,7 +1517,7 @@ inline bool plan_forward_th(int B, int C, int H, int W, int L, int elem_bytes, G
             if (npl * g.nbase > T) continue;  // at most one base tile per thread
             if (fT && T != fT) continue;
             for (int bps = 1; bps <= 6; ++bps) {
-                if (bps * T > 768) continue;  // register file: kernels are built for 128 / 84 registers
+                if (bps * T > (k == 7 ? 512 : 768)) continue;  // register file: kernels are built for 128 / 84 registers (7 x 7: 128)
                 if (fBps && bps != fBps) continue;
                 if (bps * (bytes + 1024) > SMEM_PER_SM) continue;
                 const int rounds = (npl * M + T - 1) / T;
@@ -1516,11 +1553,11 @@ inline bool plan_forward_th(int B, int C, int H, int W, int L, int elem_bytes, G
 
 // Weight-gradient plan: per class c with n_c tiles (x NPL) allocate ceil(n_c NPL / rounds) threads, smallest
 // `rounds` that fits the thread limit.  tune bits 14-19: planes per unit.
-inline bool plan_wgrad_th(int B, int C, int H, int W, int L, int elem_bytes, Geom &best, unsigned tune, int th) {
+inline bool plan_wgrad_th(int k, int B, int C, int H, int W, int L, int elem_bytes, Geom &best, unsigned tune, int th) {
     const int fNpl = (tune >> 14) & 63, fBps = 0;
     const bool no_bulk = (tune >> 20) & 1;
     Geom g = {};
-    fill_common(g, B, C, H, W, L, elem_bytes, th);
+    fill_common(g, B, C, H, W, L, elem_bytes, th, k);
     const int slot = layout_slot(g, true, false);
     const int ncls = 1 + 4 * L;
     const double teff = tile_score(g);
@@ -1541,7 +1578,7 @@ inline bool plan_wgrad_th(int B, int C, int H, int W, int L, int elem_bytes, Geo
             if (tot > MAX_THREADS) continue;
             const int T = (tot + 31) & ~31;
             long long arrays = (long long)npl * slot;
-            const long long scratch = (long long)T * (KK + 1);
+            const long long scratch = (long long)T * (k * k + 1);
             if (scratch > arrays) arrays = scratch;
             bool any = false;
             const bool can_bulk = (g.plane_bytes % 16 == 0) && !no_bulk;
@@ -1552,7 +1589,9 @@ inline bool plan_wgrad_th(int B, int C, int H, int W, int L, int elem_bytes, Geo
                 const long long bytes = smem_floats * 4;
                 if (bytes > SMEM_LIMIT) continue;
                 any = true;
-                for (int bps = 1; bps <= 4; ++bps) {
+                // (small planes have blocks of one or two warps: up to sixteen of them keep an SM busy; with four at most, the backward of 7 x 7
+                // kernels took 194 us instead of 116 on 110 x 139 planes of 7 x 7 and 486 instead of 299 on 88 x 515 of 6 x 7)
+                for (int bps = 1; bps <= 16; ++bps) {
                     if (bps * T > 512) continue;  // 128 registers per thread
                     if (fBps && bps != fBps) continue;
                     if (bps * (bytes + 1024) > SMEM_PER_SM) continue;
@@ -1590,10 +1629,10 @@ inline bool plan_wgrad_th(int B, int C, int H, int W, int L, int elem_bytes, Geo
 
 // Fused-backward plan: one round (every tile its own thread), both input pyramids plus Z in shared memory, no
 // bulk prefetch unless it fits.  tune bits 14-19: planes per unit (shared with the weight-gradient plan).
-inline bool plan_bwd_fused_th(int B, int C, int H, int W, int L, int elem_bytes, Geom &best, unsigned tune, int th) {
+inline bool plan_bwd_fused_th(int k, int B, int C, int H, int W, int L, int elem_bytes, Geom &best, unsigned tune, int th) {
     const int fNpl = (tune >> 14) & 63, fBps = 0;
     Geom g = {};
-    fill_common(g, B, C, H, W, L, elem_bytes, th);
+    fill_common(g, B, C, H, W, L, elem_bytes, th, k);
     const int slot = layout_slot(g, true, true);
     const int M = g.lvl_start[L + 1] + g.nbase;
     const double teff = tile_score(g, 1.03);
@@ -1602,7 +1641,7 @@ inline bool plan_bwd_fused_th(int B, int C, int H, int W, int L, int elem_bytes,
         if (npl > 1 && npl > C) break;
         if (fNpl && npl != fNpl) continue;
         if (npl * M > 256) break;
-        const int wtab = npl * (1 + 4 * L) * WT_STRIDE;
+        const int wtab = npl * (1 + 4 * L) * table_stride(k);
         const int T = (npl * M + 31) & ~31;
         long long arrays = (long long)npl * slot;
         const long long scratch = (long long)T * (KK + 2) + 2LL * npl * (1 + 4 * L);  // flush scratch: sums, tags, run starts and ends
@@ -1653,28 +1692,28 @@ inline bool plan_bwd_fused_th(int B, int C, int H, int W, int L, int elem_bytes,
 }
 
 // Each plan is searched for both tile heights; tune bit 22 forces 8 rows, bit 23 forces 4 rows.
-inline bool search_forward(int B, int C, int H, int W, int L, int elem_bytes, Geom &best, unsigned tune) {
+inline bool search_forward(int k, int B, int C, int H, int W, int L, int elem_bytes, Geom &best, unsigned tune) {
     best.score = -1.0;
     bool ok = false;
-    if (!((tune >> 23) & 1)) ok |= plan_forward_th(B, C, H, W, L, elem_bytes, best, tune, 8);
-    if (!((tune >> 22) & 1)) ok |= plan_forward_th(B, C, H, W, L, elem_bytes, best, tune, 4);
+    if (!((tune >> 23) & 1)) ok |= plan_forward_th(k, B, C, H, W, L, elem_bytes, best, tune, 8);
+    if (!((tune >> 22) & 1)) ok |= plan_forward_th(k, B, C, H, W, L, elem_bytes, best, tune, 4);
     if (ok) deepen_prefetch(best);
     return ok;
 }
-inline bool search_wgrad(int B, int C, int H, int W, int L, int elem_bytes, Geom &best, unsigned tune) {
+inline bool search_wgrad(int k, int B, int C, int H, int W, int L, int elem_bytes, Geom &best, unsigned tune) {
     best.score = -1.0;
     bool ok = false;
-    if (!((tune >> 23) & 1)) ok |= plan_wgrad_th(B, C, H, W, L, elem_bytes, best, tune, 8);
-    if (!((tune >> 22) & 1)) ok |= plan_wgrad_th(B, C, H, W, L, elem_bytes, best, tune, 4);
+    if (!((tune >> 23) & 1)) ok |= plan_wgrad_th(k, B, C, H, W, L, elem_bytes, best, tune, 8);
+    if (!((tune >> 22) & 1)) ok |= plan_wgrad_th(k, B, C, H, W, L, elem_bytes, best, tune, 4);
     if (ok) deepen_prefetch(best);
     return ok;
 }
-inline bool search_bwd_fused(int B, int C, int H, int W, int L, int elem_bytes, Geom &best, unsigned tune) {
-    if ((tune >> 21) & 1) return false;  // bit 21: never fuse
+inline bool search_bwd_fused(int k, int B, int C, int H, int W, int L, int elem_bytes, Geom &best, unsigned tune) {
+    if (((tune >> 21) & 1) || k == 7) return false;  // bit 21: never fuse; 49 sums, 49 weights and a tile do not fit 128 registers
     best.score = -1.0;
     bool ok = false;
-    if (!((tune >> 23) & 1)) ok |= plan_bwd_fused_th(B, C, H, W, L, elem_bytes, best, tune, 8);
-    if (!((tune >> 22) & 1)) ok |= plan_bwd_fused_th(B, C, H, W, L, elem_bytes, best, tune, 4);
+    if (!((tune >> 23) & 1)) ok |= plan_bwd_fused_th(k, B, C, H, W, L, elem_bytes, best, tune, 8);
+    if (!((tune >> 22) & 1)) ok |= plan_bwd_fused_th(k, B, C, H, W, L, elem_bytes, best, tune, 4);
     if (ok) deepen_prefetch(best);
     return ok;
 }
@@ -1682,10 +1721,10 @@ inline bool search_bwd_fused(int B, int C, int H, int W, int L, int elem_bytes, 
 // The searches above walk a few thousand candidates (tens of microseconds of host time), more than a small
 // layer's kernels take on the GPU, so every entry point looks its plan up in a small process-wide cache first.
 struct PlanKey {
-    int kind, B, C, H, W, L, elem_bytes;
+    int kind, k, B, C, H, W, L, elem_bytes;
     unsigned tune;
     bool operator==(const PlanKey &o) const {
-        return kind == o.kind && B == o.B && C == o.C && H == o.H && W == o.W && L == o.L && elem_bytes == o.elem_bytes &&
+        return kind == o.kind && k == o.k && B == o.B && C == o.C && H == o.H && W == o.W && L == o.L && elem_bytes == o.elem_bytes &&
                tune == o.tune;
     }
 };
@@ -1694,10 +1733,10 @@ struct PlanEntry {
     bool ok;
     Geom g;
 };
-inline bool cached_plan(int kind, int B, int C, int H, int W, int L, int elem_bytes, Geom &best, unsigned tune) {
+inline bool cached_plan(int kind, int k, int B, int C, int H, int W, int L, int elem_bytes, Geom &best, unsigned tune) {
     static std::mutex mu;
     static std::vector<PlanEntry> cache;
-    const PlanKey key = {kind, B, C, H, W, L, elem_bytes, tune};
+    const PlanKey key = {kind, k, B, C, H, W, L, elem_bytes, tune};
     {
         std::lock_guard<std::mutex> lock(mu);
         for (const PlanEntry &e : cache)
@@ -1709,9 +1748,9 @@ inline bool cached_plan(int kind, int B, int C, int H, int W, int L, int elem_by
     PlanEntry e;
     e.key = key;
     e.g = Geom{};
-    e.ok = kind == 0   ? search_forward(B, C, H, W, L, elem_bytes, e.g, tune)
-           : kind == 1 ? search_wgrad(B, C, H, W, L, elem_bytes, e.g, tune)
-                       : search_bwd_fused(B, C, H, W, L, elem_bytes, e.g, tune);
+    e.ok = kind == 0   ? search_forward(k, B, C, H, W, L, elem_bytes, e.g, tune)
+           : kind == 1 ? search_wgrad(k, B, C, H, W, L, elem_bytes, e.g, tune)
+                       : search_bwd_fused(k, B, C, H, W, L, elem_bytes, e.g, tune);
     {
         std::lock_guard<std::mutex> lock(mu);
         if (cache.size() >= 256) cache.clear();  // bounded: a process cycling through more shapes just searches again
@@ -1720,46 +1759,47 @@ inline bool cached_plan(int kind, int B, int C, int H, int W, int L, int elem_by
     if (e.ok) best = e.g;
     return e.ok;
 }
-inline bool plan_forward(int B, int C, int H, int W, int L, int elem_bytes, Geom &best, unsigned tune = 0) {
-    return cached_plan(0, B, C, H, W, L, elem_bytes, best, tune);
+inline bool plan_forward(int B, int C, int H, int W, int L, int elem_bytes, Geom &best, unsigned tune = 0, int k = 5) {
+    return cached_plan(0, k, B, C, H, W, L, elem_bytes, best, tune);
 }
-inline bool plan_wgrad(int B, int C, int H, int W, int L, int elem_bytes, Geom &best, unsigned tune = 0) {
-    return cached_plan(1, B, C, H, W, L, elem_bytes, best, tune);
+inline bool plan_wgrad(int B, int C, int H, int W, int L, int elem_bytes, Geom &best, unsigned tune = 0, int k = 5) {
+    return cached_plan(1, k, B, C, H, W, L, elem_bytes, best, tune);
 }
-inline bool plan_bwd_fused(int B, int C, int H, int W, int L, int elem_bytes, Geom &best, unsigned tune = 0) {
-    return cached_plan(2, B, C, H, W, L, elem_bytes, best, tune);
+inline bool plan_bwd_fused(int B, int C, int H, int W, int L, int elem_bytes, Geom &best, unsigned tune = 0, int k = 5) {
+    return cached_plan(2, k, B, C, H, W, L, elem_bytes, best, tune);
 }
 
 inline int dtype_bytes(int dtype) { return dtype == 0 ? 4 : 2; }
 
 // Human-readable launch plan of a descriptor (threads, blocks per SM, planes per unit, tile rows, ring depth).
-inline void describe(int B, int C, int H, int W, int L, int elem_bytes, unsigned tune, char *buf, size_t n) {
+inline void describe(int B, int C, int H, int W, int L, int elem_bytes, unsigned tune, char *buf, size_t n, int k = 5) {
     Geom f, b;
     int o = 0;
-    if (plan_forward(B, C, H, W, L, elem_bytes, f, tune))
+    if (plan_forward(B, C, H, W, L, elem_bytes, f, tune, k))
         o += snprintf(buf + o, n - o, "plane fwd[T=%d bps=%d npl=%d th=%d ring=%d]", f.nthreads, f.blocks_per_sm, f.NPL, f.th,
                       f.bulk ? f.nstage : 0);
-    if (o < (int)n && plan_bwd_fused(B, C, H, W, L, elem_bytes, b, tune))
+    if (o < (int)n && plan_bwd_fused(B, C, H, W, L, elem_bytes, b, tune, k))
         snprintf(buf + o, n - o, " bwd[fused T=%d bps=%d npl=%d th=%d ring=%d np=%d]", b.nthreads, b.blocks_per_sm, b.NPL, b.th,
                  b.bulk ? b.nstage : 0, b.np);
-    else if (o < (int)n && plan_wgrad(B, C, H, W, L, elem_bytes, b, tune))
+    else if (o < (int)n && plan_wgrad(B, C, H, W, L, elem_bytes, b, tune, k))
         snprintf(buf + o, n - o, " bwd[split wgrad T=%d bps=%d th=%d ring=%d np=%d]", b.nthreads, b.blocks_per_sm, b.th,
                  b.bulk ? b.nstage : 0, b.np);
 }
 
 inline bool supported(int H, int W, int k, int L, int dtype) {
-    if (k != 5) return false;
+    if (k != 5 && k != 7) return false;
     Geom g;
-    return plan_forward(2, 2, H, W, L, dtype_bytes(dtype), g) && plan_wgrad(2, 2, H, W, L, dtype_bytes(dtype), g);
+    return plan_forward(2, 2, H, W, L, dtype_bytes(dtype), g, 0, k) && plan_wgrad(2, 2, H, W, L, dtype_bytes(dtype), g, 0, k);
 }
 
 // Workspace: the status words (256 bytes reserved; see common.cuh), then for backward the base partials
-// [C][np][26] and the level partials [L][C][np][4][25] (float).
+// [C][np][KK+1] and the level partials [L][C][np][4][KK] (float).
 constexpr size_t STATUS_BYTES = 256;
 inline size_t forward_workspace_bytes(int, int, int, int, int) { return STATUS_BYTES; }
-inline size_t backward_workspace_bytes(int B, int C, int H, int W, int L, int elem_bytes, unsigned tune = 0) {
+inline size_t backward_workspace_bytes(int B, int C, int H, int W, int L, int elem_bytes, unsigned tune = 0, int k = 5) {
     Geom g;
-    if (!plan_bwd_fused(B, C, H, W, L, elem_bytes, g, tune) && !plan_wgrad(B, C, H, W, L, elem_bytes, g, tune)) return 0;
+    if (!plan_bwd_fused(B, C, H, W, L, elem_bytes, g, tune, k) && !plan_wgrad(B, C, H, W, L, elem_bytes, g, tune, k)) return 0;
+    const size_t KK = (size_t)k * k;
     return STATUS_BYTES + sizeof(float) * ((size_t)C * g.np * (KK + 1) + (size_t)L * C * g.np * 4 * KK);
 }
 
@@ -1791,7 +1831,8 @@ cudaError_t launch_fwd(const Geom &g, const T *x, const float *w0, const float *
                                    out, status)) != cudaSuccess)                                    \
             return e;                                                                               \
     }
-#define WT_LAUNCH_FWD_TH(MAXT_, MINB_, TH_) { if (g.taps == 3) WT_LAUNCH_FWD_KT(MAXT_, MINB_, TH_, 3) else WT_LAUNCH_FWD_KT(MAXT_, MINB_, TH_, 5) }
+// (7 x 7 kernels: builds of 128 registers only)
+#define WT_LAUNCH_FWD_TH(MAXT_, MINB_, TH_) { if (g.taps == 3) WT_LAUNCH_FWD_KT(MAXT_, MINB_, TH_, 3) else if (g.taps == 7) WT_LAUNCH_FWD_KT(MAXT_, ((MINB_) * (MAXT_) > 512 ? 512 / (MAXT_) : (MINB_)), TH_, 7) else WT_LAUNCH_FWD_KT(MAXT_, MINB_, TH_, 5) }
 #define WT_LAUNCH_FWD(MAXT_, MINB_) { if (g.th == 8) WT_LAUNCH_FWD_TH(MAXT_, MINB_, 8) else WT_LAUNCH_FWD_TH(MAXT_, MINB_, 4) }
     if (g.nthreads <= 128 && g.blocks_per_sm <= 3) {
         WT_LAUNCH_FWD(128, 3)
@@ -1813,7 +1854,8 @@ cudaError_t forward(int B, int C, int H, int W, int L, const T *x, const float *
                     const float *wl, const float *sl, T *out, char *ws, cudaStream_t st, unsigned tag, unsigned tune = 0,
                     bool no_copy = false, int taps = 5) {
     Geom g;
-    if (!plan_forward(B, C, H, W, L, (int)sizeof(T), g, tune)) return cudaErrorInvalidValue;
+    const int k = taps == 7 ? 7 : 5;
+    if (!plan_forward(B, C, H, W, L, (int)sizeof(T), g, tune, k)) return cudaErrorInvalidValue;
     g.no_copy = no_copy;
     g.tag = tag;
     g.alarm = call_alarm;
@@ -1829,7 +1871,8 @@ cudaError_t backward(int B, int C, int H, int W, int L, const T *x, const T *go,
                      unsigned tune = 0, bool no_copy = false, int taps = 5) {
     Geom gw, gf;
     cudaError_t e;
-    if (plan_bwd_fused(B, C, H, W, L, (int)sizeof(T), gw, tune)) {
+    const int k = taps == 7 ? 7 : 5, KK = k * k;
+    if (plan_bwd_fused(B, C, H, W, L, (int)sizeof(T), gw, tune, k)) {
         gw.no_copy = no_copy;
         gw.tag = tag;
         gw.alarm = call_alarm;
@@ -1863,7 +1906,7 @@ cudaError_t backward(int B, int C, int H, int W, int L, const T *x, const T *go,
         ep->grp = gw.NPL; ep->B = B; ep->units = gw.units; ep->nblocks = gw.nblocks;
         return cudaSuccess;
     }
-    if (!plan_wgrad(B, C, H, W, L, (int)sizeof(T), gw, tune) || !plan_forward(B, C, H, W, L, (int)sizeof(T), gf, tune))
+    if (!plan_wgrad(B, C, H, W, L, (int)sizeof(T), gw, tune, k) || !plan_forward(B, C, H, W, L, (int)sizeof(T), gf, tune, k))
         return cudaErrorInvalidValue;
     gw.no_copy = gf.no_copy = no_copy;
     gw.tag = gf.tag = tag;
@@ -1881,7 +1924,7 @@ cudaError_t backward(int B, int C, int H, int W, int L, const T *x, const T *go,
                                    status)) != cudaSuccess)                                        \
             return e;                                                                              \
     }
-#define WT_LAUNCH_WG(MAXT_, MINB_, TH_) { if (taps == 3) WT_LAUNCH_WG_KT(MAXT_, MINB_, TH_, 3) else WT_LAUNCH_WG_KT(MAXT_, MINB_, TH_, 5) }
+#define WT_LAUNCH_WG(MAXT_, MINB_, TH_) { if (taps == 3) WT_LAUNCH_WG_KT(MAXT_, MINB_, TH_, 3) else if (taps == 7) WT_LAUNCH_WG_KT(MAXT_, MINB_, TH_, 7) else WT_LAUNCH_WG_KT(MAXT_, MINB_, TH_, 5) }
     if (gw.nthreads <= 128) {
         if (gw.th == 8) WT_LAUNCH_WG(128, 4, 8) else WT_LAUNCH_WG(128, 4, 4)
     } else {

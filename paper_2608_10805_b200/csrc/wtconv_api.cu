@@ -228,10 +228,10 @@ wtconv_status forward_tk(const wtconv_desc *d, const void *x, const float *w0, c
                        : WTCONV_ERR_CUDA;
     }
     if (use_plane_path(d)) {
-        if constexpr (K == 5)
+        if constexpr (K != 3)
             return wt::plane::forward<T>(d->B, d->C, d->H, d->W, d->L, (const T *)x, w0, s0, b0, wl, sl, (T *)out, ws,
                                          st, next_status_tag(), d->flags >> 8,
-                                         (d->flags & WTCONV_FLAG_TEST_NO_COPY) != 0, taps) == cudaSuccess
+                                         (d->flags & WTCONV_FLAG_TEST_NO_COPY) != 0, K == 7 ? 7 : taps) == cudaSuccess
                        ? WTCONV_OK
                        : WTCONV_ERR_CUDA;
     }
@@ -296,11 +296,11 @@ wtconv_status backward_tk(const wtconv_desc *d, const void *x, const void *g, co
         }
     }
     if (use_plane_path(d)) {
-        if constexpr (K == 5) {
+        if constexpr (K != 3) {
             wt::EpiloguePtrs ep = {};
             if (wt::plane::backward<T>(d->B, d->C, d->H, d->W, d->L, (const T *)x, (const T *)g, w0, s0, wl, sl,
                                        (T *)gx, ws, &ep, st, next_status_tag(), d->flags >> 8,
-                                       (d->flags & WTCONV_FLAG_TEST_NO_COPY) != 0, taps) != cudaSuccess)
+                                       (d->flags & WTCONV_FLAG_TEST_NO_COPY) != 0, K == 7 ? 7 : taps) != cudaSuccess)
                 return WTCONV_ERR_CUDA;
             return launch_epilogue(d, ep, w0, s0, b0, wl, sl, gw0, gs0, gb0, gwl, gsl, st);
         }
@@ -403,7 +403,8 @@ Route find_route(const wtconv_desc *d) {
         // launch-plan overrides other than the planes per unit address the block-per-plane kernels
         if (!(d->flags & WTCONV_FLAG_NO_TEAM) && !((d->flags >> 8) & ~(63u << 8)))
             r.team = wt::team::supported(d->B, d->C, d->H, d->W, d->k, d->L, d->dtype, team_force_g(d));
-        r.plane = r.team || wt::plane::supported(d->H, d->W, d->k, d->L, d->dtype);
+        // (7 x 7 kernels: launch-plan overrides leave them on the per-level kernels, which have no plan to override)
+        r.plane = r.team || (!(d->k == 7 && (d->flags >> 8)) && wt::plane::supported(d->H, d->W, d->k, d->L, d->dtype));
         // Large planes (k = 5): windows with levels 1-2 on chip, deeper levels on the whole-plane kernels over a carrier.
         // Measured on B200: with 16-byte aligned rows the per-level tiled kernels are as fast or faster (they stream whole
         // rows), with unaligned rows (225-wide 16-bit planes) they fall to element loads and the window kernels win.
@@ -423,7 +424,7 @@ Route find_route(const wtconv_desc *d) {
         r.family_bytes[1] = align_up(wt::team::backward_workspace_bytes(d->B, d->C, d->H, d->W, d->L, eb, team_force_g(d)));
     } else if (r.plane) {
         r.family_bytes[0] = align_up(wt::plane::forward_workspace_bytes(d->B, d->C, d->H, d->W, d->L));
-        r.family_bytes[1] = align_up(wt::plane::backward_workspace_bytes(d->B, d->C, d->H, d->W, d->L, eb, d->flags >> 8));
+        r.family_bytes[1] = align_up(wt::plane::backward_workspace_bytes(d->B, d->C, d->H, d->W, d->L, eb, d->flags >> 8, d->k));
     } else if (r.window) {
         const auto p = wt::window::ws_plan(d->B, d->C, d->H, d->W, d->L, eb);
         r.family_bytes[0] = align_up(p.fwd_bytes);
@@ -550,7 +551,7 @@ const char *family_name(const wtconv_desc *d) {
         const wtconv_desc d5 = as_k5(d);
         return family_name(&d5);
     }
-    return use_ref_chain(d) ? "reference-chain" : use_team_path(d) ? "team" : use_plane_path(d) ? "plane" : use_window_path(d) ? "window" : "tiled";
+    return use_ref_chain(d) ? "reference-chain" : use_team_path(d) ? "team" : use_plane_path(d) && d->k != 7 ? "plane" : use_window_path(d) ? "window" : "tiled";
 }
 void describe_family(const wtconv_desc *d, char *buf, size_t n) {
     if (use_k3_embedding(d)) {
@@ -573,7 +574,7 @@ void describe_family(const wtconv_desc *d, char *buf, size_t n) {
                  wf.WH, wf.WW, wf.g.nthreads, wf.g.blocks_per_sm, wf.nbuf, wf.aligned ? "aligned rows" : "unaligned rows", wb.WH, wb.WW,
                  wb.g.nthreads, wb.g.blocks_per_sm, wb.nbuf, wb.g.np, d->L > 2 ? " + whole-plane kernels on the level-2 carrier" : "");
     } else if (use_plane_path(d))
-        wt::plane::describe(d->B, d->C, d->H, d->W, d->L, (int)elem_bytes(d->dtype), d->flags >> 8, buf, n);
+        wt::plane::describe(d->B, d->C, d->H, d->W, d->L, (int)elem_bytes(d->dtype), d->flags >> 8, buf, n, d->k);
     else
         snprintf(buf, n, "tiled fwd[%d launches] bwd[%d launches]", d->L + 1, d->L + 2);
 }
@@ -601,7 +602,7 @@ void family_launches(const wtconv_desc *d, int (&n)[2]) {
         n[0] = 1;
         wt::plane::Geom gq;
         // fused backward + epilogue, or weight-gradient + input-gradient + epilogue (and nothing else on the stream)
-        n[1] = wt::plane::plan_bwd_fused(d->B, d->C, d->H, d->W, d->L, (int)elem_bytes(d->dtype), gq, d->flags >> 8) ? 2 : 3;
+        n[1] = wt::plane::plan_bwd_fused(d->B, d->C, d->H, d->W, d->L, (int)elem_bytes(d->dtype), gq, d->flags >> 8, d->k) ? 2 : 3;
     } else {
         n[0] = d->L + 1;
         n[1] = d->L + 2;
