@@ -137,6 +137,10 @@ __device__ __forceinline__ void worker_sync() {
     __syncwarp();
     asm volatile("bar.sync 1, 256;" ::: "memory");
 }
+template <int NT, int BAR> __device__ __forceinline__ void build_sync() {
+    __syncwarp();
+    asm volatile("bar.sync %0, %1;" ::"n"(BAR), "n"(NT) : "memory");
+}
 __device__ __forceinline__ void issuer_sync() {
     __syncwarp();
     asm volatile("bar.sync 2, 128;" ::: "memory");
@@ -418,10 +422,10 @@ __device__ __forceinline__ float folded_weight(const KGeom &g, int c, int e, boo
 // The B operand: folded weights (already in mis[0..124]) -> M_ab -> parts -> Toeplitz columns.  `parts`: [part][ab][r] rows of
 // 24 16-bit values, q = -6 .. 17, zero outside 0 .. 9, so that eight K entries of a column are four words of a row.
 // mis: [128 folded | 400 M | 528 bias sums | 544 scale, bias | 560 barriers].
-template <typename T>
+template <typename T, int NT = WORKERS, int BAR = 1>  // NT threads that meet at named barrier BAR
 __device__ __forceinline__ void build_table(char *table, char *parts, float *mis, int tid) {
-    worker_sync();
-    for (int e = tid; e < 400; e += WORKERS) {
+    build_sync<NT, BAR>();
+    for (int e = tid; e < 400; e += NT) {
         const int ab = e / 100, rq = e - ab * 100, r = rq / 10, q = rq - r * 10, a = ab >> 1, b = ab & 1;
         float m = 0.f;
 #pragma unroll
@@ -434,7 +438,7 @@ __device__ __forceinline__ void build_table(char *table, char *parts, float *mis
     }
     float scale = 1.f;
     if (std::is_same<T, __half>::value) {  // largest magnitude to [1/2, 1): no part overflows or loses bits to underflow
-        worker_sync();
+        build_sync<NT, BAR>();
         float big = 0.f;
         for (int e = tid & 31; e < 400; e += 32) big = fmaxf(big, fabsf(mis[128 + e]));
 #pragma unroll
@@ -446,14 +450,14 @@ __device__ __forceinline__ void build_table(char *table, char *parts, float *mis
     } else if (tid == 0) {
         mis[544] = 1.f;
     }
-    for (int e = tid; e < 400; e += WORKERS) {
+    for (int e = tid; e < 400; e += NT) {
         const int row = e / 10, q = e - row * 10;
         const float m = mis[128 + e] * scale;
 #pragma unroll
         for (int sp = 0; sp < 3; ++sp) reinterpret_cast<T *>(parts)[(sp * 40 + row) * 24 + 6 + q] = (T)weight_part<T>(m, sp);
     }
-    worker_sync();
-    for (int e = tid; e < TAPS * 2 * NCOL; e += WORKERS) {  // 8 K entries of one column
+    build_sync<NT, BAR>();
+    for (int e = tid; e < TAPS * 2 * NCOL; e += NT) {  // 8 K entries of one column
         const int nn = e % NCOL, rk = e / NCOL, kh = rk & 1, r = rk >> 1, sp = nn >> 4, a = (nn >> 3) & 1, oc = nn & 7;
         const unsigned *p = reinterpret_cast<const unsigned *>(parts + ((sp * 40 + (a * 2 + (oc & 1)) * 10 + r) * 24 + 6 + kh * 8 - 2 * (oc >> 1)) * 2);
         *reinterpret_cast<uint4 *>(table + r * TAP_BYTES + (kh * (NCOL / 8) + (nn >> 3)) * 128 + (nn & 7) * 16) = make_uint4(p[0], p[1], p[2], p[3]);
@@ -489,7 +493,7 @@ __device__ __forceinline__ void store8(T *p, const float *v, int left, int W) {
 // epilogue is short of registers.
 template <typename T>
 __device__ __noinline__ void group_by_taps(const char *window, unsigned row_bytes, const float *M, T *d, int pitch, int rows, int cols, float bias,
-                                           const float *__restrict__ add, int left, int KL) {
+                                           const float *__restrict__ add, int left, int KL, int chunk) {
     const int K = KL & 15, pad = (5 - K) / 2;
     const bool level = KL >= 16;
 #pragma unroll 1
@@ -502,7 +506,7 @@ __device__ __noinline__ void group_by_taps(const char *window, unsigned row_byte
             const int r = rq / 10, q = rq - r * 10, u = r - a - 2, v = q - b - 2, ul = r >> 1, vl = q >> 1, k = q + 2 * (oc >> 1);
             const bool base = u >= pad && u < 5 - pad && v >= pad && v < 5 - pad;
             if (!base && !(level && ul >= pad && ul < 5 - pad && vl >= pad && vl < 5 - pad)) continue;
-            sum = fmaf((float)*reinterpret_cast<const T *>(window + r * row_bytes + (k >> 3) * 128 + (k & 7) * 2), M[(a * 2 + b) * 100 + rq], sum);
+            sum = fmaf((float)*reinterpret_cast<const T *>(window + r * row_bytes + (k >> 3) * chunk + (k & 7) * 2), M[(a * 2 + b) * 100 + rq], sum);
         }
         sum += bias;
         if (add && oc < left) sum = fmaf(0.5f, add[oc >> 1], sum);
@@ -828,7 +832,7 @@ tensor_kernel(const __grid_constant__ KGeom g, const T *__restrict__ x, const T 
                     if (PANEL && g.deep) more = add + (u64)it.plane * (unsigned)(((g.H + 1) >> 1) * g.pitch) + (y >> 1) * g.pitch + (x0 >> 1) + 4 * j;
                     group_by_taps<T>(conv + (unsigned)row2 * row_bytes + j * 128 + img * 16, row_bytes, mis + 128, d, PANEL ? g.tw + 8 : g.W,
                                      g.H - y < 2 ? 1 : 2, PANEL ? 8 : g.W - 8 * j < 8 ? g.W - 8 * j : 8, bias, more, g.W - x0 - 8 * j,
-                                     g.K + (g.L >= 1 ? 16 : 0));
+                                     g.K + (g.L >= 1 ? 16 : 0), 128);
                 }
             }
             plane::fence_async_smem();

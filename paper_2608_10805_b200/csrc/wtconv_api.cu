@@ -7,6 +7,7 @@
 #include "tiled_kernels.cuh"
 #include "plane_kernels.cuh"
 #include "panel_host.cuh"
+#include "pyramid_kernels.cuh"
 #include "team_kernels.cuh"
 #include "window_kernels.cuh"
 #include "tiled_host.cuh"
@@ -29,6 +30,10 @@ WT_TENSOR_INSTANTIATE(__nv_bfloat16, extern)
 WT_WIDE_INSTANTIATE(__half, extern)
 WT_WIDE_INSTANTIATE(__nv_bfloat16, extern)
 }  // namespace tensor
+namespace pyramid {
+WT_PYRAMID_INSTANTIATE(__half, extern)
+WT_PYRAMID_INSTANTIATE(__nv_bfloat16, extern)
+}  // namespace pyramid
 namespace team {
 WT_TEAM_INSTANTIATE(float, extern)
 WT_TEAM_INSTANTIATE(__half, extern)
@@ -118,7 +123,8 @@ struct Route {
     bool set;
     // The FMA family (plane: any that keeps whole planes on chip; k3: 3 x 3 kernels in 5 x 5 tables of that family), and where the
     // tensor cores are taken in its place: wide = column panels, both directions.
-    bool team, plane, window, k3, wide, tensor[2];
+    // pyramid = the block-per-plane kernels of several levels with base convolution and level 1 on the tensor cores.
+    bool team, plane, window, k3, wide, tensor[2], pyramid[2];
     size_t family_bytes[2];  // workspace, forward / backward, of the family
     size_t bytes[2];         // and of what is taken
 };
@@ -131,6 +137,8 @@ bool use_plane_path(const wtconv_desc *d) { return route(d).plane; }
 bool use_window_path(const wtconv_desc *d) { return route(d).window; }
 bool use_wide_path(const wtconv_desc *d) { return route(d).wide; }
 bool use_tensor_path(const wtconv_desc *d, int bwd) { return route(d).tensor[bwd]; }
+bool use_pyramid_path(const wtconv_desc *d, int bwd) { return route(d).pyramid[bwd]; }
+wt::pyramid::Request pyramid_request(const wtconv_desc *d) { return {d->B, d->C, d->H, d->W, d->L, d->k}; }
 wt::tensor::Request tensor_request(const wtconv_desc *d, int bwd) { return {bwd, d->B, d->C, d->H, d->W, d->L, d->k}; }
 // k = 3 through the k = 5 kernels.  A 3 x 3 depthwise kernel is a 5 x 5 kernel with a border of zeros, so wherever the
 // kernels that keep planes on chip (k = 5 only) serve the shape, the parameters are copied into 5 x 5 tables at the
@@ -192,6 +200,12 @@ wtconv_status forward_tk(const wtconv_desc *d, const void *x, const float *w0, c
     if constexpr (K != 7 && sizeof(T) == 2) {
         if (taps == 5 && use_wide_path(d))
             return wt::tensor::wide_forward<T>(tensor_request(d, 0), (const T *)x, w0, s0, b0, wl, sl, (T *)out, ws, st, next_status_tag()) == cudaSuccess
+                       ? WTCONV_OK
+                       : WTCONV_ERR_CUDA;
+        if (taps == 5 && use_pyramid_path(d, 0))
+            return wt::pyramid::run<T, false>(pyramid_request(d), (const T *)x, w0, s0, b0, wl, sl, (T *)out,
+                                              ws + (use_k3_embedding(d) ? embed_layout(d).inner : 0), st, next_status_tag(),
+                                              (d->flags & WTCONV_FLAG_TEST_NO_COPY) != 0) == cudaSuccess
                        ? WTCONV_OK
                        : WTCONV_ERR_CUDA;
         if (taps == 5 && use_tensor_path(d, 0))
@@ -387,6 +401,22 @@ bool wide_serves(const wtconv_desc *d, bool on_chip) {
            panels_win(d, g.cost);
 }
 
+// What the block-per-plane kernels take forward for a 16-bit layer of several levels, fitted like on_chip_us (11 % off).
+double plane_deep_us(const wtconv_desc *d) {
+    const double planes = (double)d->B * d->C * 1e-3, tiles = planes * ((d->W + 3) / 4 * 4) * ((d->H + 3) / 4 * 4) * 1e-3;
+    const bool odd = d->W % 4 != 0;
+    return 7.2 + 2.0 * (d->k == 3) + (3.76 + 1.77 * odd + 0.22 * (d->L > 2)) * tiles + (0.5 + 0.43 * (d->L - 2)) * planes + 0.3 * (d->L - 2);
+}
+// Several levels: taken where the estimate is a tenth below that of the block-per-plane kernels.  Over 220 random shapes that takes
+// 66, which gain 1.20 x (geometric mean; three lose, by less than a tenth); taking all would lose a tenth: units are eight images of
+// a channel, so small batches and few units leave the SMs empty.
+bool pyramid_serves(const wtconv_desc *d, bool on_chip, int bwd) {
+    if (d->dtype == WTCONV_F32 || !on_chip || d->L < 2 || (d->flags & ~WTCONV_FLAG_TEST_NO_COPY)) return false;
+    wt::pyramid::PGeom g;
+    double cost;
+    return !bwd && wt::pyramid::plan(pyramid_request(d), g, cost) && 1.1 * cost < plane_deep_us(d);
+}
+
 Route find_route(const wtconv_desc *d) {
     Route r = {};
     r.key = *d;
@@ -445,6 +475,8 @@ Route find_route(const wtconv_desc *d) {
             // (behind the embedding's tables, where the family keeps its status words too)
             const size_t own = align_up(bwd ? wt::tensor::backward_bytes(tensor_request(d, 1)) : wt::tensor::STATUS_BYTES);
             r.bytes[bwd] = (r.k3 ? embed_layout(d).inner : 0) + own;
+        } else if ((r.pyramid[bwd] = d->k != 7 && pyramid_serves(d, on_chip && !(r.k3 ? r5.team : r.team), bwd))) {
+            r.bytes[bwd] = (r.k3 ? embed_layout(d).inner : 0) + align_up(wt::plane::STATUS_BYTES);
         }
     }
     return r;
@@ -686,7 +718,8 @@ wtconv_status wtconv_plan_describe(const wtconv_desc *d, char *buf, size_t n) {
     if (st != WTCONV_OK) return st;
     if (!buf || n == 0) return WTCONV_ERR_NULL;
     buf[0] = 0;
-    const bool on[2] = {use_wide_path(d) || use_tensor_path(d, 0), use_wide_path(d) || use_tensor_path(d, 1)};
+    const bool pyr[2] = {use_pyramid_path(d, 0), use_pyramid_path(d, 1)};
+    const bool on[2] = {use_wide_path(d) || use_tensor_path(d, 0) || pyr[0], use_wide_path(d) || use_tensor_path(d, 1) || pyr[1]};
     if (!on[0] && !on[1]) {
         describe_family(d, buf, n);
         return WTCONV_OK;
@@ -696,7 +729,8 @@ wtconv_status wtconv_plan_describe(const wtconv_desc *d, char *buf, size_t n) {
         if (on[bwd] && o + 1 < n) {
             buf[o++] = ' ';
             buf[o] = 0;
-            o += (size_t)wt::tensor::describe(tensor_request(d, bwd), buf + o, n - o);
+            o += (size_t)snprintf(buf + o, n - o, "%s", pyr[bwd] ? (bwd ? "bwd" : "fwd") : "");
+            if (o < n) o += (size_t)(pyr[bwd] ? wt::pyramid::describe(pyramid_request(d), buf + o, n - o) : wt::tensor::describe(tensor_request(d, bwd), buf + o, n - o));
         }
     if ((!on[0] || !on[1]) && o < n) {
         o += (size_t)snprintf(buf + o, n - o, "; the other direction: ");
@@ -715,6 +749,8 @@ wtconv_status wtconv_launch_count(const wtconv_desc *d, int32_t *fwd, int32_t *b
             n[dir] = d->L + (dir ? 4 : 2);
         else if (use_wide_path(d) || use_tensor_path(d, dir))
             n[dir] = dir ? 2 : 1;
+        else if (use_pyramid_path(d, dir))
+            n[dir] = dir ? 3 : 1;
     }
     if (fwd) *fwd = n[0];
     if (bwd) *bwd = n[1];

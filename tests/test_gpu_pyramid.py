@@ -1,0 +1,78 @@
+"""Whole planes of several levels on the tensor cores (base convolution, level 1) and FMA units (levels >= 2): against the fp64
+oracle at the edges of their tiles and units, with infinities and NaNs, and with waits that run out."""
+import pytest
+import torch
+
+from helpers import GRAD_NAMES, TOL, rel_err, run_gpu, run_oracle
+from paper_2608_10805_b200 import inputs, wtconv as wt
+
+pytestmark = pytest.mark.gpu
+
+SHAPES = [  # B, C, H, W, k, L
+    (16, 64, 28, 28, 5, 2),    # several operand arrays
+    (13, 64, 30, 26, 5, 3),    # a unit of five images, rows of pairs
+    (24, 149, 29, 31, 5, 4),   # odd rows, a row more than whole blocks of four, several units a block
+    (16, 148, 56, 56, 5, 3),   # one operand array, levels >= 2 a unit ahead
+    (8, 100, 57, 45, 3, 2),    # 3 x 3, one operand array, odd rows
+    (40, 150, 14, 14, 5, 2),   # many units a block
+    (8, 148, 61, 64, 5, 2),    # the widest plane
+    (13, 74, 40, 64, 5, 3),    # planes in batches that do not divide eight
+]
+
+
+def pyramid(B, C, H, W, k, L, dtype, flags=0):
+    return "pyramid" in wt.wtconv_plan_describe(wt.make_desc(B, C, H, W, k, L, wt.DTYPE_NAMES[dtype], flags))
+
+
+@pytest.mark.parametrize("dtype", ["f16", "bf16"])
+@pytest.mark.parametrize("shape", SHAPES, ids=lambda s: "x".join(map(str, s)))
+def test_against_the_oracle(shape, dtype):
+    w = inputs.Workload("pyramid", *shape, dtype, 500 + SHAPES.index(shape))
+    assert pyramid(*shape, dtype)
+    I = inputs.make_inputs(w, bias=SHAPES.index(shape) % 2 == 0)
+    out, grads = run_gpu(w, I)
+    ref, ref_grads = run_oracle(w, I)
+    assert rel_err(out, ref) < TOL[dtype] / 4  # the only extra error is the final rounding: 2^-8 / 2^-11
+    for n in GRAD_NAMES:
+        if ref_grads.get(n) is not None and ref_grads[n].size:
+            # parameter gradients are sums in fp32 of exact products: far inside the storage type's tolerance
+            assert rel_err(grads[n], ref_grads[n]) < (TOL[dtype] / 4 if n == "dx" else 1e-5), n
+
+
+@pytest.mark.parametrize("where", [(0, 0), (27, 27), (13, 8)])
+def test_infinities_reach_their_own_stencil_only(where):
+    """The same elements are non-finite as on the kernels that compute every product on its own."""
+    B, C, H, W, k, L = SHAPES[0]
+    assert pyramid(B, C, H, W, k, L, "bf16")
+    gen = torch.Generator(device="cuda").manual_seed(3)
+    rnd = lambda *s: torch.randn(s, generator=gen, device="cuda")
+    x = rnd(B, C, H, W).to(torch.bfloat16)
+    x[1, 5, where[0], where[1]] = float("inf")
+    x[9, 7, where[0], where[1]] = float("nan")
+    p = [0.1 * rnd(C, k, k), rnd(C), None, 0.1 * rnd(L, C, 4, k, k), rnd(L, C, 4)]
+    res = []
+    for flags in (0, wt.FLAG_NO_WINDOW):
+        d = wt.make_desc(B, C, H, W, k, L, torch.bfloat16, flags)
+        out = torch.empty_like(x)
+        wt.wtconv_forward(d, x, *p, out, wt.alloc_workspace(d))
+        res.append(out)
+    assert torch.equal(torch.isfinite(res[0]), torch.isfinite(res[1]))
+    ok = torch.isfinite(res[0])
+    assert (res[0][ok].float() - res[1][ok].float()).abs().max() <= 2.0 ** -7 * res[1][ok].float().abs().max()
+    assert int((~ok).sum()) > 0
+
+
+def test_waits_that_run_out_are_reported_and_the_next_call_is_clean():
+    B, C, H, W, k, L = SHAPES[0]
+    assert pyramid(B, C, H, W, k, L, "f16", wt.FLAG_TEST_NO_COPY)
+    x = torch.randn(B, C, H, W, device="cuda").half()
+    p = [torch.randn(C, k, k, device="cuda"), torch.randn(C, device="cuda"), None, torch.randn(L, C, 4, k, k, device="cuda"), torch.randn(L, C, 4, device="cuda")]
+    flag = torch.zeros(2, dtype=torch.int32).pin_memory()
+    out = torch.empty_like(x)
+    ws = wt.alloc_workspace(wt.make_desc(B, C, H, W, k, L, torch.float16))
+    for i, flags in enumerate((wt.FLAG_TEST_NO_COPY, 0)):
+        d = wt.make_desc(B, C, H, W, k, L, torch.float16, flags)
+        wt.wtconv_forward(d, x, *p, out, ws)
+        wt.wtconv_read_status(d, ws, flag[i:i + 1])
+    torch.cuda.synchronize()
+    assert flag.tolist() == [1, 0]
