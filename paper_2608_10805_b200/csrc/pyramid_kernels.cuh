@@ -338,7 +338,7 @@ pyramid_kernel(const __grid_constant__ PGeom g, const T *__restrict__ x, const f
     if (tid == 0) {
         *dead = 0;
         for (int i = 0; i < RING; ++i) {
-            plane::mbar_init(acc_full + i, 1);
+            plane::mbar_init(acc_full + i, 2);  // the MMAs, and the issuer for what it has seen of the loaders
             plane::mbar_init(acc_empty + i, 4);
         }
         for (int i = 0; i < MAX_BUFS; ++i) {
@@ -380,11 +380,11 @@ pyramid_kernel(const __grid_constant__ PGeom g, const T *__restrict__ x, const f
         int c = u_begin / g.upc, k = u_begin - c * g.upc, par = 0, buf = 0;
         unsigned job = 0, phase = 0;
         for (int u = u_begin; u < u_end; ++u, next(buf, phase, g.rbufs)) {
-            wait_for(r_full + buf, phase);  // (and so the loaders are done with the unit; their own barrier may be phases ahead)
+            wait_for(r_full + buf, phase);
             plane::bulk_store_wait_read();  // the output image may be written again behind the barrier
             named_sync(BAR_EPI, EPI);
             const float *mc = mis + par * MIS, *R = reinterpret_cast<const float *>(sb + g.r_off) + buf * g.r_floats;
-            const float scale = mc[544], bias = mc[545];
+            float scale = 1.f, bias = 0.f;  // the loaders' (the deep warps may be ahead of them: known once the unit's first MMAs are done)
             for (int t = 0; t < g.T; ++t) {
                 const int row2 = 2 * (16 * t + (m >> 3)), o = fdiv(row2, g.d_period), y = row2 - o * g.period, slot = o * 8 + img, b = k * 8 * g.S + slot;
                 const bool mine = o < g.S && y < g.H && b < g.B, second = y + 1 < g.H;
@@ -397,6 +397,10 @@ pyramid_kernel(const __grid_constant__ PGeom g, const T *__restrict__ x, const f
                     wait_for(acc_full + s, (job / RING) & 1u);
                     __syncwarp();
                     fence_after();
+                    if (t == 0 && j == 0) {
+                        scale = mc[544];
+                        bias = mc[545];
+                    }
                     float a[16], p1[16], p2[16];
                     const unsigned addr = tmem + s * NCOL + ((unsigned)warp << 21);
                     tensor::tmem_ld16(addr, a);
@@ -524,6 +528,7 @@ pyramid_kernel(const __grid_constant__ PGeom g, const T *__restrict__ x, const f
 #pragma unroll
                     for (int r = 0; r < TAPS; ++r) mma(tmem + s * NCOL, ad + (u64)((unsigned)r * (rowb >> 4)), bdesc + (u64)(r * (TAP_BYTES >> 4)), id, r > 0);
                     mma_commit(acc_full + s);
+                    mbar_arrive(acc_full + s);
                 }
                 __syncwarp();
             }

@@ -39,6 +39,27 @@ def test_against_the_oracle(shape, dtype):
             assert rel_err(grads[n], ref_grads[n]) < (TOL[dtype] / 4 if n == "dx" else 1e-5), n
 
 
+@pytest.mark.parametrize("dtype", ["f16", "bf16"])
+@pytest.mark.parametrize("shape", [(8, 592, 48, 48, 5, 3), (28, 608, 16, 16, 5, 4), (8, 444, 56, 56, 5, 3)], ids=lambda s: "x".join(map(str, s)))
+def test_every_unit_another_channel(shape, dtype):
+    """Levels >= 2 run ahead of the loads: a channel's scale and bias are not its neighbours'."""
+    B, C, H, W, k, L = shape
+    assert "direct" in wt.wtconv_plan_describe(wt.make_desc(*shape, wt.DTYPE_NAMES[dtype]))
+    gen = torch.Generator(device="cuda").manual_seed(4)
+    rnd = lambda *s: torch.randn(s, generator=gen, device="cuda")
+    x = rnd(B, C, H, W).to(wt.DTYPE_NAMES[dtype])
+    size = 2.0 ** (torch.arange(C, device="cuda") % 9 - 4)
+    p = [0.1 * rnd(C, k, k) * size[:, None, None], 0.5 + rnd(C).abs(), rnd(C) * size, 0.1 * rnd(L, C, 4, k, k) * size[:, None, None, None], 0.5 + rnd(L, C, 4).abs()]
+    res = []
+    for flags in (0, wt.FLAG_NO_WINDOW):
+        d = wt.make_desc(*shape, wt.DTYPE_NAMES[dtype], flags)
+        out = torch.empty_like(x)
+        wt.wtconv_forward(d, x, *p, out, wt.alloc_workspace(d))
+        res.append(out.float())
+    err, big = (res[0] - res[1]).abs().amax((0, 2, 3)), res[1].abs().amax((0, 2, 3))
+    assert (err <= 2.0 ** (-7 if dtype == "bf16" else -10) * big).all()  # the final rounding on either side
+
+
 @pytest.mark.parametrize("where", [(0, 0), (27, 27), (13, 8)])
 def test_infinities_reach_their_own_stencil_only(where):
     """The same elements are non-finite as on the kernels that compute every product on its own."""
