@@ -2,13 +2,13 @@
 // one contraction on tcgen05 (see tensor_kernels.cuh for the algebra, the operand layout and the weights' three parts), levels
 // >= 2 as fp32 FMA tiles on the low-pass band, both from the same planes in shared memory, by different warps of one block.
 //
-// A unit is 8 S images of one channel.  The roles of a block's 22 warps, each a pipeline stage:
-//   loaders (4)    the unit's planes, global memory -> operand layout (rows of an odd number of pixels are shifted in
+// A unit is 8 S images of one channel.  The roles of a block's 26 warps, each a pipeline stage:
+//   loaders (8)    the unit's planes, global memory -> operand layout (rows of an odd number of pixels are shifted in
 //                  registers), the B operand when the channel changes
-//   deep (8)       the level-2 coefficients from 4 x 4 pixels of the operand array, deeper levels from the low-pass band, their
+//   deep (12)      the level-2 coefficients from 4 x 4 pixels of the operand array, deeper levels from the low-pass band, their
 //                  convolutions (4 x 4 register tiles), Proposition 2 down to one value R per 2 x 2 pixels
 //   issuers (2)    ten MMAs of 128 x 48 x 16 per 32 rows x 8 columns x 8 images
-//   epilogue (8)   accumulators + R / 2 + bias -> global memory
+//   epilogue (4)   accumulators + R / 2 + bias -> global memory
 // With several operand arrays the next units are loaded and their levels >= 2 computed while this one's MMAs and epilogue run; where
 // only one fits (56 x 56 and the like), the deep warps read the next unit from global memory instead.
 //
@@ -98,30 +98,32 @@ __device__ __forceinline__ void load_rows(const PGeom &g, char *arr, const T *__
         }
     }
 }
-// Rows of an odd number of pixels start at any element: aligned 32-bit words, shifted by one pixel where need be.
-template <typename T>
-__device__ __forceinline__ void load_shifted(const PGeom &g, char *arr, const T *__restrict__ x, int c, int k, int warp, int lane) {
+// Rows of an odd number of pixels start at any element: aligned 32-bit words, shifted by one pixel where need be.  P chunks a row, the
+// first begins SHIFT columns to the left of the plane; arr: the plane's first row.  ZERO: images that do not exist are zeros.
+template <typename T, int SHIFT, int WARPS, bool ZERO, typename G>
+__device__ __forceinline__ void load_shifted(const G &g, char *arr, int P, const T *__restrict__ x, int c, int k, int warp, int lane) {
     constexpr int U = 2;
     const int img = lane & 7;
-    const unsigned rowb = (unsigned)g.Pc * CHUNK;
+    const unsigned rowb = (unsigned)P * CHUNK;
     const long long total = (long long)g.B * g.C * g.HW;
     const unsigned *words = reinterpret_cast<const unsigned *>(x);
     const unsigned short *pix = reinterpret_cast<const unsigned short *>(x);
     for (int o = 0; o < g.S; ++o) {
         const int b = (k * g.S + o) * 8 + img;
-        if (b >= g.B) continue;
-        const long long plane = ((long long)b * g.C + c) * g.HW;
-        for (int y0 = warp; y0 < g.H; y0 += U * (LOAD / 32)) {
-            for (int j = lane >> 3; j < g.Pc; j += 4) {
-                const int x0 = 8 * j - 4;
+        const bool there = b < g.B;
+        if (!ZERO && !there) continue;
+        const long long plane = there ? ((long long)b * g.C + c) * g.HW : 0;
+        for (int y0 = warp; y0 < g.H; y0 += U * WARPS) {
+            for (int j = lane >> 3; j < P; j += 4) {
+                const int x0 = 8 * j - SHIFT;
                 unsigned v[U][5];
 #pragma unroll
                 for (int i = 0; i < U; ++i) {
-                    const int y = y0 + i * (LOAD / 32);
+                    const int y = y0 + i * WARPS;
                     const long long e = plane + (long long)y * g.W + x0, w = e >> 1;  // (arithmetic shift: e may be negative)
 #pragma unroll
                     for (int q = 0; q < 5; ++q) v[i][q] = 0u;
-                    if (y < g.H && x0 < g.W) {
+                    if (y < g.H && x0 < g.W && there) {
                         if (w >= 0 && 2 * (w + 5) <= total) {
 #pragma unroll
                             for (int q = 0; q < 5; ++q) v[i][q] = __ldg(words + w + q);
@@ -134,7 +136,7 @@ __device__ __forceinline__ void load_shifted(const PGeom &g, char *arr, const T 
                 }
 #pragma unroll
                 for (int i = 0; i < U; ++i) {
-                    const int y = y0 + i * (LOAD / 32);
+                    const int y = y0 + i * WARPS;
                     if (y >= g.H || x0 >= g.W) continue;
                     const bool odd = (plane + (long long)y * g.W + x0) & 1;
                     unsigned h[4];
@@ -145,16 +147,16 @@ __device__ __forceinline__ void load_shifted(const PGeom &g, char *arr, const T 
                         for (int q = 0; q < 8; ++q)
                             if ((unsigned)(x0 + q) >= (unsigned)g.W) h[q >> 1] &= q & 1 ? 0x0000ffffu : 0xffff0000u;
                     }
-                    *reinterpret_cast<uint4 *>(arr + (unsigned)(o * g.period + 4 + y) * rowb + j * CHUNK + img * 16) = make_uint4(h[0], h[1], h[2], h[3]);
+                    *reinterpret_cast<uint4 *>(arr + (unsigned)(o * g.period + y) * rowb + j * CHUNK + img * 16) = make_uint4(h[0], h[1], h[2], h[3]);
                 }
             }
         }
     }
 }
 // A unit's planes on their way to L2, a line a request: what is left of the loads' latency is L2's.
-template <typename T>
-__device__ __forceinline__ void prefetch_planes(const PGeom &g, const T *__restrict__ x, int c, int k, int warp, int lane) {
-    for (int slot = warp; slot < 8 * g.S; slot += LOAD / 32) {
+template <typename T, int WARPS, typename G>
+__device__ __forceinline__ void prefetch_planes(const G &g, const T *__restrict__ x, int c, int k, int warp, int lane) {
+    for (int slot = warp; slot < 8 * g.S; slot += WARPS) {
         const int b = k * 8 * g.S + slot;
         if (b >= g.B) break;
         const char *p = reinterpret_cast<const char *>(x + ((size_t)b * g.C + c) * g.HW), *end = p + g.HW * 2;
@@ -211,55 +213,68 @@ __device__ __forceinline__ void run_tile(float *dp, const float *wtab, const Til
         if (r < rows) *reinterpret_cast<float4 *>(dp + d.z + r * zp) = make_float4(acc[r][0], acc[r][1], acc[r][2], acc[r][3]);
 }
 // Level-2 coefficients: a task is eight columns of four rows, two blocks of 4 x 4 pixels, either a chunk of the operand array or (rows
-// of whole 16-byte words) straight from global memory.  `y`: where the first block's coefficients go; in0, in1: blocks inside the
-// grid; rows: rows of pixels from here to the end of the plane (the operand array has zeros behind it).  A thread keeps its plane
-// and columns and walks down the rows.
+// of whole 16-byte words) straight from global memory; rows past the plane's H are not read from global memory (the operand array has
+// zeros there).  row: the first of the four.
+template <bool DIRECT>
+__device__ __forceinline__ void load_blocks(uint4 (&w)[4], const char *q, int row_bytes, int row, int H) {
+#pragma unroll
+    for (int h = 0; h < 4; ++h) {
+        if (DIRECT) w[h] = row + h < H ? __ldg(reinterpret_cast<const uint4 *>(q + h * row_bytes)) : make_uint4(0u, 0u, 0u, 0u);
+        else w[h] = *reinterpret_cast<const uint4 *>(q + h * row_bytes);
+    }
+}
+// `y`: where the first block's coefficients go, `sub` floats from subband to subband; in0, in1: blocks inside the grid; returns the
+// sum of their pixels.
+template <typename T>
+__device__ __forceinline__ float analyse_blocks(const uint4 (&w)[4], float *y, int sub, bool in0, bool in1) {
+    float ll[2][4], sum = 0.f;
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        const unsigned av[4] = {w[2 * h].x, w[2 * h].y, w[2 * h].z, w[2 * h].w}, bv[4] = {w[2 * h + 1].x, w[2 * h + 1].y, w[2 * h + 1].z, w[2 * h + 1].w};
+#pragma unroll
+        for (int m = 0; m < 4; ++m) {
+            const float2 t = tensor::unpack16(av[m], T()), u = tensor::unpack16(bv[m], T());
+            ll[h][m] = (t.x + t.y) + (u.x + u.y);
+        }
+    }
+    if (in0) {
+        const Haar4 h = butterfly(ll[0][0], ll[0][1], ll[1][0], ll[1][1]);
+        sum += h.ll;
+        y[0] = h.ll;
+        y[sub] = h.lh;
+        y[2 * sub] = h.hl;
+        y[3 * sub] = h.hh;
+    }
+    if (in1) {
+        const Haar4 h = butterfly(ll[0][2], ll[0][3], ll[1][2], ll[1][3]);
+        sum += h.ll;
+        y[1] = h.ll;
+        y[1 + sub] = h.lh;
+        y[1 + 2 * sub] = h.hl;
+        y[1 + 3 * sub] = h.hh;
+    }
+    return sum;
+}
+// A thread keeps its plane and columns and walks down the rows i0, i0 + di, ... of blocks; p: floats from row to row of coefficients.
 template <typename T, bool DIRECT>
-__device__ __forceinline__ void analyse(const PGeom &g, const char *q, int row_bytes, float *y, bool in0, bool in1, int i0, int di) {
-    const int H2 = g.Hl[2], p = g.pitch[2], sub = g.rowsl[2] * p;
+__device__ __forceinline__ void analyse(int H, int H2, int p, int sub, const char *q, int row_bytes, float *y, bool in0, bool in1, int i0, int di) {
 #pragma unroll 1
     for (int i = i0; i < H2; i += di, q += 4 * di * row_bytes, y += di * p) {
         uint4 w[4];
-#pragma unroll
-        for (int h = 0; h < 4; ++h) {
-            if (DIRECT) w[h] = 4 * i + h < g.H ? __ldg(reinterpret_cast<const uint4 *>(q + h * row_bytes)) : make_uint4(0u, 0u, 0u, 0u);
-            else w[h] = *reinterpret_cast<const uint4 *>(q + h * row_bytes);
-        }
-        float ll[2][4];
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            const unsigned av[4] = {w[2 * h].x, w[2 * h].y, w[2 * h].z, w[2 * h].w}, bv[4] = {w[2 * h + 1].x, w[2 * h + 1].y, w[2 * h + 1].z, w[2 * h + 1].w};
-#pragma unroll
-            for (int m = 0; m < 4; ++m) {
-                const float2 t = tensor::unpack16(av[m], T()), u = tensor::unpack16(bv[m], T());
-                ll[h][m] = (t.x + t.y) + (u.x + u.y);
-            }
-        }
-        if (in0) {
-            const Haar4 h = butterfly(ll[0][0], ll[0][1], ll[1][0], ll[1][1]);
-            y[0] = h.ll;
-            y[sub] = h.lh;
-            y[2 * sub] = h.hl;
-            y[3 * sub] = h.hh;
-        }
-        if (in1) {
-            const Haar4 h = butterfly(ll[0][2], ll[0][3], ll[1][2], ll[1][3]);
-            y[1] = h.ll;
-            y[1 + sub] = h.lh;
-            y[1 + 2 * sub] = h.hl;
-            y[1 + 3 * sub] = h.hh;
-        }
+        load_blocks<DIRECT>(w, q, row_bytes, 4 * i, H);
+        analyse_blocks<T>(w, y, sub, in0, in1);
     }
 }
-// Level l >= 3 from the low-pass band above it (reads past an odd grid meet the zeros around it).
-__device__ __forceinline__ void analyse_deeper(const PGeom &g, float *dp, int l, int nb, int tid) {
-    const int Wl = g.Wl[l], n = (int)g.d_hw[l].d, pp = g.pitch[l - 1], p = g.pitch[l], sub = g.rowsl[l] * p;
+// Level l >= 3 of nb planes from the low-pass band above it (reads past an odd grid meet the zeros around it).  in, out: the first
+// plane's grids, without their borders.
+__device__ __forceinline__ void analyse_deeper(const float *in, int pp, float *out, int p, int sub, int dslot, const FastDiv &d_hw, const FastDiv &d_w, int nb, int tid) {
+    const int Wl = (int)d_w.d, n = (int)d_hw.d;
     for (int e = tid; e < n * nb; e += DEEP) {
-        const int s = fdiv(e, g.d_hw[l]), r = e - s * n, i = fdiv(r, g.d_w[l]), j = r - i * Wl;
-        const float *q = dp + s * g.dslot + g.offY[l - 1] + (2 * i + 2) * pp + 2 * j + 2;
+        const int s = fdiv(e, d_hw), r = e - s * n, i = fdiv(r, d_w), j = r - i * Wl;
+        const float *q = in + s * dslot + 2 * i * pp + 2 * j;
         const float2 a = *reinterpret_cast<const float2 *>(q), b = *reinterpret_cast<const float2 *>(q + pp);
         const Haar4 h = butterfly(a.x, a.y, b.x, b.y);
-        float *y = dp + s * g.dslot + g.offY[l] + (i + 2) * p + j + 2;
+        float *y = out + s * dslot + i * p + j;
         y[0] = h.ll;
         y[sub] = h.lh;
         y[2 * sub] = h.hl;
@@ -315,12 +330,84 @@ __device__ __noinline__ void pixels_by_taps(const T *__restrict__ plane, int H, 
     }
 }
 
+// ------------------------------------------------------------------ the parameters' gradients
+struct Parameters {
+    const float *w0, *s0, *b0, *wl, *sl;
+};
+// Where they go, and the partial sums they come from: slot i of a channel is the i-th block's whose units meet the channel's (see
+// EpiloguePtrs); level l of partl is l * C * np * 4 * K * K floats on.
+struct Gradients {
+    float *w0, *s0, *b0, *wl, *sl;
+    const float *part0, *partl;
+    int np, upc, units, nblocks;
+    float ratio;  // blocks to a unit
+};
+// block_of_unit without a 64-bit division, whose subroutine costs the kernel's other roles registers (8 spilled: 128 x 192 x 28 x 28
+// 137 -> 146 us): a guess in fp32, one off at most, and the exact ranges.
+__device__ __forceinline__ int block_near(const Gradients &d, int v) {
+    const unsigned n = d.nblocks, whole = (unsigned)d.units / n, rest = (unsigned)d.units % n;
+    auto begin = [&](unsigned b) { return (int)(b * whole + b * rest / n); };
+    int b = (int)((float)v * d.ratio);
+    if (b >= d.nblocks) b = d.nblocks - 1;
+    while (b + 1 < d.nblocks && begin(b + 1) <= v) ++b;
+    while (b > 0 && begin(b) > v) --b;
+    return b;
+}
+// What unfold_epilogue_kernel does, class by class, a warp each and a lane a tap (at most 25 and the bias): fixed-order fp64 sums and
+// Eq. 9.  The loaders do it when they have loaded their last unit: it hides behind that unit's other stages, where a launch of its own
+// took 4 - 5 us.
+inline __device__ __noinline__ void unfold_classes(const PGeom &g, const Parameters &p, const Gradients &d, int warp, int warps, int lane) {
+    const int KK = g.K * g.K, classes = 1 + 4 * g.L;
+    for (int e = blockIdx.x * warps + warp; e < g.C * classes; e += gridDim.x * warps) {
+        const int c = e / classes, cls = e - c * classes, l = (cls - 1) >> 2, sub = (cls - 1) & 3;
+        const int n = block_near(d, (c + 1) * d.upc - 1) - block_near(d, c * d.upc) + 1;
+        const float *q, *w, *s;
+        float *to, *ts;
+        int stride = 4 * KK, taps = KK;
+        if (cls == 0) {
+            stride = KK + 1;
+            q = d.part0 + (size_t)c * d.np * stride;
+            w = p.w0 + (size_t)c * KK;
+            s = p.s0 + c;
+            to = d.w0 + (size_t)c * KK;
+            ts = d.s0 + c;
+            if (p.b0) taps = KK + 1;
+        } else {
+            const size_t f = ((size_t)l * g.C + c) * 4 + sub;
+            q = d.partl + (size_t)l * g.C * d.np * stride + ((size_t)c * d.np * 4 + sub) * KK;
+            w = p.wl + f * KK;
+            s = p.sl + f;
+            to = d.wl + f * KK;
+            ts = d.sl + f;
+        }
+        double prod = 0.0;
+        if (lane < taps) {
+            const float wv = lane < KK ? __ldg(w + lane) : __ldg(p.b0 + c), sv = __ldg(s);
+            double acc = 0.0;
+            for (int i0 = 0; i0 < n; i0 += 8) {
+                float v[8];
+#pragma unroll
+                for (int i = 0; i < 8; ++i) v[i] = i0 + i < n ? q[(size_t)(i0 + i) * stride + lane] : 0.f;
+#pragma unroll
+                for (int i = 0; i < 8; ++i) acc += (double)v[i];
+            }
+            *(lane < KK ? to + lane : d.b0 + c) = (float)((double)sv * acc);
+            prod = acc * (double)wv;
+        }
+#pragma unroll
+        for (int o = 16; o; o >>= 1) prod += __shfl_xor_sync(0xffffffffu, prod, o);
+        if (lane == 0) *ts = (float)prod;
+    }
+}
+
 // ------------------------------------------------------------------ the kernel
-// FLIP = false: out = WTConv(x).  FLIP = true: the same on grad_out with rotated kernels and no bias: grad_x.
+// FLIP = false: out = WTConv(x).  FLIP = true: the same on grad_out with rotated kernels and no bias: grad_x, and the parameters'
+// gradients from the sums of the kernel before.
 template <typename T, bool FLIP>
 __global__ void __launch_bounds__(THREADS, 1)
-pyramid_kernel(const __grid_constant__ PGeom g, const T *__restrict__ x, const float *__restrict__ w0, const float *__restrict__ s0,
-               const float *__restrict__ b0, const float *__restrict__ wl, const float *__restrict__ sl, T *__restrict__ out, int *__restrict__ status) {
+pyramid_kernel(const __grid_constant__ PGeom g, const T *__restrict__ x, const __grid_constant__ Parameters prm, const __grid_constant__ Gradients grad,
+               T *__restrict__ out, int *__restrict__ status) {
+    const float *__restrict__ w0 = prm.w0, *__restrict__ s0 = prm.s0, *__restrict__ b0 = prm.b0, *__restrict__ wl = prm.wl, *__restrict__ sl = prm.sl;
     extern __shared__ __align__(128) char sb[];
     const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
     float *mis = reinterpret_cast<float *>(sb + g.misc_off);  // two channels' worth
@@ -365,7 +452,7 @@ pyramid_kernel(const __grid_constant__ PGeom g, const T *__restrict__ x, const f
             raise_timeout(status, g.alarm, g.tag);
         }
     };
-    if (!FLIP) dependents_may_start();
+    dependents_may_start();  // (what follows is another kernel that fills the SMs, or the program's)
     wait_for_predecessor();  // shared and tensor memory only up to here
     if (blockIdx.x == 0 && tid == 0) status[STATUS_LAUNCH] = (int)g.tag;
     const int jobs = g.T * g.n;
@@ -452,6 +539,7 @@ pyramid_kernel(const __grid_constant__ PGeom g, const T *__restrict__ x, const f
         const int dt = tid - EPI;
         float *dp = reinterpret_cast<float *>(sb + g.deep_off), *wtab = reinterpret_cast<float *>(sb + g.wtab_off);
         const Tile own = find_tile(g, dt);
+        const int sub2 = g.rowsl[2] * g.pitch[2];
         // analysis: images fastest where they are neighbours in shared memory, columns where the rows come from global memory
         const int cols = g.direct ? g.W / 8 : g.Pc, combos = g.nb * cols, a_s = g.direct ? dt / cols % g.nb : dt % g.nb,
                   a_j = g.direct ? dt % cols : dt / g.nb % g.Pc, a_i = dt < DEEP / combos * combos ? dt / combos : g.Hl[2];
@@ -480,12 +568,12 @@ pyramid_kernel(const __grid_constant__ PGeom g, const T *__restrict__ x, const f
                 if (g.direct) {
                     const int b = k * 8 * g.S + slot0 + a_s;
                     if (a_s < nb && b < g.B)
-                        analyse<T, true>(g, reinterpret_cast<const char *>(x + ((size_t)b * g.C + c) * g.HW + 4 * a_i * g.W + 8 * a_j), 2 * g.W, y, true,
+                        analyse<T, true>(g.H, g.Hl[2], g.pitch[2], sub2, reinterpret_cast<const char *>(x + ((size_t)b * g.C + c) * g.HW + 4 * a_i * g.W + 8 * a_j), 2 * g.W, y, true,
                                          2 * a_j + 1 < g.Wl[2], a_i, DEEP / combos);
                 } else {
                     const int slot = slot0 + a_s;  // (chunks start four columns to the left)
                     if (a_s < nb)
-                        analyse<T, false>(g, sb + buf * g.a_bytes + ((slot >> 3) * g.period + 4 + 4 * a_i) * (int)rowb + a_j * CHUNK + (slot & 7) * 16, (int)rowb,
+                        analyse<T, false>(g.H, g.Hl[2], g.pitch[2], sub2, sb + buf * g.a_bytes + ((slot >> 3) * g.period + 4 + 4 * a_i) * (int)rowb + a_j * CHUNK + (slot & 7) * 16, (int)rowb,
                                           y - 1, a_j > 0 && 2 * a_j - 1 < g.Wl[2], 2 * a_j < g.Wl[2], a_i, DEEP / combos);
                     __syncwarp();
                     if (lane == 0 && slot0 + nb == 8 * g.S) mbar_arrive(freed + buf);
@@ -493,7 +581,8 @@ pyramid_kernel(const __grid_constant__ PGeom g, const T *__restrict__ x, const f
                 named_sync(BAR_DEEP, DEEP);
 #pragma unroll 1
                 for (int l = 3; l <= g.L; ++l) {
-                    analyse_deeper(g, dp, l, nb, dt);
+                    analyse_deeper(dp + g.offY[l - 1] + 2 * g.pitch[l - 1] + 2, g.pitch[l - 1], dp + g.offY[l] + 2 * g.pitch[l] + 2, g.pitch[l],
+                                   g.rowsl[l] * g.pitch[l], g.dslot, g.d_hw[l], g.d_w[l], nb, dt);
                     named_sync(BAR_DEEP, DEEP);
                 }
 #pragma unroll 1
@@ -561,11 +650,11 @@ pyramid_kernel(const __grid_constant__ PGeom g, const T *__restrict__ x, const f
             if (u + 1 + g.direct < u_end) {  // (the deep warps are a unit ahead where they read global memory)
                 int cp = c, kp = k + 1 + g.direct;
                 while (kp >= g.upc) { kp -= g.upc; ++cp; }
-                prefetch_planes<T>(g, x, cp, kp, lw, lane);
+                prefetch_planes<T, LOAD / 32>(g, x, cp, kp, lw, lane);
             }
             if (g.vec == 4) load_rows<T, 4>(g, arr, x, c, k, lw, lane);
             else if (g.vec == 2) load_rows<T, 2>(g, arr, x, c, k, lw, lane);
-            else load_shifted<T>(g, arr, x, c, k, lw, lane);
+            else load_shifted<T, 4, LOAD / 32, false>(g, arr + 4 * rowb, g.Pc, x, c, k, lw, lane);
             if (change) {  // the MMAs that read the old B operand have completed
                 const int v = u - u_begin, old = v - (g.rbufs > 1 ? 2 : 1);  // the last unit that may use this set of M, scale and bias
                 if (v > 0) wait_for(mma_done, (unsigned)(v - 1) & 1u);
@@ -579,8 +668,9 @@ pyramid_kernel(const __grid_constant__ PGeom g, const T *__restrict__ x, const f
             plane::fence_async_smem();
             mbar_arrive(full + buf);
         }
+        __syncwarp();
+        if (FLIP) unfold_classes(g, prm, grad, lw, LOAD / 32, lane);
     }
-    if (FLIP) dependents_may_start();
     fence_before();
     __syncthreads();
     __syncwarp();
@@ -709,8 +799,7 @@ inline bool plan(const Request &q, PGeom &out, double &cost) {  // searched once
 }
 
 template <typename T, bool FLIP>
-cudaError_t run(const Request &q, const T *x, const float *w0, const float *s0, const float *b0, const float *wl, const float *sl, T *out, char *ws,
-                cudaStream_t st, unsigned tag, bool no_copy) {
+cudaError_t run(const Request &q, const T *x, const Parameters &p, const Gradients &grad, T *out, char *ws, cudaStream_t st, unsigned tag, bool no_copy) {
     PGeom g;
     double cost;
     if (!plan(q, g, cost)) return cudaErrorInvalidValue;
@@ -720,7 +809,7 @@ cudaError_t run(const Request &q, const T *x, const float *w0, const float *s0, 
     constexpr auto kern = pyramid_kernel<T, FLIP>;
     cudaError_t e;
     if ((e = plane::opt_in_smem<kern>()) != cudaSuccess) return e;
-    return launch_overlapped(kern, (unsigned)g.nblocks, (unsigned)THREADS, (size_t)g.smem, st, g, x, w0, s0, b0, wl, sl, out, reinterpret_cast<int *>(ws));
+    return launch_overlapped(kern, (unsigned)g.nblocks, (unsigned)THREADS, (size_t)g.smem, st, g, x, p, grad, out, reinterpret_cast<int *>(ws));
 }
 
 inline int describe(const Request &q, char *buf, size_t n) {
@@ -731,11 +820,9 @@ inline int describe(const Request &q, char *buf, size_t n) {
     return o < 0 ? 0 : o;
 }
 
-#define WT_PYRAMID_INSTANTIATE(T, EXTERN)                                                                                                  \
-    EXTERN template cudaError_t run<T, false>(const Request &, const T *, const float *, const float *, const float *, const float *,     \
-                                              const float *, T *, char *, cudaStream_t, unsigned, bool);                                  \
-    EXTERN template cudaError_t run<T, true>(const Request &, const T *, const float *, const float *, const float *, const float *,      \
-                                             const float *, T *, char *, cudaStream_t, unsigned, bool);
+#define WT_PYRAMID_INSTANTIATE(T, EXTERN)                                                                                                                  \
+    EXTERN template cudaError_t run<T, false>(const Request &, const T *, const Parameters &, const Gradients &, T *, char *, cudaStream_t, unsigned, bool); \
+    EXTERN template cudaError_t run<T, true>(const Request &, const T *, const Parameters &, const Gradients &, T *, char *, cudaStream_t, unsigned, bool);
 
 }  // namespace pyramid
 }  // namespace wt

@@ -7,7 +7,7 @@
 #include "tiled_kernels.cuh"
 #include "plane_kernels.cuh"
 #include "panel_host.cuh"
-#include "pyramid_kernels.cuh"
+#include "pyramid_gradient.cuh"
 #include "team_kernels.cuh"
 #include "window_kernels.cuh"
 #include "tiled_host.cuh"
@@ -33,6 +33,8 @@ WT_WIDE_INSTANTIATE(__nv_bfloat16, extern)
 namespace pyramid {
 WT_PYRAMID_INSTANTIATE(__half, extern)
 WT_PYRAMID_INSTANTIATE(__nv_bfloat16, extern)
+WT_GRADIENT_INSTANTIATE(__half, extern)
+WT_GRADIENT_INSTANTIATE(__nv_bfloat16, extern)
 }  // namespace pyramid
 namespace team {
 WT_TEAM_INSTANTIATE(float, extern)
@@ -203,7 +205,7 @@ wtconv_status forward_tk(const wtconv_desc *d, const void *x, const float *w0, c
                        ? WTCONV_OK
                        : WTCONV_ERR_CUDA;
         if (taps == 5 && use_pyramid_path(d, 0))
-            return wt::pyramid::run<T, false>(pyramid_request(d), (const T *)x, w0, s0, b0, wl, sl, (T *)out,
+            return wt::pyramid::run<T, false>(pyramid_request(d), (const T *)x, {w0, s0, b0, wl, sl}, {}, (T *)out,
                                               ws + (use_k3_embedding(d) ? embed_layout(d).inner : 0), st, next_status_tag(),
                                               (d->flags & WTCONV_FLAG_TEST_NO_COPY) != 0) == cudaSuccess
                        ? WTCONV_OK
@@ -275,6 +277,12 @@ wtconv_status backward_tk(const wtconv_desc *d, const void *x, const void *g, co
                 return WTCONV_ERR_CUDA;
             return launch_epilogue(d, ep, w0, s0, b0, wl, sl, gw0, gs0, gb0, gwl, gsl, st);
         }
+        if (!family && use_pyramid_path(d, 1))
+            return wt::pyramid::backward<T>(pyramid_request(d), (const T *)x, (const T *)g, {w0, s0, b0, wl, sl}, {gw0, gs0, gb0, gwl, gsl}, (T *)gx,
+                                            ws + (use_k3_embedding(d) ? embed_layout(d).inner : 0), st, next_status_tag(),
+                                            (d->flags & WTCONV_FLAG_TEST_NO_COPY) != 0) == cudaSuccess
+                       ? WTCONV_OK
+                       : WTCONV_ERR_CUDA;
     }
     if constexpr (K == 3) {
         if (use_k3_embedding(d)) {
@@ -401,20 +409,26 @@ bool wide_serves(const wtconv_desc *d, bool on_chip) {
            panels_win(d, g.cost);
 }
 
-// What the block-per-plane kernels take forward for a 16-bit layer of several levels, fitted like on_chip_us (11 % off).
-double plane_deep_us(const wtconv_desc *d) {
+// What the block-per-plane kernels take for a 16-bit layer of several levels, fitted like on_chip_us (11 % off forward, 14 % backward).
+double plane_deep_us(const wtconv_desc *d, int bwd) {
     const double planes = (double)d->B * d->C * 1e-3, tiles = planes * ((d->W + 3) / 4 * 4) * ((d->H + 3) / 4 * 4) * 1e-3;
-    const bool odd = d->W % 4 != 0;
-    return 7.2 + 2.0 * (d->k == 3) + (3.76 + 1.77 * odd + 0.22 * (d->L > 2)) * tiles + (0.5 + 0.43 * (d->L - 2)) * planes + 0.3 * (d->L - 2);
+    const bool odd = d->W % 4 != 0, k3 = d->k == 3, big = d->H * d->W > 2200;
+    if (bwd)
+        return 11.1 + 7.5 * k3 + (6.0 + 4.5 * odd + 2.9 * !k3 + 0.1 * (d->L > 2) + 1.4 * big) * tiles + 1.08 * (d->L - 2) * planes + 1.1 * (d->L - 2) +
+               8.0 * (planes < 1 ? planes : 1);
+    return 7.2 + 2.0 * k3 + (3.76 + 1.77 * odd + 0.22 * (d->L > 2)) * tiles + (0.5 + 0.43 * (d->L - 2)) * planes + 0.3 * (d->L - 2);
 }
-// Several levels: taken where the estimate is a tenth below that of the block-per-plane kernels.  Over 220 random shapes that takes
-// 66, which gain 1.20 x (geometric mean; three lose, by less than a tenth); taking all would lose a tenth: units are eight images of
-// a channel, so small batches and few units leave the SMs empty.
+// Several levels: taken where the estimate is a tenth (backward, where the other side's is less certain: 15 %) below that of the
+// block-per-plane kernels.  Over 220 random shapes that takes 66 forward, which gain 1.20 x (geometric mean; three lose, by less than
+// a tenth), and over 250 others 48 backward: 1.38 x, none loses.  Taking all would lose a tenth: units are eight images of a channel,
+// so small batches and few units leave the SMs empty.
 bool pyramid_serves(const wtconv_desc *d, bool on_chip, int bwd) {
     if (d->dtype == WTCONV_F32 || !on_chip || d->L < 2 || (d->flags & ~WTCONV_FLAG_TEST_NO_COPY)) return false;
     wt::pyramid::PGeom g;
+    wt::pyramid::WGeom w;
     double cost;
-    return !bwd && wt::pyramid::plan(pyramid_request(d), g, cost) && 1.1 * cost < plane_deep_us(d);
+    if (bwd) return wt::pyramid::plan_gradient(pyramid_request(d), w, cost) && 1.15 * cost < plane_deep_us(d, 1);
+    return wt::pyramid::plan(pyramid_request(d), g, cost) && 1.1 * cost < plane_deep_us(d, 0);
 }
 
 Route find_route(const wtconv_desc *d) {
@@ -476,7 +490,7 @@ Route find_route(const wtconv_desc *d) {
             const size_t own = align_up(bwd ? wt::tensor::backward_bytes(tensor_request(d, 1)) : wt::tensor::STATUS_BYTES);
             r.bytes[bwd] = (r.k3 ? embed_layout(d).inner : 0) + own;
         } else if ((r.pyramid[bwd] = d->k != 7 && pyramid_serves(d, on_chip && !(r.k3 ? r5.team : r.team), bwd))) {
-            r.bytes[bwd] = (r.k3 ? embed_layout(d).inner : 0) + align_up(wt::plane::STATUS_BYTES);
+            r.bytes[bwd] = (r.k3 ? embed_layout(d).inner : 0) + align_up(bwd ? wt::pyramid::backward_bytes(pyramid_request(d)) : wt::plane::STATUS_BYTES);
         }
     }
     return r;
@@ -730,7 +744,7 @@ wtconv_status wtconv_plan_describe(const wtconv_desc *d, char *buf, size_t n) {
             buf[o++] = ' ';
             buf[o] = 0;
             o += (size_t)snprintf(buf + o, n - o, "%s", pyr[bwd] ? (bwd ? "bwd" : "fwd") : "");
-            if (o < n) o += (size_t)(pyr[bwd] ? wt::pyramid::describe(pyramid_request(d), buf + o, n - o) : wt::tensor::describe(tensor_request(d, bwd), buf + o, n - o));
+            if (o < n) o += (size_t)(pyr[bwd] ? (bwd ? wt::pyramid::describe_backward : wt::pyramid::describe)(pyramid_request(d), buf + o, n - o) : wt::tensor::describe(tensor_request(d, bwd), buf + o, n - o));
         }
     if ((!on[0] || !on[1]) && o < n) {
         o += (size_t)snprintf(buf + o, n - o, "; the other direction: ");
@@ -750,7 +764,7 @@ wtconv_status wtconv_launch_count(const wtconv_desc *d, int32_t *fwd, int32_t *b
         else if (use_wide_path(d) || use_tensor_path(d, dir))
             n[dir] = dir ? 2 : 1;
         else if (use_pyramid_path(d, dir))
-            n[dir] = dir ? 3 : 1;
+            n[dir] = dir ? 2 : 1;
     }
     if (fwd) *fwd = n[0];
     if (bwd) *bwd = n[1];

@@ -39,6 +39,32 @@ def test_against_the_oracle(shape, dtype):
             assert rel_err(grads[n], ref_grads[n]) < (TOL[dtype] / 4 if n == "dx" else 1e-5), n
 
 
+BACKWARD_SHAPES = [  # B, C, H, W, k, L
+    (13, 64, 30, 26, 5, 3),    # a unit of five images, copies of pairs
+    (61, 96, 29, 31, 5, 4),    # odd rows, a last unit that is not full, a row more than whole blocks of four
+    (16, 148, 56, 56, 5, 3),   # one pair of operand arrays, planes in two batches, four-row tiles
+    (40, 148, 57, 45, 5, 2),   # odd rows, one pair of arrays
+    (64, 150, 14, 14, 3, 2),   # 3 x 3, four octets a unit, several channels a block
+    (61, 64, 14, 13, 5, 5),    # levels down to one coefficient, units of four octets
+    (8, 148, 61, 64, 5, 2),    # the widest plane
+    (13, 74, 40, 64, 5, 3),    # rows of whole 16-byte words
+]
+
+
+@pytest.mark.parametrize("dtype", ["f16", "bf16"])
+@pytest.mark.parametrize("shape", BACKWARD_SHAPES, ids=lambda s: "x".join(map(str, s)))
+def test_backward_against_the_oracle(shape, dtype):
+    w = inputs.Workload("pyramid", *shape, dtype, 600 + BACKWARD_SHAPES.index(shape))
+    assert "pyramid gradients" in wt.wtconv_plan_describe(wt.make_desc(*shape, wt.DTYPE_NAMES[dtype]))
+    I = inputs.make_inputs(w, bias=BACKWARD_SHAPES.index(shape) % 2 == 0)
+    _, grads = run_gpu(w, I)
+    _, ref_grads = run_oracle(w, I)
+    for n in GRAD_NAMES:
+        if ref_grads.get(n) is not None and ref_grads[n].size:
+            # as above: grad_x is rounded once, parameter gradients are sums in fp32 of exact products
+            assert rel_err(grads[n], ref_grads[n]) < (TOL[dtype] / 4 if n == "dx" else 1e-5), n
+
+
 @pytest.mark.parametrize("dtype", ["f16", "bf16"])
 @pytest.mark.parametrize("shape", [(8, 592, 48, 48, 5, 3), (28, 608, 16, 16, 5, 4), (8, 444, 56, 56, 5, 3)], ids=lambda s: "x".join(map(str, s)))
 def test_every_unit_another_channel(shape, dtype):
@@ -94,6 +120,22 @@ def test_waits_that_run_out_are_reported_and_the_next_call_is_clean():
     for i, flags in enumerate((wt.FLAG_TEST_NO_COPY, 0)):
         d = wt.make_desc(B, C, H, W, k, L, torch.float16, flags)
         wt.wtconv_forward(d, x, *p, out, ws)
+        wt.wtconv_read_status(d, ws, flag[i:i + 1])
+    torch.cuda.synchronize()
+    assert flag.tolist() == [1, 0]
+
+
+def test_backward_waits_that_run_out_are_reported_and_the_next_call_is_clean():
+    B, C, H, W, k, L = BACKWARD_SHAPES[0]
+    assert "pyramid gradients" in wt.wtconv_plan_describe(wt.make_desc(B, C, H, W, k, L, torch.float16, wt.FLAG_TEST_NO_COPY))
+    x, g = (torch.randn(B, C, H, W, device="cuda").half() for _ in range(2))
+    p = [torch.randn(C, k, k, device="cuda"), torch.randn(C, device="cuda"), None, torch.randn(L, C, 4, k, k, device="cuda"), torch.randn(L, C, 4, device="cuda")]
+    flag = torch.zeros(2, dtype=torch.int32).pin_memory()
+    grads = [torch.empty_like(x)] + [None if q is None else torch.empty_like(q) for q in p]
+    ws = wt.alloc_workspace(wt.make_desc(B, C, H, W, k, L, torch.float16))
+    for i, flags in enumerate((wt.FLAG_TEST_NO_COPY, 0)):
+        d = wt.make_desc(B, C, H, W, k, L, torch.float16, flags)
+        wt.wtconv_backward(d, x, g, *p, *grads, ws)
         wt.wtconv_read_status(d, ws, flag[i:i + 1])
     torch.cuda.synchronize()
     assert flag.tolist() == [1, 0]
