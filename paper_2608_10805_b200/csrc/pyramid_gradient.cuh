@@ -47,30 +47,6 @@ struct WGeom {
     unsigned tag;
 };
 
-// One tensor's rows into the operand layout, PIX pixels a copy; images that do not exist are zeros.  arr: the plane's first row.  A lane
-// walks down the rows of one image (of two): few warps issue all copies of a unit, so the loop is as short as it can be.
-template <int PIX, typename T>
-__device__ __forceinline__ void copy_rows(const WGeom &g, char *arr, int P, int shift, const T *__restrict__ x, int c, int k, int warp, int lane) {
-    const int pieces = g.W / PIX, lp = pieces > 16 ? 5 : pieces > 8 ? 4 : pieces > 4 ? 3 : 2;  // log2 of the lanes to a row
-    const int q = lane & ((1 << lp) - 1), per = (WLOAD / 32) * (32 >> lp), first = warp * (32 >> lp) + (lane >> lp);  // rows under way, this lane's
-    const int col = PIX * q + shift, rowb = P * CHUNK, dy = per >= 8 ? per / 8 : 1, sstep = dy * g.W * 2, dstep = dy * rowb;
-    if (q >= pieces) return;
-    const unsigned to = plane::smem_addr(arr) + (col >> 3) * CHUNK + (col & 7) * 2;
-    for (int o = 0; o < g.S; ++o)
-        for (int img = first & 7; img < 8; img += per) {
-            const int y0 = first >> 3, b = (k * g.S + o) * 8 + img;
-            const int bytes = b < g.B ? 2 * PIX : 0;
-            const char *src = reinterpret_cast<const char *>(b < g.B ? x + ((size_t)b * g.C + c) * g.HW + y0 * g.W + PIX * q : x);
-            const int step = b < g.B ? sstep : 0;
-            unsigned dst = to + (o * g.period + y0) * rowb + img * 16;
-#pragma unroll 4
-            for (int y = y0; y < g.H; y += dy, src += step, dst += dstep) {
-                if (PIX == 8) asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(bytes) : "memory");
-                else asm volatile("cp.async.ca.shared.global [%0], [%1], %2, %3;" ::"r"(dst), "l"(src), "n"(2 * PIX), "r"(bytes) : "memory");
-            }
-        }
-}
-
 template <int TH>
 __device__ __forceinline__ void gradient_tile(const float *D, int pd, const float *Y, int p, float (&acc)[25]) {
     float d[TH][4];
@@ -341,14 +317,14 @@ pyramid_gradient_kernel(const __grid_constant__ WGeom g, const T *__restrict__ x
             if (g.no_copy) break;  // test mode: nothing is copied and nobody is told
             char *xa = sb + buf * (g.x_bytes + g.g_bytes) + 4 * g.Px * CHUNK, *ga = sb + buf * (g.x_bytes + g.g_bytes) + g.x_bytes;
             if (g.W % 8 == 0) {
-                copy_rows<8>(g, ga, g.n, 0, go, c, k, lw, lane);
-                copy_rows<4>(g, xa, g.Px, 4, x, c, k, lw, lane);
+                copy_rows<8, WLOAD / 32>(g, ga, g.n, 0, go, c, k, lw, lane);
+                copy_rows<4, WLOAD / 32>(g, xa, g.Px, 4, x, c, k, lw, lane);
             } else if (g.W % 4 == 0) {
-                copy_rows<4>(g, ga, g.n, 0, go, c, k, lw, lane);
-                copy_rows<4>(g, xa, g.Px, 4, x, c, k, lw, lane);
+                copy_rows<4, WLOAD / 32>(g, ga, g.n, 0, go, c, k, lw, lane);
+                copy_rows<4, WLOAD / 32>(g, xa, g.Px, 4, x, c, k, lw, lane);
             } else if (g.W % 2 == 0) {
-                copy_rows<2>(g, ga, g.n, 0, go, c, k, lw, lane);
-                copy_rows<2>(g, xa, g.Px, 4, x, c, k, lw, lane);
+                copy_rows<2, WLOAD / 32>(g, ga, g.n, 0, go, c, k, lw, lane);
+                copy_rows<2, WLOAD / 32>(g, xa, g.Px, 4, x, c, k, lw, lane);
             } else {
                 load_shifted<T, 0, WLOAD / 32, true>(g, ga, g.n, go, c, k, lw, lane);
                 load_shifted<T, 4, WLOAD / 32, true>(g, xa, g.Px, x, c, k, lw, lane);

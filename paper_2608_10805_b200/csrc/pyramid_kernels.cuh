@@ -2,8 +2,8 @@
 // one contraction on tcgen05 (see tensor_kernels.cuh for the algebra, the operand layout and the weights' three parts), levels
 // >= 2 as fp32 FMA tiles on the low-pass band, both from the same planes in shared memory, by different warps of one block.
 //
-// A unit is 8 S images of one channel.  The roles of a block's 26 warps, each a pipeline stage:
-//   loaders (8)    the unit's planes, global memory -> operand layout (rows of an odd number of pixels are shifted in
+// A unit is 8 S images of one channel.  The roles of a block's 26 (22) warps, each a pipeline stage:
+//   loaders (8, 4) the unit's planes, global memory -> operand layout (rows of an odd number of pixels are shifted in
 //                  registers), the B operand when the channel changes
 //   deep (12)      the level-2 coefficients from 4 x 4 pixels of the operand array, deeper levels from the low-pass band, their
 //                  convolutions (4 x 4 register tiles), Proposition 2 down to one value R per 2 x 2 pixels
@@ -37,7 +37,8 @@ using tensor::TAP_BYTES;
 using tensor::TAPS;
 using tensor::u64;
 
-constexpr int EPI = 128, DEEP = 384, ISS = 2, LOAD = 256, THREADS = EPI + DEEP + 32 * ISS + LOAD;
+constexpr int EPI = 128, DEEP = 384, ISS = 2, OTHERS = EPI + DEEP + 32 * ISS;  // threads and (ISS) warps of the roles but the loaders
+constexpr int LOAD = 256, FEW = 128;  // loaders: through registers, or issuing asynchronous copies
 constexpr int RING = 8, MAXL = 8, MAX_BUFS = 4, WS = plane::WT_STRIDE;
 constexpr int BAR_DEEP = 3, BAR_LOAD = 4, BAR_EPI = 5;  // named barriers
 constexpr int CHUNK = 144;                 // bytes from one chunk of eight images to the next: one image's chunks fall on different banks
@@ -98,6 +99,30 @@ __device__ __forceinline__ void load_rows(const PGeom &g, char *arr, const T *__
         }
     }
 }
+// One tensor's rows into the operand layout, PIX pixels a copy; images that do not exist are zeros.  arr: the plane's first row.  A lane
+// walks down the rows of one image (of two): few warps issue all copies of a unit, so the loop is as short as it can be.
+template <int PIX, int WARPS, typename T, typename G>
+__device__ __forceinline__ void copy_rows(const G &g, char *arr, int P, int shift, const T *__restrict__ x, int c, int k, int warp, int lane) {
+    const int pieces = g.W / PIX, lp = pieces > 16 ? 5 : pieces > 8 ? 4 : pieces > 4 ? 3 : 2;  // log2 of the lanes to a row
+    const int q = lane & ((1 << lp) - 1), per = WARPS * (32 >> lp), first = warp * (32 >> lp) + (lane >> lp);  // rows under way, this lane's
+    const int col = PIX * q + shift, rowb = P * CHUNK, dy = per >= 8 ? per / 8 : 1, sstep = dy * g.W * 2, dstep = dy * rowb;
+    if (q >= pieces) return;
+    const unsigned to = plane::smem_addr(arr) + (col >> 3) * CHUNK + (col & 7) * 2;
+    for (int o = 0; o < g.S; ++o)
+        for (int img = first & 7; img < 8; img += per) {
+            const int y0 = first >> 3, b = (k * g.S + o) * 8 + img;
+            const int bytes = b < g.B ? 2 * PIX : 0;
+            const char *src = reinterpret_cast<const char *>(b < g.B ? x + ((size_t)b * g.C + c) * g.HW + y0 * g.W + PIX * q : x);
+            const int step = b < g.B ? sstep : 0;
+            unsigned dst = to + (o * g.period + y0) * rowb + img * 16;
+#pragma unroll 4
+            for (int y = y0; y < g.H; y += dy, src += step, dst += dstep) {
+                if (PIX == 8) asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(bytes) : "memory");
+                else asm volatile("cp.async.ca.shared.global [%0], [%1], %2, %3;" ::"r"(dst), "l"(src), "n"(2 * PIX), "r"(bytes) : "memory");
+            }
+        }
+}
+
 // Rows of an odd number of pixels start at any element: aligned 32-bit words, shifted by one pixel where need be.  P chunks a row, the
 // first begins SHIFT columns to the left of the plane; arr: the plane's first row.  ZERO: images that do not exist are zeros.
 template <typename T, int SHIFT, int WARPS, bool ZERO, typename G>
@@ -403,11 +428,12 @@ inline __device__ __noinline__ void unfold_classes(const PGeom &g, const Paramet
 // ------------------------------------------------------------------ the kernel
 // FLIP = false: out = WTConv(x).  FLIP = true: the same on grad_out with rotated kernels and no bias: grad_x, and the parameters'
 // gradients from the sums of the kernel before.
-template <typename T, bool FLIP>
-__global__ void __launch_bounds__(THREADS, 1)
+template <typename T, bool FLIP, int LOAD>
+__global__ void __launch_bounds__(OTHERS + LOAD, 1)
 pyramid_kernel(const __grid_constant__ PGeom g, const T *__restrict__ x, const __grid_constant__ Parameters prm, const __grid_constant__ Gradients grad,
                T *__restrict__ out, int *__restrict__ status) {
     const float *__restrict__ w0 = prm.w0, *__restrict__ s0 = prm.s0, *__restrict__ b0 = prm.b0, *__restrict__ wl = prm.wl, *__restrict__ sl = prm.sl;
+    constexpr int THREADS = OTHERS + LOAD;
     extern __shared__ __align__(128) char sb[];
     const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
     float *mis = reinterpret_cast<float *>(sb + g.misc_off);  // two channels' worth
@@ -652,9 +678,12 @@ pyramid_kernel(const __grid_constant__ PGeom g, const T *__restrict__ x, const _
                 while (kp >= g.upc) { kp -= g.upc; ++cp; }
                 prefetch_planes<T, LOAD / 32>(g, x, cp, kp, lw, lane);
             }
-            if (g.vec == 4) load_rows<T, 4>(g, arr, x, c, k, lw, lane);
+            if (LOAD == FEW && g.vec == 4) copy_rows<4, LOAD / 32>(g, arr + 4 * rowb, g.Pc, 4, x, c, k, lw, lane);
+            else if (LOAD == FEW) copy_rows<2, LOAD / 32>(g, arr + 4 * rowb, g.Pc, 4, x, c, k, lw, lane);
+            else if (g.vec == 4) load_rows<T, 4>(g, arr, x, c, k, lw, lane);
             else if (g.vec == 2) load_rows<T, 2>(g, arr, x, c, k, lw, lane);
             else load_shifted<T, 4, LOAD / 32, false>(g, arr + 4 * rowb, g.Pc, x, c, k, lw, lane);
+            if (LOAD == FEW) asm volatile("cp.async.wait_all;" ::: "memory");
             if (change) {  // the MMAs that read the old B operand have completed
                 const int v = u - u_begin, old = v - (g.rbufs > 1 ? 2 : 1);  // the last unit that may use this set of M, scale and bias
                 if (v > 0) wait_for(mma_done, (unsigned)(v - 1) & 1u);
@@ -806,10 +835,14 @@ cudaError_t run(const Request &q, const T *x, const Parameters &p, const Gradien
     g.tag = tag;
     g.alarm = call_alarm;
     g.no_copy = no_copy;
-    constexpr auto kern = pyramid_kernel<T, FLIP>;
-    cudaError_t e;
-    if ((e = plane::opt_in_smem<kern>()) != cudaSuccess) return e;
-    return launch_overlapped(kern, (unsigned)g.nblocks, (unsigned)THREADS, (size_t)g.smem, st, g, x, p, grad, out, reinterpret_cast<int *>(ws));
+    // Four warps that issue asynchronous copies leave the other roles 16 more registers a thread (88), but are slower than eight that load through
+    // registers where units are small: forward, 128 x 96 x 56 x 56 (3136 pixels an image and octet) 126 -> 121 us, 128 x 192 x 28 x 28
+    // (1568) 68.2 -> 62.9; 64 x 192 x 28 x 28 with four levels (784) 48.0 -> 49.3, 16 x 64 x 14 x 14 8.9 -> 9.5.
+    constexpr auto few = pyramid_kernel<T, FLIP, FEW>, many = pyramid_kernel<T, FLIP, LOAD>;
+    const bool copies = g.vec > 1 && g.S * g.HW >= 1500;
+    const cudaError_t e = copies ? plane::opt_in_smem<few>() : plane::opt_in_smem<many>();
+    if (e != cudaSuccess) return e;
+    return launch_overlapped(copies ? few : many, (unsigned)g.nblocks, (unsigned)(OTHERS + (copies ? FEW : LOAD)), (size_t)g.smem, st, g, x, p, grad, out, reinterpret_cast<int *>(ws));
 }
 
 inline int describe(const Request &q, char *buf, size_t n) {
