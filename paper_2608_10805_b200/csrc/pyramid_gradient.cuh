@@ -10,8 +10,8 @@
 //   issuers (2)    one half of the window each: an MMA of 128 x 64 x 16 per 16 rows x 8 columns x 8 images
 //   loaders (4)    asynchronous copies of both tensors' rows into the operand layout (rows of an odd number of pixels are shifted in
 //                  registers)
-// Measured with grad_x, bf16, against the block-per-plane kernels: 128 x 96 x 56 x 56, three levels, 376 -> 245 us; 128 x 192 x 28 x 28,
-// two levels, 229 -> 139; 64 x 192 x 28 x 28, four levels, 145 -> 95.  What bounds it now, by time stamps of the roles: where one pair
+// Measured with grad_x, bf16, against the block-per-plane kernels: 128 x 96 x 56 x 56, three levels, 376 -> 240 us; 128 x 192 x 28 x 28,
+// two levels, 229 -> 132; 64 x 192 x 28 x 28, four levels, 145 -> 95.  What bounds it now, by time stamps of the roles: where one pair
 // of arrays fills an SM (56 x 56) a unit's copies (5300 of 18600 cycles, 16 a copy instruction), its two analyses (4400 and 2900) and
 // the first batch's tiles (2700) follow one another; with several pairs (28 x 28) the deep warps' passes do (two of 4500 cycles).
 // Eight loader warps instead of four left 72 registers a thread: 254 -> 272 us.  One launch for this and grad_x's kernel, block by
@@ -39,6 +39,7 @@ struct WGeom {
     int rowsd[MAXL + 1], pitchd[MAXL + 1], offD[MAXL + 1], tiles[MAXL + 1];                          // grad_out, no borders
     int tpc[MAXL + 1], cls0[MAXL + 1];  // threads to a class of a level, the level's first thread
     int th;                             // rows of a tile: four, or two where that leaves most threads idle
+    int turns;                          // tiles a thread
     int taps;                           // taps flushed at a time
     int deep_off, scr_off, misc_off, zero_end, smem;
     int nblocks, np, no_copy;
@@ -342,12 +343,15 @@ pyramid_gradient_kernel(const __grid_constant__ WGeom g, const T *__restrict__ x
 }
 
 // ------------------------------------------------------------------ host side
+inline int trips(const WGeom &g) { return g.W % 2 ? g.S * ((g.H + 7) / 8) * ((g.n + 3) / 4 + (g.Px + 3) / 4) : 0; }  // a loader's, of shifted rows
+// Microseconds of a backward call, fitted to the same shapes as the forward's (7 % off).
+inline double estimate(const WGeom &g, double grad_x) {
+    const int rounds = (g.units + g.nblocks - 1) / g.nblocks, changes = (rounds + g.upc - 1) / g.upc, passes = (8 * g.S + g.nb - 1) / g.nb;
+    return 3.8 + 1.115 * grad_x + rounds * (1.24 + 0.317 * trips(g) + passes * (1.44 + 0.108 * (g.L - 2) + 0.45 * g.turns * g.th)) + 1.5 * changes;
+}
 inline bool search_gradient(const Request &q, WGeom &best, double &best_cost) {
     using tensor::up;
     if ((q.K != 3 && q.K != 5) || q.L < 2 || q.L > MAXL || q.H < 4 || q.W < 4 || q.W > 64 || q.H > 128) return false;
-    PGeom flip;
-    double flip_cost;
-    if (!plan(q, flip, flip_cost)) return false;
     WGeom g = {};
     g.B = q.B; g.C = q.C; g.H = q.H; g.W = q.W; g.HW = q.H * q.W; g.L = q.L; g.K = q.K;
     g.n = (q.W + 7) / 8;
@@ -411,16 +415,16 @@ inline bool search_gradient(const Request &q, WGeom &best, double &best_cost) {
                     if (used <= DEEP || turns >= 4096) break;
                 }
                 if (used > DEEP) continue;
+                h.turns = turns;
                 h.upc = (q.B + 8 * S - 1) / (8 * S);
                 if ((long long)h.upc * q.C > 0x3fffffffLL) continue;
                 h.units = h.upc * q.C;
                 h.nblocks = plane::NUM_SMS < h.units ? plane::NUM_SMS : h.units;
-                // Microseconds with grad_x's kernel, fitted to 319 shapes between 1 x 16 x 8 x 8 and 128 x 768 x 70 x 64 (7 % off): the deep
-                // warps' passes and tiles and the shifted rows' round trips of each round of units, the sums of each channel
+                // What the candidates are compared by: the deep warps' passes and tiles and the shifted rows' round trips of each round of
+                // units, the sums of each channel
                 const int rounds = (h.units + h.nblocks - 1) / h.nblocks, changes = (rounds + h.upc - 1) / h.upc, passes = (8 * S + nb - 1) / nb;
-                const int trips = q.W % 2 ? S * ((q.H + 7) / 8) * ((h.n + 3) / 4 + (h.Px + 3) / 4) : 0;
-                const double per = 0.65 + 0.39 * trips + passes * (0.46 + 0.08 * (q.L - 2) + 0.515 * turns * h.th);
-                const double cost = 8.0 + 1.2 * flip_cost + rounds * per + 1.7 * changes;
+                const double per = 0.65 + 0.39 * trips(h) + passes * (0.46 + 0.08 * (q.L - 2) + 0.515 * turns * h.th);
+                const double cost = rounds * per + 1.7 * changes;
                 if (!found || cost < best_cost) {
                     best = h;
                     best_cost = cost;
@@ -456,7 +460,10 @@ inline bool plan_gradient(const Request &q, WGeom &out, double &cost) {  // sear
     }
     GradientEntry e = {};
     e.q = q;
-    e.ok = search_gradient(q, e.g, e.cost);
+    PGeom flip;
+    double grad_x;
+    e.ok = plan(q, flip, grad_x) && search_gradient(q, e.g, e.cost);
+    if (e.ok) e.cost = estimate(e.g, grad_x);
     {
         std::lock_guard<std::mutex> lock(mu);
         if (cache.size() >= 256) cache.clear();

@@ -12,8 +12,8 @@
 // With several operand arrays the next units are loaded and their levels >= 2 computed while this one's MMAs and epilogue run; where
 // only one fits (56 x 56 and the like), the deep warps read the next unit from global memory instead.
 //
-// Measured forward against the block-per-plane kernels, bf16: 128 x 96 x 56 x 56, three levels, 188 -> 125 us; 128 x 192 x 28 x 28,
-// two levels, 107 -> 70; 64 x 384 x 14 x 14, three levels, 58 -> 52; 64 x 96 x 30 x 30 46 -> 30, 64 x 96 x 57 x 55 143 -> 113.  What
+// Measured forward against the block-per-plane kernels, bf16: 128 x 96 x 56 x 56, three levels, 188 -> 121 us; 128 x 192 x 28 x 28,
+// two levels, 107 -> 63; 64 x 384 x 14 x 14, three levels, 58 -> 52; 64 x 96 x 30 x 30 46 -> 30, 64 x 96 x 57 x 55 143 -> 113.  What
 // bounds it now is instruction issue (2.1 of 4 a cycle, most warps waiting for their own last instruction) beside shared memory,
 // whose cycles the MMAs' A operand takes a third of.
 #pragma once
@@ -712,6 +712,14 @@ struct Request {
     bool operator==(const Request &o) const { return B == o.B && C == o.C && H == o.H && W == o.W && L == o.L && K == o.K; }
 };
 
+inline bool copied(const PGeom &g) { return g.vec > 1 && g.S * g.HW >= 1500; }
+// Microseconds of a plan, fitted to 390 shapes between 1 x 16 x 8 x 8 and 128 x 768 x 70 x 64 (7 % off): MMA jobs, tiles (dearer where
+// nothing overlaps them or the loaders take the registers), passes and shifted rows of each round of units, a B operand a channel.
+inline double estimate(const PGeom &g) {
+    const int rounds = (g.units + g.nblocks - 1) / g.nblocks, changes = (rounds + g.upc - 1) / g.upc, passes = (8 * g.S + g.nb - 1) / g.nb;
+    const double tile = 0.0333 + (g.bufs == 1 && !g.direct ? 0.0316 : 0) + (copied(g) ? 0 : 0.0126), shift = g.vec == 1 ? 0.0014 : g.vec == 2 ? 0.00038 : 0;
+    return 6.0 + rounds * (0.225 + 0.39 * g.T * g.n + tile * g.S * g.items + 0.2 * passes * (g.L + 1) + shift * g.S * g.HW) + 0.85 * changes;
+}
 inline bool search(const Request &q, PGeom &best, double &best_cost) {
     using tensor::up;
     if ((q.K != 3 && q.K != 5) || q.L < 2 || q.L > MAXL || q.H < 4 || q.W < 4 || q.W > 64 || q.H > 128) return false;
@@ -779,8 +787,8 @@ inline bool search(const Request &q, PGeom &best, double &best_cost) {
                 if ((long long)h.upc * q.C > 0x3fffffffLL) continue;
                 h.units = h.upc * q.C;
                 h.nblocks = plane::NUM_SMS < h.units ? plane::NUM_SMS : h.units;
-                // Microseconds, fitted to 220 shapes between 1 x 16 x 9 x 9 and 128 x 768 x 64 x 64 (9 % off): tiles, blocks of the
-                // analysis, the deep warps' barriers and shifted rows of each round of units, a B operand a channel
+                // What the candidates are compared by: tiles, blocks of the analysis, the deep warps' barriers and shifted rows of each round
+                // of units, a B operand a channel
                 const int rounds = (h.units + h.nblocks - 1) / h.nblocks, changes = (rounds + h.upc - 1) / h.upc, passes = (8 * S + nb - 1) / nb;
                 const double blocks = 8.0 * S * ((q.H + 3) / 4) * h.Pc, odd = h.vec == 4 ? 0 : S * q.H * q.W / 8.0;
                 const double per = 0.0003 * h.T * h.n + (0.067 + (h.bufs == 1 && !h.direct ? 0.018 : 0)) * S * h.items + 0.0053 * blocks +
@@ -818,6 +826,7 @@ inline bool plan(const Request &q, PGeom &out, double &cost) {  // searched once
     Entry e = {};
     e.q = q;
     e.ok = search(q, e.g, e.cost);
+    if (e.ok) e.cost = estimate(e.g);
     {
         std::lock_guard<std::mutex> lock(mu);
         if (cache.size() >= 256) cache.clear();
@@ -839,7 +848,7 @@ cudaError_t run(const Request &q, const T *x, const Parameters &p, const Gradien
     // registers where units are small: forward, 128 x 96 x 56 x 56 (3136 pixels an image and octet) 126 -> 121 us, 128 x 192 x 28 x 28
     // (1568) 68.2 -> 62.9; 64 x 192 x 28 x 28 with four levels (784) 48.0 -> 49.3, 16 x 64 x 14 x 14 8.9 -> 9.5.
     constexpr auto few = pyramid_kernel<T, FLIP, FEW>, many = pyramid_kernel<T, FLIP, LOAD>;
-    const bool copies = g.vec > 1 && g.S * g.HW >= 1500;
+    const bool copies = copied(g);
     const cudaError_t e = copies ? plane::opt_in_smem<few>() : plane::opt_in_smem<many>();
     if (e != cudaSuccess) return e;
     return launch_overlapped(copies ? few : many, (unsigned)g.nblocks, (unsigned)(OTHERS + (copies ? FEW : LOAD)), (size_t)g.smem, st, g, x, p, grad, out, reinterpret_cast<int *>(ws));

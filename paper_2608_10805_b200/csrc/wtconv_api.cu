@@ -409,26 +409,25 @@ bool wide_serves(const wtconv_desc *d, bool on_chip) {
            panels_win(d, g.cost);
 }
 
-// What the block-per-plane kernels take for a 16-bit layer of several levels, fitted like on_chip_us (11 % off forward, 14 % backward).
+// What the block-per-plane kernels take for a 16-bit layer of several levels, fitted like on_chip_us (10 % off forward, 14 % backward).
 double plane_deep_us(const wtconv_desc *d, int bwd) {
     const double planes = (double)d->B * d->C * 1e-3, tiles = planes * ((d->W + 3) / 4 * 4) * ((d->H + 3) / 4 * 4) * 1e-3;
     const bool odd = d->W % 4 != 0, k3 = d->k == 3, big = d->H * d->W > 2200;
     if (bwd)
         return 11.1 + 7.5 * k3 + (6.0 + 4.5 * odd + 2.9 * !k3 + 0.1 * (d->L > 2) + 1.4 * big) * tiles + 1.08 * (d->L - 2) * planes + 1.1 * (d->L - 2) +
                8.0 * (planes < 1 ? planes : 1);
-    return 7.2 + 2.0 * k3 + (3.76 + 1.77 * odd + 0.22 * (d->L > 2)) * tiles + (0.5 + 0.43 * (d->L - 2)) * planes + 0.3 * (d->L - 2);
+    return 7.3 + 3.0 * k3 + (2.55 + 1.59 * odd + 1.05 * !k3 + 0.42 * (d->L > 2) + 0.43 * big) * tiles + (0.75 + 0.35 * (d->L - 2)) * planes + 0.5 * (d->L - 2);
 }
-// Several levels: taken where the estimate is a tenth (backward, where the other side's is less certain: 15 %) below that of the
-// block-per-plane kernels.  Over 220 random shapes that takes 66 forward, which gain 1.20 x (geometric mean; three lose, by less than
-// a tenth), and over 250 others 48 backward: 1.38 x, none loses.  Taking all would lose a tenth: units are eight images of a channel,
-// so small batches and few units leave the SMs empty.
+// Several levels: taken where the estimate is 15 % (backward 20 %) below that of the block-per-plane kernels.  Over 390 random shapes
+// that takes 91 forward, which gain 1.26 x (geometric mean; four lose more than 2 %), and 89 backward: 1.45 x, none loses.  Taking all
+// would lose a tenth: units are eight images of a channel, so small batches and few units leave the SMs empty.
 bool pyramid_serves(const wtconv_desc *d, bool on_chip, int bwd) {
     if (d->dtype == WTCONV_F32 || !on_chip || d->L < 2 || (d->flags & ~WTCONV_FLAG_TEST_NO_COPY)) return false;
     wt::pyramid::PGeom g;
     wt::pyramid::WGeom w;
     double cost;
-    if (bwd) return wt::pyramid::plan_gradient(pyramid_request(d), w, cost) && 1.15 * cost < plane_deep_us(d, 1);
-    return wt::pyramid::plan(pyramid_request(d), g, cost) && 1.1 * cost < plane_deep_us(d, 0);
+    if (bwd) return wt::pyramid::plan_gradient(pyramid_request(d), w, cost) && 1.2 * cost < plane_deep_us(d, 1);
+    return wt::pyramid::plan(pyramid_request(d), g, cost) && 1.15 * cost < plane_deep_us(d, 0);
 }
 
 Route find_route(const wtconv_desc *d) {

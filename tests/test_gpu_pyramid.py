@@ -9,12 +9,12 @@ from paper_2608_10805_b200 import inputs, wtconv as wt
 pytestmark = pytest.mark.gpu
 
 SHAPES = [  # B, C, H, W, k, L
-    (16, 64, 28, 28, 5, 2),    # several operand arrays
+    (32, 148, 28, 28, 5, 2),   # several operand arrays
     (13, 64, 30, 26, 5, 3),    # a unit of five images, rows of pairs
     (24, 149, 29, 31, 5, 4),   # odd rows, a row more than whole blocks of four, several units a block
     (16, 148, 56, 56, 5, 3),   # one operand array, levels >= 2 a unit ahead
-    (8, 100, 57, 45, 3, 2),    # 3 x 3, one operand array, odd rows
-    (40, 150, 14, 14, 5, 2),   # many units a block
+    (8, 148, 57, 45, 3, 2),    # 3 x 3, one operand array, odd rows
+    (64, 150, 14, 14, 5, 2),   # many units a block
     (8, 148, 61, 64, 5, 2),    # the widest plane
     (13, 74, 40, 64, 5, 3),    # planes in batches that do not divide eight
 ]
