@@ -438,7 +438,7 @@ pyramid_kernel(const __grid_constant__ PGeom g, const T *__restrict__ x, const _
     const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
     float *mis = reinterpret_cast<float *>(sb + g.misc_off);  // two channels' worth
     u64 *acc_full = reinterpret_cast<u64 *>(mis + 2 * MIS), *acc_empty = acc_full + RING, *full = acc_empty + RING, *freed = full + MAX_BUFS,
-        *r_full = freed + MAX_BUFS, *r_free = r_full + MAX_BUFS, *mma_done = r_free + MAX_BUFS, *fin = mma_done + 1;
+        *r_full = freed + MAX_BUFS, *r_free = r_full + MAX_BUFS, *mma_done = r_free + MAX_BUFS, *set_free = mma_done + MAX_BUFS, *fin = set_free + 2;
     volatile int *dead = reinterpret_cast<volatile int *>(fin + 1);
     unsigned *tmem_slot = reinterpret_cast<unsigned *>(fin + 1) + 1;
     const int u_begin = (int)((long long)blockIdx.x * g.units / gridDim.x), u_end = (int)((long long)(blockIdx.x + 1) * g.units / gridDim.x);
@@ -456,11 +456,12 @@ pyramid_kernel(const __grid_constant__ PGeom g, const T *__restrict__ x, const _
         }
         for (int i = 0; i < MAX_BUFS; ++i) {
             plane::mbar_init(full + i, LOAD);
-            plane::mbar_init(freed + i, ISS + (g.direct ? 0 : DEEP / 32));
+            plane::mbar_init(freed + i, DEEP / 32);
+            plane::mbar_init(mma_done + i, ISS);
             plane::mbar_init(r_full + i, DEEP / 32);
             plane::mbar_init(r_free + i, EPI / 32);
         }
-        plane::mbar_init(mma_done, ISS);
+        for (int i = 0; i < 2; ++i) plane::mbar_init(set_free + i, EPI / 32);
         plane::mbar_init(fin, ISS);
     }
     __syncwarp();
@@ -544,7 +545,10 @@ pyramid_kernel(const __grid_constant__ PGeom g, const T *__restrict__ x, const _
             }
             plane::fence_async_smem();
             __syncwarp();
-            if (lane == 0) mbar_arrive(r_free + buf);
+            if (lane == 0) {
+                mbar_arrive(r_free + buf);
+                if (k + 1 == g.upc) mbar_arrive(set_free + par);  // the channel's last unit
+            }
             named_sync(BAR_EPI, EPI);
             // ---- whole 16-byte words by one bulk copy a plane, the pixels before and behind them one by one (sixteen lanes a plane)
             for (int slot = warp * 2 + (lane >> 4); slot < 8 * g.S; slot += EPI / 16) {
@@ -647,10 +651,7 @@ pyramid_kernel(const __grid_constant__ PGeom g, const T *__restrict__ x, const _
                 }
                 __syncwarp();
             }
-            if (elected) {
-                mma_commit(freed + buf);
-                mma_commit(mma_done);
-            }
+            if (elected) mma_commit(mma_done + buf);
             __syncwarp();
         }
         if (elected) mma_commit(fin);  // nothing may be in flight when tensor and shared memory are given back
@@ -659,19 +660,22 @@ pyramid_kernel(const __grid_constant__ PGeom g, const T *__restrict__ x, const _
     } else {
         // ---------------------------------------------------------------- loaders
         const int lt = tid - (THREADS - LOAD), lw = lt >> 5;
-        int c = u_begin / g.upc, k = u_begin - c * g.upc, c_prev = -1, par = 1, buf = 0;
+        // A wait for a barrier's phase says something only if the phase before it is known to be over (the parity is all it sees), so
+        // every barrier's phases are waited for in turn: `freed` and `mma_done` of an array each time it is loaded, mma_done of the
+        // unit before's array, whose last phase was waited for when that unit was loaded, at a change of channel; set_free when a
+        // set of M, scale and bias is written again, which is every second channel.
+        int c = u_begin / g.upc, k = u_begin - c * g.upc, channels = 0, buf = 0;
         unsigned phase = 0;
         for (int u = u_begin; u < u_end; ++u, next(buf, phase, g.bufs)) {
             char *arr = sb + buf * g.a_bytes;
-            const bool change = c != c_prev;
+            const bool change = u == u_begin || k == 0;
             float wreg = 0.f, breg = 0.f;
             if (change) {
                 wreg = lt < 125 ? folded(g, c, lt, FLIP, w0, s0, wl, sl) : 0.f;
                 if (lt == 0 && !FLIP && b0) breg = __ldg(s0 + c) * __ldg(b0 + c);
-                par ^= 1;
-                c_prev = c;
             }
-            wait_for(freed + buf, phase ^ 1u);
+            if (!g.direct) wait_for(freed + buf, phase ^ 1u);
+            wait_for(mma_done + buf, phase ^ 1u);
             if (g.no_copy) break;  // test mode: nothing is copied and nobody is told
             if (u + 1 + g.direct < u_end) {  // (the deep warps are a unit ahead where they read global memory)
                 int cp = c, kp = k + 1 + g.direct;
@@ -685,10 +689,11 @@ pyramid_kernel(const __grid_constant__ PGeom g, const T *__restrict__ x, const _
             else load_shifted<T, 4, LOAD / 32, false>(g, arr + 4 * rowb, g.Pc, x, c, k, lw, lane);
             if (LOAD == FEW) asm volatile("cp.async.wait_all;" ::: "memory");
             if (change) {  // the MMAs that read the old B operand have completed
-                const int v = u - u_begin, old = v - (g.rbufs > 1 ? 2 : 1);  // the last unit that may use this set of M, scale and bias
-                if (v > 0) wait_for(mma_done, (unsigned)(v - 1) & 1u);
-                if (old >= 0) wait_for(r_free + old % g.rbufs, (unsigned)(old / g.rbufs) & 1u);
-                float *mc = mis + par * MIS;
+                const int set = channels & 1;
+                if (u > u_begin) wait_for(mma_done + (buf ? buf : g.bufs) - 1, buf ? phase : phase ^ 1u);
+                if (channels > 1) wait_for(set_free + set, ((channels >> 1) - 1) & 1u);  // the epilogue has left the channel before the last
+                ++channels;
+                float *mc = mis + set * MIS;
                 if (lt < 125) mc[lt] = wreg;
                 if (lt == 0) mc[545] = breg;
                 tensor::build_table<T, LOAD, BAR_LOAD>(sb + g.table_off, sb + g.parts_off, mc, lt);
@@ -780,7 +785,7 @@ inline bool search(const Request &q, PGeom &best, double &best_cost) {
                 // the last tile's MMAs read up to 32 T + 8 rows; those behind the array feed no output, but lie inside the block's memory
                 const int reach = (h.bufs - 1) * h.a_bytes + (32 * h.T + 8) * h.Pc * CHUNK;
                 h.out_off = o; o += 8 * S * h.out_stride;
-                h.misc_off = o; o += 2 * MIS * 4 + (2 * RING + 4 * MAX_BUFS + 2) * 8 + 16;
+                h.misc_off = o; o += 2 * MIS * 4 + (2 * RING + 5 * MAX_BUFS + 3) * 8 + 16;
                 h.smem = up(o > reach ? o : reach, 128);
                 if (h.smem > plane::SMEM_LIMIT) continue;
                 h.upc = (q.B + 8 * S - 1) / (8 * S);

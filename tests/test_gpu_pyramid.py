@@ -86,6 +86,38 @@ def test_every_unit_another_channel(shape, dtype):
     assert (err <= 2.0 ** (-7 if dtype == "bf16" else -10) * big).all()  # the final rounding on either side
 
 
+@pytest.mark.parametrize("dtype", ["f16", "bf16"])
+@pytest.mark.parametrize("shape,buffers,backward", [((16, 768, 14, 14, 5, 2), 4, False), ((24, 768, 14, 14, 5, 2), 4, True), ((72, 300, 14, 14, 5, 3), 4, True),
+                                                    ((128, 600, 12, 12, 5, 3), 3, True)], ids=lambda s: str(s).replace(", ", "x"))
+def test_the_next_channels_weights_wait_for_units_under_way(shape, buffers, backward, dtype):
+    """Three or four operand arrays and few MMAs a unit: several loaded units wait for their MMAs when a channel's weights, scale and
+    bias are replaced.  Channels differ by powers of two, each is compared by itself, in calls that follow one another."""
+    B, C, H, W, k, L = shape
+    plan = wt.wtconv_plan_describe(wt.make_desc(*shape, wt.DTYPE_NAMES[dtype]))
+    S, T, n, bufs, units = (int(plan.split("fwd[pyramid")[1].split(q)[1].split()[0].strip(",")) for q in (" S=", " T=", " n=", " buffers=", " units="))
+    assert bufs == buffers and T * n <= 6 and units >= 4 * 148 and ("pyramid gradients" in plan) == backward
+    gen = torch.Generator(device="cuda").manual_seed(6)
+    rnd = lambda *s: torch.randn(s, generator=gen, device="cuda")
+    x, g = (rnd(B, C, H, W).to(wt.DTYPE_NAMES[dtype]) for _ in range(2))
+    size = 2.0 ** (5 * torch.arange(C, device="cuda") % 9 - 4)
+    p = [0.1 * rnd(C, k, k) * size[:, None, None], 0.5 + rnd(C).abs(), rnd(C) * size, 0.1 * rnd(L, C, 4, k, k) * size[:, None, None, None], 0.5 + rnd(L, C, 4).abs()]
+    res = []
+    for flags, calls in ((wt.FLAG_NO_WINDOW, 1), (0, 6)):
+        d = wt.make_desc(*shape, wt.DTYPE_NAMES[dtype], flags)
+        ws = wt.alloc_workspace(d)
+        outs = [[torch.empty_like(x), torch.empty_like(x)] + [torch.empty_like(q) for q in p] for _ in range(calls)]
+        for o in outs:
+            wt.wtconv_forward(d, x, *p, o[0], ws)
+            wt.wtconv_backward(d, x, g, *p, *o[1:], ws)
+        res += outs
+    per_channel = lambda t, dim: t.float().movedim(dim, 0).flatten(1).abs().amax(1)
+    for o in res[1:]:
+        for i, dim in ((0, 1), (1, 1), (2, 0), (5, 1)):  # out, grad_x, the weights' gradients
+            err = per_channel(o[i].float() - res[0][i].float(), dim)
+            # activations: the final rounding on either side; weight gradients: sums of thousands of products in fp32
+            assert (err <= (2.0 ** (-7 if dtype == "bf16" else -10) if i < 2 else 1e-4) * per_channel(res[0][i], dim)).all(), i
+
+
 @pytest.mark.parametrize("where", [(0, 0), (27, 27), (13, 8)])
 def test_infinities_reach_their_own_stencil_only(where):
     """The same elements are non-finite as on the kernels that compute every product on its own."""
