@@ -159,9 +159,9 @@ pyramid_gradient_kernel(const __grid_constant__ WGeom g, const T *__restrict__ x
                     for (int ab = 0; ab < 4; ++ab)
 #pragma unroll
                         for (int pq = 0; pq < 4; ++pq)
-                            sum += tensor::haar_sign(cls - 1, ab >> 1, ab & 1) * tensor::haar_sign(cls - 1, pq >> 1, pq & 1) *
+                            sum += 0.25f * tensor::haar_sign(cls - 1, ab >> 1, ab & 1) * tensor::haar_sign(cls - 1, pq >> 1, pq & 1) *
                                    mis[ab * 100 + (2 * uu + (pq >> 1)) * 10 + 2 * vv + (pq & 1)];
-                    partl[(slot * 4 + cls - 1) * KK + t] = 0.25f * sum;
+                    partl[(slot * 4 + cls - 1) * KK + t] = sum;
                 }
             }
             // (the next channel's spill and dM wait behind this unit's barriers: all of a warp's reads lie before its next drain's end)
@@ -250,8 +250,7 @@ pyramid_gradient_kernel(const __grid_constant__ WGeom g, const T *__restrict__ x
                         for (int h = 0; h < 4; ++h) s[h] += q[j + h];
                     }
                     for (; j < g.tpc[m]; ++j) s[0] += q[j];
-                    // (a coefficient of level m is 2^m times the transform's, on either side)
-                    partl[(size_t)(m - 1) * g.C * g.np * 4 * KK + (slot * 4 + (cls & 3)) * KK + uu * g.K + vv] = ((s[0] + s[1]) + (s[2] + s[3])) * (1.f / (float)(1 << 2 * m));
+                    partl[(size_t)(m - 1) * g.C * g.np * 4 * KK + (slot * 4 + (cls & 3)) * KK + uu * g.K + vv] = (s[0] + s[1]) + (s[2] + s[3]);
                 }
                 named_sync(BAR_DEEP, DEEP);
             }
@@ -266,7 +265,7 @@ pyramid_gradient_kernel(const __grid_constant__ WGeom g, const T *__restrict__ x
             if (dt == 0) {
                 float sum = 0.f;
                 for (int i = 0; i < DEEP / 32; ++i) sum += mis[400 + i];
-                part0[slot * (KK + 1) + KK] = sum;
+                part0[slot * (KK + 1) + KK] = 4.f * sum;  // (quarters: level-2 coefficients)
             }
         }
     } else if (warp < (WDRAIN + DEEP) / 32 + WISS) {

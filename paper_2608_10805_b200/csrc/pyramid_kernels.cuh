@@ -200,11 +200,10 @@ __device__ __forceinline__ float folded(const PGeom &g, int c, int e, bool flip,
     return __ldg(wl + ((size_t)c * 4 + cls - 1) * KK + u * g.K + v) * __ldg(sl + (size_t)c * 4 + cls - 1);
 }
 
-// Eq. 5 without its factor: the coefficients of level l are 2^l times the transform's, and the folded weights carry 2^-l (powers of
-// two: nothing is rounded).
+// Eq. 5 with its factor inside the second sums (a power of two: the results are haar_butterfly's, but no sum is larger than they are).
 __device__ __forceinline__ Haar4 butterfly(float a, float b, float c, float d) {
-    const float s0 = a + b, s1 = c + d, d0 = a - b, d1 = c - d;
-    return {s0 + s1, s0 - s1, d0 + d1, d0 - d1};
+    const float s0 = a + b, d0 = a - b, s1 = 0.5f * (c + d), d1 = 0.5f * (c - d);
+    return {fmaf(0.5f, s0, s1), fmaf(0.5f, s0, -s1), fmaf(0.5f, d0, d1), fmaf(0.5f, d0, -d1)};
 }
 struct Tile {
     int src, wt, z, meta;  // window, folded weights, output (float indices); meta: bit 31 valid, window pitch, Z pitch << 10, rows to store << 20
@@ -248,8 +247,8 @@ __device__ __forceinline__ void load_blocks(uint4 (&w)[4], const char *q, int ro
         else w[h] = *reinterpret_cast<const uint4 *>(q + h * row_bytes);
     }
 }
-// `y`: where the first block's coefficients go, `sub` floats from subband to subband; in0, in1: blocks inside the grid; returns the
-// sum of their pixels.
+// `y`: where the first block's coefficients go, `sub` floats from subband to subband; in0, in1: blocks inside the grid; returns a
+// quarter of the sum of their pixels.
 template <typename T>
 __device__ __forceinline__ float analyse_blocks(const uint4 (&w)[4], float *y, int sub, bool in0, bool in1) {
     float ll[2][4], sum = 0.f;
@@ -259,7 +258,7 @@ __device__ __forceinline__ float analyse_blocks(const uint4 (&w)[4], float *y, i
 #pragma unroll
         for (int m = 0; m < 4; ++m) {
             const float2 t = tensor::unpack16(av[m], T()), u = tensor::unpack16(bv[m], T());
-            ll[h][m] = (t.x + t.y) + (u.x + u.y);
+            ll[h][m] = fmaf(0.5f, t.x + t.y, 0.5f * (u.x + u.y));
         }
     }
     if (in0) {
@@ -584,7 +583,7 @@ pyramid_kernel(const __grid_constant__ PGeom g, const T *__restrict__ x, const _
                     const int cls = e / 25, t = e - cls * 25, tt = FLIP ? 24 - t : t, uu = tt / 5 - pad, vv = tt % 5 - pad;
                     const size_t f = ((size_t)(1 + (cls >> 2)) * g.C + c) * 4 + (cls & 3);
                     const bool in = uu >= 0 && uu < g.K && vv >= 0 && vv < g.K;
-                    wtab[cls * WS + t] = in ? __ldg(wl + f * KK + uu * g.K + vv) * __ldg(sl + f) * (1.f / (float)(4 << (cls >> 2))) : 0.f;
+                    wtab[cls * WS + t] = in ? __ldg(wl + f * KK + uu * g.K + vv) * __ldg(sl + f) : 0.f;
                 }
                 c_prev = c;
             }

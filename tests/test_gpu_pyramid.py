@@ -1,5 +1,6 @@
 """Whole planes of several levels on the tensor cores (base convolution, level 1) and FMA units (levels >= 2): against the fp64
 oracle at the edges of their tiles and units, with infinities and NaNs, and with waits that run out."""
+import numpy as np
 import pytest
 import torch
 
@@ -116,6 +117,25 @@ def test_the_next_channels_weights_wait_for_units_under_way(shape, buffers, back
             err = per_channel(o[i].float() - res[0][i].float(), dim)
             # activations: the final rounding on either side; weight gradients: sums of thousands of products in fp32
             assert (err <= (2.0 ** (-7 if dtype == "bf16" else -10) if i < 2 else 1e-4) * per_channel(res[0][i], dim)).all(), i
+
+
+def test_the_range_of_the_coefficients():
+    """Values whose plain sums over a coefficient's pixels (and products of such sums) are beyond fp32, while the transform's own
+    coefficients, outputs and gradients are not."""
+    shape = B, C, H, W, k, L = 128, 64, 16, 16, 5, 5
+    plan = wt.wtconv_plan_describe(wt.make_desc(*shape, "bf16"))
+    assert "fwd[pyramid" in plan and "pyramid gradients" in plan
+    w = inputs.Workload("range", *shape, "bf16", 78)
+    data = inputs.make_inputs(w)
+    data["s0"][:], data["sl"][:] = 1, 1
+    shade = {n: 1 + np.abs(data[n]) / 64 for n in ("x", "g")}  # (at most 1.1)
+    for x_exp, g_exp in ((121, -121), (-121, 121), (56, 54)):
+        for n, e in (("x", x_exp), ("g", g_exp)):
+            data[n] = torch.from_numpy(np.float32(2.0 ** e) * shade[n]).bfloat16().float().numpy()
+        out, grads = run_gpu(w, data, guarded=False)
+        ref, ref_grads = run_oracle(w, data)
+        for got, want, tol in ((out, ref, TOL["bf16"] / 4), *((grads[n], ref_grads[n], TOL["bf16"] / 4 if n == "dx" else 1e-5) for n in GRAD_NAMES if n != "db0")):
+            assert np.abs(want).max() < 3e38 and rel_err(got, want) < tol
 
 
 @pytest.mark.parametrize("where", [(0, 0), (27, 27), (13, 8)])
