@@ -38,7 +38,7 @@ using tensor::TAPS;
 using tensor::u64;
 
 constexpr int EPI = 128, DEEP = 384, ISS = 2, OTHERS = EPI + DEEP + 32 * ISS;  // threads and (ISS) warps of the roles but the loaders
-constexpr int LOAD = 256, FEW = 128;  // loaders: through registers, or issuing asynchronous copies
+constexpr int MANY = 256, FEW = 128;  // loaders: through registers, or issuing asynchronous copies
 constexpr int RING = 8, MAXL = 8, MAX_BUFS = 4, WS = plane::WT_STRIDE;
 constexpr int BAR_DEEP = 3, BAR_LOAD = 4, BAR_EPI = 5;  // named barriers
 constexpr int CHUNK = 144;                 // bytes from one chunk of eight images to the next: one image's chunks fall on different banks
@@ -74,13 +74,13 @@ __device__ __forceinline__ void named_sync(int id, int count) {
 // an instruction, and the chunks' distance keeps an image's pieces on different banks.  A lane's addresses are worked out once an
 // octet: a warp alone issues an instruction every four to five cycles, so what counts here, as in the other roles, is how many
 // instructions a unit takes.
-template <typename T, int PIX>
+template <typename T, int PIX, int WARPS>
 __device__ __forceinline__ void load_rows(const PGeom &g, char *arr, const T *__restrict__ x, int c, int k, int warp, int lane) {
     using V = typename std::conditional<PIX == 4, uint2, unsigned>::type;
     constexpr int U = 7;
     const int pieces = g.W / PIX, lp = pieces > 16 ? 5 : pieces > 8 ? 4 : pieces > 4 ? 3 : 2;  // log2 of the lanes to a row
     const int sets = lp - 2, q = lane & ((1 << lp) - 1), col = PIX * q + 4;                      // log2 of the warps that share a row's images
-    const int img = ((warp & ((1 << sets) - 1)) << (5 - lp)) + (lane >> lp), y0 = warp >> sets, dy = (LOAD / 32) >> sets;
+    const int img = ((warp & ((1 << sets) - 1)) << (5 - lp)) + (lane >> lp), y0 = warp >> sets, dy = WARPS >> sets;
     const int rowb = g.Pc * CHUNK, sstep = dy * g.W * 2, dstep = dy * rowb;
     if (q >= pieces) return;
     for (int o = 0; o < g.S; ++o) {
@@ -227,10 +227,12 @@ __device__ __forceinline__ Tile find_tile(const PGeom &g, int it) {
     d.meta = (int)(0x80000000u | (unsigned)g.pitch[l] | ((unsigned)g.zpitch[l] << 10) | ((unsigned)rows << 20));
     return d;
 }
+// KT = 3: the zeros around 3 x 3 kernels in their 5 x 5 tables meet no coefficient (which may be an infinity).
+template <int KT>
 __device__ __forceinline__ void run_tile(float *dp, const float *wtab, const Tile &d) {
     float w[25], acc[4][4];
     plane::load_weights(wtab + d.wt, w);
-    plane::conv_tile<4>(dp + d.src, d.meta & 0x3ff, w, acc);
+    plane::conv_tile<4, false, KT>(dp + d.src, d.meta & 0x3ff, w, acc);
     const int zp = (d.meta >> 10) & 0x3ff, rows = (d.meta >> 20) & 0xf;
 #pragma unroll
     for (int r = 0; r < 4; ++r)
@@ -427,7 +429,7 @@ inline __device__ __noinline__ void unfold_classes(const PGeom &g, const Paramet
 // ------------------------------------------------------------------ the kernel
 // FLIP = false: out = WTConv(x).  FLIP = true: the same on grad_out with rotated kernels and no bias: grad_x, and the parameters'
 // gradients from the sums of the kernel before.
-template <typename T, bool FLIP, int LOAD>
+template <typename T, bool FLIP, int LOAD, int KT>
 __global__ void __launch_bounds__(OTHERS + LOAD, 1)
 pyramid_kernel(const __grid_constant__ PGeom g, const T *__restrict__ x, const __grid_constant__ Parameters prm, const __grid_constant__ Gradients grad,
                T *__restrict__ out, int *__restrict__ status) {
@@ -615,7 +617,7 @@ pyramid_kernel(const __grid_constant__ PGeom g, const T *__restrict__ x, const _
                     named_sync(BAR_DEEP, DEEP);
                 }
 #pragma unroll 1
-                for (int it = dt; it < total; it += DEEP) run_tile(dp, wtab, it == dt ? own : find_tile(g, it));  // (one copy of the tile code)
+                for (int it = dt; it < total; it += DEEP) run_tile<KT>(dp, wtab, it == dt ? own : find_tile(g, it));  // (one copy of the tile code)
                 named_sync(BAR_DEEP, DEEP);
                 synthesise(g, dp, R, slot0, nb, s_s, s_j, s_i, DEEP / sets);
             }
@@ -683,8 +685,8 @@ pyramid_kernel(const __grid_constant__ PGeom g, const T *__restrict__ x, const _
             }
             if (LOAD == FEW && g.vec == 4) copy_rows<4, LOAD / 32>(g, arr + 4 * rowb, g.Pc, 4, x, c, k, lw, lane);
             else if (LOAD == FEW) copy_rows<2, LOAD / 32>(g, arr + 4 * rowb, g.Pc, 4, x, c, k, lw, lane);
-            else if (g.vec == 4) load_rows<T, 4>(g, arr, x, c, k, lw, lane);
-            else if (g.vec == 2) load_rows<T, 2>(g, arr, x, c, k, lw, lane);
+            else if (g.vec == 4) load_rows<T, 4, LOAD / 32>(g, arr, x, c, k, lw, lane);
+            else if (g.vec == 2) load_rows<T, 2, LOAD / 32>(g, arr, x, c, k, lw, lane);
             else load_shifted<T, 4, LOAD / 32, false>(g, arr + 4 * rowb, g.Pc, x, c, k, lw, lane);
             if (LOAD == FEW) asm volatile("cp.async.wait_all;" ::: "memory");
             if (change) {  // the MMAs that read the old B operand have completed
@@ -840,6 +842,13 @@ inline bool plan(const Request &q, PGeom &out, double &cost) {  // searched once
     return e.ok;
 }
 
+template <typename T, bool FLIP, int LOAD, int KT>
+cudaError_t launch(const PGeom &g, const T *x, const Parameters &p, const Gradients &grad, T *out, char *ws, cudaStream_t st) {
+    constexpr auto kern = pyramid_kernel<T, FLIP, LOAD, KT>;
+    const cudaError_t e = plane::opt_in_smem<kern>();
+    if (e != cudaSuccess) return e;
+    return launch_overlapped(kern, (unsigned)g.nblocks, (unsigned)(OTHERS + LOAD), (size_t)g.smem, st, g, x, p, grad, out, reinterpret_cast<int *>(ws));
+}
 template <typename T, bool FLIP>
 cudaError_t run(const Request &q, const T *x, const Parameters &p, const Gradients &grad, T *out, char *ws, cudaStream_t st, unsigned tag, bool no_copy) {
     PGeom g;
@@ -851,11 +860,9 @@ cudaError_t run(const Request &q, const T *x, const Parameters &p, const Gradien
     // Four warps that issue asynchronous copies leave the other roles 16 more registers a thread (88), but are slower than eight that load through
     // registers where units are small: forward, 128 x 96 x 56 x 56 (3136 pixels an image and octet) 126 -> 121 us, 128 x 192 x 28 x 28
     // (1568) 68.2 -> 62.9; 64 x 192 x 28 x 28 with four levels (784) 48.0 -> 49.3, 16 x 64 x 14 x 14 8.9 -> 9.5.
-    constexpr auto few = pyramid_kernel<T, FLIP, FEW>, many = pyramid_kernel<T, FLIP, LOAD>;
     const bool copies = copied(g);
-    const cudaError_t e = copies ? plane::opt_in_smem<few>() : plane::opt_in_smem<many>();
-    if (e != cudaSuccess) return e;
-    return launch_overlapped(copies ? few : many, (unsigned)g.nblocks, (unsigned)(OTHERS + (copies ? FEW : LOAD)), (size_t)g.smem, st, g, x, p, grad, out, reinterpret_cast<int *>(ws));
+    if (q.K == 3) return copies ? launch<T, FLIP, FEW, 3>(g, x, p, grad, out, ws, st) : launch<T, FLIP, MANY, 3>(g, x, p, grad, out, ws, st);
+    return copies ? launch<T, FLIP, FEW, 5>(g, x, p, grad, out, ws, st) : launch<T, FLIP, MANY, 5>(g, x, p, grad, out, ws, st);
 }
 
 inline int describe(const Request &q, char *buf, size_t n) {

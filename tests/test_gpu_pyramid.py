@@ -4,7 +4,7 @@ import numpy as np
 import pytest
 import torch
 
-from helpers import GRAD_NAMES, TOL, rel_err, run_gpu, run_oracle
+from helpers import GRAD_NAMES, TOL, rel_err, run_gpu, run_oracle, to_dev
 from paper_2608_10805_b200 import inputs, wtconv as wt
 
 pytestmark = pytest.mark.gpu
@@ -136,6 +136,41 @@ def test_the_range_of_the_coefficients():
         ref, ref_grads = run_oracle(w, data)
         for got, want, tol in ((out, ref, TOL["bf16"] / 4), *((grads[n], ref_grads[n], TOL["bf16"] / 4 if n == "dx" else 1e-5) for n in GRAD_NAMES if n != "db0")):
             assert np.abs(want).max() < 3e38 and rel_err(got, want) < tol
+
+
+NON_FINITE_SHAPES = [(64, 96, 28, 28, 5, 2), (13, 96, 30, 26, 3, 3), (61, 96, 29, 31, 5, 4), (16, 148, 56, 56, 5, 3), (64, 192, 14, 13, 5, 3)]
+
+
+def with_infinities(shape, dtype):
+    """Infinities and NaNs at the planes' edges and in the middle, those of x and of grad_out in channels of their own."""
+    B, C, H, W, k, L = shape
+    w = inputs.Workload("pyramid", *shape, dtype, 930)
+    plan = wt.wtconv_plan_describe(wt.make_desc(*shape, wt.DTYPE_NAMES[dtype]))
+    assert "fwd[pyramid" in plan and "pyramid gradients" in plan
+    data = inputs.make_inputs(w)
+    for n, channels in (("x", (0, 1, 2, C - 1)), ("g", (4, 5, 6, C - 2))):
+        for c, (b, y, x_, v) in zip(channels, ((0, H // 2, W // 2, np.inf), (1, 0, W - 1, np.nan), (B - 1, H - 1, 0, -np.inf), (2, H - 1, W - 1, np.inf))):
+            data[n][b, c, y, x_] = v
+    return w, data
+
+
+def run_unchecked(w, data, flags=0):
+    dt = wt.DTYPE_NAMES[w.dtype]
+    out, grads = wt.forward_backward(wt.make_desc(w.B, w.C, w.H, w.W, w.k, w.L, dt, flags), to_dev(data["x"], dt), to_dev(data["g"], dt), to_dev(data["w0"]),
+                                     to_dev(data["s0"]), None, to_dev(data["wl"]), to_dev(data["sl"]))
+    return out.double().cpu().numpy(), {n: v.double().cpu().numpy() for n, v in grads.items() if v is not None}
+
+
+@pytest.mark.parametrize("dtype", ["f16", "bf16"])
+@pytest.mark.parametrize("shape", NON_FINITE_SHAPES, ids=lambda s: "x".join(map(str, s)))
+def test_outputs_and_grad_x_are_non_finite_where_the_oracles_are(shape, dtype):
+    w, data = with_infinities(shape, dtype)
+    out, grads = run_unchecked(w, data)
+    ref, ref_grads = run_oracle(w, data)
+    for a, want in ((out, ref), (grads["dx"], ref_grads["dx"])):
+        fin = np.isfinite(want)
+        assert 0 < fin.sum() < fin.size and (np.isfinite(a) == fin).all()
+        assert rel_err(a[fin], want[fin]) < TOL[dtype] / 4
 
 
 @pytest.mark.parametrize("where", [(0, 0), (27, 27), (13, 8)])
