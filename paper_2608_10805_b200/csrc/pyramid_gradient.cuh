@@ -503,6 +503,7 @@ cudaError_t backward(const Request &q, const T *x, const T *go, const Parameters
     to.units = g.units;
     to.nblocks = g.nblocks;
     to.ratio = (float)g.nblocks / (float)g.units;
+    to.x = x;
     return run<T, true>(q, go, p, to, gx, ws, st, tag, no_copy);
 }
 

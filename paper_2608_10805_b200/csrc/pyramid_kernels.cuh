@@ -367,6 +367,7 @@ struct Gradients {
     const float *part0, *partl;
     int np, upc, units, nblocks;
     float ratio;  // blocks to a unit
+    const void *x;  // the layer's input
 };
 // block_of_unit without a 64-bit division, whose subroutine costs the kernel's other roles registers (8 spilled: 128 x 192 x 28 x 28
 // 137 -> 146 us): a guess in fp32, one off at most, and the exact ranges.
@@ -379,10 +380,49 @@ __device__ __forceinline__ int block_near(const Gradients &d, int v) {
     while (b > 0 && begin(b) > v) --b;
     return b;
 }
+// One class (0: base convolution, 1 .. 4: level 1) of a channel's weight gradients by a warp, every product on its own, from global memory: the
+// contraction multiplies the zeros around the planes (to whole groups of 16 rows and chunks of 8 columns) too, so that an infinity or
+// NaN has reached taps that do not meet it.  x, go: the channel's planes of the first image.  Returns tap `lane` of 5 x 5.
+template <typename T>
+__device__ __noinline__ double taps_of_class(const PGeom &g, const T *__restrict__ x, const T *__restrict__ go, int cls, int lane) {
+    const int s = cls ? 1 : 0, h = (g.H + s) >> s, w = (g.W + s) >> s;
+    const float sy = (cls - 1) & 1 ? -1.f : 1.f, sx = (cls - 1) & 2 ? -1.f : 1.f;
+    const size_t image = (size_t)g.C * g.HW;
+    auto at = [&](const T *q, int i, int j) {  // a pixel, or the class's coefficient (Eq. 5)
+        auto pixel = [&](int y, int xx) { return y < g.H && xx < g.W ? (float)q[y * g.W + xx] : 0.f; };
+        return cls ? 0.5f * ((pixel(2 * i, 2 * j) + sx * pixel(2 * i, 2 * j + 1)) + sy * (pixel(2 * i + 1, 2 * j) + sx * pixel(2 * i + 1, 2 * j + 1))) : pixel(i, j);
+    };
+    double total = 0.0;
+#pragma unroll 1
+    for (int b = 0; b < g.B; ++b, x += image, go += image) {
+        float acc[25];
+#pragma unroll
+        for (int t = 0; t < 25; ++t) acc[t] = 0.f;
+#pragma unroll 1
+        for (int e = lane; e < h * w; e += 32) {
+            const int i = e / w, j = e - i * w;
+            const float v = at(go, i, j);
+#pragma unroll
+            for (int t = 0; t < 25; ++t) {
+                const int y = i + t / 5 - 2, xx = j + t % 5 - 2;
+                if ((unsigned)y < (unsigned)h && (unsigned)xx < (unsigned)w) acc[t] = fmaf(v, at(x, y, xx), acc[t]);
+            }
+        }
+#pragma unroll
+        for (int t = 0; t < 25; ++t) {
+#pragma unroll
+            for (int o = 16; o; o >>= 1) acc[t] += __shfl_xor_sync(0xffffffffu, acc[t], o);
+            if (lane == t) total += (double)acc[t];
+        }
+    }
+    return total;
+}
 // What unfold_epilogue_kernel does, class by class, a warp each and a lane a tap (at most 25 and the bias): fixed-order fp64 sums and
 // Eq. 9.  The loaders do it when they have loaded their last unit: it hides behind that unit's other stages, where a launch of its own
 // took 4 - 5 us.
-inline __device__ __noinline__ void unfold_classes(const PGeom &g, const Parameters &p, const Gradients &d, int warp, int warps, int lane) {
+// Classes of base convolution and level 1 whose sums are not finite are computed again, see taps_of_class.
+template <typename T>
+__device__ __noinline__ void unfold_classes(const PGeom &g, const Parameters &p, const Gradients &d, const T *__restrict__ go, int warp, int warps, int lane) {
     const int KK = g.K * g.K, classes = 1 + 4 * g.L;
     for (int e = blockIdx.x * warps + warp; e < g.C * classes; e += gridDim.x * warps) {
         const int c = e / classes, cls = e - c * classes, l = (cls - 1) >> 2, sub = (cls - 1) & 3;
@@ -406,17 +446,18 @@ inline __device__ __noinline__ void unfold_classes(const PGeom &g, const Paramet
             to = d.wl + f * KK;
             ts = d.sl + f;
         }
-        double prod = 0.0;
+        double prod = 0.0, acc = 0.0;
+        if (lane < taps)
+            for (int i = 0; i < n; ++i) acc += (double)q[(size_t)i * stride + lane];
+        if (cls < 5 && __any_sync(0xffffffffu, lane < KK && !(fabs(acc) < 1e300))) {
+            const size_t first = (size_t)c * g.HW;
+            const double again = taps_of_class<T>(g, static_cast<const T *>(d.x) + first, go + first, cls, lane);
+            const int pad = (5 - g.K) / 2;
+            const double mine = __shfl_sync(0xffffffffu, again, lane < KK ? (lane / g.K + pad) * 5 + lane % g.K + pad : 0);
+            if (lane < KK) acc = mine;
+        }
         if (lane < taps) {
             const float wv = lane < KK ? __ldg(w + lane) : __ldg(p.b0 + c), sv = __ldg(s);
-            double acc = 0.0;
-            for (int i0 = 0; i0 < n; i0 += 8) {
-                float v[8];
-#pragma unroll
-                for (int i = 0; i < 8; ++i) v[i] = i0 + i < n ? q[(size_t)(i0 + i) * stride + lane] : 0.f;
-#pragma unroll
-                for (int i = 0; i < 8; ++i) acc += (double)v[i];
-            }
             *(lane < KK ? to + lane : d.b0 + c) = (float)((double)sv * acc);
             prod = acc * (double)wv;
         }
@@ -704,7 +745,7 @@ pyramid_kernel(const __grid_constant__ PGeom g, const T *__restrict__ x, const _
             mbar_arrive(full + buf);
         }
         __syncwarp();
-        if (FLIP) unfold_classes(g, prm, grad, lw, LOAD / 32, lane);
+        if (FLIP) unfold_classes<T>(g, prm, grad, x, lw, LOAD / 32, lane);
     }
     fence_before();
     __syncthreads();

@@ -173,6 +173,20 @@ def test_outputs_and_grad_x_are_non_finite_where_the_oracles_are(shape, dtype):
         assert rel_err(a[fin], want[fin]) < TOL[dtype] / 4
 
 
+@pytest.mark.parametrize("dtype", ["f16", "bf16"])
+@pytest.mark.parametrize("shape", NON_FINITE_SHAPES, ids=lambda s: "x".join(map(str, s)))
+def test_weight_gradients_are_non_finite_where_their_taps_meet_it(shape, dtype):
+    """Base convolution and level 1: where the oracle's are (which multiplies grad_out with zeros around x: not further there).  Levels
+    >= 2: no further than on the block-per-plane kernels."""
+    w, data = with_infinities(shape, dtype)
+    grads, family, ref = run_unchecked(w, data)[1], run_unchecked(w, data, wt.FLAG_NO_WINDOW)[1], run_oracle(w, data)[1]
+    for a, want in ((grads["dw0"], ref["dw0"]), (grads["dwl"][0], ref["dwl"][0])):
+        fin, got = np.isfinite(want), np.isfinite(a)
+        assert 0 < fin.sum() < fin.size and got[fin].all() and (got == fin)[:4].all() and (got == fin)[-1].all() and not got[4].any()
+        assert rel_err(a[fin], want[fin]) < 1e-5
+    assert all(np.isfinite(grads[n][np.isfinite(family[n])]).all() for n in ("dwl", "dsl", "ds0"))
+
+
 @pytest.mark.parametrize("where", [(0, 0), (27, 27), (13, 8)])
 def test_infinities_reach_their_own_stencil_only(where):
     """The same elements are non-finite as on the kernels that compute every product on its own."""
