@@ -820,10 +820,11 @@ struct EpiloguePtrs {
     bool deep_all;  // levels >= 2 come from kernels that write every slot, whatever the one above does
 };
 
-// Bound by latency alone (a few KB a block): a thread an entry where a block can have that many (epilogue_threads), eight partial
-// sums requested at a time, and a warp for each scale gradient.  Against 128 threads in several passes and one thread adding a
-// class's products after one another, a training step of 16 x 96 x 56 x 56 f32, three levels, went from 180 to 172 us with 7 x 7
-// kernels (638 entries a channel) and from 92.3 to 90.8 with 3 x 3 ones in 5 x 5 tables (326).
+// Bound by latency alone (a few KB a block): a thread an entry where a block can have that many (epilogue_threads), and a warp for each
+// scale gradient.  Against 128 threads in several passes and one thread adding a class's products after one another, a backward of
+// 16 x 96 x 56 x 56 f32, three levels, takes 103 us instead of 107 with 7 x 7 kernels (638 entries a channel) and 53.8 instead of 56.4
+// with 3 x 3 ones in 5 x 5 tables (326).  The sum over the slots is left to the compiler: eight slots at a time, the last of them
+// predicated, took 35 us instead of 19 for a backward of 67 x 26 x 16 x 16, two levels (67 slots).
 constexpr int EPILOGUE_MAX_THREADS = 512;
 inline int epilogue_threads(int KK, int L) {
     const int n = (KK + 1 + L * 4 * KK + 31) / 32 * 32;
@@ -871,13 +872,7 @@ unfold_epilogue_kernel(int C, int K, int L, EpiloguePtrs ep, const float *__rest
             dst = dwl + ((size_t)l * C + c) * nl + t;
         }
         double acc = 0.0;  // fixed slot order, fp64: the batch sum does not depend on the launch geometry's timing
-        for (int i0 = 0; i0 < n; i0 += 8) {
-            float v[8];
-#pragma unroll
-            for (int i = 0; i < 8; ++i) v[i] = i0 + i < n ? q[(size_t)(i0 + i) * stride] : 0.f;
-#pragma unroll
-            for (int i = 0; i < 8; ++i) acc += (double)v[i];
-        }
+        for (int i = 0; i < n; ++i) acc += (double)q[(size_t)i * stride];
         prod[e] = acc * (double)wv;
         if (dst) *dst = (float)((double)sv * acc);  // Eq. 9: dW = s dWfold, db = s dbfold
     }
