@@ -85,7 +85,8 @@ typedef enum {
  * limit is tiny, so every wait for a copy runs out; the kernels record it in the status word and return
  * normally with nothing in flight (outputs are then invalid by design).  Never set it in production. */
 #define WTCONV_FLAG_TEST_NO_COPY 2u
-#define WTCONV_FLAG_NO_TEAM 4u /* never take the team kernels for small planes (used to test the block-per-plane kernels on them) */
+#define WTCONV_FLAG_NO_TEAM 4u /* never take the team kernels for small planes, nor the per-level kernels for 7 x 7 kernels on planes that the
+                                 * block-per-plane kernels serve (used to test the block-per-plane kernels on them) */
 #define WTCONV_FLAG_NO_WINDOW 64u /* never take the window kernels for large planes (used to test the tiled path on them) */
 /* Large planes are served by the window kernels (levels 1-2 on chip, about 2.2 N elements of HBM traffic) when their
  * rows are not 16-byte multiples, and by the tiled kernels (per-level launches, Q_fused - 2 N of traffic, but faster

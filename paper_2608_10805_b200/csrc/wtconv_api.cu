@@ -430,6 +430,40 @@ bool pyramid_serves(const wtconv_desc *d, bool on_chip, int bwd) {
     return wt::pyramid::plan(pyramid_request(d), g, cost) && 1.15 * cost < plane_deep_us(d, 0);
 }
 
+// 7 x 7 kernels on whole planes: block per plane, or the per-level kernels.  The latter win where planes are few (a block per plane
+// leaves SMs empty, and its chain of stages is longer) and without levels on large 16-bit planes, where they only stream.  Both directions
+// follow one answer, because a workspace keeps its status words in one place: the block-per-plane kernels are taken where both
+// estimates (microseconds, fitted to 444 shapes of up to 74 x 74 with up to three levels, 9 - 14 % off) are a fifth below (without levels, forward: three
+// tenths).  Of 484 measured shapes that takes 285, 3.3 x as fast (geometric mean of both directions), none slower in either.
+bool seven_on_planes(const wtconv_desc *d) {
+    wt::plane::Geom g;
+    if (!wt::plane::supported(d->H, d->W, 7, d->L, d->dtype) ||
+        !wt::plane::plan_forward(d->B, d->C, d->H, d->W, d->L, (int)elem_bytes(d->dtype), g, 0, 7))
+        return false;
+    if (d->flags & WTCONV_FLAG_NO_TEAM) return true;
+    const double planes = (double)d->B * d->C * 1e-3, px = planes * d->H * d->W * 1e-3, tiles = planes * ((d->W + 3) / 4 * 4) * ((d->H + 3) / 4 * 4) * 1e-3;
+    const double unit = 0.1 * g.NPL * d->H * d->W / g.nthreads, late = !g.bulk && d->W % 4 ? unit : 0;  // a thread's pixels of a unit; fetched one by one
+    const bool odd = d->W % 4 != 0, unaligned = d->W * elem_bytes(d->dtype) % 16 != 0;
+    if (d->L == 0) {
+        if (d->dtype != WTCONV_F32 && d->H * d->W > 1500) return false;
+        const double level[2] = {3.79 + (7.17 + 1.98 * unaligned) * planes + (2.35 + 0.63 * unaligned) * px,
+                                 9.81 + (31.2 + 7.75 * unaligned) * planes + (3.72 + 1.68 * unaligned) * px};
+        return 1.4 * (4.63 + 4.2 * tiles + 0.28 * planes + 1.33 * late + 1.05 * unit) < level[0] &&
+               1.25 * (13.1 + (9.98 + 0.4 * odd) * tiles + 1.17 * planes + 2.5 * late + 2.7 * unit) < level[1];
+    }
+    double grids = 0, coefficients = 0;  // 32 x 32 tiles and coefficients of a plane's levels
+    const double base = (d->H + 31) / 32 * ((d->W + 31) / 32);
+    for (int l = 1, h = (d->H + 1) / 2, w = (d->W + 1) / 2; l <= d->L; ++l, h = (h + 1) / 2, w = (w + 1) / 2) {
+        grids += 4.0 * ((h + 31) / 32) * ((w + 31) / 32);
+        coefficients += 4.0 * h * w;
+    }
+    const double all = planes * (coefficients + d->H * d->W) * 1e-3;
+    const double level[2] = {5.63 + 2.5 * d->L + planes * (3.83 * base + 2.84 * grids) + 0.72 * all,
+                             11.5 + 5.0 * d->L + planes * (15.5 * base + 11.7 * grids) + 0.61 * all};
+    return 1.25 * (6.88 + 0.55 * d->L + (6.56 + 1.46 * odd) * tiles + (0.38 + 0.4 * d->L) * planes + 0.89 * late - 0.38 * unit) < level[0] &&
+           1.25 * (17.6 + 2.39 * d->L + (14.66 + 2.4 * odd) * tiles + (0.71 + 1.33 * d->L) * planes + 1.22 * late + 0.1 * unit) < level[1];
+}
+
 Route find_route(const wtconv_desc *d) {
     Route r = {};
     r.key = *d;
@@ -447,7 +481,7 @@ Route find_route(const wtconv_desc *d) {
         if (!(d->flags & WTCONV_FLAG_NO_TEAM) && !((d->flags >> 8) & ~(63u << 8)))
             r.team = wt::team::supported(d->B, d->C, d->H, d->W, d->k, d->L, d->dtype, team_force_g(d));
         // (7 x 7 kernels: launch-plan overrides leave them on the per-level kernels, which have no plan to override)
-        r.plane = r.team || (!(d->k == 7 && (d->flags >> 8)) && wt::plane::supported(d->H, d->W, d->k, d->L, d->dtype));
+        r.plane = r.team || (d->k == 7 ? !(d->flags >> 8) && seven_on_planes(d) : wt::plane::supported(d->H, d->W, d->k, d->L, d->dtype));
         // Large planes (k = 5): windows with levels 1-2 on chip, deeper levels on the whole-plane kernels over a carrier.
         // Measured on B200: with 16-byte aligned rows the per-level tiled kernels are as fast or faster (they stream whole
         // rows), with unaligned rows (225-wide 16-bit planes) they fall to element loads and the window kernels win.

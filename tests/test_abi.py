@@ -100,6 +100,16 @@ def test_plan_and_launch_count(lib):
     assert wt.wtconv_plan_name(d3t) == "tiled" and wt.wtconv_launch_count(d3t) == (4, 5)
 
 
+def test_seven_by_seven_kernels_take_whole_planes_where_that_is_faster(lib):
+    """Few planes, and large 16-bit planes without levels, stay on the per-level kernels: one launch a level and direction, one more
+    for the parameter gradients."""
+    for shape, plane in (((16, 96, 56, 56, 7, 3, "f32"), True), ((49, 419, 11, 11, 7, 0, "bf16"), True), ((2, 55, 56, 56, 7, 1, "f32"), False),
+                         ((2, 29, 63, 63, 7, 0, "f32"), False), ((106, 123, 47, 44, 7, 0, "f16"), False), ((2, 15, 15, 13, 7, 0, "bf16"), False)):
+        d = wt.make_desc(*shape)
+        assert wt.wtconv_plan_describe(d).startswith("plane" if plane else "tiled"), shape
+        assert wt.wtconv_launch_count(d) == ((1, 3) if plane else (d.L + 1, d.L + 2)), shape
+
+
 def test_scratch_memory_accounting(lib):
     """Device memory the layer needs beyond its inputs and outputs.  Whole-plane kernels keep every intermediate
     on chip: the forward needs only a status word and the backward its per-block gradient partials, a few
