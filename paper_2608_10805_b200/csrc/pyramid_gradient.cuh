@@ -43,7 +43,7 @@ struct WGeom {
     int taps;                           // taps flushed at a time
     int deep_off, scr_off, misc_off, zero_end, smem;
     int nblocks, np, no_copy;
-    FastDiv d_n, d_tx[MAXL + 1], d_nt[MAXL + 1], d_hw[MAXL + 1], d_w[MAXL + 1];
+    FastDiv d_tx[MAXL + 1], d_nt[MAXL + 1], d_hw[MAXL + 1], d_w[MAXL + 1];
     int *alarm;
     unsigned tag;
 };
@@ -355,7 +355,6 @@ inline bool search_gradient(const Request &q, WGeom &best, double &best_cost) {
     g.B = q.B; g.C = q.C; g.H = q.H; g.W = q.W; g.HW = q.H * q.W; g.L = q.L; g.K = q.K;
     g.n = (q.W + 7) / 8;
     g.Px = g.n + 1;
-    g.d_n = make_fastdiv(g.n);
     const int th = up(q.H, 2);
     g.period = th + 4;
     g.Hl[0] = q.H; g.Wl[0] = q.W;

@@ -493,7 +493,7 @@ __device__ __forceinline__ void store8(T *p, const float *v, int left, int W) {
 // epilogue is short of registers.
 template <typename T>
 __device__ __noinline__ void group_by_taps(const char *window, unsigned row_bytes, const float *M, T *d, int pitch, int rows, int cols, float bias,
-                                           const float *__restrict__ add, int left, int KL, int chunk) {
+                                           const float *__restrict__ add, int left, int KL) {
     const int K = KL & 15, pad = (5 - K) / 2;
     const bool level = KL >= 16;
 #pragma unroll 1
@@ -506,7 +506,7 @@ __device__ __noinline__ void group_by_taps(const char *window, unsigned row_byte
             const int r = rq / 10, q = rq - r * 10, u = r - a - 2, v = q - b - 2, ul = r >> 1, vl = q >> 1, k = q + 2 * (oc >> 1);
             const bool base = u >= pad && u < 5 - pad && v >= pad && v < 5 - pad;
             if (!base && !(level && ul >= pad && ul < 5 - pad && vl >= pad && vl < 5 - pad)) continue;
-            sum = fmaf((float)*reinterpret_cast<const T *>(window + r * row_bytes + (k >> 3) * chunk + (k & 7) * 2), M[(a * 2 + b) * 100 + rq], sum);
+            sum = fmaf((float)*reinterpret_cast<const T *>(window + r * row_bytes + (k >> 3) * 128 + (k & 7) * 2), M[(a * 2 + b) * 100 + rq], sum);
         }
         sum += bias;
         if (add && oc < left) sum = fmaf(0.5f, add[oc >> 1], sum);
@@ -832,7 +832,7 @@ tensor_kernel(const __grid_constant__ KGeom g, const T *__restrict__ x, const T 
                     if (PANEL && g.deep) more = add + (u64)it.plane * (unsigned)(((g.H + 1) >> 1) * g.pitch) + (y >> 1) * g.pitch + (x0 >> 1) + 4 * j;
                     group_by_taps<T>(conv + (unsigned)row2 * row_bytes + j * 128 + img * 16, row_bytes, mis + 128, d, PANEL ? g.tw + 8 : g.W,
                                      g.H - y < 2 ? 1 : 2, PANEL ? 8 : g.W - 8 * j < 8 ? g.W - 8 * j : 8, bias, more, g.W - x0 - 8 * j,
-                                     g.K + (g.L >= 1 ? 16 : 0), 128);
+                                     g.K + (g.L >= 1 ? 16 : 0));
                 }
             }
             plane::fence_async_smem();
