@@ -343,10 +343,11 @@ pyramid_gradient_kernel(const __grid_constant__ WGeom g, const T *__restrict__ x
 
 // ------------------------------------------------------------------ host side
 inline int trips(const WGeom &g) { return g.W % 2 ? g.S * ((g.H + 7) / 8) * ((g.n + 3) / 4 + (g.Px + 3) / 4) : 0; }  // a loader's, of shifted rows
-// Microseconds of a backward call, fitted to the same shapes as the forward's (7 % off).
+// Microseconds of a backward call, fitted to the same plans as the forward's (4 % off; its choice is as fast as the other constants' was).
 inline double estimate(const WGeom &g, double grad_x) {
     const int rounds = (g.units + g.nblocks - 1) / g.nblocks, changes = (rounds + g.upc - 1) / g.upc, passes = (8 * g.S + g.nb - 1) / g.nb;
-    return 3.8 + 1.115 * grad_x + rounds * (1.24 + 0.317 * trips(g) + passes * (1.44 + 0.108 * (g.L - 2) + 0.45 * g.turns * g.th)) + 1.5 * changes;
+    const int blocks = (g.nb * g.Px * ((g.H + 3) / 4) + DEEP - 1) / DEEP;
+    return 3.37 + 1.224 * grad_x + rounds * (0.536 + 0.315 * trips(g) + (0.404 + 0.00065 * g.HW) * g.S + passes * (0.579 + 0.257 * (g.L - 2) + 0.224 * blocks + 0.1395 * g.turns * g.th)) + 1.54 * changes;
 }
 inline bool search_gradient(const Request &q, WGeom &best, double &best_cost) {
     using tensor::up;
@@ -418,11 +419,7 @@ inline bool search_gradient(const Request &q, WGeom &best, double &best_cost) {
                 if ((long long)h.upc * q.C > 0x3fffffffLL) continue;
                 h.units = h.upc * q.C;
                 h.nblocks = plane::NUM_SMS < h.units ? plane::NUM_SMS : h.units;
-                // What the candidates are compared by: the deep warps' passes and tiles and the shifted rows' round trips of each round of
-                // units, the sums of each channel
-                const int rounds = (h.units + h.nblocks - 1) / h.nblocks, changes = (rounds + h.upc - 1) / h.upc, passes = (8 * S + nb - 1) / nb;
-                const double per = 0.65 + 0.39 * trips(h) + passes * (0.46 + 0.08 * (q.L - 2) + 0.515 * turns * h.th);
-                const double cost = rounds * per + 1.7 * changes;
+                const double cost = estimate(h, 0.0);
                 if (!found || cost < best_cost) {
                     best = h;
                     best_cost = cost;

@@ -760,12 +760,15 @@ struct Request {
 };
 
 inline bool copied(const PGeom &g) { return g.vec > 1 && g.S * g.HW >= 1500; }
-// Microseconds of a plan, fitted to 390 shapes between 1 x 16 x 8 x 8 and 128 x 768 x 70 x 64 (7 % off): MMA jobs, tiles (dearer where
-// nothing overlaps them or the loaders take the registers), passes and shifted rows of each round of units, a B operand a channel.
+// Microseconds of a plan, by which the candidates and then the kernels of a layer are compared: MMA jobs, tiles (dearer where nothing
+// overlaps them or the loaders take the registers), passes, blocks of the analysis, octets and shifted rows of each round of units, a B operand
+// a channel.  Fitted to two plans each of 295 shapes between 2 x 24 x 4 x 4 and 128 x 800 x 110 x 64 (5 % off).  (A second set of
+// constants had chosen the plan; where the two differ, on one shape in five, this one's choice is 1.8 % faster among the layers it is taken for.)
 inline double estimate(const PGeom &g) {
     const int rounds = (g.units + g.nblocks - 1) / g.nblocks, changes = (rounds + g.upc - 1) / g.upc, passes = (8 * g.S + g.nb - 1) / g.nb;
-    const double tile = 0.0333 + (g.bufs == 1 && !g.direct ? 0.0316 : 0) + (copied(g) ? 0 : 0.0126), shift = g.vec == 1 ? 0.0014 : g.vec == 2 ? 0.00038 : 0;
-    return 6.0 + rounds * (0.225 + 0.39 * g.T * g.n + tile * g.S * g.items + 0.2 * passes * (g.L + 1) + shift * g.S * g.HW) + 0.85 * changes;
+    const int blocks = (g.nb * (g.direct ? g.n : g.Pc) * ((g.H + 3) / 4) + DEEP - 1) / DEEP;  // a deep thread's, of the analysis of one pass
+    const double tile = (g.K == 3 ? 0.0182 : 0.0259) + (g.bufs == 1 && !g.direct ? 0.0388 : 0) + (copied(g) ? 0 : 0.0112), shift = g.vec == 1 ? 0.00138 : g.vec == 2 ? 0.00049 : 0;
+    return 6.19 + rounds * (0.301 * g.T * g.n + (0.61 + tile * g.items + shift * g.HW) * g.S + (0.194 * (g.L + 1) + 0.146 * blocks) * passes) + 0.65 * changes;
 }
 inline bool search(const Request &q, PGeom &best, double &best_cost) {
     using tensor::up;
@@ -834,13 +837,7 @@ inline bool search(const Request &q, PGeom &best, double &best_cost) {
                 if ((long long)h.upc * q.C > 0x3fffffffLL) continue;
                 h.units = h.upc * q.C;
                 h.nblocks = plane::NUM_SMS < h.units ? plane::NUM_SMS : h.units;
-                // What the candidates are compared by: tiles, blocks of the analysis, the deep warps' barriers and shifted rows of each round
-                // of units, a B operand a channel
-                const int rounds = (h.units + h.nblocks - 1) / h.nblocks, changes = (rounds + h.upc - 1) / h.upc, passes = (8 * S + nb - 1) / nb;
-                const double blocks = 8.0 * S * ((q.H + 3) / 4) * h.Pc, odd = h.vec == 4 ? 0 : S * q.H * q.W / 8.0;
-                const double per = 0.0003 * h.T * h.n + (0.067 + (h.bufs == 1 && !h.direct ? 0.018 : 0)) * S * h.items + 0.0053 * blocks +
-                                   0.205 * passes * (q.L + 1) + 0.0086 * odd;
-                const double cost = 5.9 + rounds * per + 0.65 * changes;
+                const double cost = estimate(h);
                 ahead = ahead || h.direct;
                 if (!found || cost < best_cost) {
                     best = h;
@@ -873,7 +870,6 @@ inline bool plan(const Request &q, PGeom &out, double &cost) {  // searched once
     Entry e = {};
     e.q = q;
     e.ok = search(q, e.g, e.cost);
-    if (e.ok) e.cost = estimate(e.g);
     {
         std::lock_guard<std::mutex> lock(mu);
         if (cache.size() >= 256) cache.clear();

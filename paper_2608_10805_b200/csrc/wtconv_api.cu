@@ -409,25 +409,35 @@ bool wide_serves(const wtconv_desc *d, bool on_chip) {
            panels_win(d, g.cost);
 }
 
-// What the block-per-plane kernels take for a 16-bit layer of several levels, fitted like on_chip_us (10 % off forward, 14 % backward).
+// What the block-per-plane kernels take for a 16-bit layer of several levels, in microseconds, from their plan: rounds of units, a thread's
+// tiles of a round, rows fetched pixel by pixel; fitted to 320 shapes (6 % off).
 double plane_deep_us(const wtconv_desc *d, int bwd) {
-    const double planes = (double)d->B * d->C * 1e-3, tiles = planes * ((d->W + 3) / 4 * 4) * ((d->H + 3) / 4 * 4) * 1e-3;
-    const bool odd = d->W % 4 != 0, k3 = d->k == 3, big = d->H * d->W > 2200;
+    wt::plane::Geom g;
+    const int eb = (int)elem_bytes(d->dtype);
+    const bool split = bwd && !wt::plane::plan_bwd_fused(d->B, d->C, d->H, d->W, d->L, eb, g);
+    if ((!bwd || split) && !(bwd ? wt::plane::plan_wgrad : wt::plane::plan_forward)(d->B, d->C, d->H, d->W, d->L, eb, g, 0, 5)) return 0;
+    const double planes = (double)d->B * d->C * 1e-3, tiles = planes * ((d->W + 3) / 4 * 4) * ((d->H + 3) / 4 * 4) * 1e-3, first = planes < 1 ? planes : 1;
+    const int rounds = (g.units + g.nblocks - 1) / g.nblocks, all = g.NPL * (g.lvl_start[d->L + 1] + g.nbase), more = d->L - 2;
+    const double work = (double)((all + g.nthreads - 1) / g.nthreads) * g.th * g.blocks_per_sm, px = (double)g.NPL * d->H * d->W / g.nthreads;
+    const bool odd = d->W % 4 != 0, k3 = d->k == 3;
     if (bwd)
-        return 11.1 + 7.5 * k3 + (6.0 + 4.5 * odd + 2.9 * !k3 + 0.1 * (d->L > 2) + 1.4 * big) * tiles + 1.08 * (d->L - 2) * planes + 1.1 * (d->L - 2) +
-               8.0 * (planes < 1 ? planes : 1);
-    return 7.3 + 3.0 * k3 + (2.55 + 1.59 * odd + 1.05 * !k3 + 0.42 * (d->L > 2) + 0.43 * big) * tiles + (0.75 + 0.35 * (d->L - 2)) * planes + 0.5 * (d->L - 2);
+        return 7.2 + 3.4 * k3 + 0.97 * more + (-0.72 - 1.97 * k3 + 1.65 * odd + 1.32 * (odd && !k3) + 0.25 * (more > 0) + 7.76 * split + 5.4 * (g.th == 8)) * tiles +
+               (0.56 + 0.61 * more) * planes + 6.6 * first + 3.6 * split + rounds * (3.66 + 0.0476 * work + 0.09 * more + (g.bulk ? 0 : 0.137) * px - 0.0363 * g.blocks_per_sm * px);
+    return 3.7 + 2.27 * k3 + 0.66 * more + (2.39 - 0.91 * k3 + 0.99 * odd + 0.17 * (odd && !k3) + 0.35 * (more > 0)) * tiles + (0.53 + 0.26 * more) * planes + 2.0 * first +
+           rounds * (1.33 + 0.0154 * work + (g.bulk ? 0 : 0.083) * px);
 }
-// Several levels: taken where the estimate is 15 % (backward 20 %) below that of the block-per-plane kernels.  Over 390 random shapes
-// that takes 91 forward, which gain 1.26 x (geometric mean; four lose more than 2 %), and 89 backward: 1.45 x, none loses.  Taking all
-// would lose a tenth: units are eight images of a channel, so small batches and few units leave the SMs empty.
+// Several levels: taken where their estimate is 8 - 13 % below that of the block-per-plane kernels (units are eight images of a channel: small
+// batches and few units leave the SMs empty).  Over 630 random shapes, a third of them beyond the fitted range (up to 8 levels, planes of 4
+// columns or 128 rows, single images), that takes 292 forward, which gain 1.23 x (geometric mean), and 312 backward: 1.30 x.  Ten and eleven of
+// them lose more than 2 %: layers of one or two units a block, most of them with rows that are not 8-byte multiples, 17 x 45 x 31 x 20 (five
+// levels, forward 9.5 -> 10.4 us), 18 x 81 x 15 x 62 (15.6 -> 18.8), 9 x 138 x 19 x 17 (3 x 3, backward 27.1 -> 30.5), 88 x 582 x 7 x 7 (180 -> 194).
 bool pyramid_serves(const wtconv_desc *d, bool on_chip, int bwd) {
     if (d->dtype == WTCONV_F32 || !on_chip || d->L < 2 || (d->flags & ~WTCONV_FLAG_TEST_NO_COPY)) return false;
     wt::pyramid::PGeom g;
     wt::pyramid::WGeom w;
     double cost;
-    if (bwd) return wt::pyramid::plan_gradient(pyramid_request(d), w, cost) && 1.2 * cost < plane_deep_us(d, 1);
-    return wt::pyramid::plan(pyramid_request(d), g, cost) && 1.15 * cost < plane_deep_us(d, 0);
+    if (bwd) return wt::pyramid::plan_gradient(pyramid_request(d), w, cost) && (d->W % 2 ? 1.13 : 1.1) * cost < plane_deep_us(d, 1);
+    return wt::pyramid::plan(pyramid_request(d), g, cost) && (d->W % 4 ? 1.12 : 1.08) * cost < plane_deep_us(d, 0);
 }
 
 // 7 x 7 kernels on whole planes: block per plane, or the per-level kernels.  The latter win where planes are few (a block per plane
