@@ -142,9 +142,10 @@ wtconv_status wtconv_level_shape(const wtconv_desc *desc, int level, int32_t *Hl
 wtconv_status wtconv_workspace_bytes(const wtconv_desc *desc, size_t *fwd_bytes, size_t *bwd_bytes);
 
 /* Name of the kernels a descriptor dispatches to ("team" = small planes, several per thread team; "plane" =
- * one block per whole plane in shared memory; "window" = large planes cut into windows with levels 1-2 on chip;
- * "tiled" = per-level tiled kernels, and the name of all 7 x 7 kernels, whose planes of up to about 70 x 70 stay on one SM too
- * (wtconv_plan_describe tells which kernels run); "tensor" = base convolution, level 1 and synthesis as one contraction on the
+ * whole planes in shared memory, one block for one or more of them: all levels as FP32 tiles, or, 16-bit activations with two or more
+ * levels, base convolution and level 1 on the tensor cores beside them (wtconv_plan_describe tells which, a direction each:
+ * "fwd[pyramid", "bwd[pyramid gradients"); "window" = large planes cut into windows with levels 1-2 on chip;
+ * "tiled" = per-level tiled kernels; "tensor" = base convolution, level 1 and synthesis as one contraction on the
  * tensor cores (16-bit activations), "panel" = the same in column panels of wide planes, levels >= 2 through HBM;
  * "reference-chain" = the comparator).  Where the two directions are served differently: both names, forward/backward
  * ("team/tensor").  Host call; returns NULL for an invalid desc. */

@@ -640,7 +640,7 @@ const char *family_name(const wtconv_desc *d) {
         const wtconv_desc d5 = as_k5(d);
         return family_name(&d5);
     }
-    return use_ref_chain(d) ? "reference-chain" : use_team_path(d) ? "team" : use_plane_path(d) && d->k != 7 ? "plane" : use_window_path(d) ? "window" : "tiled";
+    return use_ref_chain(d) ? "reference-chain" : use_team_path(d) ? "team" : use_plane_path(d) ? "plane" : use_window_path(d) ? "window" : "tiled";
 }
 void describe_family(const wtconv_desc *d, char *buf, size_t n) {
     if (use_k3_embedding(d)) {
