@@ -145,7 +145,8 @@ wtconv_status wtconv_workspace_bytes(const wtconv_desc *desc, size_t *fwd_bytes,
  * whole planes in shared memory, one block for one or more of them: all levels as FP32 tiles, or, 16-bit activations with two or more
  * levels, base convolution and level 1 on the tensor cores beside them (wtconv_plan_describe tells which, a direction each:
  * "fwd[pyramid", "bwd[pyramid gradients"); "window" = large planes cut into windows with levels 1-2 on chip;
- * "tiled" = per-level tiled kernels; "tensor" = base convolution, level 1 and synthesis as one contraction on the
+ * "tiled" = per-level tiled kernels, and the name of all 7 x 7 layers, whose planes of up to about 70 x 70 run on the block-per-plane
+ * kernels where planes are many (wtconv_plan_describe begins with the family that runs); "tensor" = base convolution, level 1 and synthesis as one contraction on the
  * tensor cores (16-bit activations), "panel" = the same in column panels of wide planes, levels >= 2 through HBM;
  * "reference-chain" = the comparator).  Where the two directions are served differently: both names, forward/backward
  * ("team/tensor").  Host call; returns NULL for an invalid desc. */

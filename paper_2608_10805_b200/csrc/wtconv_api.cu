@@ -640,7 +640,7 @@ const char *family_name(const wtconv_desc *d) {
         const wtconv_desc d5 = as_k5(d);
         return family_name(&d5);
     }
-    return use_ref_chain(d) ? "reference-chain" : use_team_path(d) ? "team" : use_plane_path(d) ? "plane" : use_window_path(d) ? "window" : "tiled";
+    return use_ref_chain(d) ? "reference-chain" : use_team_path(d) ? "team" : use_plane_path(d) && d->k != 7 ? "plane" : use_window_path(d) ? "window" : "tiled";
 }
 void describe_family(const wtconv_desc *d, char *buf, size_t n) {
     if (use_k3_embedding(d)) {
@@ -665,7 +665,9 @@ void describe_family(const wtconv_desc *d, char *buf, size_t n) {
     } else if (use_plane_path(d))
         wt::plane::describe(d->B, d->C, d->H, d->W, d->L, (int)elem_bytes(d->dtype), d->flags >> 8, buf, n, d->k);
     else
-        snprintf(buf, n, "tiled fwd[%d launches] bwd[%d launches]", d->L + 1, d->L + 2);
+        snprintf(buf, n, "tiled fwd[%d launches] bwd[%d launches]%s", d->L + 1, d->L + 2,
+                 d->k == 7 && !(d->flags & WTCONV_FLAG_TILED_ONLY) && !(d->flags >> 8) && wt::plane::supported(d->H, d->W, 7, d->L, d->dtype)
+                     ? " (faster here than the block-per-plane kernels)" : "");
 }
 void family_launches(const wtconv_desc *d, int (&n)[2]) {
     if (use_k3_embedding(d)) {  // the k = 5 path's launches + the table kernel (+ the gradient copy in the backward)

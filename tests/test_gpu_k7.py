@@ -20,14 +20,33 @@ SHAPES = [(3, 5, 7, 7, 3), (2, 16, 14, 14, 1), (2, 8, 28, 28, 2), (3, 4, 33, 29,
 @pytest.mark.parametrize("B,C,H,W,L", SHAPES)
 def test_against_the_oracle(B, C, H, W, L, dtype):
     wl = Workload("k7_%dx%d_L%d" % (H, W, L), B, C, H, W, 7, L, dtype, 700 + H + W)
-    flags = wt.FLAG_NO_TEAM  # (few planes: the per-level kernels otherwise)
-    assert "plane" in wt.wtconv_plan_describe(wt.make_desc(B, C, H, W, 7, L, wt.DTYPE_NAMES[dtype], flags))
+    assert "plane" in wt.wtconv_plan_describe(wt.make_desc(B, C, H, W, 7, L, wt.DTYPE_NAMES[dtype]))
     I = inputs.make_inputs(wl, bias=True)
-    assert_close(wl, run_gpu(wl, I, flags=flags), run_oracle(wl, I))
+    assert_close(wl, run_gpu(wl, I), run_oracle(wl, I))
 
 
 @pytest.mark.parametrize("seed", range(12))
 def test_against_the_per_level_kernels(seed):
+    rng = np.random.default_rng(seed)
+    H, W, L = int(rng.integers(2, 66)), int(rng.integers(2, 66)), int(rng.integers(0, 6))
+    wl = Workload("k7_%d" % seed, int(rng.integers(1, 7)), int(rng.integers(1, 40)), H, W, 7, L, ["f32", "f16", "bf16"][seed % 3], 40 + seed)
+    I = inputs.make_inputs(wl, bias=seed % 2 == 0)
+    a, b = run_gpu(wl, I), run_gpu(wl, I, flags=wt.FLAG_TILED_ONLY)
+    assert_close(wl, a, b, tol=2 * TOL[wl.dtype])  # each side is within the tolerance of the exact result
+
+
+@pytest.mark.parametrize("dtype", ["f32", "f16", "bf16"])
+@pytest.mark.parametrize("B,C,H,W,L", SHAPES)
+def test_block_per_plane_kernels_against_the_oracle(B, C, H, W, L, dtype):
+    """Few planes take the per-level kernels, unless these are kept away."""
+    wl = Workload("k7_%dx%d_L%d" % (H, W, L), B, C, H, W, 7, L, dtype, 700 + H + W)
+    assert wt.wtconv_plan_describe(wt.make_desc(B, C, H, W, 7, L, wt.DTYPE_NAMES[dtype], wt.FLAG_NO_TEAM)).startswith("plane")
+    I = inputs.make_inputs(wl, bias=True)
+    assert_close(wl, run_gpu(wl, I, flags=wt.FLAG_NO_TEAM), run_oracle(wl, I))
+
+
+@pytest.mark.parametrize("seed", range(12))
+def test_block_per_plane_kernels_against_the_per_level_kernels(seed):
     rng = np.random.default_rng(seed)
     H, W, L = int(rng.integers(2, 66)), int(rng.integers(2, 66)), int(rng.integers(0, 6))
     wl = Workload("k7_%d" % seed, int(rng.integers(1, 7)), int(rng.integers(1, 40)), H, W, 7, L, ["f32", "f16", "bf16"][seed % 3], 40 + seed)
