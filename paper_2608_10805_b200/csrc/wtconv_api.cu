@@ -354,6 +354,13 @@ bool static_takes_family(const wtconv_desc *d) {
     const Route &r = route(d);
     return r.bytes[1] > (size_t)WTCONV_STATIC_SCRATCH_BYTES && r.family_bytes[1] <= (size_t)WTCONV_STATIC_SCRATCH_BYTES;
 }
+// 7 x 7 layers whose per-level kernels need more than the built-in array: the block-per-plane kernels need partial sums only.
+wtconv_desc static_desc(const wtconv_desc *d) {
+    wtconv_desc on_planes = *d;
+    on_planes.flags |= WTCONV_FLAG_NO_TEAM;
+    const bool takes = d->k == 7 && bwd_ws_bytes(d) > (size_t)WTCONV_STATIC_SCRATCH_BYTES && bwd_ws_bytes(&on_planes) <= (size_t)WTCONV_STATIC_SCRATCH_BYTES;
+    return takes ? on_planes : *d;
+}
 
 // What the kernels that keep a plane on one SM (or a team of them) take for a 16-bit layer with at most one level, in
 // microseconds: fitted to 3000 shapes between 1 x 16 x 7 x 7 and 128 x 768 x 64 x 64 (13 % off; k = 3 in 5 x 5 tables 11 %).
@@ -1024,11 +1031,14 @@ wtconv_status wtconv_read_status(const wtconv_desc *d, void *workspace, int32_t 
     if (st != WTCONV_OK) return st;
     if (!h_flag) return WTCONV_ERR_NULL;
     bool wide = use_wide_path(d);
+    wtconv_desc in_scratch;
     if (!workspace) {  // the scratch array built into the library (wtconv_backward_static)
         void *scratch = nullptr;
         if ((st = check_device()) != WTCONV_OK) return st;
         if ((st = static_scratch_for_current_device(&scratch)) != WTCONV_OK) return st;
         workspace = scratch;
+        in_scratch = static_desc(d);
+        d = &in_scratch;
         wide = wide && !static_takes_family(d);
     }
     if ((uintptr_t)workspace & (ALIGN - 1)) return WTCONV_ERR_ALIGNMENT;
@@ -1063,6 +1073,8 @@ wtconv_status wtconv_backward_static(const wtconv_desc *d, const void *x, const 
                                      void *stream) {
     wtconv_status st = validate_desc(d);
     if (st != WTCONV_OK) return st;
+    const wtconv_desc in_scratch = static_desc(d);
+    d = &in_scratch;
     const bool family = static_takes_family(d);
     if (!family && bwd_ws_bytes(d) > (size_t)WTCONV_STATIC_SCRATCH_BYTES) return WTCONV_ERR_WORKSPACE;  // shape needs more scratch than is built in
     if ((st = check_device()) != WTCONV_OK) return st;

@@ -110,6 +110,16 @@ def test_seven_by_seven_kernels_take_whole_planes_where_that_is_faster(lib):
         assert wt.wtconv_launch_count(d) == ((1, 3) if plane else (d.L + 1, d.L + 2)), shape
 
 
+def test_static_backward_takes_seven_by_seven_layers_whose_per_level_kernels_need_more(lib):
+    """The block-per-plane kernels keep partial sums only: a misaligned activation is refused behind the size check, before any launch."""
+    P = ctypes.c_void_p
+    a = P(256)  # never dereferenced
+    for shape in ((4, 121, 55, 137, 7, 1, "f16"), (1, 164, 55, 125, 7, 2, "bf16")):
+        d = wt.make_desc(*shape)
+        assert wt.wtconv_plan_describe(d).startswith("tiled") and wt.wtconv_workspace_bytes(d)[1] > wt.STATIC_SCRATCH_BYTES
+        assert lib.wtconv_backward_static(ctypes.byref(d), P(264), a, a, a, None, a, a, P(1 << 40), a, a, None, a, a, None) != 7
+
+
 def test_scratch_memory_accounting(lib):
     """Device memory the layer needs beyond its inputs and outputs.  Whole-plane kernels keep every intermediate
     on chip: the forward needs only a status word and the backward its per-block gradient partials, a few
