@@ -16,6 +16,7 @@ pytestmark = pytest.mark.gpu
     (Workload("ag_plane", 2, 4, 28, 28, 5, 2, "f32", 31), True),
     (Workload("ag_odd_bf16", 3, 5, 7, 7, 5, 2, "bf16", 32), False),
     (Workload("ag_tiled_k3", 2, 3, 20, 33, 3, 2, "f32", 33), True),
+    (Workload("ag_pyramid", 61, 64, 14, 13, 5, 5, "bf16", 35), True),
     (Workload("ag_base_only", 2, 3, 9, 12, 5, 0, "f32", 34), False),
 ], ids=lambda v: v.name if isinstance(v, Workload) else str(v))
 def test_module_gradients_match_oracle(wl, bias):

@@ -18,6 +18,8 @@ CASES = [
     Workload("conc_b", 2, 6, 56, 56, 5, 3, "bf16", 62),
     Workload("conc_c", 1, 3, 90, 75, 5, 3, "f32", 63),   # tiled path
     Workload("conc_d", 6, 16, 7, 7, 5, 2, "f16", 64),
+    Workload("conc_e", 61, 64, 14, 13, 5, 5, "bf16", 65),  # several levels, partly on the tensor cores
+    Workload("conc_f", 61, 64, 14, 13, 5, 5, "bf16", 66),  # (the same kernels at once on two streams)
 ]
 
 

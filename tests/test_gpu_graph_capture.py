@@ -20,6 +20,7 @@ pytestmark = pytest.mark.gpu
 @pytest.mark.parametrize("wl", [
     Workload("graph_stage4", 4, 16, 7, 7, 5, 2, "bf16", 41),     # team kernels
     Workload("graph_stage2", 2, 8, 28, 28, 5, 2, "f32", 42),
+    Workload("graph_pyramid", 61, 64, 14, 13, 5, 5, "bf16", 44),  # several levels, partly on the tensor cores
     Workload("graph_tiled", 1, 3, 90, 75, 5, 3, "f32", 43),      # tiled path (several launches per call)
 ], ids=lambda w: w.name)
 def test_step_replays_from_a_cuda_graph(wl):

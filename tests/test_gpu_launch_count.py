@@ -8,6 +8,7 @@ pytestmark = pytest.mark.gpu
 
 SHAPES = [
     (2, 8, 56, 56, 5, 3, "f32", 0, "plane"), (3, 10, 40, 36, 5, 3, "f32", 0, "plane"), (12, 32, 7, 7, 5, 1, "f32", 0, "team"),
+    (64, 64, 20, 24, 7, 2, "f32", 0, "tiled"), (61, 64, 14, 13, 5, 5, "bf16", 0, "plane"),  # (block-per-plane kernels; several levels on tensor cores)
     (2, 8, 56, 56, 3, 3, "f32", 0, "plane"), (2, 6, 20, 24, 7, 2, "f32", 0, "tiled"), (1, 2, 99, 201, 5, 2, "f32", 0, "window"),
     (1, 2, 225, 225, 5, 5, "f32", 0, "window"), (1, 2, 225, 225, 3, 4, "f32", 0, "window"),
     (24, 40, 31, 30, 5, 1, "bf16", 0, "tensor"), (33, 96, 50, 56, 3, 1, "bf16", 0, "tensor"), (33, 48, 50, 56, 3, 1, "bf16", 0, "plane/tensor"), (128, 768, 7, 7, 5, 1, "bf16", 0, "team/tensor"),

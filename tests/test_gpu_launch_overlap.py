@@ -19,6 +19,7 @@ LAYERS = [Workload("ov_plane_28", 6, 24, 28, 28, 5, 2, "bf16", 81),   # fused ba
           Workload("ov_team_7", 12, 32, 7, 7, 5, 2, "bf16", 86),      # team kernels
           Workload("ov_split_40", 3, 10, 40, 36, 5, 3, "f32", 83),    # split backward (weight-gradient + input-gradient kernels)
           Workload("ov_plane_14", 8, 40, 14, 14, 5, 1, "f16", 84),
+          Workload("ov_pyramid_14", 61, 64, 14, 13, 5, 5, "bf16", 87),  # several levels, partly on the tensor cores, both directions
           Workload("ov_tiled_k7", 2, 6, 20, 24, 7, 2, "f32", 85)]     # per-level kernels between the persistent ones
 
 
@@ -26,6 +27,7 @@ def test_layers_share_one_workspace_back_to_back():
     descs = [wt.make_desc(w.B, w.C, w.H, w.W, w.k, w.L, wt.DTYPE_NAMES[w.dtype], 0) for w in LAYERS]
     plans = [wt.wtconv_plan_name(d) for d in descs]
     assert {"plane", "team", "tiled", "tensor"} <= {n for p in plans for n in p.split("/")}, plans
+    assert any("fwd[pyramid" in t and "bwd[pyramid gradients" in t for t in map(wt.wtconv_plan_describe, descs))
     nbytes = max(max(wt.wtconv_workspace_bytes(d)) for d in descs)
     ws = torch.full((nbytes,), 0xFF, dtype=torch.uint8, device="cuda")
     Is = [inputs.make_inputs(w) for w in LAYERS]

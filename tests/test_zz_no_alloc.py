@@ -36,6 +36,7 @@ def _grads_like(x, w0, s0, b0, wl_, sl):
                                 Workload("na_odd", 3, 5, 7, 7, 5, 2, "bf16", 42),
                                 Workload("na_team", 6, 16, 7, 7, 5, 2, "bf16", 43),         # team kernels
                                 Workload("na_tensor", 6, 16, 7, 7, 5, 1, "bf16", 47),       # tensor-core kernels
+                                Workload("na_pyramid", 61, 64, 14, 13, 5, 5, "bf16", 49),   # several levels, partly on the tensor cores
                                 Workload("na_tiled", 1, 3, 90, 75, 5, 3, "f32", 44)],      # tiled path: Z^l and carriers in the array
                          ids=lambda w: w.name)
 def test_static_scratch_backward_matches_workspace_backward_twice(wl):
