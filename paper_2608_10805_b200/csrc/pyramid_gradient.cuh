@@ -436,36 +436,14 @@ inline bool search_gradient(const Request &q, WGeom &best, double &best_cost) {
     }
     return true;
 }
-struct GradientEntry {
-    Request q;
-    bool ok;
-    double cost;
-    WGeom g;
-};
-inline bool plan_gradient(const Request &q, WGeom &out, double &cost) {  // searched once and kept (bounded)
-    static std::mutex mu;
-    static std::vector<GradientEntry> cache;
-    {
-        std::lock_guard<std::mutex> lock(mu);
-        for (const GradientEntry &e : cache)
-            if (e.q == q) {
-                if (e.ok) { out = e.g; cost = e.cost; }
-                return e.ok;
-            }
-    }
-    GradientEntry e = {};
-    e.q = q;
-    PGeom flip;
-    double grad_x;
-    e.ok = plan(q, flip, grad_x) && search_gradient(q, e.g, e.cost);
-    if (e.ok) e.cost = estimate(e.g, grad_x);
-    {
-        std::lock_guard<std::mutex> lock(mu);
-        if (cache.size() >= 256) cache.clear();
-        cache.push_back(e);
-    }
-    if (e.ok) { out = e.g; cost = e.cost; }
-    return e.ok;
+inline bool plan_gradient(const Request &q, WGeom &out, double &cost) {
+    return kept_plan(q, out, cost, [&](WGeom &g, double &c) {
+        PGeom flip;
+        double grad_x;
+        if (!plan(q, flip, grad_x) || !search_gradient(q, g, c)) return false;
+        c = estimate(g, grad_x);
+        return true;
+    });
 }
 inline size_t backward_bytes(const Request &q) {
     WGeom g;

@@ -190,16 +190,6 @@ __device__ __forceinline__ void prefetch_planes(const G &g, const T *__restrict_
 }
 
 // ------------------------------------------------------------------ levels >= 2
-// One folded weight (Eq. 8) of base convolution and level 1: as tensor::folded_weight.
-__device__ __forceinline__ float folded(const PGeom &g, int c, int e, bool flip, const float *__restrict__ w0, const float *__restrict__ s0,
-                                        const float *__restrict__ wl, const float *__restrict__ sl) {
-    const int KK = g.K * g.K, pad = (5 - g.K) / 2;
-    const int cls = e / 25, t = e - cls * 25, tt = flip ? 24 - t : t, u = tt / 5 - pad, v = tt % 5 - pad;
-    if (u < 0 || u >= g.K || v < 0 || v >= g.K) return 0.f;
-    if (cls == 0) return __ldg(w0 + (size_t)c * KK + u * g.K + v) * __ldg(s0 + c);
-    return __ldg(wl + ((size_t)c * 4 + cls - 1) * KK + u * g.K + v) * __ldg(sl + (size_t)c * 4 + cls - 1);
-}
-
 // Eq. 5 with its factor inside the second sums (a power of two: the results are haar_butterfly's, but no sum is larger than they are).
 __device__ __forceinline__ Haar4 butterfly(float a, float b, float c, float d) {
     const float s0 = a + b, d0 = a - b, s1 = 0.5f * (c + d), d1 = 0.5f * (c - d);
@@ -713,7 +703,7 @@ pyramid_kernel(const __grid_constant__ PGeom g, const T *__restrict__ x, const _
             const bool change = u == u_begin || k == 0;
             float wreg = 0.f, breg = 0.f;
             if (change) {
-                wreg = lt < 125 ? folded(g, c, lt, FLIP, w0, s0, wl, sl) : 0.f;
+                wreg = lt < 125 ? tensor::folded_weight(g, c, lt, FLIP, w0, s0, wl, sl) : 0.f;
                 if (lt == 0 && !FLIP && b0) breg = __ldg(s0 + c) * __ldg(b0 + c);
             }
             if (!g.direct) wait_for(freed + buf, phase ^ 1u);
@@ -850,13 +840,15 @@ inline bool search(const Request &q, PGeom &best, double &best_cost) {
     return found;
 }
 
-struct Entry {
-    Request q;
-    bool ok;
-    double cost;
-    PGeom g;
-};
-inline bool plan(const Request &q, PGeom &out, double &cost) {  // searched once and kept (bounded)
+// A plan is searched once and kept (bounded); `find(geom, cost)` searches.
+template <typename G, typename F>
+bool kept_plan(const Request &q, G &out, double &cost, F find) {
+    struct Entry {
+        Request q;
+        bool ok;
+        double cost;
+        G g;
+    };
     static std::mutex mu;
     static std::vector<Entry> cache;
     {
@@ -869,7 +861,7 @@ inline bool plan(const Request &q, PGeom &out, double &cost) {  // searched once
     }
     Entry e = {};
     e.q = q;
-    e.ok = search(q, e.g, e.cost);
+    e.ok = find(e.g, e.cost);
     {
         std::lock_guard<std::mutex> lock(mu);
         if (cache.size() >= 256) cache.clear();
@@ -900,6 +892,9 @@ cudaError_t run(const Request &q, const T *x, const Parameters &p, const Gradien
     const bool copies = copied(g);
     if (q.K == 3) return copies ? launch<T, FLIP, FEW, 3>(g, x, p, grad, out, ws, st) : launch<T, FLIP, MANY, 3>(g, x, p, grad, out, ws, st);
     return copies ? launch<T, FLIP, FEW, 5>(g, x, p, grad, out, ws, st) : launch<T, FLIP, MANY, 5>(g, x, p, grad, out, ws, st);
+}
+inline bool plan(const Request &q, PGeom &out, double &cost) {
+    return kept_plan(q, out, cost, [&](PGeom &g, double &c) { return search(q, g, c); });
 }
 
 inline int describe(const Request &q, char *buf, size_t n) {

@@ -411,7 +411,8 @@ __device__ __forceinline__ void repack(char *arr, const char *raw, const Item *i
 __device__ __forceinline__ float haar_sign(int sub, int a, int b) { return ((sub & 1) & a) ^ ((sub >> 1) & b) ? -1.f : 1.f; }
 
 // One folded weight (Eq. 8) of channel c: classes base, LL, LH, HL, HH x 25 taps (3 x 3 kernels sit in the middle of 5 x 5).
-__device__ __forceinline__ float folded_weight(const KGeom &g, int c, int e, bool flip, const float *__restrict__ w0, const float *__restrict__ s0,
+template <typename G>
+__device__ __forceinline__ float folded_weight(const G &g, int c, int e, bool flip, const float *__restrict__ w0, const float *__restrict__ s0,
                                                const float *__restrict__ wl, const float *__restrict__ sl) {
     const int KK = g.K * g.K, pad = (5 - g.K) / 2;
     const int cls = e / 25, t = e - cls * 25, tt = flip ? 24 - t : t, u = tt / 5 - pad, v = tt % 5 - pad;
