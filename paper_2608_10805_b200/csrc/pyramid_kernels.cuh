@@ -341,6 +341,7 @@ __device__ __noinline__ void pixels_by_taps(const T *__restrict__ plane, int H, 
             if (!base && !(ul >= pad && ul < 5 - pad && vl >= pad && vl < 5 - pad)) continue;
             const float p = (unsigned)yy < (unsigned)H && (unsigned)xx < (unsigned)W ? (float)plane[yy * W + xx] : 0.f;
             sum = fmaf(p, M[(a * 2 + b) * 100 + rq], sum);
+            if (sum != sum) break;  // (a NaN stays one)
         }
         d[a * W + oc] = (T)fmaf(0.5f, more[oc >> 1], sum + bias);
     }
@@ -370,11 +371,13 @@ __device__ __forceinline__ int block_near(const Gradients &d, int v) {
     while (b > 0 && begin(b) > v) --b;
     return b;
 }
-// One class (0: base convolution, 1 .. 4: level 1) of a channel's weight gradients by a warp, every product on its own, from global memory: the
+// One class (0: base convolution, 1 .. 4: level 1) of a channel's weight gradients by a warp whose sums are not all finite.  The
 // contraction multiplies the zeros around the planes (to whole groups of 16 rows and chunks of 8 columns) too, so that an infinity or
-// NaN has reached taps that do not meet it.  x, go: the channel's planes of the first image.  Returns tap `lane` of 5 x 5.
+// NaN has reached taps that do not meet it.  Taps that do meet one inside the plane keep their sum (any product with it is not finite);
+// the others are added again, every product on its own, from global memory.  x, go: the channel's planes of the first image; sum: tap
+// `lane` of 5 x 5 (lanes < 25).  The search for what a tap meets ends when every tap has met something: with NaNs everywhere at once.
 template <typename T>
-__device__ __noinline__ double taps_of_class(const PGeom &g, const T *__restrict__ x, const T *__restrict__ go, int cls, int lane) {
+__device__ __noinline__ double taps_of_class(const PGeom &g, const T *__restrict__ x, const T *__restrict__ go, int cls, int lane, double sum) {
     const int s = cls ? 1 : 0, h = (g.H + s) >> s, w = (g.W + s) >> s;
     const float sy = (cls - 1) & 1 ? -1.f : 1.f, sx = (cls - 1) & 2 ? -1.f : 1.f;
     const size_t image = (size_t)g.C * g.HW;
@@ -382,30 +385,48 @@ __device__ __noinline__ double taps_of_class(const PGeom &g, const T *__restrict
         auto pixel = [&](int y, int xx) { return y < g.H && xx < g.W ? (float)q[y * g.W + xx] : 0.f; };
         return cls ? 0.5f * ((pixel(2 * i, 2 * j) + sx * pixel(2 * i, 2 * j + 1)) + sy * (pixel(2 * i + 1, 2 * j) + sx * pixel(2 * i + 1, 2 * j + 1))) : pixel(i, j);
     };
-    double total = 0.0;
+    unsigned todo = __ballot_sync(0xffffffffu, lane < 25 && !(fabs(sum) < 1e300));
 #pragma unroll 1
-    for (int b = 0; b < g.B; ++b, x += image, go += image) {
-        float acc[25];
-#pragma unroll
-        for (int t = 0; t < 25; ++t) acc[t] = 0.f;
-#pragma unroll 1
+    for (int b = 0; b < g.B && todo; ++b) {
+        const T *px = x + b * image, *pg = go + b * image;
+        unsigned met = 0;
+#pragma unroll 4
         for (int e = lane; e < h * w; e += 32) {
             const int i = e / w, j = e - i * w;
-            const float v = at(go, i, j);
-#pragma unroll
-            for (int t = 0; t < 25; ++t) {
-                const int y = i + t / 5 - 2, xx = j + t % 5 - 2;
-                if ((unsigned)y < (unsigned)h && (unsigned)xx < (unsigned)w) acc[t] = fmaf(v, at(x, y, xx), acc[t]);
-            }
+            const bool in_x = !(fabsf(at(px, i, j)) <= 3.4028235e38f), in_g = !(fabsf(at(pg, i, j)) <= 3.4028235e38f);
+            if (in_x || in_g)
+#pragma unroll 1
+                for (int t = 0; t < 25; ++t) {  // the partner: grad_out's coefficient t off x's, x's off grad_out's
+                    const int dy = t / 5 - 2, dx = t % 5 - 2;
+                    if ((in_x && (unsigned)(i - dy) < (unsigned)h && (unsigned)(j - dx) < (unsigned)w) ||
+                        (in_g && (unsigned)(i + dy) < (unsigned)h && (unsigned)(j + dx) < (unsigned)w))
+                        met |= 1u << t;
+                }
         }
-#pragma unroll
-        for (int t = 0; t < 25; ++t) {
-#pragma unroll
-            for (int o = 16; o; o >>= 1) acc[t] += __shfl_xor_sync(0xffffffffu, acc[t], o);
-            if (lane == t) total += (double)acc[t];
-        }
+        todo &= ~__reduce_or_sync(0xffffffffu, met);
     }
-    return total;
+#pragma unroll 1
+    while (todo) {
+        const int t = __ffs(todo) - 1, dy = t / 5 - 2, dx = t % 5 - 2, i0 = dy < 0 ? -dy : 0, j0 = dx < 0 ? -dx : 0, hh = h - (dy < 0 ? -dy : dy), ww = w - (dx < 0 ? -dx : dx);
+        todo &= todo - 1;
+        double total = 0.0;
+#pragma unroll 1
+        for (int b = 0; b < g.B; ++b) {
+            const T *px = x + b * image, *pg = go + b * image;
+            float acc = 0.f;
+            if (hh > 0 && ww > 0)
+#pragma unroll 4
+                for (int e = lane; e < hh * ww; e += 32) {
+                    const int i = i0 + e / ww, j = j0 + e % ww;
+                    acc = fmaf(at(pg, i, j), at(px, i + dy, j + dx), acc);
+                }
+#pragma unroll
+            for (int o = 16; o; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+            total += (double)acc;
+        }
+        if (lane == t) sum = total;
+    }
+    return sum;
 }
 // What unfold_epilogue_kernel does, class by class, a warp each and a lane a tap (at most 25 and the bias): fixed-order fp64 sums and
 // Eq. 9.  The loaders do it when they have loaded their last unit: it hides behind that unit's other stages, where a launch of its own
@@ -441,10 +462,12 @@ __device__ __noinline__ void unfold_classes(const PGeom &g, const Parameters &p,
             for (int i = 0; i < n; ++i) acc += (double)q[(size_t)i * stride + lane];
         if (cls < 5 && __any_sync(0xffffffffu, lane < KK && !(fabs(acc) < 1e300))) {
             const size_t first = (size_t)c * g.HW;
-            const double again = taps_of_class<T>(g, static_cast<const T *>(d.x) + first, go + first, cls, lane);
-            const int pad = (5 - g.K) / 2;
-            const double mine = __shfl_sync(0xffffffffu, again, lane < KK ? (lane / g.K + pad) * 5 + lane % g.K + pad : 0);
-            if (lane < KK) acc = mine;
+            const int pad = (5 - g.K) / 2, u = lane / 5 - pad, v = lane % 5 - pad;  // (lanes are taps of 5 x 5 there)
+            const bool in = lane < 25 && u >= 0 && u < g.K && v >= 0 && v < g.K;
+            const double mine = __shfl_sync(0xffffffffu, acc, in ? u * g.K + v : 0);
+            const double again = taps_of_class<T>(g, static_cast<const T *>(d.x) + first, go + first, cls, lane, in ? mine : 0.0);
+            const double back = __shfl_sync(0xffffffffu, again, lane < KK ? (lane / g.K + pad) * 5 + lane % g.K + pad : 0);
+            if (lane < KK) acc = back;
         }
         if (lane < taps) {
             const float wv = lane < KK ? __ldg(w + lane) : __ldg(p.b0 + c), sv = __ldg(s);
@@ -870,6 +893,9 @@ bool kept_plan(const Request &q, G &out, double &cost, F find) {
     if (e.ok) { out = e.g; cost = e.cost; }
     return e.ok;
 }
+inline bool plan(const Request &q, PGeom &out, double &cost) {
+    return kept_plan(q, out, cost, [&](PGeom &g, double &c) { return search(q, g, c); });
+}
 
 template <typename T, bool FLIP, int LOAD, int KT>
 cudaError_t launch(const PGeom &g, const T *x, const Parameters &p, const Gradients &grad, T *out, char *ws, cudaStream_t st) {
@@ -892,9 +918,6 @@ cudaError_t run(const Request &q, const T *x, const Parameters &p, const Gradien
     const bool copies = copied(g);
     if (q.K == 3) return copies ? launch<T, FLIP, FEW, 3>(g, x, p, grad, out, ws, st) : launch<T, FLIP, MANY, 3>(g, x, p, grad, out, ws, st);
     return copies ? launch<T, FLIP, FEW, 5>(g, x, p, grad, out, ws, st) : launch<T, FLIP, MANY, 5>(g, x, p, grad, out, ws, st);
-}
-inline bool plan(const Request &q, PGeom &out, double &cost) {
-    return kept_plan(q, out, cost, [&](PGeom &g, double &c) { return search(q, g, c); });
 }
 
 inline int describe(const Request &q, char *buf, size_t n) {
