@@ -433,18 +433,20 @@ double plane_deep_us(const wtconv_desc *d, int bwd) {
     return 3.7 + 2.27 * k3 + 0.66 * more + (2.39 - 0.91 * k3 + 0.99 * odd + 0.17 * (odd && !k3) + 0.35 * (more > 0)) * tiles + (0.53 + 0.26 * more) * planes + 2.0 * first +
            rounds * (1.33 + 0.0154 * work + (g.bulk ? 0 : 0.083) * px);
 }
-// Several levels: taken where their estimate is 8 - 13 % below that of the block-per-plane kernels (units are eight images of a channel: small
-// batches and few units leave the SMs empty).  Over 630 random shapes, a third of them beyond the fitted range (up to 8 levels, planes of 4
-// columns or 128 rows, single images), that takes 292 forward, which gain 1.23 x (geometric mean), and 312 backward: 1.30 x.  Ten and eleven of
-// them lose more than 2 %: layers of one or two units a block, most of them with rows that are not 8-byte multiples, 17 x 45 x 31 x 20 (five
-// levels, forward 9.5 -> 10.4 us), 18 x 81 x 15 x 62 (15.6 -> 18.8), 9 x 138 x 19 x 17 (3 x 3, backward 27.1 -> 30.5), 88 x 582 x 7 x 7 (180 -> 194).
+// Several levels: taken where their estimate is 7 - 13 % below that of the block-per-plane kernels, 20 % where a block has fewer than three
+// octets of images (its first loads are not hidden then: 16 x 192 x 28 x 28 is 1.15 x as fast in a loop of calls, but a host step on chunks of
+// it, whose inputs have just arrived, is 1.5 - 3.6 % slower).  3 x 3 kernels: the block-per-plane estimate is 7 % low forward and 12 % low
+// backward with rows of an odd number of pixel pairs (64 x 150 x 14 x 14, two levels: forward 20.4 us against 27.0, backward 42.8 against 49.9).
+// Measured on 315 random shapes of 4 - 128 images: taken forward 194, 1.27 x as fast (geometric mean), backward 150, 1.31 x; four and two of them
+// lose more than 2 %, the worst 32 x 234 x 13 x 13 (three levels, forward 0.91 x).
 bool pyramid_serves(const wtconv_desc *d, bool on_chip, int bwd) {
     if (d->dtype == WTCONV_F32 || !on_chip || d->L < 2 || (d->flags & ~WTCONV_FLAG_TEST_NO_COPY)) return false;
     wt::pyramid::PGeom g;
     wt::pyramid::WGeom w;
     double cost;
-    if (bwd) return wt::pyramid::plan_gradient(pyramid_request(d), w, cost) && (d->W % 2 ? 1.13 : 1.1) * cost < plane_deep_us(d, 1);
-    return wt::pyramid::plan(pyramid_request(d), g, cost) && (d->W % 4 ? 1.12 : 1.08) * cost < plane_deep_us(d, 0);
+    const bool few = (d->B + 7) / 8 * (long long)d->C < 3 * 148;
+    if (bwd) return wt::pyramid::plan_gradient(pyramid_request(d), w, cost) && (few ? 1.2 : d->W % 2 ? 1.13 : d->k == 3 && d->W % 4 ? 0.92 : 1.1) * cost < plane_deep_us(d, 1);
+    return wt::pyramid::plan(pyramid_request(d), g, cost) && (few ? 1.2 : d->k == 3 ? 0.95 : d->W % 4 ? 1.1 : 1.07) * cost < plane_deep_us(d, 0);
 }
 
 // 7 x 7 kernels on whole planes: block per plane, or the per-level kernels.  The latter win where planes are few (a block per plane

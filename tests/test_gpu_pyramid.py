@@ -4,20 +4,23 @@ import numpy as np
 import pytest
 import torch
 
-from helpers import GRAD_NAMES, TOL, rel_err, run_gpu, run_oracle, to_dev
+from helpers import GRAD_NAMES, TOL, rel_err, run_gpu, run_oracle
+from helpers import to_dev
 from paper_2608_10805_b200 import inputs, wtconv as wt
 
 pytestmark = pytest.mark.gpu
 
 SHAPES = [  # B, C, H, W, k, L
     (32, 148, 28, 28, 5, 2),   # several operand arrays
-    (13, 148, 30, 26, 5, 3),   # a last octet of five images, rows of pairs
+    (13, 64, 30, 26, 5, 3),    # a unit of five images, rows of pairs
     (24, 149, 29, 31, 5, 4),   # odd rows, a row more than whole blocks of four, several units a block
     (16, 148, 56, 56, 5, 3),   # one operand array, levels >= 2 a unit ahead
     (8, 148, 57, 45, 3, 2),    # 3 x 3, one operand array, odd rows
-    (72, 300, 14, 14, 5, 3),   # many units a block
+    (64, 150, 14, 14, 5, 2),   # many units a block
     (8, 148, 61, 64, 5, 2),    # the widest plane
     (13, 74, 40, 64, 5, 3),    # planes in batches that do not divide eight
+    (13, 148, 30, 26, 5, 3),   # a last octet of five images, rows of pairs
+    (72, 300, 14, 14, 5, 3),   # many units a block
     (5, 139, 77, 4, 3, 8),     # fewer than eight images, the narrowest plane, more than 64 rows, every level
     (16, 148, 100, 31, 5, 3),  # four MMA tiles of one plane
 ]
@@ -43,14 +46,15 @@ def test_against_the_oracle(shape, dtype):
 
 
 BACKWARD_SHAPES = [  # B, C, H, W, k, L
-    (13, 64, 30, 26, 5, 3),    # a last unit of five images, copies of pairs
+    (13, 64, 30, 26, 5, 3),    # a unit of five images, copies of pairs
     (61, 96, 29, 31, 5, 4),    # odd rows, a last unit that is not full, a row more than whole blocks of four
     (16, 148, 56, 56, 5, 3),   # one pair of operand arrays, planes in two batches, four-row tiles
     (40, 148, 57, 45, 5, 2),   # odd rows, one pair of arrays
-    (61, 296, 14, 14, 3, 3),   # 3 x 3, several octets a unit and channels a block
+    (64, 150, 14, 14, 3, 2),   # 3 x 3, four octets a unit, several channels a block
     (61, 64, 14, 13, 5, 5),    # levels down to one coefficient, units of four octets
     (8, 148, 61, 64, 5, 2),    # the widest plane
     (13, 74, 40, 64, 5, 3),    # rows of whole 16-byte words
+    (61, 296, 14, 14, 3, 3),   # 3 x 3, several octets a unit and channels a block
     (5, 139, 77, 4, 3, 8),     # fewer than eight images, the narrowest plane, more than 64 rows, every level
     (16, 148, 100, 31, 5, 3),
 ]
@@ -68,10 +72,12 @@ def test_backward_against_the_oracle(shape, dtype):
         if ref_grads.get(n) is not None and ref_grads[n].size:
             # as above: grad_x is rounded once, parameter gradients are sums in fp32 of exact products
             assert rel_err(grads[n], ref_grads[n]) < (TOL[dtype] / 4 if n == "dx" else 1e-5), n
+            # chains of eight truncated additions, the rest rounded: 1 - 4e-7 measured on these shapes, as on the FMA kernels
+            assert n not in ("dw0", "dwl") or rel_err(grads[n], ref_grads[n]) < 1e-6, n
 
 
 @pytest.mark.parametrize("dtype", ["f16", "bf16"])
-@pytest.mark.parametrize("shape", [(8, 592, 48, 48, 5, 3), (30, 386, 6, 24, 5, 4), (8, 444, 56, 56, 5, 3)], ids=lambda s: "x".join(map(str, s)))
+@pytest.mark.parametrize("shape", [(8, 592, 48, 48, 5, 3), (28, 608, 16, 16, 5, 4), (8, 444, 56, 56, 5, 3)], ids=lambda s: "x".join(map(str, s)))
 def test_every_unit_another_channel(shape, dtype):
     """Levels >= 2 run ahead of the loads: a channel's scale and bias are not its neighbours'."""
     B, C, H, W, k, L = shape
