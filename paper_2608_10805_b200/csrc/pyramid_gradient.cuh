@@ -14,6 +14,9 @@
 // two levels, 229 -> 132; 64 x 192 x 28 x 28, four levels, 145 -> 95.  What bounds it now, by time stamps of the roles: where one pair
 // of arrays fills an SM (56 x 56) a unit's copies (5300 of 18600 cycles, 16 a copy instruction), its two analyses (4400 and 2900) and
 // the first batch's tiles (2700) follow one another; with several pairs (28 x 28) the deep warps' passes do (two of 4500 cycles).
+// Relative error of the weight gradients against fp64 (2-norm; base, all levels; in brackets the block-per-plane kernels): 128 x 96 x 56 x 56
+// bf16 1.6e-7, 2.0e-7 (3.3e-7, 5.7e-7), f16 2.1e-7, 2.3e-7 (6.5e-7, 5.8e-7); 128 x 192 x 28 x 28 bf16 1.4e-7, 1.5e-7 (2.4e-7, 4.3e-7),
+// f16 2.0e-7, 2.0e-7 (4.9e-7, 4.5e-7); over 20 smaller shapes 0.8 - 2.1e-7 (0.9 - 3.5e-7), no entry off by more than 3.6e-7 of the largest.
 // Eight loader warps instead of four left 72 registers a thread: 254 -> 272 us.  One launch for this and grad_x's kernel, block by
 // block, 250 -> 264: the second's set-up is no longer hidden.
 #pragma once
