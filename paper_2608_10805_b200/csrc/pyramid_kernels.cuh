@@ -912,9 +912,9 @@ cudaError_t run(const Request &q, const T *x, const Parameters &p, const Gradien
     g.tag = tag;
     g.alarm = call_alarm;
     g.no_copy = no_copy;
-    // Four warps that issue asynchronous copies leave the other roles 16 more registers a thread (88), but are slower than eight that load through
-    // registers where units are small: forward, 128 x 96 x 56 x 56 (3136 pixels an image and octet) 126 -> 121 us, 128 x 192 x 28 x 28
-    // (1568) 68.2 -> 62.9; 64 x 192 x 28 x 28 with four levels (784) 48.0 -> 49.3, 16 x 64 x 14 x 14 8.9 -> 9.5.
+    // Four warps that issue asynchronous copies (80 registers a thread; 72 with eight) are slower than eight that load through registers where
+    // units are small: forward, 128 x 96 x 56 x 56 (3136 pixels an image and octet) 126 -> 121 us, 128 x 192 x 28 x 28 (1568) 68.2 -> 62.9;
+    // 64 x 192 x 28 x 28 with four levels (784) 48.0 -> 49.3, 16 x 64 x 14 x 14 8.9 -> 9.5.  Nothing was measured between 784 and 1568.
     const bool copies = copied(g);
     if (q.K == 3) return copies ? launch<T, FLIP, FEW, 3>(g, x, p, grad, out, ws, st) : launch<T, FLIP, MANY, 3>(g, x, p, grad, out, ws, st);
     return copies ? launch<T, FLIP, FEW, 5>(g, x, p, grad, out, ws, st) : launch<T, FLIP, MANY, 5>(g, x, p, grad, out, ws, st);
